@@ -373,21 +373,18 @@ const char *fpsa_last_error(const fpsa_ctx *ctx);
  *   h [K], sigma_t [K]          cell widths and total cross sections
  *   q [K][2][N]                 nodal ANGULAR source (values at the ordinates)
  *   psi [K][2][N]               output angular flux
- * The per-(cell, ordinate) coefficient scratch lives in a fixed __device__
- * array of FPSA_SWEEP_NOALLOC_MAX_CELL_ANGLES x 6 doubles (6.3 MB) that every GPU
- * loading the library holds until the process exits; no call allocates device
- * memory. K * N above that limit, or N > 256, returns FPSA_ENOTSUP; malformed
+ * The call is one kernel launch that uses no scratch in device memory (the
+ * coefficients stay in registers, the maps of the cell chunks in shared memory), so
+ * calls on several streams are independent. K * N above
+ * FPSA_SWEEP_NOALLOC_MAX_CELL_ANGLES, or N > 256, returns FPSA_ENOTSUP; malformed
  * arguments return FPSA_EINVAL; a refused launch returns FPSA_ECUDA (the launch's
  * own status: an error left pending by earlier, unrelated work is not cleared).
  * Work is enqueued on `stream` (cudaStream_t, NULL = legacy default) and the
  * call returns without synchronising. The first call on a device does a one-time
- * set-up with that device current: it looks up the arrays' device addresses and
- * copies the ordinate tables of every even N <= 256 into a second fixed array
- * (a synchronous copy); make that first call before any stream capture. Later
- * calls copy nothing from host memory. All calls share the one scratch array and
- * leave their coefficients in it (each call rewrites every coefficient it reads
- * before the sweep): calls whose work overlaps on the GPU (e.g. on two streams)
- * race and must be serialised by the caller.
+ * set-up with that device current: it looks up the address of a fixed array and
+ * copies the ordinate tables of every even N <= 256 into it (a synchronous copy);
+ * make that first call before any stream capture. Later calls copy nothing from
+ * host memory.
  */
 #define FPSA_SWEEP_NOALLOC_MAX_CELL_ANGLES 131072
 int fpsa_sweep_noalloc(int32_t n_ordinates, int32_t n_cells, const double *h, const double *sigma_t,

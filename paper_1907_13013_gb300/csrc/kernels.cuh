@@ -61,22 +61,20 @@ __global__ void k_sweep_coef(const double *__restrict__ mu, const double *__rest
 }
 
 // ---------------------------------------------------------------------------
-// Transport sweep L psi = q (Eq. trsi / Eq. predict), one block per
-// (ordinate, instance, rhs). The sequential recurrence over cells
-// x_{k+1} = alpha_k x_k + beta_k (x = outflow of cell k, beta_k its outflow
-// for zero inflow) is an affine map per cell; affine maps compose
-// associatively, so each thread composes the maps of a contiguous chunk of
-// cells (pass 1), the block scans the chunk maps (warp shuffles, then across
-// warps), and each thread re-sweeps its chunk from the exact inflow (pass 2).
+// Transport sweep L psi = q (Eq. trsi / Eq. predict). The sequential recurrence
+// over cells x_{k+1} = alpha_k x_k + beta_k (x = outflow of cell k, beta_k its
+// outflow for zero inflow) is an affine map per cell; affine maps compose
+// associatively, so chunks of cells are composed independently, the chunk maps are
+// combined, and each chunk is swept again from its exact inflow.
 //
 // Edge inflow x0 of ordinate n (upwind edge s: left for mu > 0):
 //   vacuum edge       x0 = psi_inc[r][b][s][n] (given incoming flux; 0 if none)
 //   reflective edge   x0 = outflow at s of the mirror ordinate n' = N-1-n. With the
-//                     whole-slab maps x -> A x + E of n and n' for zero inflow
-//                     (the totals pass, kTotals = true, writes them to tot), this is
-//                     A' x0' + E' with x0' the inflow of n' at the far edge: its
-//                     given flux, or, if that edge reflects too, A x0 + E, so that
-//                     x0 = (A' E + E') / (1 - A A')  (|A A'| < 1 for sigma_t > 0).
+//                     whole-slab maps x -> A x + E of n and n' for zero inflow,
+//                     this is A' x0' + E' with x0' the inflow of n' at the far edge:
+//                     its given flux, or, if that edge reflects too, A x0 + E, so
+//                     that x0 = (A' E + E') / (1 - A A')  (|A A'| < 1 for
+//                     sigma_t > 0).
 // The mirror-ordinate coupling is thus exact per sweep (no lagged edge values).
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -93,141 +91,16 @@ constexpr int32_t kBcReflect = 1;
 
 constexpr int kSweepBatch = 8;  // cells whose inputs one thread requests together
 
-template <typename T, int NT, bool kTotals = false>
-__global__ void __launch_bounds__(NT) k_sweep(const T *__restrict__ q, T *__restrict__ psi,
-                                              const T *__restrict__ coef, const double *__restrict__ mu,
-                                              const int32_t *__restrict__ off, const int32_t *__restrict__ Kc,
-                                              int N, int sumK, const T *__restrict__ psi_inc = nullptr,
-                                              const int32_t *__restrict__ bc = nullptr, T *__restrict__ tot = nullptr) {
-    __shared__ Affine<T> warp_tot[NT / 32];
-    const int n = blockIdx.x, b = blockIdx.y, r = blockIdx.z, B = gridDim.y;
-    const int K = Kc[b], o = off[b];
-    const bool fwd = mu[n] > 0.0;
-    const int nu_ = fwd ? 0 : 1, nd_ = 1 - nu_;
-    const int chunk = (K + NT - 1) / NT;
-    const int p0 = min((int)threadIdx.x * chunk, K), p1 = min(p0 + chunk, K);
-    const size_t base = ((size_t)r * sumK + o) * 2 * N + n;
-    const T *qb = q + base;
-    T *pb_ = psi + base;
-    const T *cb = coef + (size_t)o * 6 * N + n;
-
-    // pass 1: the chunk's affine map, inputs requested kSweepBatch cells at a time
-    // (all loads of a batch in flight together, then the dependent recurrence)
-    Affine<T> m{T(1), T(0)};
-    for (int pb = p0; pb < p1; pb += kSweepBatch) {
-        T qu[kSweepBatch], qd[kSweepBatch], al[kSweepBatch], gdu[kSweepBatch], gdd[kSweepBatch];
-#pragma unroll
-        for (int t = 0; t < kSweepBatch; ++t) {
-            const int p = pb + t;
-            if (p < p1) {
-                const int c = fwd ? p : K - 1 - p;
-                const T *cc = cb + (size_t)c * 6 * N;
-                qu[t] = qb[(size_t)(2 * c + nu_) * N];
-                qd[t] = qb[(size_t)(2 * c + nd_) * N];
-                al[t] = cc[0];
-                gdu[t] = cc[4 * N];
-                gdd[t] = cc[5 * N];
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < kSweepBatch; ++t)
-            if (pb + t < p1) {
-                m.b = al[t] * m.b + (gdu[t] * qu[t] + gdd[t] * qd[t]);
-                m.a = al[t] * m.a;
-            }
-    }
-    // inclusive scan over the block (thread order = sweep order)
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    Affine<T> inc = m;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        T pa = __shfl_up_sync(0xffffffffu, inc.a, d);
-        T pbv = __shfl_up_sync(0xffffffffu, inc.b, d);
-        if (lane >= d) inc = compose(Affine<T>{pa, pbv}, inc);
-    }
-    if (lane == 31) warp_tot[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        Affine<T> t = (lane < NT / 32) ? warp_tot[lane] : Affine<T>{T(1), T(0)};
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            T pa = __shfl_up_sync(0xffffffffu, t.a, d);
-            T pbv = __shfl_up_sync(0xffffffffu, t.b, d);
-            if (lane >= d) t = compose(Affine<T>{pa, pbv}, t);
-        }
-        if (lane < NT / 32) warp_tot[lane] = t;  // inclusive prefix over warps
-    }
-    __syncthreads();
-    if (kTotals) {
-        if (threadIdx.x == 0) {
-            const Affine<T> t = warp_tot[NT / 32 - 1];
-            T *o = tot + (((size_t)r * B + b) * N + n) * 2;
-            o[0] = t.a;
-            o[1] = t.b;
-        }
-        return;
-    }
-    // inflow at the upwind edge
-    const int s = fwd ? 0 : 1;
-    const size_t ib = (size_t)r * B + b;
-    T x0 = psi_inc ? psi_inc[(ib * 2 + s) * N + n] : T(0);
-    if (bc && bc[2 * b + s] == kBcReflect) {
-        const int nm = N - 1 - n;
-        const T *tn = tot + (ib * N + n) * 2, *tm = tot + (ib * N + nm) * 2;
-        if (bc[2 * b + 1 - s] == kBcReflect) {
-            x0 = (tm[0] * tn[1] + tm[1]) / (T(1) - tn[0] * tm[0]);
-        } else {
-            const T far = psi_inc ? psi_inc[(ib * 2 + 1 - s) * N + nm] : T(0);
-            x0 = tm[0] * far + tm[1];
-        }
-    }
-    // exclusive prefix for this thread, applied to the inflow x0
-    T before_warp = (wid > 0) ? warp_tot[wid - 1].a * x0 + warp_tot[wid - 1].b : x0;
-    T inc_b_full = inc.a * before_warp + inc.b;  // inclusive, thread-level
-    T x = __shfl_up_sync(0xffffffffu, inc_b_full, 1);
-    if (lane == 0) x = before_warp;
-
-    // pass 2: re-sweep the chunk from its exact inflow, in batches as in pass 1
-    for (int pb = p0; pb < p1; pb += kSweepBatch) {
-        T qu[kSweepBatch], qd[kSweepBatch], cf[6][kSweepBatch];
-#pragma unroll
-        for (int t = 0; t < kSweepBatch; ++t) {
-            const int p = pb + t;
-            if (p < p1) {
-                const int c = fwd ? p : K - 1 - p;
-                const T *cc = cb + (size_t)c * 6 * N;
-                qu[t] = qb[(size_t)(2 * c + nu_) * N];
-                qd[t] = qb[(size_t)(2 * c + nd_) * N];
-#pragma unroll
-                for (int k = 0; k < 6; ++k) cf[k][t] = cc[(size_t)k * N];
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < kSweepBatch; ++t) {
-            const int p = pb + t;
-            if (p < p1) {
-                const int c = fwd ? p : K - 1 - p;
-                // cf: 0 alpha, 1 a_u, 2 G_uu, 3 G_ud, 4 G_du, 5 G_dd
-                const T pu = cf[2][t] * qu[t] + cf[3][t] * qd[t] + cf[1][t] * x;
-                const T pd = cf[4][t] * qu[t] + cf[5][t] * qd[t] + cf[0][t] * x;
-                pb_[(size_t)(2 * c + nu_) * N] = pu;
-                pb_[(size_t)(2 * c + nd_) * N] = pd;
-                x = pd;
-            }
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
-// Segmented transport sweep (the same recurrence, maps and edge inflows as
-// k_sweep), laid out for coalesced access: a block holds 32 ordinates of one
+// Segmented transport sweep (the recurrence, maps and edge inflows above), laid
+// out for coalesced access: a block holds 32 ordinates of one
 // direction in its lanes (consecutive n: one 128-byte line per cell value) and
 // kSegWarps chunks of cpt consecutive cells (in sweep order) in its warps, so a
 // segment covers kSegWarps * cpt cells and a (direction, 32-ordinate group,
 // instance, rhs) is swept by nseg blocks along the slab (nseg <= kSegMax):
 //   k_sweep_maps   each chunk's affine map (x -> a x + b for the chunk's outflow)
 //                  and their composition over the segment, written per ordinate;
-//   k_sweep_apply  the segment's inflow: the edge inflow (as in k_sweep, the
+//   k_sweep_apply  the segment's inflow: the edge inflow (above; the
 //                  whole-slab maps of n and of its mirror composed from all
 //                  segment maps at a reflective edge) carried through the maps of
 //                  the segments before it, then through the chunk maps before

@@ -839,149 +839,6 @@ __global__ void k_bcr_invert(T *__restrict__ A, const BcrItem *__restrict__ item
     gj_smem_body(Ag, n2, Ag, n2, true, n2, growth, status);
 }
 
-// Register-tiled Gauss-Jordan inversion for n2 = 2N in {32, 64, 128}: 16 warps;
-// warp w owns the columns w + 16 j (j < n2/16), lane t the rows t + 32 i
-// (i < n2/32), so every thread holds an (n2/32) x (n2/16) tile in registers and
-// column k lives in one warp. Pivoting is implicit: step k picks, among rows not
-// yet used, the row p_k of largest |a[p][k]| (partial pivoting without moving
-// rows; the comparison key is |a| rounded to FP32). The in-place update is the
-// usual one with row p_k as pivot row; at the end the array X holds
-// A^{-1}[r][c] = X[p_r][q_c] with q the inverse of p (row p_k carries step k's
-// identity column). Written back transposed.
-//
-// One block barrier per step: the pivot row reaches the other lanes of each warp
-// by shuffles (every warp holds all rows of its columns), only column k goes
-// through shared memory, and the warp owning column k+1 updates that column first
-// and picks pivot k+1 (look-ahead) while the other warps are still updating.
-// Body shared by the in-place kernel and the strided sub-block variant: src / dst
-// are N2 x N2 row-major with leading dimensions lds / ldd; transposed output when
-// tout; growth may be NULL.
-template <typename T, int RI>
-__device__ __forceinline__ void gj_pick_pivot(const T (&colv)[RI], unsigned used, int lane, int &p) {
-    // key 0: no candidate; else the FP32 bits of |v| plus one (|v| >= 0 orders as unsigned)
-    unsigned best = 0u;
-    int bi = 0;
-#pragma unroll
-    for (int i = 0; i < RI; ++i) {
-        const unsigned key = (used >> i) & 1u ? 0u : __float_as_uint(fabsf((float)colv[i])) + 1u;
-        if (key > best) { best = key; bi = lane + 32 * i; }
-    }
-    const unsigned m = __reduce_max_sync(0xffffffffu, best);
-    const unsigned who = __ballot_sync(0xffffffffu, best == m);
-    p = __shfl_sync(0xffffffffu, bi, __ffs(who) - 1);
-}
-
-// rv[j] = (row ip of lane pl's register tile)[j] * inv, broadcast to the warp by
-// shuffles; ip and pl are warp-uniform, so the row is chosen by a branch.
-template <typename T, int RI, int CJ>
-__device__ __forceinline__ void gj_pivot_row(const T (&x)[RI][CJ], int ip, int pl, T inv, T (&rv)[CJ]) {
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-        if (i == ip) {
-#pragma unroll
-            for (int j = 0; j < CJ; ++j) rv[j] = __shfl_sync(0xffffffffu, x[i][j], pl) * inv;
-        }
-}
-
-// x[I][j] = rv[j] for every j except jskip (the look-ahead column, already set).
-template <typename T, int RI, int CJ, int I>
-__device__ __forceinline__ void gj_set_row_i(T (&x)[RI][CJ], const T (&rv)[CJ], int jskip) {
-    if constexpr (I < RI) {
-#pragma unroll
-        for (int j = 0; j < CJ; ++j)
-            if (j != jskip) x[I][j] = rv[j];
-    }
-}
-
-template <typename T, int RI, int CJ>
-__device__ __forceinline__ void gj_set_row_elem(T (&x)[RI][CJ], int ip, int j, T val) {
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-        if (i == ip) x[i][j] = val;
-}
-
-template <typename T, int N2>
-struct GjShared {
-    T (*colbuf)[N2];
-    int *s_p, *perm, *iperm;
-};
-
-// One elimination step k = 16 JK + wk with the look-ahead column register JN
-// (JN = CJ: no look-ahead, the last step).
-template <typename T, int N2, int JK, int JN>
-__device__ __forceinline__ void gj_step(T (&x)[N2 / 32][N2 / 16], const GjShared<T, N2> &sh, unsigned &used,
-                                        bool &bad, int lane, int w, int wk) {
-    constexpr int RI = N2 / 32, CJ = N2 / 16;
-    const int k = 16 * JK + wk, b = k & 1;
-    const int p = sh.s_p[b];
-    const T pv = sh.colbuf[b][p];
-    if (pv == T(0) || !isfinite(pv)) bad = true;
-    const T inv = __frcp_rn(pv);  // correctly rounded, as 1 / pv
-    const int ip = p >> 5, pl = p & 31;
-    if (lane == pl) used |= 1u << ip;
-    T f[RI], rv[CJ];
-#pragma unroll
-    for (int i = 0; i < RI; ++i) f[i] = sh.colbuf[b][lane + 32 * i];
-    gj_pivot_row<T, RI, CJ>(x, ip, pl, inv, rv);  // pivot row of this warp's columns, from lane pl
-    if (w == wk) {  // column k: its old value is replaced, not updated
-        rv[JK] = inv;
-#pragma unroll
-        for (int i = 0; i < RI; ++i) x[i][JK] = T(0);
-    }
-    bool ahead = false;
-    if constexpr (JN < CJ) {
-        ahead = w == ((wk + 1) & 15);
-        if (ahead) {
-            // look-ahead: update column k+1 now and pick pivot k+1
-            T colv[RI];
-#pragma unroll
-            for (int i = 0; i < RI; ++i) x[i][JN] = fma(-f[i], rv[JN], x[i][JN]);
-            if (lane == pl) gj_set_row_elem<T, RI, CJ>(x, ip, JN, rv[JN]);
-#pragma unroll
-            for (int i = 0; i < RI; ++i) {
-                colv[i] = x[i][JN];
-                sh.colbuf[b ^ 1][lane + 32 * i] = colv[i];
-            }
-            int pn;
-            gj_pick_pivot<T, RI>(colv, used, lane, pn);
-            if (lane == 0) {
-                sh.s_p[b ^ 1] = pn;
-                sh.perm[k + 1] = pn;
-                sh.iperm[pn] = k + 1;
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < CJ; ++j) {
-        if (j == JN && ahead) continue;
-#pragma unroll
-        for (int i = 0; i < RI; ++i) x[i][j] = fma(-f[i], rv[j], x[i][j]);
-    }
-    // the pivot row becomes the scaled row (its own update used f = pv)
-    if (lane == pl) {
-        const int js = ahead ? JN : -1;
-        switch (ip) {
-            case 0: gj_set_row_i<T, RI, CJ, 0>(x, rv, js); break;
-            case 1: gj_set_row_i<T, RI, CJ, 1>(x, rv, js); break;
-            case 2: gj_set_row_i<T, RI, CJ, 2>(x, rv, js); break;
-            default: gj_set_row_i<T, RI, CJ, 3>(x, rv, js); break;
-        }
-    }
-    __syncthreads();
-}
-
-// All steps with column register JK (k = 16 JK .. 16 JK + 15), then JK + 1.
-template <typename T, int N2, int JK>
-__device__ __forceinline__ void gj_steps(T (&x)[N2 / 32][N2 / 16], const GjShared<T, N2> &sh, unsigned &used,
-                                         bool &bad, int lane, int w) {
-    constexpr int CJ = N2 / 16;
-    if constexpr (JK < CJ) {
-        for (int wk = 0; wk < 15; ++wk) gj_step<T, N2, JK, JK>(x, sh, used, bad, lane, w, wk);
-        gj_step<T, N2, JK, JK + 1>(x, sh, used, bad, lane, w, 15);
-        gj_steps<T, N2, JK + 1>(x, sh, used, bad, lane, w);
-    }
-}
-
 // One row of CJ values to / from shared memory in 16-byte (CJ % 4 == 0) or 8-byte vectors.
 template <int CJ>
 __device__ __forceinline__ void gj_st_row(float *d, const float (&v)[CJ]) {
@@ -1195,16 +1052,49 @@ __device__ __forceinline__ void gj_panel_body(const float *src, int lds, float *
     if (bad) atomicExch(status, 1);
 }
 
+// x[i] of the warp-uniform row register i (select chain: registers take no run-time index).
+template <int RI>
+__device__ __forceinline__ double gj_pick(const double (&x)[RI], int i) {
+    double v = x[0];
+#pragma unroll
+    for (int k = 1; k < RI; ++k) v = (i == k) ? x[k] : v;
+    return v;
+}
+
+// Register-tiled Gauss-Jordan inversion (FP64) for n2 = N2 in {32, 64, 128}: 16 warps;
+// warp w owns the columns w + 16 j (j < N2/16), lane t the rows t + 32 i (i < N2/32),
+// so every thread holds an (N2/32) x (N2/16) tile in registers and column k lives in one
+// warp. Pivoting is implicit: step k picks, among rows not yet used, the row p_k of
+// largest |a[p][k]| (partial pivoting without moving rows; magnitudes compared to 13
+// mantissa bits, the row index in the key's low 7 bits, so one warp reduction picks it).
+//
+// The elimination leaves the pivot rows unscaled: with f[r] = x[r][k] / pivot (0 in the
+// pivot row), X -= f (x) X[p_k][:], where column k first becomes the unit column of p_k;
+// row p_k is divided by its pivot once, at the end. At the end the array X holds
+// A^{-1}[r][c] = X[p_r][q_c] / pivot_r with q the inverse of p. Written back transposed.
+//
+// What bounds it is FP64 arithmetic (two FP64 FMAs a clock and SM: the N2^2 of a step
+// take 4.2 us at N2 = 128), so everything but those FMAs runs once per step, in the warp
+// that owns column k + 1: it updates that column first (look-ahead), picks pivot k + 1 and
+// publishes f, while the other warps still update. Scaling the pivot row and dividing by
+// the pivot in every warp instead took 17 FP64 instructions a step and warp beside the 32
+// FMAs (2000 cells of N2 = 128, all levels: 18.8 ms, now 14.5; 100 cells of N2 = 64: 1.57
+// ms, now 1.03; 200 cells of N2 = 32: 0.55 ms, now 0.33).
+// One block barrier per step: the pivot row reaches the lanes of each warp by shuffles.
+// Body shared by the in-place kernel and the strided sub-block variant: src / dst
+// are N2 x N2 row-major with leading dimensions lds / ldd; transposed output when
+// tout; growth may be NULL.
 template <typename T, int N2>
 __device__ __forceinline__ void gj_reg_body(const T *src, int lds, T *dst, int ldd, bool tout,
                                             unsigned long long *__restrict__ growth, int *__restrict__ status) {
+    static_assert(sizeof(T) == 8 && N2 <= 128, "FP64; the row index must fit the key's 7 bits");
     constexpr int RI = N2 / 32, CJ = N2 / 16;
-    __shared__ T colbuf[2][N2];
+    __shared__ T colbuf[2][N2], rinv[N2];
     __shared__ int s_p[2], perm[N2], iperm[N2];
     __shared__ double s_red[16];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     T x[RI][CJ];
-    T amax = T(0);  // growth bookkeeping in T (FP64 only for the final product)
+    T amax = T(0);
 #pragma unroll
     for (int i = 0; i < RI; ++i)
 #pragma unroll
@@ -1214,112 +1104,88 @@ __device__ __forceinline__ void gj_reg_body(const T *src, int lds, T *dst, int l
         }
     unsigned used = 0u;  // bit i: row lane + 32 i has been a pivot row
     bool bad = false;
-    if (w == 0) {  // pivot of step 0 (column 0 = x[.][0] of warp 0)
-        T colv[RI];
+    // the owner of column k: pick pivot k among the rows not yet used, publish f and the pivot
+    auto publish = [&](int k, const T (&colv)[RI]) {
+        unsigned best = 0u;
 #pragma unroll
         for (int i = 0; i < RI; ++i) {
-            colv[i] = x[i][0];
-            colbuf[0][lane + 32 * i] = colv[i];
+            const unsigned mag = ((unsigned)__double2hiint(colv[i]) & 0x7fffff80u) + 0x80u;
+            best = max(best, (used >> i) & 1u ? 0u : (mag | (unsigned)(lane + 32 * i)));
         }
-        int pn;
-        gj_pick_pivot<T, RI>(colv, used, lane, pn);
+        const int p = (int)(__reduce_max_sync(0xffffffffu, best) & 127u);
+        const T pv = __shfl_sync(0xffffffffu, gj_pick<RI>(colv, p >> 5), p & 31);
+        if (pv == T(0) || !isfinite(pv)) bad = true;
+        const T inv = T(1) / pv;
+#pragma unroll
+        for (int i = 0; i < RI; ++i) colbuf[k & 1][lane + 32 * i] = (lane + 32 * i == p) ? T(0) : colv[i] * inv;
         if (lane == 0) {
-            s_p[0] = pn;
-            perm[0] = pn;
-            iperm[pn] = 0;
+            s_p[k & 1] = p;
+            rinv[p] = inv;
+            perm[k] = p;
+            iperm[p] = k;
         }
+    };
+    if (w == 0) {
+        T colv[RI];
+#pragma unroll
+        for (int i = 0; i < RI; ++i) colv[i] = x[i][0];
+        publish(0, colv);
     }
     __syncthreads();
-    // step k = 16 JK + wk: column k is x[.][JK] of warp wk. JK is a compile-time index
-    // (the loop over it is unrolled) so the owner's and the look-ahead column's
-    // registers are addressed statically; the look-ahead column is JK (wk < 15) or
-    // JK + 1 (wk = 15).
-    // (FP32; the FP64 tile is register-bound, so there the loop stays rolled)
-    if constexpr (sizeof(T) == 4) {
-        GjShared<T, N2> sh{colbuf, s_p, perm, iperm};
-        gj_steps<T, N2, 0>(x, sh, used, bad, lane, w);
-    } else {
-        for (int k = 0; k < N2; ++k) {
-            const int b = k & 1;
-            const int p = s_p[b];
-            const T pv = colbuf[b][p];
-            if (pv == T(0) || !isfinite(pv)) bad = true;
-            const T inv = T(1) / pv;
-            const int ip = p >> 5, pl = p & 31;
-            if (lane == pl) used |= 1u << ip;
-            T f[RI], rv[CJ];
-    #pragma unroll
-            for (int i = 0; i < RI; ++i) f[i] = colbuf[b][lane + 32 * i];
-            // pivot row values of this warp's columns, from lane pl
-            gj_pivot_row<T, RI, CJ>(x, ip, pl, inv, rv);
-            const bool own = w == (k & 15);
-            const int jk = k >> 4;
-            if (own) {  // column k: its old value is replaced, not updated
-    #pragma unroll
-                for (int j = 0; j < CJ; ++j)
-                    if (j == jk) {
-                        rv[j] = inv;
-    #pragma unroll
-                        for (int i = 0; i < RI; ++i) x[i][j] = T(0);
-                    }
+    for (int k = 0; k < N2; ++k) {
+        const int p = s_p[k & 1], ip = p >> 5, pl = p & 31;
+        if (lane == pl) used |= 1u << ip;
+        T f[RI];
+#pragma unroll
+        for (int i = 0; i < RI; ++i) f[i] = colbuf[k & 1][lane + 32 * i];
+        const int jk = w == (k & 15) ? k >> 4 : -1;                         // column k, if this warp's
+        const int jn = k + 1 < N2 && w == ((k + 1) & 15) ? (k + 1) >> 4 : -1;  // column k + 1
+        // X[:][j] -= f X[p][j]; column k first becomes the unit column of the pivot row
+        auto update = [&](int j) {
+            T col[RI];
+#pragma unroll
+            for (int i = 0; i < RI; ++i) col[i] = x[i][j];
+            T xp = __shfl_sync(0xffffffffu, gj_pick<RI>(col, ip), pl);
+            if (j == jk) {
+                xp = T(1);
+#pragma unroll
+                for (int i = 0; i < RI; ++i) col[i] = (lane + 32 * i == p) ? T(1) : T(0);
             }
-            const bool ahead = k + 1 < N2 && w == ((k + 1) & 15);
-            const int jn = (k + 1) >> 4;
-            if (ahead) {
-                // look-ahead: update column k+1 now and pick pivot k+1
-                T colv[RI];
-    #pragma unroll
-                for (int j = 0; j < CJ; ++j)
-                    if (j == jn) {
-    #pragma unroll
-                        for (int i = 0; i < RI; ++i) x[i][j] = fma(-f[i], rv[j], x[i][j]);
-                        if (lane == pl) gj_set_row_elem<T, RI, CJ>(x, ip, j, rv[j]);
-    #pragma unroll
-                        for (int i = 0; i < RI; ++i) colv[i] = x[i][j];
-                    }
-    #pragma unroll
-                for (int i = 0; i < RI; ++i) colbuf[b ^ 1][lane + 32 * i] = colv[i];
-                int pn;
-                gj_pick_pivot<T, RI>(colv, used, lane, pn);
-                if (lane == 0) {
-                    s_p[b ^ 1] = pn;
-                    perm[k + 1] = pn;
-                    iperm[pn] = k + 1;
+#pragma unroll
+            for (int i = 0; i < RI; ++i) x[i][j] = fma(-f[i], xp, col[i]);
+        };
+        if (jn >= 0) {
+            T colv[RI];
+#pragma unroll
+            for (int j = 0; j < CJ; ++j)
+                if (j == jn) {
+                    update(j);
+#pragma unroll
+                    for (int i = 0; i < RI; ++i) colv[i] = x[i][j];
                 }
-            }
-    #pragma unroll
-            for (int j = 0; j < CJ; ++j) {
-                if (ahead && j == jn) continue;
-    #pragma unroll
-                for (int i = 0; i < RI; ++i) x[i][j] = fma(-f[i], rv[j], x[i][j]);
-            }
-            // the pivot row becomes the scaled row (its own update used f = pv)
-            if (lane == pl) {
-                const int js = ahead ? jn : -1;
-                switch (ip) {
-                    case 0: gj_set_row_i<T, RI, CJ, 0>(x, rv, js); break;
-                    case 1: gj_set_row_i<T, RI, CJ, 1>(x, rv, js); break;
-                    case 2: gj_set_row_i<T, RI, CJ, 2>(x, rv, js); break;
-                    default: gj_set_row_i<T, RI, CJ, 3>(x, rv, js); break;
-                }
-            }
-            __syncthreads();
+            publish(k + 1, colv);
         }
+#pragma unroll
+        for (int j = 0; j < CJ; ++j)
+            if (j != jn) update(j);
+        __syncthreads();
     }
-    // Thread holds X[row][col] = A^{-1}[r][c] with perm[r] = row (r = iperm[row]) and
-    // iperm[c] = col (c = perm[col]); written transposed when tout.
+    // X[row][col] / pivot of the row = A^{-1}[r][c], r = iperm[row], c = perm[col]
     T ainv = T(0);
 #pragma unroll
-    for (int i = 0; i < RI; ++i)
+    for (int i = 0; i < RI; ++i) {
+        const int row = lane + 32 * i, r = iperm[row];
+        const T sc = rinv[row];
 #pragma unroll
         for (int j = 0; j < CJ; ++j) {
-            const int row = lane + 32 * i, col = w + 16 * j;
-            const int r = iperm[row], c = perm[col];
-            if (tout) dst[(size_t)c * ldd + r] = x[i][j];
-            else dst[(size_t)r * ldd + c] = x[i][j];
-            ainv = fmax(ainv, fabs(x[i][j]));
-            if (!isfinite(x[i][j])) bad = true;
+            const int c = perm[w + 16 * j];
+            const T v = x[i][j] * sc;
+            if (tout) dst[(size_t)c * ldd + r] = v;
+            else dst[(size_t)r * ldd + c] = v;
+            ainv = fmax(ainv, fabs(v));
+            if (!isfinite(v)) bad = true;
         }
+    }
     for (int o = 16; o > 0; o >>= 1) {
         amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
         ainv = fmax(ainv, __shfl_xor_sync(0xffffffffu, ainv, o));

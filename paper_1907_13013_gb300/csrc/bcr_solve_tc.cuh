@@ -169,12 +169,13 @@ template <int RT>
 __global__ void __launch_bounds__(tcs::kThreads) k_bcr_solve_tc(
     const unsigned char *__restrict__ Atc, const float *__restrict__ Bc, const float *__restrict__ Cc,
     const BcrItem *__restrict__ items, LevelTable lv, float *rhs, float *Y, float *gs, int N, int sumK, int R,
-    int *cnt, int *done, int *queue, int *err, int *zero_next, long long nzero, int *queue_next) {
+    int *cnt, int *done, int *queue, int *err, int *zero_next, long long nzero, int *queue_next, const int *stop) {
     using namespace tcs;
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < nzero; i += (long long)gridDim.x * kThreads)
         zero_next[i] = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) *queue_next = 0;
     tc::grid_dependency_wait();
+    if (stopped(stop)) return;
     extern __shared__ __align__(128) unsigned char smem_tcs[];
     const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2, MT = n2 / 128, ald = aux_ld(n2);
     const Plan pl = Plan::make(n2, RT);

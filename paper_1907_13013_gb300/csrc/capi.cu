@@ -64,6 +64,7 @@ struct PathBuffers {
 
 }  // namespace
 
+constexpr unsigned kConvSlots = 4;  // at most two reports are under way at once
 constexpr double kGrowthLimit = 1e14;  // default pivot-growth limit of the FP block factorization
 
 struct fpsa_ctx {
@@ -117,7 +118,6 @@ struct fpsa_ctx {
     double *d_result = nullptr;
     int *d_steps = nullptr;      // refinement steps taken by a batch graph's loop
     cudaEvent_t ad_ev[4] = {};   // MIXED: first residual and first inner step, timed once per solve
-    double *h_result = nullptr;  // pinned
 
     // adjoint
     bool fwd_ready = false;      // d_phi_fwd holds the last converged forward moments
@@ -142,7 +142,13 @@ struct fpsa_ctx {
     unsigned char *d_tc_ops = nullptr;  // D_hi, D_lo, M_hi, M_lo (BF16, core-matrix layout)
     // [0]: a bounded device wait ran out (tensor-core or BCR dataflow); [1]: the polls a
     // BCR dataflow wait makes before it gives up (fpsa_set_limits)
-    int *d_dev_err = nullptr, *h_flag = nullptr;
+    int *d_dev_err = nullptr;
+    // convergence reports (k_sweep_maps, k_conv_report): the stop flag lies before d_dev_err,
+    // so that one memset clears both; slots in pinned host memory, used in turn
+    int *d_stop = nullptr;
+    ConvSlot *h_slots = nullptr;
+    unsigned conv_seq = 0;
+    int *h_flag = nullptr;  // pinned, after the slots
     double growth_limit = kGrowthLimit;  // fpsa_set_xs: FPSA_EPIVOT above this pivot growth
     int tc_grid = 0;
 
@@ -732,16 +738,19 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
 // psi = L^{-1} q for every (ordinate, instance, rhs) with the given incoming edge
 // fluxes inc (NULL: none): the segmented sweep (chunk / segment maps, then the
 // re-sweep from each segment's inflow; reflective edges take their whole-slab maps
-// from the segment maps).
+// from the segment maps). rep: the convergence report of the iteration before, made by
+// one more block of the maps kernel (slot NULL: none).
 template <typename T>
-int sweep(fpsa_ctx *ctx, PathBuffers<T> &p, const T *q, T *psi, const T *inc) {
+int sweep(fpsa_ctx *ctx, PathBuffers<T> &p, const T *q, T *psi, const T *inc, const ConvReport &rep = {}) {
     const Geometry &g = ctx->geo;
     const int cpt = ctx->sweep_cpt, nseg = (g.Kmax + kSegWarps * cpt - 1) / (kSegWarps * cpt);
     const dim3 grid(2 * ((g.N / 2 + 31) / 32), nseg, g.R * g.B);
     {
         Launch L_(ctx, FPSA_PHASE_SWEEP);
-        CK(launch_pdl(k_sweep_maps<T>, grid, dim3(kSegWarps * 32), 0, ctx->stream, q, (const T *)p.coef, ctx->d_off,
-                      ctx->d_K, g.N, g.sumK, g.B, cpt, nseg, p.cmap, p.smap));
+        dim3 mgrid = grid;
+        if (rep.slot) mgrid.y += 1;
+        CK(launch_pdl(k_sweep_maps<T>, mgrid, dim3(kSegWarps * 32), 0, ctx->stream, q, (const T *)p.coef, ctx->d_off,
+                      ctx->d_K, g.N, g.sumK, g.B, cpt, nseg, p.cmap, p.smap, rep));
     }
     {
         Launch L_(ctx, FPSA_PHASE_SWEEP);
@@ -786,7 +795,7 @@ void plan_solve_shape(fpsa_ctx *ctx) {
 // be launched as a programmatic dependent of the kernel before it.
 // The tensor-core solve (k_bcr_solve_tc): an ordinary launch of two CTAs per SM
 // that takes its units from a queue; counters as the cooperative solve's.
-int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs) {
+int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *stop) {
     const Geometry &g = ctx->geo;
     const size_t n = ctx->flow_n;
     int *cnt = ctx->d_flow + 2 * n * ctx->flow_parity, *done = cnt + n;
@@ -800,7 +809,7 @@ int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs) {
         return launch_pdl(kern, dim3(ctx->tcs_grid), dim3(tcs::kThreads), smem, ctx->stream,
                           (const unsigned char *)ctx->d_tcs_A, (const float *)p.Bc, (const float *)p.Cc,
                           (const BcrItem *)ctx->d_items_all, ctx->lvt[0], rhs, p.ybuf, ctx->d_tcs_g, g.N, g.sumK,
-                          g.R, cnt, done, queue, ctx->d_dev_err, zero_next, (long long)(2 * n), queue_next);
+                          g.R, cnt, done, queue, ctx->d_dev_err, zero_next, (long long)(2 * n), queue_next, stop);
     };
     switch (RT) {
         case 16: CK(go(k_bcr_solve_tc<16>)); break;
@@ -811,10 +820,11 @@ int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs) {
     return FPSA_OK;
 }
 
+// stop: the flag at which the solve is skipped (NULL: none; its counters are zeroed either way).
 template <typename T>
-int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs) {
+int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs, const int *stop = nullptr) {
     if constexpr (sizeof(T) == sizeof(float))
-        if (ctx->tcs_rt && ctx->tuning.solve_engine != 1) return bcr_solve_tc(ctx, p, rhs);
+        if (ctx->tcs_rt && ctx->tuning.solve_engine != 1) return bcr_solve_tc(ctx, p, rhs, stop);
     const Geometry &g = ctx->geo;
     int N = g.N, sumK = g.sumK, R = g.R;
     const BcrItem *items = ctx->d_items_all;
@@ -829,7 +839,8 @@ int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs) {
     const T *G = p.G;
     void *args[] = {(void *)&A,   (void *)&Bc,  (void *)&Cc,   (void *)&items, (void *)&lv,
                     (void *)&rhs, (void *)&Y,   (void *)&N,    (void *)&sumK,  (void *)&R,
-                    (void *)&cnt, (void *)&done, (void *)&err, (void *)&G,     (void *)&zero_next, (void *)&nzero};
+                    (void *)&cnt, (void *)&done, (void *)&err, (void *)&G,     (void *)&zero_next, (void *)&nzero,
+                    (void *)&stop};
     const int grid = ctx->coop_grid[sizeof(T) == 8 ? 1 : 0];
     const int RC = solve_rc(R);
     const void *kern = coop_kernel<T>(RC, N);
@@ -870,9 +881,45 @@ int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs) {
     return FPSA_OK;
 }
 
-template <typename T>
+// The next report's target: the change of phi_0 against tol (a negative tol: reported only).
+ConvReport next_report(fpsa_ctx *ctx, double tol) {
+    const unsigned seq = ++ctx->conv_seq;
+    return ConvReport{ctx->d_conv, ctx->geo.R * ctx->geo.B, tol, ctx->d_dev_err, ctx->d_stop,
+                      ctx->h_slots + seq % kConvSlots, seq};
+}
+
+// Make report r by a kernel of its own (no sweep follows to carry it).
+int report_alone(fpsa_ctx *ctx, const ConvReport &r) {
+    Launch L_(ctx, FPSA_PHASE_CONVERGENCE);
+    CK(launch_pdl(k_conv_report, dim3(1), dim3(256), 0, ctx->stream, r));
+    return FPSA_OK;
+}
+
+// Wait for report r. The stream is asked now and then, so that a failed launch ends the wait.
+int wait_report(fpsa_ctx *ctx, const ConvReport &r, double &e, int &err) {
+    const volatile ConvSlot *s = r.slot;
+    auto arrived = [&]() { return __atomic_load_n(const_cast<const unsigned *>(&s->seq), __ATOMIC_ACQUIRE) == r.seq; };
+    for (unsigned n = 1; !arrived(); ++n) {
+        if (n % 4096) continue;
+        const cudaError_t q = cudaStreamQuery(ctx->stream);
+        if (q == cudaErrorNotReady) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        CK(q);
+        if (!arrived()) return fail(ctx, FPSA_ECUDA, "the stream ended without a convergence report");
+    }
+    e = s->e;
+    err = s->err;
+    return FPSA_OK;
+}
+
 // Qm: source moments (may be NULL), Qa: nodal angular source (may be NULL), inc:
 // incoming edge fluxes (may be NULL). phi_out may be NULL (the iterate stays in p.phi).
+// The host launches iteration it + 1 before it waits for the test of iteration it, whose
+// report that iteration's first kernel makes: the GPU never waits for the host. When it
+// turns out to have been the last one, what was launched behind it leaves phi alone.
+template <typename T>
 int solve_fp64(fpsa_ctx *ctx, PathBuffers<T> &p, const fpsa_opts &o, const double *phi0, int mem, double *phi_out,
                fpsa_stats &stats, const T *Qm, const T *Qa, const T *inc) {
     const Geometry &g = ctx->geo;
@@ -891,52 +938,51 @@ int solve_fp64(fpsa_ctx *ctx, PathBuffers<T> &p, const fpsa_opts &o, const doubl
         CK(cudaMemsetAsync(p.phi, 0, ncol * N * sizeof(T), st));
     }
     CK(cudaMemsetAsync(ctx->d_conv, 0, (size_t)g.R * g.B * 2 * sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(ctx->d_dev_err, 0, sizeof(int), st));
+    CK(cudaMemsetAsync(ctx->d_stop, 0, 2 * sizeof(int), st));  // and d_dev_err
     {
         Launch L_(ctx, FPSA_PHASE_CONTRACT);
         k_scatter<T><<<cgrid, kContractThreads, csm / 2, st>>>(p.phi, p.sigma_s, Qm, p.MT, p.q, N, g.sumK, Qa);
     }
     CK(cudaGetLastError());
     const int every = o.check_every > 0 ? o.check_every : 1;
+    auto tested = [&](int i) { return i >= 1 && (i % every == 0 || i == o.max_iterations); };
     int status = FPSA_ENOTCONV;
     double e = INFINITY;
-    int it = 0;
-    for (it = 1; it <= o.max_iterations; ++it) {
-        int rc0 = sweep(ctx, p, p.q, p.psi, inc);
-        if (rc0) return rc0;
-        if (fpsa) {
-            {
-                Launch L_(ctx, FPSA_PHASE_CONTRACT);
-                k_fp_rhs<T><<<cgrid, kContractThreads, csm, st>>>(p.psi, p.phi, p.phi_half, p.sigma_s, ctx->d_h, p.DT,
-                                                                   p.MT, p.rhs, N, g.sumK);
-            }
-            int rc = bcr_solve(ctx, p, p.rhs);
-            if (rc) return rc;
-            {
-                Launch L_(ctx, FPSA_PHASE_CONTRACT);
-                k_update_scatter<T><<<cgrid, kContractThreads, csm, st>>>(p.ybuf, p.phi_half, p.phi, p.sigma_s, Qm, p.DT,
-                                                                           p.MT, p.q, ctx->d_cell_inst, g.B, ctx->d_conv,
-                                                                           N, g.sumK, Qa);
-            }
+    int it = 0;  // iterations whose test is known
+    for (int launched = 1;; ++launched) {
+        const bool last = launched > o.max_iterations;  // no iteration left to launch: its report alone
+        ConvReport rep{};
+        if (tested(launched - 1)) rep = next_report(ctx, o.tol);
+        if (last) {
+            const int rc0 = report_alone(ctx, rep);
+            if (rc0) return rc0;
         } else {
-            {
-                Launch L_(ctx, FPSA_PHASE_CONTRACT);
-                k_update_scatter<T><<<cgrid, kContractThreads, csm, st>>>(p.psi, (const T *)nullptr, p.phi, p.sigma_s,
-                                                                           Qm, p.DT, p.MT, p.q, ctx->d_cell_inst, g.B,
-                                                                           ctx->d_conv, N, g.sumK, Qa);
+            int rc0 = sweep(ctx, p, p.q, p.psi, inc, rep);
+            if (rc0) return rc0;
+            if (fpsa) {
+                {
+                    Launch L_(ctx, FPSA_PHASE_CONTRACT);
+                    CK(launch_pdl(k_fp_rhs<T>, cgrid, dim3(kContractThreads), csm, st, (const T *)p.psi,
+                                  (const T *)p.phi, p.phi_half, (const T *)p.sigma_s, (const double *)ctx->d_h,
+                                  (const T *)p.DT, (const T *)p.MT, p.rhs, N, g.sumK));
+                }
+                int rc = bcr_solve(ctx, p, p.rhs, (const int *)ctx->d_stop);
+                if (rc) return rc;
             }
+            Launch L_(ctx, FPSA_PHASE_CONTRACT);
+            CK(launch_pdl(k_update_scatter<T>, cgrid, dim3(kContractThreads), csm, st,
+                          (const T *)(fpsa ? p.ybuf : p.psi), (const T *)(fpsa ? p.phi_half : nullptr), p.phi,
+                          (const T *)p.sigma_s, Qm, (const T *)p.DT, (const T *)p.MT, p.q,
+                          (const int32_t *)ctx->d_cell_inst, g.B, ctx->d_conv, N, g.sumK, Qa,
+                          (const int *)ctx->d_stop));
         }
         CK(cudaGetLastError());
-        if (it % every == 0 || it == o.max_iterations) {
-            {
-                Launch L_(ctx, FPSA_PHASE_CONVERGENCE);
-                k_conv_finalize<<<1, 256, 0, st>>>(ctx->d_conv, g.R * g.B, ctx->d_result);
-            }
-            CK(cudaMemcpyAsync(ctx->h_result, ctx->d_result, sizeof(double), cudaMemcpyDeviceToHost, st));
-            CK(cudaMemcpyAsync(ctx->h_flag, ctx->d_dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
-            e = ctx->h_result[0];
-            if (*ctx->h_flag) {
+        if (rep.slot) {
+            int flag = 0;
+            const int rcw = wait_report(ctx, rep, e, flag);
+            if (rcw) return rcw;
+            it = launched - 1;
+            if (flag) {
                 status = fail(ctx, FPSA_ETIMEOUT, "a bounded device wait ran out (BCR dataflow)");
                 break;
             }
@@ -949,8 +995,8 @@ int solve_fp64(fpsa_ctx *ctx, PathBuffers<T> &p, const fpsa_opts &o, const doubl
                 break;
             }
         }
+        if (last) break;
     }
-    if (it > o.max_iterations) it = o.max_iterations;
     stats.iterations = it;
     stats.outer_iterations = it;
     stats.sweeps = it;
@@ -1007,10 +1053,10 @@ int mixed_plan(fpsa_ctx *ctx, const fpsa_opts &o, MixedPlan &mp) {
 }
 
 // The FP64 residual of a refinement step: phi = D psi64, the convergence maxima, the
-// residual source of the next inner solve (k_mixed_residual), then the relative change
-// of phi_0 into d_result (k_conv_finalize).
+// residual source of the next inner solve (k_mixed_residual); with finalize (batch
+// graphs) the relative change of phi_0 goes into d_result (k_conv_finalize).
 int mixed_residual_launch(fpsa_ctx *ctx, const MixedPlan &mp, const double *Qm, const double *Qa, const double *inc,
-                          bool gmres) {
+                          bool gmres, bool finalize) {
     const Geometry &g = ctx->geo;
     const int N = g.N;
     cudaStream_t st = ctx->stream;
@@ -1037,7 +1083,7 @@ int mixed_residual_launch(fpsa_ctx *ctx, const MixedPlan &mp, const double *Qm, 
                       ctx->d_K, g.B, ctx->d_conv, f.qang, N, g.sumK, Qa, inc, ctx->d_bc,
                       gmres ? (float *)nullptr : f.q, gmres ? (float *)nullptr : f.phi));
     }
-    {
+    if (finalize) {
         Launch L_(ctx, FPSA_PHASE_CONVERGENCE);
         CK(launch_pdl(k_conv_finalize, dim3(1), dim3(256), 0, st, ctx->d_conv, g.R * g.B, ctx->d_result));
     }
@@ -1045,10 +1091,14 @@ int mixed_residual_launch(fpsa_ctx *ctx, const MixedPlan &mp, const double *Qm, 
     return FPSA_OK;
 }
 
-// inner_k FP32 FPSA (fpsa) or SI iterations of the correction equation from zero
-// (f.phi = 0 and f.q = f.qang were written by the residual kernel), then
-// psi64 += dpsi (FP64). Adds the sweeps launched to `sweeps`.
-int mixed_inner_launch(fpsa_ctx *ctx, const MixedPlan &mp, int inner_k, bool fpsa, int &sweeps) {
+// FP32 FPSA (fpsa) or SI iterations j0 .. inner_k of the correction equation from zero
+// (f.phi = 0 and f.q = f.qang were written by the residual kernel), each but the first
+// preceded by the update from the one before; with finish, psi64 += dpsi (FP64) after
+// the last. (j0, inner_k, finish) = (1, 1, false) launches the first iteration alone,
+// with the convergence report rep, skipping its BCR solve when that report raises *stop;
+// (2, k, true) the rest.
+int mixed_inner_launch(fpsa_ctx *ctx, const MixedPlan &mp, int j0, int inner_k, bool fpsa, bool finish,
+                       const ConvReport &rep = {}) {
     const Geometry &g = ctx->geo;
     const int N = g.N;
     cudaStream_t st = ctx->stream;
@@ -1059,11 +1109,28 @@ int mixed_inner_launch(fpsa_ctx *ctx, const MixedPlan &mp, int inner_k, bool fps
     const int tc_blocks = mp.tc_blocks;
     const size_t tc_smem = mp.tc_smem;
     const TcOps tcops = mp.tcops;
-    for (int j = 1; j <= inner_k; ++j) {
-        int rcs = sweep(ctx, f, f.q, f.psi, (const float *)nullptr);
+    const float *vin = fpsa ? f.ybuf : f.psi, *base = fpsa ? f.phi_half : nullptr;
+    for (int j = j0; j <= inner_k; ++j) {
+        if (j > 1) {
+            Launch L_(ctx, FPSA_PHASE_CONTRACT);
+            if (use_tc && tc_big)
+                CK(launch_pdl(k_tc_update_scatter_big, dim3(tc_blocks), dim3(128), tc_smem, st, vin, base, f.phi,
+                              (const float *)f.sigma_s, tcops, f.q, (const float *)f.qang, N, g.sumK, g.R,
+                              ctx->d_dev_err));
+            else if (use_tc && tc_full)
+                CK(launch_pdl(k_tc_update_scatter_tile, dim3(tc_blocks), dim3(128), tc_smem, st, vin, base, f.phi,
+                              (const float *)f.sigma_s, tcops, f.q, (const float *)f.qang, N, g.sumK, g.R,
+                              ctx->d_dev_err));
+            else if (use_tc)
+                k_tc_update_scatter<<<tc_blocks, 128, tc_smem, st>>>(vin, base, f.phi, f.sigma_s, tcops, f.q,
+                                                                     f.qang, N, g.sumK, g.R, ctx->d_dev_err);
+            else
+                k_update_scatter<float><<<cgrid, kContractThreads, contract_smem<float>(N), st>>>(
+                    vin, base, f.phi, f.sigma_s, (const float *)nullptr, f.DT, f.MT, f.q, ctx->d_cell_inst, g.B,
+                    (unsigned long long *)nullptr, N, g.sumK, f.qang, nullptr);
+        }
+        int rcs = sweep(ctx, f, f.q, f.psi, (const float *)nullptr, rep);
         if (rcs) return rcs;
-        ++sweeps;
-        const float *vin = f.psi, *base = nullptr;
         if (fpsa) {
             {
                 Launch L_(ctx, FPSA_PHASE_CONTRACT);
@@ -1082,31 +1149,11 @@ int mixed_inner_launch(fpsa_ctx *ctx, const MixedPlan &mp, int inner_k, bool fps
                     k_fp_rhs<float><<<cgrid, kContractThreads, contract_smem<float>(N), st>>>(
                         f.psi, f.phi, f.phi_half, f.sigma_s, ctx->d_h, f.DT, f.MT, f.rhs, N, g.sumK);
             }
-            int rc = bcr_solve(ctx, f, f.rhs);
+            int rc = bcr_solve(ctx, f, f.rhs, rep.slot ? (const int *)ctx->d_stop : nullptr);
             if (rc) return rc;
-            vin = f.ybuf;
-            base = f.phi_half;
-        }
-        if (j < inner_k) {
-            Launch L_(ctx, FPSA_PHASE_CONTRACT);
-            if (use_tc && tc_big)
-                CK(launch_pdl(k_tc_update_scatter_big, dim3(tc_blocks), dim3(128), tc_smem, st, vin, base, f.phi,
-                              (const float *)f.sigma_s, tcops, f.q, (const float *)f.qang, N, g.sumK, g.R,
-                              ctx->d_dev_err));
-            else if (use_tc && tc_full)
-                CK(launch_pdl(k_tc_update_scatter_tile, dim3(tc_blocks), dim3(128), tc_smem, st, vin, base, f.phi,
-                              (const float *)f.sigma_s, tcops, f.q, (const float *)f.qang, N, g.sumK, g.R,
-                              ctx->d_dev_err));
-            else if (use_tc)
-                k_tc_update_scatter<<<tc_blocks, 128, tc_smem, st>>>(vin, base, f.phi, f.sigma_s, tcops, f.q,
-                                                                     f.qang, N, g.sumK, g.R, ctx->d_dev_err);
-            else
-                k_update_scatter<float><<<cgrid, kContractThreads, contract_smem<float>(N), st>>>(
-                    vin, base, f.phi, f.sigma_s, (const float *)nullptr, f.DT, f.MT, f.q, ctx->d_cell_inst, g.B,
-                    (unsigned long long *)nullptr, N, g.sumK, f.qang);
         }
     }
-    {
+    if (finish) {
         Launch L_(ctx, FPSA_PHASE_RESIDUAL);
         CK(launch_pdl(k_mixed_accumulate, dim3(4 * 152), dim3(256), 0, st, p.psi, (const float *)f.psi,
                       fpsa ? (const float *)f.ybuf : (const float *)nullptr, mp.nang));
@@ -1137,7 +1184,7 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
     const double inner_tol = o.inner_tol > 0 ? o.inner_tol : 1e-5;
     int krylov = 0;
     ctx->gm_use_tc = mp.use_tc;  // the inner GMRES solves of GMRES-IR too
-    CK(cudaMemsetAsync(ctx->d_dev_err, 0, sizeof(int), st));
+    CK(cudaMemsetAsync(ctx->d_stop, 0, 2 * sizeof(int), st));  // and d_dev_err
 
     CK(cudaMemsetAsync(p.phi, 0, nang * sizeof(double), st));
     if (phi0) {
@@ -1160,14 +1207,26 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
         for (int i = 0; i < 4; ++i) CK(cudaEventCreate(&ctx->ad_ev[i]));
     for (outer = 1; outer <= o.max_iterations + 1; ++outer) {
         if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[0], st));
-        int rcr = mixed_residual_launch(ctx, mp, Qm, Qa, inc, gmres);
+        int rcr = mixed_residual_launch(ctx, mp, Qm, Qa, inc, gmres, false);
         if (rcr) return rcr;
         if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[1], st));
-        CK(cudaMemcpyAsync(ctx->h_result, ctx->d_result, sizeof(double), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(ctx->h_flag, ctx->d_dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        e = ctx->h_result[0];
-        if (*ctx->h_flag) {
+        // The test's report: SI and FPSA launch the first inner iteration behind the residual
+        // (every step that goes on has one) and let it carry the report, so that the GPU does not
+        // wait while the host decides; if this was the last residual, that iteration leaves
+        // psi64 and phi alone and its BCR solve is skipped.
+        const ConvReport rep = next_report(ctx, (outer > 1 || phi0) ? o.tol : -1.0);
+        const bool ahead = !gmres && outer <= o.max_iterations;
+        if (ahead) {
+            if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[2], st));
+            rcr = mixed_inner_launch(ctx, mp, 1, 1, fpsa, false, rep);
+        } else {
+            rcr = report_alone(ctx, rep);
+        }
+        if (rcr) return rcr;
+        int flag = 0;
+        rcr = wait_report(ctx, rep, e, flag);
+        if (rcr) return rcr;
+        if (flag) {
             status = fail(ctx, FPSA_ETIMEOUT, "a bounded device wait ran out (tensor-core contraction or BCR dataflow)");
             break;
         }
@@ -1237,7 +1296,8 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
         e_prev = e;
         k_before = k_last;
         k_last = inner_k;
-        if (time_first && outer == 2) {  // the first step's events have completed (synchronised above)
+        if (time_first && outer == 2) {
+            CK(cudaEventSynchronize(ctx->ad_ev[3]));  // (already reached: the report came after it)
             float t_res = 0.f, t_step = 0.f;
             if (cudaEventElapsedTime(&t_res, ctx->ad_ev[0], ctx->ad_ev[1]) == cudaSuccess &&
                 cudaEventElapsedTime(&t_step, ctx->ad_ev[2], ctx->ad_ev[3]) == cudaSuccess)
@@ -1246,9 +1306,9 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
         }
         if (!adaptive_on && inner_k > inner) inner_k = inner;
         k_last = inner_k;
-        if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[2], st));
-        int rci = mixed_inner_launch(ctx, mp, inner_k, fpsa, sweeps);
+        int rci = mixed_inner_launch(ctx, mp, 2, inner_k, fpsa, true);
         if (rci) return rci;
+        sweeps += inner_k;
         if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[3], st));
     }
     stats.iterations = gmres ? krylov : sweeps;
@@ -1424,7 +1484,7 @@ int gm_update(fpsa_ctx *ctx, PathBuffers<T> &p, const T *y, const T *base, T *ou
     const dim3 cgrid((g.sumK + kContractCells - 1) / kContractCells, g.R);
     k_update_scatter<T><<<cgrid, kContractThreads, contract_smem<T>(N), st>>>(
         y, base, out, p.sigma_s, (const T *)nullptr, p.DT, p.MT, p.q, ctx->d_cell_inst, g.B,
-        (unsigned long long *)nullptr, N, g.sumK, (const T *)nullptr);
+        (unsigned long long *)nullptr, N, g.sumK, (const T *)nullptr, nullptr);
     CK(cudaGetLastError());
     return FPSA_OK;
 }
@@ -1684,7 +1744,6 @@ int capture_mixed_loop(fpsa_ctx *ctx, const MixedPlan &mp, const fpsa_opts &o, i
         restore();
         return fail(ctx, FPSA_ECUDA, "batch graph: stream capture refused");
     }
-    int sw = 0;
     if (cudaMemsetAsync(ctx->d_dev_err, 0, sizeof(int), cs) != cudaSuccess ||
         cudaMemsetAsync(ctx->d_steps, 0, sizeof(int), cs) != cudaSuccess ||
         cudaMemsetAsync(p.phi, 0, mp.nang * sizeof(double), cs) != cudaSuccess ||
@@ -1694,7 +1753,7 @@ int capture_mixed_loop(fpsa_ctx *ctx, const MixedPlan &mp, const fpsa_opts &o, i
         restore();
         return fail(ctx, FPSA_ECUDA, "batch graph: capture of the prologue failed");
     }
-    rc = mixed_residual_launch(ctx, mp, p.Q, nullptr, inc, false);
+    rc = mixed_residual_launch(ctx, mp, p.Q, nullptr, inc, false, true);
     if (rc) {
         end_capture_on_error();
         restore();
@@ -1736,8 +1795,8 @@ int capture_mixed_loop(fpsa_ctx *ctx, const MixedPlan &mp, const fpsa_opts &o, i
             return fail(ctx, FPSA_ECUDA, "batch graph: capture of the loop body failed");
         }
     }
-    rc = mixed_inner_launch(ctx, mp, inner, fpsa, sw);
-    if (!rc) rc = mixed_residual_launch(ctx, mp, p.Q, nullptr, inc, false);
+    rc = mixed_inner_launch(ctx, mp, 1, inner, fpsa, true);
+    if (!rc) rc = mixed_residual_launch(ctx, mp, p.Q, nullptr, inc, false, true);
     if (!rc) {
         k_batch_cond<<<1, 32, 0, cs>>>(handle, ctx->d_result, ctx->d_dev_err, ctx->d_steps, o.tol, o.max_iterations);
         if (cudaGetLastError() != cudaSuccess) rc = fail(ctx, FPSA_ECUDA, "batch graph: loop test launch failed");
@@ -1785,8 +1844,7 @@ void fpsa_destroy(fpsa_ctx *ctx) {
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : ctx->ad_ev)
         if (e) cudaEventDestroy(e);
-    if (ctx->h_result) cudaFreeHost(ctx->h_result);
-    if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
+    if (ctx->h_slots) cudaFreeHost(ctx->h_slots);
     delete ctx;
 }
 
@@ -1844,12 +1902,15 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
         CK(dalloc(ctx, &ctx->d_in_ss, (size_t)g.sumK * g.L1));
         CK(dalloc(ctx, &ctx->d_in_q, (size_t)g.R * g.sumK * 2 * g.L1));
         CK(dalloc(ctx, &ctx->d_xs_err, 2));
-        CK(dalloc(ctx, &ctx->d_dev_err, 2));
+        CK(dalloc(ctx, &ctx->d_stop, 3));
+        ctx->d_dev_err = ctx->d_stop + 1;
         {
-            const int e0[2] = {0, (int)kFlowSpinLimit};
-            CK(cudaMemcpy(ctx->d_dev_err, e0, sizeof(e0), cudaMemcpyHostToDevice));
+            const int e0[3] = {0, 0, (int)kFlowSpinLimit};
+            CK(cudaMemcpy(ctx->d_stop, e0, sizeof(e0), cudaMemcpyHostToDevice));
         }
-        CK(cudaMallocHost(&ctx->h_flag, sizeof(int)));
+        CK(cudaMallocHost(&ctx->h_slots, kConvSlots * sizeof(ConvSlot) + sizeof(int)));
+        std::memset(ctx->h_slots, 0, kConvSlots * sizeof(ConvSlot) + sizeof(int));
+        ctx->h_flag = reinterpret_cast<int *>(ctx->h_slots + kConvSlots);
         {
             const int nchunk = (g.R + solve_rc(g.R) - 1) / solve_rc(g.R);
             ctx->flow_n = (size_t)nchunk * g.sumK;
@@ -1861,7 +1922,6 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
         CK(dalloc(ctx, &ctx->d_status, 1));
         CK(dalloc(ctx, &ctx->d_result, 2));
         CK(dalloc(ctx, &ctx->d_steps, 1));
-        CK(cudaMallocHost(&ctx->h_result, 2 * sizeof(double)));
         CK(cudaMemcpy(ctx->d_off, g.off.data(), g.B * sizeof(int32_t), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->d_K, g.K.data(), g.B * sizeof(int32_t), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->d_cell_inst, g.cell_inst.data(), g.sumK * sizeof(int32_t), cudaMemcpyHostToDevice));

@@ -92,6 +92,79 @@ constexpr int32_t kBcReflect = 1;
 constexpr int kSweepBatch = 8;  // cells whose inputs one thread requests together
 
 // ---------------------------------------------------------------------------
+// Convergence test (Eq. iterate): the worst relative change over (rhs, instance),
+// max_rb conv_d / conv_a (NaN if any value was non-finite), by one block; resets the
+// accumulators. The result is valid in thread 0.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double worst_change(unsigned long long *conv, int nrb) {
+    __shared__ double red[32];
+    double worst = 0.0;
+    bool bad = false;
+    for (int i = threadIdx.x; i < nrb; i += blockDim.x) {
+        const double d = __longlong_as_double((long long)__ldcg(conv + 2 * i));
+        const double a = __longlong_as_double((long long)__ldcg(conv + 2 * i + 1));
+        if (!isfinite(d) || !isfinite(a)) bad = true;
+        worst = fmax(worst, (a > 0.0) ? d / a : (d > 0.0 ? INFINITY : 0.0));
+        conv[2 * i] = 0ull;
+        conv[2 * i + 1] = 0ull;
+    }
+    for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = worst;
+    const bool any_bad = __syncthreads_or(bad) != 0;
+    if (threadIdx.x != 0) return 0.0;
+    for (int i = 1; i < (int)((blockDim.x + 31) >> 5); ++i) worst = fmax(worst, red[i]);
+    return any_bad ? (double)NAN : worst;
+}
+
+// The result in device memory (batch graphs: k_batch_cond tests it there).
+static __global__ void k_conv_finalize(unsigned long long *conv, int nrb, double *out) {
+    tc::grid_dependency_wait();  // inputs of the previous kernel (programmatic dependent launch)
+    const double e = worst_change(conv, nrb);
+    if (threadIdx.x == 0) out[0] = e;
+}
+
+// The test as a side task of the NEXT iteration's first kernel, instead of a kernel and
+// a copy of its own that the host waits for with nothing queued behind: the host always
+// has one more iteration in the stream than it has results for (200 cells at N = 16, FP64
+// source iteration: 42 us an iteration with the kernel, two copies and a wait, 17.6 so). A report goes to a slot
+// in pinned host memory that the host polls (e and err, then the sequence number); when
+// the iteration it speaks of was the last one (converged, not finite, or a bounded wait
+// ran out) it also raises *stop, at which the kernels queued behind leave the state as it is.
+struct ConvSlot {
+    double e;
+    int err;
+    unsigned seq;
+};
+struct ConvReport {
+    unsigned long long *conv;
+    int nrb;
+    double tol;
+    const int *err;
+    int *stop;
+    ConvSlot *slot;  // NULL: no report
+    unsigned seq;
+};
+__device__ __forceinline__ void conv_report(const ConvReport &r) {  // one block
+    const double e = worst_change(r.conv, r.nrb);
+    if (threadIdx.x == 0) {
+        const int err = *(volatile const int *)r.err;
+        if (e < r.tol || isnan(e) || err) *(volatile int *)r.stop = 1;
+        volatile ConvSlot *s = r.slot;
+        s->e = e;
+        s->err = err;
+        __threadfence_system();
+        s->seq = r.seq;
+    }
+}
+// The report alone (no iteration follows).
+static __global__ void k_conv_report(ConvReport r) {
+    tc::grid_dependency_wait();
+    conv_report(r);
+}
+// Has a report ended the iteration? (stop NULL: never)
+__device__ __forceinline__ bool stopped(const int *stop) { return stop && *(volatile const int *)stop != 0; }
+
+// ---------------------------------------------------------------------------
 // Segmented transport sweep (the recurrence, maps and edge inflows above), laid
 // out for coalesced access: a block holds 32 ordinates of one
 // direction in its lanes (consecutive n: one 128-byte line per cell value) and
@@ -139,8 +212,12 @@ __global__ void __launch_bounds__(kSegWarps * 32) k_sweep_maps(const T *__restri
                                                                const int32_t *__restrict__ off,
                                                                const int32_t *__restrict__ Kc, int N, int sumK, int B,
                                                                int cpt, int nseg, T *__restrict__ cmap,
-                                                               T *__restrict__ smap) {
+                                                               T *__restrict__ smap, ConvReport rep) {
     tc::grid_dependency_wait();  // inputs of the previous kernel (programmatic dependent launch)
+    if ((int)blockIdx.y == nseg) {  // launched only with a report to make
+        if (blockIdx.x == 0 && blockIdx.z == 0) conv_report(rep);
+        return;
+    }
     __shared__ Affine<T> part[kSegWarps][32];
     const SweepLane L = sweep_lane(N, off, Kc, B);
     const int seg = blockIdx.y, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -407,8 +484,9 @@ __global__ void k_update_scatter(const T *__restrict__ v, const T *__restrict__ 
                                  const T *__restrict__ DT, const T *__restrict__ MT, T *__restrict__ q,
                                  const int32_t *__restrict__ cell_inst, int B,
                                  unsigned long long *__restrict__ conv, int N, int sumK,
-                                 const T *__restrict__ Qang = nullptr) {
+                                 const T *__restrict__ Qang, const int *stop) {
     tc::grid_dependency_wait();  // inputs of the previous kernel (programmatic dependent launch)
+    const bool halt = stopped(stop);  // tested below, before anything is written
     extern __shared__ unsigned char smem_raw[];
     T *Xs = reinterpret_cast<T *>(smem_raw);
     T *Ys = Xs + 2 * kContractCells * N;
@@ -421,6 +499,7 @@ __global__ void k_update_scatter(const T *__restrict__ v, const T *__restrict__ 
     __syncthreads();
     block_contract(Xs, N, DT, N, ncols, Ys, N);
     __syncthreads();
+    if (halt) return;
     for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
         const int c = idx / N, l = idx - c * N;
         const int g = g0 + c / 2;
@@ -584,34 +663,6 @@ __global__ void k_expand(const T *__restrict__ x, const T *__restrict__ MT, T *_
     for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) Xs[idx] = x[colbase * N + idx];
     __syncthreads();
     block_contract(Xs, N, MT, N, ncols, out + colbase * N, N);
-}
-
-// Worst relative change over (rhs, instance); resets the accumulators.
-// out[0] = max_rb conv_d / conv_a (NaN if any value was non-finite).
-static __global__ void k_conv_finalize(unsigned long long *conv, int nrb, double *out) {
-    tc::grid_dependency_wait();  // inputs of the previous kernel (programmatic dependent launch)
-    __shared__ double red[256];
-    double worst = 0.0;
-    bool bad = false;
-    for (int i = threadIdx.x; i < nrb; i += blockDim.x) {
-        double d = __longlong_as_double((long long)conv[2 * i]);
-        double a = __longlong_as_double((long long)conv[2 * i + 1]);
-        if (!isfinite(d) || !isfinite(a)) bad = true;
-        double e = (a > 0.0) ? d / a : (d > 0.0 ? INFINITY : 0.0);
-        worst = fmax(worst, e);
-        conv[2 * i] = 0ull;
-        conv[2 * i + 1] = 0ull;
-    }
-    red[threadIdx.x] = bad ? NAN : worst;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            double x = red[threadIdx.x], y = red[threadIdx.x + s];
-            red[threadIdx.x] = (isnan(x) || isnan(y)) ? NAN : fmax(x, y);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[0] = red[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -1793,10 +1844,11 @@ __global__ void __launch_bounds__(NT, 2) k_bcr_solve_flow(const T *__restrict__ 
                                                        LevelTable lv, T *rhs, T *Y, int N, int sumK, int R, int *cnt,
                                                        int *done, int *err,
                                                        const T *__restrict__ G /* coarse step: staged only */,
-                                                       int *zero_next, long long nzero) {
+                                                       int *zero_next, long long nzero, const int *stop) {
     for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < nzero; i += (long long)gridDim.x * NT)
         zero_next[i] = 0;
     tc::grid_dependency_wait();
+    if (stopped(stop)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sm = reinterpret_cast<T *>(smem_raw);
     const unsigned limit = flow_spin_limit(err);
@@ -2178,7 +2230,7 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
                                                             const BcrItem *__restrict__ items, LevelTable lv, T *rhs,
                                                             T *Y, int N, int sumK, int R, int *cnt, int *done,
                                                             int *err, const T *__restrict__ G, int *zero_next,
-                                                            long long nzero) {
+                                                            long long nzero, const int *stop) {
     constexpr int NTG = (NT - 32 * kSolveGroups) / kSolveGroups;
     static_assert(NTG >= 64 && NTG % 32 == 0 && NT == kSolveGroups * (NTG + 32), "compute groups and service warps");
     // the next solve's counters (the other half of the double-buffered pair) start at zero
@@ -2292,9 +2344,10 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
             }
         }
         tc::grid_dependency_wait();  // later copies may carry the previous kernel's right-hand sides
+        const bool halt = stopped(stop);
         Pos cur{0, 0, 0, 0, 0, 0, 0, false}, nxt{0, 0, 0, 0, 0, 0, 0, false};
         int k = sw;
-        for (;; k += kSolveGroups) {
+        for (; !halt; k += kSolveGroups) {
             locate(cur, blockIdx.x + k * (int)gridDim.x);
             if (!cur.valid) break;
             gbar_sync(3 + k % ns + ns * sw, kHandoff);  // group sw is done with unit k
@@ -2339,6 +2392,7 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
     const Group gr{(int)threadIdx.x - grp * NTG, 1 + grp};
     T *smg = sm + grp * base;
     tc::grid_dependency_wait();  // the right-hand sides come from the previous kernel
+    if (stopped(stop)) return;   // the service warps wait for the copies in flight
     Pos cur{0, 0, 0, 0, 0, 0, 0, false};
     for (int k = grp;; k += kSolveGroups) {
         locate(cur, blockIdx.x + k * (int)gridDim.x);

@@ -102,44 +102,84 @@ __global__ void __launch_bounds__(256) k_bgemm(int n, T alpha, BMat<T> A, BMat<T
         }
 }
 
-// max|A| of each block of the batch (before inversion), for the growth check.
-template <typename T>
-__global__ void k_bamax(BMat<T> M, int n, const BcrItem *__restrict__ items, double *__restrict__ amax) {
-    const T *p = bmat_ptr(M, items, blockIdx.x);
-    double m = 0.0;
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x)
-        m = fmax(m, fabs((double)p[(size_t)(idx / n) * M.ld + idx % n]));
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+// Block-wide maximum of |v| (valid in thread 0), for blocks of up to 1024 threads.
+__device__ __forceinline__ double block_max(double m) {
     __shared__ double red[32];
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r = fmax(r, red[i]);
-        amax[blockIdx.x] = r;
+    if (threadIdx.x == 0)
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, red[i]);
+    return m;
+}
+
+// max|A| of each block of the batch (contiguous, n even; before inversion), for
+// the growth check, into the zeroed amax[e] (as the bits of a non-negative double, whose
+// order is that of the values). Bound by the read of the blocks (131 MB at n = 256 and 500
+// items): kMaxSplit thread blocks per item, 16-byte loads eight deep (one block of single
+// loads per item took 144 us there, 561 us at n = 512).
+constexpr int kMaxSplit = 8;
+template <typename T>
+__global__ void __launch_bounds__(256) k_bamax(BMat<T> M, int n, const BcrItem *__restrict__ items,
+                                               unsigned long long *__restrict__ amax) {
+    using VT = typename VecOf<T>::type;
+    const VT *p = reinterpret_cast<const VT *>(bmat_ptr(M, items, blockIdx.x));
+    const int words = n * n / VecOf<T>::V, per = (words + kMaxSplit - 1) / kMaxSplit;
+    const int w0 = blockIdx.y * per, w1 = min(words, w0 + per);
+    T m = T(0);
+    for (int i = w0 + threadIdx.x; i < w1; i += 8 * 256) {
+        VT v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + 256 * u < w1) v[u] = __ldcg(p + i + 256 * u);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + 256 * u < w1) {
+                m = fmax(m, fmax(fabs(v[u].x), fabs(v[u].y)));
+                if constexpr (VecOf<T>::V == 4) m = fmax(m, fmax(fabs(v[u].z), fabs(v[u].w)));
+            }
     }
+    const double b = block_max((double)m);
+    if (threadIdx.x == 0) atomicMax(amax + blockIdx.x, dkey(b));
 }
 
 // In-place transpose of each n x n inverse (row-major -> the transposed layout of
-// the BCR solve) with the growth check max|A| max|A^{-1}| and a finiteness check.
+// the BCR solve) with the growth check max|A| max|A^{-1}| and a finiteness check. One
+// block per item and pair of mirrored 32 x 32 tiles (blockIdx.y counts the tiles on and
+// above the diagonal), both read and written by whole rows: one pass over the blocks at
+// memory rate (element by element, one block per item: 113 us at n = 256 and 500 items).
 template <typename T>
-__global__ void k_btranspose(BMat<T> M, int n, const BcrItem *__restrict__ items, const double *__restrict__ amax,
-                             unsigned long long *__restrict__ growth, int *__restrict__ status) {
+__global__ void __launch_bounds__(256) k_btranspose(BMat<T> M, int n, const BcrItem *__restrict__ items,
+                                                    const unsigned long long *__restrict__ amax,
+                                                    unsigned long long *__restrict__ growth, int *__restrict__ status) {
+    __shared__ T ta[32][33], tb[32][33];
     T *p = bmat_ptr(M, items, blockIdx.x);
-    double m = 0.0;
-    bool bad = false;
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-        const int i = idx / n, j = idx % n;
-        if (j < i) continue;
-        T *x = p + (size_t)i * M.ld + j, *y = p + (size_t)j * M.ld + i;
-        const T a = *x, b = *y;
-        *x = b;
-        *y = a;
-        m = fmax(m, fmax(fabs((double)a), fabs((double)b)));
-        if (!isfinite((double)a) || !isfinite((double)b)) bad = true;
+    int bi = 0, rest = blockIdx.y;
+    for (int row = (n + 31) / 32; rest >= row; --row) {
+        rest -= row;
+        ++bi;
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(growth, dkey(m * amax[blockIdx.x]));
+    const int i0 = 32 * bi, j0 = 32 * (bi + rest), x = threadIdx.x & 31, y0 = threadIdx.x >> 5;
+    T m = T(0);
+    bool bad = false;
+    auto take = [&](T v) {
+        m = fmax(m, fabs(v));
+        if (!isfinite(v)) bad = true;
+        return v;
+    };
+#pragma unroll
+    for (int y = y0; y < 32; y += 8) {
+        if (i0 + y < n && j0 + x < n) ta[y][x] = take(p[(size_t)(i0 + y) * M.ld + j0 + x]);
+        if (j0 + y < n && i0 + x < n) tb[y][x] = take(p[(size_t)(j0 + y) * M.ld + i0 + x]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int y = y0; y < 32; y += 8) {
+        if (i0 + y < n && j0 + x < n) p[(size_t)(i0 + y) * M.ld + j0 + x] = tb[x][y];
+        if (j0 + y < n && i0 + x < n) p[(size_t)(j0 + y) * M.ld + i0 + x] = ta[x][y];
+    }
+    const double b = block_max((double)m);
+    if (threadIdx.x == 0) atomicMax(growth, dkey(b * __longlong_as_double((long long)amax[blockIdx.x])));
     if (bad) atomicExch(status, 1);
 }
 

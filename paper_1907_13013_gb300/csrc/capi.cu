@@ -59,7 +59,7 @@ struct PathBuffers {
     T *G = nullptr;                          // coarse step of the BCR solve: inverse of the coarse system [n][n]
     // recursive block inversion (2N too large for one CTA): per-depth scratch X, Y
     std::vector<T *> inv_scratch;
-    double *inv_amax = nullptr;
+    unsigned long long *inv_amax = nullptr;
 };
 
 }  // namespace
@@ -401,7 +401,12 @@ int alloc_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
             CK(dalloc(ctx, &p.inv_amax, kLargeChunk));
             CK(raise_smem_limit((const void *)k_binv_smem_rm<T>, (int)kSmemLimit));
         }
-        CK(raise_smem_limit((const void *)k_bcr_schur<T>, (int)schur_smem<T>(g.N)));
+        switch (schur_tile(h2)) {
+            case 1: CK(raise_smem_limit((const void *)k_bcr_schur<T, 1>, (int)schur_tile_smem<T>(h2))); break;
+            case 2: CK(raise_smem_limit((const void *)k_bcr_schur<T, 2>, (int)schur_tile_smem<T>(h2))); break;
+            case 4: CK(raise_smem_limit((const void *)k_bcr_schur<T, 4>, (int)schur_tile_smem<T>(h2))); break;
+            default: CK(raise_smem_limit((const void *)k_bcr_schur<T, 8>, (int)schur_tile_smem<T>(h2))); break;
+        }
     }
     {
         const int cs = (int)contract_smem<T>(g.N);
@@ -519,10 +524,13 @@ int invert_level(fpsa_ctx *ctx, PathBuffers<T> &p, const BcrItem *items, int ni,
         const BMat<T> M{p.A, (long long)n2 * n2, n2, 1};
         for (int c0 = 0; c0 < ni; c0 += kLargeChunk) {
             const int ne = std::min(kLargeChunk, ni - c0);
-            k_bamax<T><<<ne, 256, 0, st>>>(M, n2, items + c0, p.inv_amax);
+            CK(cudaMemsetAsync(p.inv_amax, 0, ne * sizeof(*p.inv_amax), st));
+            k_bamax<T><<<dim3(ne, kMaxSplit), 256, 0, st>>>(M, n2, items + c0, p.inv_amax);
             int rc = invert_inplace(ctx, p, M, n2, items + c0, ne, 0);
             if (rc) return rc;
-            k_btranspose<T><<<ne, 256, 0, st>>>(M, n2, items + c0, p.inv_amax, ctx->d_growth, ctx->d_status);
+            const int nt = (n2 + 31) / 32;
+            k_btranspose<T><<<dim3(ne, nt * (nt + 1) / 2), 256, 0, st>>>(M, n2, items + c0, p.inv_amax, ctx->d_growth,
+                                                                         ctx->d_status);
         }
     }
     CK(cudaGetLastError());
@@ -685,8 +693,14 @@ int setup_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
         CK(cudaGetLastError());
         if (!fused) {
             Launch L_(ctx, FPSA_PHASE_BCR_SCHUR);
-            k_bcr_schur<T><<<ni, 256, schur_smem<T>(N), st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N,
-                                                              schur_staged<T>(N) ? 1 : 0);
+            const dim3 grid(ni, 4);
+            const size_t sm = schur_tile_smem<T>(h2);
+            switch (schur_tile(h2)) {
+                case 1: k_bcr_schur<T, 1><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
+                case 2: k_bcr_schur<T, 2><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
+                case 4: k_bcr_schur<T, 4><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
+                default: k_bcr_schur<T, 8><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
+            }
         }
         CK(cudaGetLastError());
     }

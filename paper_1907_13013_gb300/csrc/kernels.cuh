@@ -1382,11 +1382,117 @@ __device__ __forceinline__ void schur_body(T *__restrict__ A, T *__restrict__ Bc
     }
 }
 
+// The Schur updates of a level as a kernel of its own (blocks that are not inverted in
+// registers). Each of an item's four updates,
+//   out (mode 1: -=, mode 2: = -) (M Ainv[r0 .., c0 ..]) W,
+// is one block: it forms X = M Ainv[..] and then X W, 256 threads with TI x TI outputs
+// each, the operands through shared memory in k-chunks of kSchurK and X kept there,
+// transposed, as the second product's left operand. What bounds it is FP32 (FP64)
+// arithmetic, 4 h2^3 operations an update: TI x TI register tiles make that 2 TI shared
+// loads for TI^2 FMAs (2 x 2 tiles, and one block for all four updates, took 978 us a
+// level at h2 = 128 and 113 us at h2 = 64).
+constexpr int kSchurK = 16;
+constexpr int schur_tile(int h2) { return h2 <= 16 ? 1 : (h2 <= 32 ? 2 : (h2 <= 64 ? 4 : 8)); }
 template <typename T>
-__global__ void k_bcr_schur(T *__restrict__ A, T *__restrict__ Bc, T *__restrict__ Cc,
-                            const BcrItem *__restrict__ items, int N, int staged) {
-    extern __shared__ unsigned char smem_raw[];
-    schur_body(A, Bc, Cc, items[blockIdx.x], N, staged, smem_raw);
+constexpr size_t schur_tile_smem(int h2) {  // X^T, then the chunks of both operands
+    return ((size_t)h2 * (16 * schur_tile(h2) + 1) + (size_t)2 * kSchurK * (16 * schur_tile(h2) + 1)) * sizeof(T);
+}
+
+// acc[i][j] += sum_k L[k][16 i + ty] Rt[k][16 j + tx], k < nk (rows of ld values)
+template <typename T, int TI>
+__device__ __forceinline__ void schur_mma(const T *L, const T *Rt, int ld, int nk, int tx, int ty, T (&acc)[TI][TI]) {
+    for (int k = 0; k < nk; ++k) {
+        T l[TI], r[TI];
+#pragma unroll
+        for (int i = 0; i < TI; ++i) l[i] = L[k * ld + 16 * i + ty];
+#pragma unroll
+        for (int j = 0; j < TI; ++j) r[j] = Rt[k * ld + 16 * j + tx];
+#pragma unroll
+        for (int i = 0; i < TI; ++i)
+#pragma unroll
+            for (int j = 0; j < TI; ++j) acc[i][j] = fma(l[i], r[j], acc[i][j]);
+    }
+}
+
+template <typename T, int TI>
+__global__ void __launch_bounds__(256) k_bcr_schur(T *__restrict__ A, T *__restrict__ Bc, T *__restrict__ Cc,
+                                                   const BcrItem *__restrict__ items, int N) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const BcrItem it = items[blockIdx.x];
+    const int task = blockIdx.y, right = task < 2;
+    if (right ? it.right < 0 : it.left < 0) return;
+    const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2, W = 16 * TI, ld = W + 1;
+    const int Lm = 0, Lp = h2, Rm = N, Rp = N + h2;
+    const T *Ai = A + (size_t)it.cell * n2 * n2;  // transposed inverse: Ainv[r][c] = Ai[c * n2 + r]
+    const T *Bi = Bc + (size_t)it.s_cell * hh, *Ci = Cc + (size_t)it.s_cell * hh;
+    const T *M, *V;  // left and right factors of the update; Ainv's sub-block starts at (r0, c0)
+    T *out;
+    int r0, c0, ldo, mode;
+    if (right) {
+        M = Bc + (size_t)it.s_right * hh;
+        r0 = Rp;
+        c0 = task == 0 ? Rm : Lp;
+        V = task == 0 ? Ci : Bi;
+        out = task == 0 ? A + (size_t)it.right * n2 * n2 + (size_t)Lp * n2 + Lm : Bc + (size_t)it.s_right_next * hh;
+    } else {
+        M = Cc + (size_t)it.s_left * hh;
+        r0 = Lm;
+        c0 = task == 2 ? Lp : Rm;
+        V = task == 2 ? Bi : Ci;
+        out = task == 2 ? A + (size_t)it.left * n2 * n2 + (size_t)Rm * n2 + Rp : Cc + (size_t)it.s_left_next * hh;
+    }
+    mode = (task & 1) ? 2 : 1;
+    ldo = (task & 1) ? h2 : n2;
+    if (task == 3 && it.right < 0) {  // no right neighbour: the next coupling is zero
+        for (int idx = threadIdx.x; idx < hh; idx += 256) out[idx] = T(0);
+        return;
+    }
+    T *Xt = reinterpret_cast<T *>(smem_raw), *Ls = Xt + (size_t)h2 * ld, *Rs = Ls + kSchurK * ld;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    T acc[TI][TI];
+    auto clear = [&]() {
+#pragma unroll
+        for (int i = 0; i < TI; ++i)
+#pragma unroll
+            for (int j = 0; j < TI; ++j) acc[i][j] = T(0);
+    };
+    clear();
+    const T *P = Ai + (size_t)c0 * n2 + r0;  // Ainv[r0 + k][c0 + q] = P[q * n2 + k]
+    for (int k0 = 0; k0 < h2; k0 += kSchurK) {
+        for (int idx = threadIdx.x; idx < kSchurK * W; idx += 256) {  // k fastest: both are contiguous in k
+            const int kk = idx % kSchurK, p = idx / kSchurK;
+            const bool in = k0 + kk < h2 && p < h2;
+            Ls[kk * ld + p] = in ? M[(size_t)p * h2 + k0 + kk] : T(0);
+            Rs[kk * ld + p] = in ? P[(size_t)p * n2 + k0 + kk] : T(0);
+        }
+        __syncthreads();
+        schur_mma<T, TI>(Ls, Rs, ld, kSchurK, tx, ty, acc);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < TI; ++i)
+#pragma unroll
+        for (int j = 0; j < TI; ++j)
+            if (16 * j + tx < h2) Xt[(16 * j + tx) * ld + 16 * i + ty] = acc[i][j];
+    clear();
+    for (int k0 = 0; k0 < h2; k0 += kSchurK) {
+        for (int idx = threadIdx.x; idx < kSchurK * W; idx += 256) {  // q fastest: rows of V are contiguous
+            const int q = idx % W, kk = idx / W;
+            Rs[kk * ld + q] = (k0 + kk < h2 && q < h2) ? V[(size_t)(k0 + kk) * h2 + q] : T(0);
+        }
+        __syncthreads();
+        schur_mma<T, TI>(Xt + (size_t)k0 * ld, Rs, ld, min(kSchurK, h2 - k0), tx, ty, acc);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < TI; ++i)
+#pragma unroll
+        for (int j = 0; j < TI; ++j) {
+            const int p = 16 * i + ty, q = 16 * j + tx;
+            if (p >= h2 || q >= h2) continue;
+            T *o = out + (size_t)p * ldo + q;
+            *o = mode == 1 ? *o - acc[i][j] : -acc[i][j];
+        }
 }
 
 // ---------------------------------------------------------------------------

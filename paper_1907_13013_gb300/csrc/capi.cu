@@ -151,6 +151,7 @@ struct fpsa_ctx {
     int *h_flag = nullptr;  // pinned, after the slots
     double growth_limit = kGrowthLimit;  // fpsa_set_xs: FPSA_EPIVOT above this pivot growth
     int tc_grid = 0;
+    int tc_cols = 0;                    // columns per block of the few-column contractions (0: not used)
 
     // built-in profiler: launch counters (always) and event pairs (when on)
     bool prof_on = false;
@@ -603,6 +604,17 @@ int setup_tc(fpsa_ctx *ctx) {
     CK(raise_smem_limit((const void *)k_tc_update_scatter_tile, smem));
     CK(raise_smem_limit((const void *)k_tc_fp_rhs_moments<false>, smem));
     CK(raise_smem_limit((const void *)k_tc_moments_axpy<false>, smem));
+    ctx->tc_cols = tc::col_tile(ctx->geo.sumK, ctx->geo.R, nsm);
+    if (ctx->tc_cols) {
+        const int cs = (int)tc::ColPlan::make(N, ctx->tc_cols).total;
+        const void *fr[3] = {(const void *)k_tc_fp_rhs_cols<16>, (const void *)k_tc_fp_rhs_cols<32>,
+                             (const void *)k_tc_fp_rhs_cols<64>};
+        const void *us[3] = {(const void *)k_tc_update_scatter_cols<16>, (const void *)k_tc_update_scatter_cols<32>,
+                             (const void *)k_tc_update_scatter_cols<64>};
+        const int i = ctx->tc_cols == 16 ? 0 : (ctx->tc_cols == 32 ? 1 : 2);
+        CK(raise_smem_limit(fr[i], cs));
+        CK(raise_smem_limit(us[i], cs));
+    }
     int per_sm = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_update_scatter, 128, smem));
     ctx->tc_grid = std::max(1, std::min(per_sm, 2)) * nsm;
@@ -1047,6 +1059,17 @@ struct MixedPlan {
     size_t tc_smem;
 };
 
+void tc_plan(const fpsa_ctx *ctx, MixedPlan &mp) {  // its tensor-core part (ctx->tc_able)
+    const Geometry &g = ctx->geo;
+    const int N = g.N;
+    mp.tcops = TcOps{ctx->d_tc_ops, ctx->d_tc_ops + 2 * (size_t)N * N * sizeof(__nv_bfloat16)};
+    const int tc_tiles = ((2 * g.sumK + 127) / 128) * g.R;
+    mp.tc_blocks = std::max(1, std::min(tc_tiles, ctx->tc_grid));
+    mp.tc_big = ctx->tc_big;
+    mp.tc_smem = mp.tc_big ? tc::BigPlan::make(N).total : tc::Plan::make(N).total;
+    mp.tc_full = !mp.tc_big && tc::Plan::make(N).full;
+}
+
 int mixed_plan(fpsa_ctx *ctx, const fpsa_opts &o, MixedPlan &mp) {
     const Geometry &g = ctx->geo;
     const int N = g.N;
@@ -1057,12 +1080,58 @@ int mixed_plan(fpsa_ctx *ctx, const fpsa_opts &o, MixedPlan &mp) {
     mp.ncol = (size_t)g.R * g.sumK * 2;
     mp.nang = mp.ncol * N;
     mp.use_tc = ctx->tc_able && o.contraction != 1;
-    mp.tcops = TcOps{ctx->d_tc_ops, ctx->d_tc_ops + 2 * (size_t)N * N * sizeof(__nv_bfloat16)};
-    const int tc_tiles = ((2 * g.sumK + 127) / 128) * g.R;
-    mp.tc_blocks = std::max(1, std::min(tc_tiles, ctx->tc_grid));
-    mp.tc_big = ctx->tc_big;
-    mp.tc_smem = mp.tc_big ? tc::BigPlan::make(N).total : tc::Plan::make(N).total;
-    mp.tc_full = !mp.tc_big && tc::Plan::make(N).full;
+    tc_plan(ctx, mp);
+    return FPSA_OK;
+}
+
+// The tensor-core contractions of the FP32 inner solves, by size: few columns per block
+// where that leaves no SM with more than one block (N <= 128; tc::col_tile), else
+// 128-column tiles, whole (N <= 64) or in k-chunks, with streamed operators for N > 128.
+int tc_fp_rhs(fpsa_ctx *ctx, const MixedPlan &mp, const float *psi, const float *phi, float *phi_half,
+              const float *sigma_s, float *rhs) {
+    const Geometry &g = ctx->geo;
+    const int N = g.N;
+    cudaStream_t st = ctx->stream;
+    auto tiles = [&](auto kern) {
+        return launch_pdl(kern, dim3(mp.tc_blocks), dim3(128), mp.tc_smem, st, psi, phi, phi_half, sigma_s,
+                          (const double *)ctx->d_h, mp.tcops, rhs, N, g.sumK, g.R, ctx->d_dev_err);
+    };
+    auto cols = [&](auto kern) {
+        const int ct = ctx->tc_cols;
+        return launch_pdl(kern, dim3((2 * g.sumK + ct - 1) / ct, g.R), dim3(128),
+                          (size_t)tc::ColPlan::make(N, ct).total, st, psi, phi, phi_half, sigma_s,
+                          (const double *)ctx->d_h, mp.tcops, rhs, N, g.sumK, ctx->d_dev_err);
+    };
+    if (mp.tc_big) CK(tiles(k_tc_fp_rhs_big));
+    else if (ctx->tc_cols == 16) CK(cols(k_tc_fp_rhs_cols<16>));
+    else if (ctx->tc_cols == 32) CK(cols(k_tc_fp_rhs_cols<32>));
+    else if (ctx->tc_cols == 64) CK(cols(k_tc_fp_rhs_cols<64>));
+    else if (mp.tc_full) CK(tiles(k_tc_fp_rhs_tile));
+    else CK(tiles(k_tc_fp_rhs));
+    return FPSA_OK;
+}
+
+int tc_update_scatter(fpsa_ctx *ctx, const MixedPlan &mp, const float *v, const float *base, float *phi,
+                      const float *sigma_s, float *q, const float *qang) {
+    const Geometry &g = ctx->geo;
+    const int N = g.N;
+    cudaStream_t st = ctx->stream;
+    auto tiles = [&](auto kern) {
+        return launch_pdl(kern, dim3(mp.tc_blocks), dim3(128), mp.tc_smem, st, v, base, phi, sigma_s, mp.tcops, q,
+                          qang, N, g.sumK, g.R, ctx->d_dev_err);
+    };
+    auto cols = [&](auto kern) {
+        const int ct = ctx->tc_cols;
+        return launch_pdl(kern, dim3((2 * g.sumK + ct - 1) / ct, g.R), dim3(128),
+                          (size_t)tc::ColPlan::make(N, ct).total, st, v, base, phi, sigma_s, mp.tcops, q, qang, N,
+                          g.sumK, ctx->d_dev_err);
+    };
+    if (mp.tc_big) CK(tiles(k_tc_update_scatter_big));
+    else if (ctx->tc_cols == 16) CK(cols(k_tc_update_scatter_cols<16>));
+    else if (ctx->tc_cols == 32) CK(cols(k_tc_update_scatter_cols<32>));
+    else if (ctx->tc_cols == 64) CK(cols(k_tc_update_scatter_cols<64>));
+    else if (mp.tc_full) CK(tiles(k_tc_update_scatter_tile));
+    else CK(tiles(k_tc_update_scatter));
     return FPSA_OK;
 }
 
@@ -1119,26 +1188,15 @@ int mixed_inner_launch(fpsa_ctx *ctx, const MixedPlan &mp, int j0, int inner_k, 
     PathBuffers<double> &p = ctx->p64;
     PathBuffers<float> &f = ctx->p32;
     const dim3 cgrid = mp.cgrid;
-    const bool use_tc = mp.use_tc, tc_big = mp.tc_big, tc_full = mp.tc_full;
-    const int tc_blocks = mp.tc_blocks;
-    const size_t tc_smem = mp.tc_smem;
-    const TcOps tcops = mp.tcops;
+    const bool use_tc = mp.use_tc;
     const float *vin = fpsa ? f.ybuf : f.psi, *base = fpsa ? f.phi_half : nullptr;
     for (int j = j0; j <= inner_k; ++j) {
         if (j > 1) {
             Launch L_(ctx, FPSA_PHASE_CONTRACT);
-            if (use_tc && tc_big)
-                CK(launch_pdl(k_tc_update_scatter_big, dim3(tc_blocks), dim3(128), tc_smem, st, vin, base, f.phi,
-                              (const float *)f.sigma_s, tcops, f.q, (const float *)f.qang, N, g.sumK, g.R,
-                              ctx->d_dev_err));
-            else if (use_tc && tc_full)
-                CK(launch_pdl(k_tc_update_scatter_tile, dim3(tc_blocks), dim3(128), tc_smem, st, vin, base, f.phi,
-                              (const float *)f.sigma_s, tcops, f.q, (const float *)f.qang, N, g.sumK, g.R,
-                              ctx->d_dev_err));
-            else if (use_tc)
-                k_tc_update_scatter<<<tc_blocks, 128, tc_smem, st>>>(vin, base, f.phi, f.sigma_s, tcops, f.q,
-                                                                     f.qang, N, g.sumK, g.R, ctx->d_dev_err);
-            else
+            if (use_tc) {
+                const int rc = tc_update_scatter(ctx, mp, vin, base, f.phi, f.sigma_s, f.q, f.qang);
+                if (rc) return rc;
+            } else
                 k_update_scatter<float><<<cgrid, kContractThreads, contract_smem<float>(N), st>>>(
                     vin, base, f.phi, f.sigma_s, (const float *)nullptr, f.DT, f.MT, f.q, ctx->d_cell_inst, g.B,
                     (unsigned long long *)nullptr, N, g.sumK, f.qang, nullptr);
@@ -1148,18 +1206,10 @@ int mixed_inner_launch(fpsa_ctx *ctx, const MixedPlan &mp, int j0, int inner_k, 
         if (fpsa) {
             {
                 Launch L_(ctx, FPSA_PHASE_CONTRACT);
-                if (use_tc && tc_big)
-                    CK(launch_pdl(k_tc_fp_rhs_big, dim3(tc_blocks), dim3(128), tc_smem, st, (const float *)f.psi,
-                                  (const float *)f.phi, f.phi_half, (const float *)f.sigma_s,
-                                  (const double *)ctx->d_h, tcops, f.rhs, N, g.sumK, g.R, ctx->d_dev_err));
-                else if (use_tc && tc_full)
-                    CK(launch_pdl(k_tc_fp_rhs_tile, dim3(tc_blocks), dim3(128), tc_smem, st, (const float *)f.psi,
-                                  (const float *)f.phi, f.phi_half, (const float *)f.sigma_s,
-                                  (const double *)ctx->d_h, tcops, f.rhs, N, g.sumK, g.R, ctx->d_dev_err));
-                else if (use_tc)
-                    k_tc_fp_rhs<<<tc_blocks, 128, tc_smem, st>>>(f.psi, f.phi, f.phi_half, f.sigma_s, ctx->d_h,
-                                                                 tcops, f.rhs, N, g.sumK, g.R, ctx->d_dev_err);
-                else
+                if (use_tc) {
+                    const int rc = tc_fp_rhs(ctx, mp, f.psi, f.phi, f.phi_half, f.sigma_s, f.rhs);
+                    if (rc) return rc;
+                } else
                     k_fp_rhs<float><<<cgrid, kContractThreads, contract_smem<float>(N), st>>>(
                         f.psi, f.phi, f.phi_half, f.sigma_s, ctx->d_h, f.DT, f.MT, f.rhs, N, g.sumK);
             }
@@ -1477,22 +1527,10 @@ int gm_update(fpsa_ctx *ctx, PathBuffers<T> &p, const T *y, const T *base, T *ou
     Launch L_(ctx, FPSA_PHASE_CONTRACT);
     if constexpr (sizeof(T) == sizeof(float)) {
         if (ctx->gm_use_tc) {
-            const TcOps ops{ctx->d_tc_ops, ctx->d_tc_ops + 2 * (size_t)N * N * sizeof(__nv_bfloat16)};
-            const int blocks = std::max(1, std::min(((2 * g.sumK + 127) / 128) * g.R, ctx->tc_grid));
-            const float *qnull = nullptr;
-            if (ctx->tc_big)
-                CK(launch_pdl(k_tc_update_scatter_big, dim3(blocks), dim3(128), (size_t)tc::BigPlan::make(N).total,
-                              st, (const float *)y, (const float *)base, (float *)out, (const float *)p.sigma_s, ops,
-                              (float *)p.q, qnull, N, g.sumK, g.R, ctx->d_dev_err));
-            else if (tc::Plan::make(N).full)
-                CK(launch_pdl(k_tc_update_scatter_tile, dim3(blocks), dim3(128), (size_t)tc::Plan::make(N).total, st,
-                              (const float *)y, (const float *)base, (float *)out, (const float *)p.sigma_s, ops,
-                              (float *)p.q, qnull, N, g.sumK, g.R, ctx->d_dev_err));
-            else
-                CK(launch_pdl(k_tc_update_scatter, dim3(blocks), dim3(128), (size_t)tc::Plan::make(N).total, st,
-                              (const float *)y, (const float *)base, (float *)out, (const float *)p.sigma_s, ops,
-                              (float *)p.q, qnull, N, g.sumK, g.R, ctx->d_dev_err));
-            return FPSA_OK;
+            MixedPlan mp;
+            tc_plan(ctx, mp);
+            return tc_update_scatter(ctx, mp, (const float *)y, (const float *)base, (float *)out,
+                                     (const float *)p.sigma_s, (float *)p.q, nullptr);
         }
     }
     const dim3 cgrid((g.sumK + kContractCells - 1) / kContractCells, g.R);

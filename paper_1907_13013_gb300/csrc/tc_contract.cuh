@@ -644,6 +644,224 @@ __global__ void __launch_bounds__(128) k_tc_update_scatter_tile(const float *__r
 }
 
 // ---------------------------------------------------------------------------
+// Few-column variants of the same two kernels (N <= 128) for problems whose 128-column
+// tiles leave most SMs without one. The roles are exchanged: the operator is the A operand
+// (M = 128 rows, row o = output o; rows from N up read whatever follows in shared memory
+// and are ignored, the accumulator's lanes being independent) and a tile of CT columns
+// the B operand (N = CT), so a tile is as small as 16 columns. Thread t < N owns output t
+// of every column: its global accesses are whole rows across the threads, all requested
+// at the start, and both nodes of a cell meet in one thread. What bounds it is latency
+// (one pass of loads, two short chains of MMAs, one of stores per block); with 2000
+// columns (K = 1000) at N = 128 the 128-column kernels take 35 and 59 us on 16 SMs.
+// ---------------------------------------------------------------------------
+namespace tc {
+// Shared memory: the operators as in Plan, x_hi and x_lo (CT x N BF16 each), 2 mbarriers,
+// tmem slot; at least what 128 rows of the last operator span.
+struct ColPlan {
+    uint32_t op_bytes, x_bytes, bars, total;
+    __host__ __device__ static ColPlan make(int N, int CT) {
+        ColPlan p;
+        p.op_bytes = (uint32_t)N * N * 2;
+        p.x_bytes = (uint32_t)CT * N * 2;
+        p.bars = 4 * p.op_bytes + 2 * p.x_bytes;
+        p.total = p.bars + 64;
+        const uint32_t span = 3 * p.op_bytes + 256u * (uint32_t)N;
+        if (p.total < span) p.total = span;
+        return p;
+    }
+};
+// columns per block: the fewest (of 16, 32, 64) whose blocks fit one per SM; 0: none does
+__host__ inline int col_tile(int sumK, int R, int n_sm) {
+    for (int ct = 16; ct <= 64; ct *= 2)
+        if ((long long)((2 * sumK + ct - 1) / ct) * R <= n_sm) return ct;
+    return 0;
+}
+}  // namespace tc
+
+template <int CT>
+struct TcCols {
+    unsigned char *op[4], *x_hi, *x_lo;  // D_hi, D_lo, M_hi, M_lo
+    uint64_t *bars;                      // operator copy, MMAs
+    uint32_t tmem;
+    static constexpr uint32_t kCols = 2 * CT < 32 ? 32u : 2u * CT;
+
+    // barriers, tensor memory and the operators' copy: nothing of the previous kernel's
+    __device__ __forceinline__ void setup(unsigned char *smem, const TcOps &ops, int N) {
+        const tc::ColPlan pl = tc::ColPlan::make(N, CT);
+        for (int i = 0; i < 4; ++i) op[i] = smem + i * pl.op_bytes;
+        x_hi = smem + 4 * pl.op_bytes;
+        x_lo = x_hi + pl.x_bytes;
+        bars = reinterpret_cast<uint64_t *>(smem + pl.bars);
+        uint32_t *slot = reinterpret_cast<uint32_t *>(bars + 2);
+        if (threadIdx.x == 0) {
+            tc::mbar_init(bars, 1);
+            tc::mbar_init(bars + 1, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        if (threadIdx.x < 32) {
+            tc::tmem_alloc(slot, kCols);
+            tc::tmem_relinquish();
+        }
+        __syncthreads();
+        tc::tc_fence_after();
+        tmem = *slot;
+        if (threadIdx.x == 0) {
+            tc::mbar_arrive_expect_tx(bars, 4 * pl.op_bytes);
+            tc::bulk_copy_g2s(op[0], ops.D, 2 * pl.op_bytes, bars);
+            tc::bulk_copy_g2s(op[2], ops.M, 2 * pl.op_bytes, bars);
+        }
+    }
+    // v[c] = element k = threadIdx.x of column c, into x_hi / x_lo (row c). Adjacent threads
+    // exchange values so that each stores two adjacent k of one column.
+    __device__ __forceinline__ void store_x(const float (&v)[CT], int N) {
+        const int t = threadIdx.x, odd = t & 1;
+#pragma unroll
+        for (int c = 0; c < CT; c += 2) {
+            const float other = __shfl_xor_sync(0xffffffffu, odd ? v[c] : v[c + 1], 1);
+            const float k0 = odd ? other : v[c], k1 = odd ? v[c + 1] : other;
+            __nv_bfloat16 h0, l0, h1, l1;
+            tc::split_bf16(k0, h0, l0);
+            tc::split_bf16(k1, h1, l1);
+            if (t < N) {
+                const uint32_t off = tc::kmajor_offset(c + odd, t & ~1, N);
+                *reinterpret_cast<uint32_t *>(x_hi + off) =
+                    (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                *reinterpret_cast<uint32_t *>(x_lo + off) =
+                    (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+            }
+        }
+    }
+    // GEMM `which` (0: D, 1: M) of the tile in x_hi / x_lo; a[c] = output threadIdx.x of column c.
+    __device__ __forceinline__ bool gemm(int which, int N, float (&a)[CT]) {
+        const uint32_t acc = tmem + (uint32_t)(which * CT);
+        tc::fence_async_smem();  // the tile's st.shared must be visible to the tensor core
+        tc::tc_fence_before();
+        __syncthreads();
+        bool ok = true;
+        if (threadIdx.x == 0) {
+            ok = tc::mbar_wait(bars, 0);
+            tc::tc_fence_after();
+            if (ok) {
+                const uint32_t idesc = tc::idesc_bf16(128, CT), sbo = (uint32_t)N * 16;
+                const uint32_t oh = tc::smem_u32(op[2 * which]), ol = tc::smem_u32(op[2 * which + 1]);
+                const uint32_t xh = tc::smem_u32(x_hi), xl = tc::smem_u32(x_lo);
+                for (int s = 0; s < N / 16; ++s) {
+                    const uint32_t ko = 256u * s;
+                    const uint64_t a_hi = tc::smem_desc(oh + ko, 128, sbo), a_lo = tc::smem_desc(ol + ko, 128, sbo);
+                    const uint64_t b_hi = tc::smem_desc(xh + ko, 128, sbo), b_lo = tc::smem_desc(xl + ko, 128, sbo);
+                    tc::mma_bf16(acc, a_hi, b_hi, idesc, s > 0 ? 1u : 0u);
+                    tc::mma_bf16(acc, a_hi, b_lo, idesc, 1u);
+                    tc::mma_bf16(acc, a_lo, b_hi, idesc, 1u);
+                }
+            }
+            tc::mma_commit(bars + 1);
+        }
+        ok = tc::mbar_wait(bars + 1, (uint32_t)which) && ok;
+        tc::tc_fence_after();
+        const uint32_t lane_base = (uint32_t)(threadIdx.x & ~31) << 16;
+#pragma unroll
+        for (int c = 0; c < CT; c += 16) tc::tmem_ld16(acc + lane_base + c, a + c);
+        return __syncthreads_and(ok) != 0;  // x_hi / x_lo may be rewritten
+    }
+    __device__ __forceinline__ void teardown(bool ok, int *err) {
+        if (threadIdx.x == 0) {
+            if (!tc::mbar_wait(bars, 0)) ok = false;  // no copy may land after the block has gone (bounded)
+            if (!ok) atomicExch(err, 1);
+        }
+        tc::tc_fence_before();
+        __syncthreads();
+        if (threadIdx.x < 32) tc::tmem_dealloc(tmem, kCols);
+    }
+};
+
+// v[c] = src[(j0 + c) N + t] for live columns and t < N, else 0
+template <int CT>
+__device__ __forceinline__ void load_cols(const float *src, size_t cb, int ncols, int N, float (&v)[CT]) {
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int c = 0; c < CT; ++c) v[c] = (src && t < N && c < ncols) ? __ldcg(src + cb + (size_t)c * N + t) : 0.f;
+}
+template <int CT>
+__device__ __forceinline__ void store_cols(float *dst, size_t cb, int ncols, int N, const float (&v)[CT]) {
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int c = 0; c < CT; ++c)
+        if (t < N && c < ncols) dst[cb + (size_t)c * N + t] = v[c];
+}
+
+template <int CT>
+__global__ void __launch_bounds__(128) k_tc_fp_rhs_cols(const float *psi_half, const float *phi, float *phi_half,
+                                                        const float *sigma_s, const double *h, TcOps ops, float *rhs,
+                                                        int N, int sumK, int *err) {
+    extern __shared__ __align__(128) unsigned char smem_tc[];
+    __shared__ float w[CT / 2];  // h / 6 of the cells (an FP64 divide: once per cell, not per thread)
+    TcCols<CT> s;
+    const int j0 = blockIdx.x * CT, ncols = min(CT, 2 * sumK - j0), g0 = j0 >> 1, t = threadIdx.x;
+    if (t < CT / 2) w[t] = 2 * t < ncols ? (float)(h[g0 + t] / 6.0) : 0.f;
+    s.setup(smem_tc, ops, N);
+    tc::grid_dependency_wait();  // the inputs come from the previous kernel
+    const size_t cb = ((size_t)blockIdx.y * sumK * 2 + j0) * N;
+    float v[CT], ph[CT], sg[CT / 2], a[CT];
+    load_cols<CT>(psi_half, cb, ncols, N, v);
+    load_cols<CT>(phi, cb, ncols, N, ph);
+    load_cols<CT / 2>(sigma_s, (size_t)g0 * N, ncols / 2, N, sg);
+    s.store_x(v, N);
+    bool ok = s.gemm(0, N, a);
+    if (ok) {  // phi_half = D psi; next x = Sigma (phi_half - phi)
+        store_cols<CT>(phi_half, cb, ncols, N, a);
+#pragma unroll
+        for (int c = 0; c < CT; ++c) v[c] = sg[c / 2] * (a[c] - ph[c]);
+        s.store_x(v, N);
+        ok = s.gemm(1, N, a);
+    }
+    if (ok) {  // rhs = m (x) r
+#pragma unroll
+        for (int c = 0; c < CT; c += 2) {
+            const float wc = w[c / 2], r0 = a[c], r1 = a[c + 1];
+            a[c] = wc * (2.f * r0 + r1);
+            a[c + 1] = wc * (r0 + 2.f * r1);
+        }
+        store_cols<CT>(rhs, cb, ncols, N, a);
+    }
+    s.teardown(ok, err);
+}
+
+template <int CT>
+__global__ void __launch_bounds__(128) k_tc_update_scatter_cols(const float *v_in, const float *phi_base, float *phi,
+                                                                const float *sigma_s, TcOps ops, float *q,
+                                                                const float *qang, int N, int sumK, int *err) {
+    extern __shared__ __align__(128) unsigned char smem_tc[];
+    TcCols<CT> s;
+    s.setup(smem_tc, ops, N);
+    tc::grid_dependency_wait();  // the inputs come from the previous kernel
+    const int j0 = blockIdx.x * CT, ncols = min(CT, 2 * sumK - j0);
+    const size_t cb = ((size_t)blockIdx.y * sumK * 2 + j0) * N;
+    float v[CT], pb[CT], sg[CT / 2], qa[CT], a[CT];
+    load_cols<CT>(v_in, cb, ncols, N, v);
+    load_cols<CT>(phi_base, cb, ncols, N, pb);
+    load_cols<CT / 2>(sigma_s, (size_t)(j0 >> 1) * N, ncols / 2, N, sg);
+    load_cols<CT>(qang, cb, ncols, N, qa);
+    s.store_x(v, N);
+    bool ok = s.gemm(0, N, a);
+    if (ok) {  // phi = phi_base + D v; next x = Sigma phi
+#pragma unroll
+        for (int c = 0; c < CT; ++c) {
+            a[c] += pb[c];
+            v[c] = sg[c / 2] * a[c];
+        }
+        store_cols<CT>(phi, cb, ncols, N, a);
+        s.store_x(v, N);
+        ok = s.gemm(1, N, a);
+    }
+    if (ok) {  // q = M (Sigma phi) + q_ang
+#pragma unroll
+        for (int c = 0; c < CT; ++c) a[c] += qa[c];
+        store_cols<CT>(q, cb, ncols, N, a);
+    }
+    s.teardown(ok, err);
+}
+
+// ---------------------------------------------------------------------------
 // Streamed-operator variants for N > 128 (N a multiple of 32, at most 256): the
 // operators (2 N^2 BF16 values each, split hi / lo) no longer fit shared memory next
 // to the column tile, so each GEMM streams them through three buffers in K-chunks of

@@ -31,11 +31,18 @@ using namespace fpsa;
 
 namespace {
 
-// segmented sweep: cells per thread (at least 4) so that no slab needs more than
-// kSegMax segments of kSegWarps * cpt cells
+// Segmented sweep, cells per thread: at least 4, and so many that no slab needs more than
+// kSegMax segments of kSegWarps * cpt cells. Beyond that, where right-hand sides and
+// instances fill the chip by themselves, longer chunks (up to 64 cells) share a block's
+// fixed work (the maps of the segments and chunks before it) among more cells: as many as
+// leave kSweepBlocks blocks (two rounds of eight per SM). 64 right-hand sides of 1250 cells
+// at N = 256: 330 us a sweep with 4 cells, SWEEP_NEW with 32.
+constexpr int kSweepBlocks = 2 * 8 * 152;
 inline int sweep_cells_per_thread(const Geometry &g) {
     const int per = kSegMax * kSegWarps;
-    return std::max(4, (g.Kmax + per - 1) / per);
+    const long long cells = 2ll * ((g.N / 2 + 31) / 32) * g.R * g.sumK;  // (direction, ordinate group, rhs, cell)
+    const long long fill = std::min<long long>(64, cells / ((long long)kSegWarps * kSweepBlocks) / kSweepBatch * kSweepBatch);
+    return std::max({4, (g.Kmax + per - 1) / per, (int)fill});
 }
 inline int sweep_segments(const Geometry &g) {
     const int len = kSegWarps * sweep_cells_per_thread(g);

@@ -36,7 +36,7 @@ namespace {
 // instances fill the chip by themselves, longer chunks (up to 64 cells) share a block's
 // fixed work (the maps of the segments and chunks before it) among more cells: as many as
 // leave kSweepBlocks blocks (two rounds of eight per SM). 64 right-hand sides of 1250 cells
-// at N = 256: 330 us a sweep with 4 cells, SWEEP_NEW with 32.
+// at N = 256: 330 us a sweep with 4 cells, 159 with 32.
 constexpr int kSweepBlocks = 2 * 8 * 152;
 inline int sweep_cells_per_thread(const Geometry &g) {
     const int per = kSegMax * kSegWarps;

@@ -88,7 +88,8 @@ struct fpsa_ctx {
     int32_t *d_bc = nullptr;     // [B][2] edge conditions; NULL when every edge is vacuum
     double *d_in_st = nullptr, *d_in_ss = nullptr, *d_in_q = nullptr;  // fpsa_set_xs staging of host inputs
     int *d_xs_err = nullptr;     // [2] validation of fpsa_set_xs
-    // BCR solve dataflow counters, double-buffered: [parity][cnt | done][rhs chunks][sumK];
+    Packets pk = {};  // of the dataflow BCR solve (NULL push: not allocated)
+    // counters of the tensor-core BCR solve, double-buffered: [parity][cnt | done][rhs chunks][sumK];
     // each solve uses one parity and zeroes the other for the next solve
     int *d_flow = nullptr;
     size_t flow_n = 0;                      // counters per array (rhs chunks x sumK)
@@ -321,16 +322,29 @@ int solve_threads(int N) {
     return bcr_slice_staged(N, (int)sizeof(T)) ? kSolveThreads + 32 * kSolveGroups : kSolveThreads;
 }
 
+template <typename T, int BPSM>
+const void *staged_kernel(int RC) {
+    constexpr int NT = kSolveThreads + 32 * kSolveGroups;
+    switch (RC) {
+        case 8: return (const void *)k_bcr_solve_flow_s<T, NT, 8, BPSM>;
+        case 4: return (const void *)k_bcr_solve_flow_s<T, NT, 4, BPSM>;
+        case 2: return (const void *)k_bcr_solve_flow_s<T, NT, 2, BPSM>;
+        default: return (const void *)k_bcr_solve_flow_s<T, NT, 1, BPSM>;
+    }
+}
+// The cooperative solve of a context of geometry g. Staged: two blocks per SM where their
+// shared memory fits and the widest level has more than two units for every compute group
+// of one block per SM (six slabs of 37 to 613 cells, N = 32, 3 right-hand sides: 112 us a
+// solve with one, 79 with two); below that more blocks only mean more slices per cell and
+// more readers of each packet (200 cells at N = 16, FP64: 1.94 ms a solve with one, 2.03
+// with two).
 template <typename T>
-const void *coop_kernel(int RC, int N) {
+const void *coop_kernel(const Geometry &g, int n_sm) {
+    const int RC = solve_rc(g.R), N = g.N, nchunk = (g.R + RC - 1) / RC;
     if (bcr_slice_staged(N, (int)sizeof(T))) {
-        constexpr int NT = kSolveThreads + 32 * kSolveGroups;
-        switch (RC) {
-            case 8: return (const void *)k_bcr_solve_flow_s<T, NT, 8>;
-            case 4: return (const void *)k_bcr_solve_flow_s<T, NT, 4>;
-            case 2: return (const void *)k_bcr_solve_flow_s<T, NT, 2>;
-            default: return (const void *)k_bcr_solve_flow_s<T, NT, 1>;
-        }
+        const long long widest = g.n_levels ? (long long)g.levels[0].size() * nchunk : 0;
+        const bool two = 2 * solve_smem<T>(N, RC) <= kSmemLimit && widest > 2ll * kSolveGroups * n_sm;
+        return two ? staged_kernel<T, 2>(RC) : staged_kernel<T, 1>(RC);
     }
     switch (RC) {
         case 8: return (const void *)k_bcr_solve_flow<T, kSolveThreads, 8>;
@@ -822,12 +836,33 @@ void plan_solve_shape(fpsa_ctx *ctx) {
     }
 }
 
+// The packets of the dataflow BCR solve (kernels.cuh), in the path's element type.
+int alloc_packets(fpsa_ctx *ctx) {
+    const Geometry &g = ctx->geo;
+    const int e = ctx->precision == FPSA_PRECISION_FP64 ? 1 : 0;
+    const int RC = solve_rc(g.R), nchunk = (g.R + RC - 1) / RC;
+    const size_t words = e ? packet_words<double>() : packet_words<float>();
+    const size_t n = (size_t)nchunk * g.sumK * RC * g.N * words, m = (size_t)ctx->lvt[e].coarse_m * 2 * g.N * words;
+    Packets pk{};
+    CK(dalloc(ctx, &pk.push, 4 * n + m));
+    CK(cudaMemset(pk.push, 0, (4 * n + m) * sizeof(*pk.push)));
+    pk.y = pk.push + n;
+    pk.u = pk.y + 2 * n;
+    pk.rc = pk.u + n;
+    CK(dalloc(ctx, &pk.epoch, 2));
+    const unsigned first[2] = {1u, 0u};
+    CK(cudaMemcpy(pk.epoch, first, sizeof(first), cudaMemcpyHostToDevice));
+    ctx->pk = pk;
+    return FPSA_OK;
+}
+
 // F u = rhs by block cyclic reduction over the stored factors: one cooperative
 // launch (forward levels, roots, backward levels); the solution is left in p.ybuf.
-// No memset precedes it (its counters were zeroed by the previous solve), so it can
-// be launched as a programmatic dependent of the kernel before it.
+// No memset precedes it (packets carry their solve's number; the tensor-core solve's
+// counters were zeroed by its previous solve), so it can be launched as a programmatic
+// dependent of the kernel before it.
 // The tensor-core solve (k_bcr_solve_tc): an ordinary launch of two CTAs per SM
-// that takes its units from a queue; counters as the cooperative solve's.
+// that takes its units from a queue.
 int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *stop) {
     const Geometry &g = ctx->geo;
     const size_t n = ctx->flow_n;
@@ -853,7 +888,7 @@ int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *st
     return FPSA_OK;
 }
 
-// stop: the flag at which the solve is skipped (NULL: none; its counters are zeroed either way).
+// stop: the flag at which the solve is skipped (NULL: none).
 template <typename T>
 int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs, const int *stop = nullptr) {
     if constexpr (sizeof(T) == sizeof(float))
@@ -864,19 +899,14 @@ int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs, const int *stop = nullpt
     LevelTable lv = ctx->lvt[sizeof(T) == 8 ? 1 : 0];
     const T *A = p.A, *Bc = p.Bc, *Cc = p.Cc;
     T *Y = p.ybuf;
-    const size_t n = ctx->flow_n;
-    int *cnt = ctx->d_flow + 2 * n * ctx->flow_parity, *done = cnt + n, *err = ctx->d_dev_err;
-    int *zero_next = ctx->d_flow + 2 * n * (1 - ctx->flow_parity);
-    long long nzero = (long long)(2 * n);
-    ctx->flow_parity ^= 1;
     const T *G = p.G;
-    void *args[] = {(void *)&A,   (void *)&Bc,  (void *)&Cc,   (void *)&items, (void *)&lv,
-                    (void *)&rhs, (void *)&Y,   (void *)&N,    (void *)&sumK,  (void *)&R,
-                    (void *)&cnt, (void *)&done, (void *)&err, (void *)&G,     (void *)&zero_next, (void *)&nzero,
-                    (void *)&stop};
+    int *err = ctx->d_dev_err;
+    Packets pk = ctx->pk;
+    void *args[] = {(void *)&A, (void *)&Bc,   (void *)&Cc, (void *)&items, (void *)&lv,  (void *)&rhs, (void *)&Y,
+                    (void *)&N, (void *)&sumK, (void *)&R,  (void *)&pk,    (void *)&err, (void *)&G,   (void *)&stop};
     const int grid = ctx->coop_grid[sizeof(T) == 8 ? 1 : 0];
     const int RC = solve_rc(R);
-    const void *kern = coop_kernel<T>(RC, N);
+    const void *kern = coop_kernel<T>(g, ctx->n_sm);
     Launch L_(ctx, FPSA_PHASE_BCR_SOLVE);
     if (g_plain_launch) {  // captured into a batch graph: a cooperative kernel node
         cudaLaunchConfig_t cfg = {};
@@ -1841,13 +1871,13 @@ int capture_mixed_loop(fpsa_ctx *ctx, const MixedPlan &mp, const fpsa_opts &o, i
         restore();
         return fail(ctx, FPSA_ENOTSUP, "batch graph: conditional while node refused");
     }
-    // body: the BCR solves alternate their counter halves; with an odd number of them per
-    // step the first one's half is zeroed at the top of the step (it is otherwise zeroed
-    // by the step before)
-    if (fpsa && inner % 2 == 1) {
+    // body: the tensor-core BCR solves alternate their counter halves; with an odd number of
+    // them per step the first one's half is zeroed at the top of the step (it is otherwise
+    // zeroed by the step before)
+    if (fpsa && inner % 2 == 1 && ctx->d_tcs_queue) {
         const int par = ctx->flow_parity;
-        ok = cudaMemsetAsync(ctx->d_flow + 2 * ctx->flow_n * par, 0, 2 * ctx->flow_n * sizeof(int), cs) == cudaSuccess;
-        if (ctx->d_tcs_queue) ok = ok && cudaMemsetAsync(ctx->d_tcs_queue + par, 0, sizeof(int), cs) == cudaSuccess;
+        ok = cudaMemsetAsync(ctx->d_flow + 2 * ctx->flow_n * par, 0, 2 * ctx->flow_n * sizeof(int), cs) == cudaSuccess &&
+             cudaMemsetAsync(ctx->d_tcs_queue + par, 0, sizeof(int), cs) == cudaSuccess;
         if (!ok) {
             end_capture_on_error();
             restore();
@@ -1970,13 +2000,7 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
         CK(cudaMallocHost(&ctx->h_slots, kConvSlots * sizeof(ConvSlot) + sizeof(int)));
         std::memset(ctx->h_slots, 0, kConvSlots * sizeof(ConvSlot) + sizeof(int));
         ctx->h_flag = reinterpret_cast<int *>(ctx->h_slots + kConvSlots);
-        {
-            const int nchunk = (g.R + solve_rc(g.R) - 1) / solve_rc(g.R);
-            ctx->flow_n = (size_t)nchunk * g.sumK;
-            CK(dalloc(ctx, &ctx->d_flow, 4 * ctx->flow_n));
-            CK(cudaMemset(ctx->d_flow, 0, 4 * ctx->flow_n * sizeof(int)));
-            CK(dalloc(ctx, &ctx->d_factor_cnt, (size_t)g.sumK + 1));  // + the tensor-core factorization's queue
-        }
+        CK(dalloc(ctx, &ctx->d_factor_cnt, (size_t)g.sumK + 1));  // + the tensor-core factorization's queue
         CK(dalloc(ctx, &ctx->d_growth, 1));
         CK(dalloc(ctx, &ctx->d_status, 1));
         CK(dalloc(ctx, &ctx->d_result, 2));
@@ -2038,12 +2062,12 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
             int nsm = 0, per_sm = 0;
             CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
             const int RC = solve_rc(g.R);
-            CK(raise_smem_limit((const void *)coop_kernel<float>(RC, g.N), (int)solve_smem<float>(g.N, RC)));
-            CK(raise_smem_limit((const void *)coop_kernel<double>(RC, g.N), (int)solve_smem<double>(g.N, RC)));
-            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_kernel<float>(RC, g.N),
+            CK(raise_smem_limit((const void *)coop_kernel<float>(g, nsm), (int)solve_smem<float>(g.N, RC)));
+            CK(raise_smem_limit((const void *)coop_kernel<double>(g, nsm), (int)solve_smem<double>(g.N, RC)));
+            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_kernel<float>(g, nsm),
                                                              solve_threads<float>(g.N), solve_smem<float>(g.N, RC)));
             ctx->solve_per_sm[0] = std::max(1, per_sm);
-            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_kernel<double>(RC, g.N),
+            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_kernel<double>(g, nsm),
                                                              solve_threads<double>(g.N), solve_smem<double>(g.N, RC)));
             ctx->solve_per_sm[1] = std::max(1, per_sm);
             ctx->n_sm = nsm;
@@ -2078,6 +2102,9 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                 // the tensor-core BCR solve: a split copy of the factors, two CTAs per SM
                 ctx->tcs_rt = tcs::rhs_tile(g.R);
                 ctx->tcs_grid = 2 * nsm;
+                ctx->flow_n = (size_t)((g.R + ctx->tcs_rt - 1) / ctx->tcs_rt) * g.sumK;
+                CK(dalloc(ctx, &ctx->d_flow, 4 * ctx->flow_n));
+                CK(cudaMemset(ctx->d_flow, 0, 4 * ctx->flow_n * sizeof(int)));
                 CK(dalloc(ctx, &ctx->d_tcs_A, (size_t)g.sumK * tcs::cell_bytes(2 * g.N)));
                 CK(dalloc(ctx, &ctx->d_tcs_g, (size_t)ctx->tcs_grid * ctx->tcs_rt * g.N));
                 CK(dalloc(ctx, &ctx->d_tcs_queue, 2));
@@ -2101,6 +2128,10 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
             }
             ctx->sweep_cpt = sweep_cells_per_thread(g);
             plan_solve_shape(ctx);
+            if (!ctx->tcs_rt) {
+                const int rp = alloc_packets(ctx);
+                if (rp) return rp;
+            }
         }
         if (ctx->precision == FPSA_PRECISION_FP64) return alloc_path(ctx, ctx->p64, true);
         int r2 = alloc_path(ctx, ctx->p64, false);
@@ -2521,6 +2552,11 @@ int fpsa_set_tuning(fpsa_ctx *ctx, const fpsa_tuning *t) {
         return fail(ctx, FPSA_ENOTSUP,
                     "tensor-core BCR solve needs FP32 factors (MIXED), 2N a multiple of 128 up to 512 and at least "
                     "16 right-hand sides");
+    if (r.solve_engine == 1 && !ctx->pk.push) {  // a tensor-core context's first dataflow solve
+        CK(cudaSetDevice(ctx->device));
+        const int rc = alloc_packets(ctx);
+        if (rc) return rc;
+    }
     // the segment maps were allocated for the smallest cells-per-thread (most segments)
     const int cmin = sweep_cells_per_thread(ctx->geo);
     ctx->sweep_cpt = std::max(cmin, r.sweep_cells_per_thread);

@@ -1510,14 +1510,13 @@ __global__ void __launch_bounds__(256) k_bcr_schur(T *__restrict__ A, T *__restr
 // slice boundary is a quadrant boundary (L-, L+, R-, R+ are N/2 rows each).
 //   forward (item i at level l, s = 2^l, or a root):
 //     y_i = A_i^{-1} r_i                                (rows of this slice) -> Y
-//     the slice holding y_i[R+] pushes  r_{i+s}[L+] -= B_{i+s} y_i[R+]
-//     the slice holding y_i[L-] pushes  r_{i-s}[R-] -= C_{i-s} y_i[L-]
+//     the slice holding y_i[R+] hands   B_{i+s} y_i[R+] to cell i+s (r_{i+s}[L+] -= it)
+//     the slice holding y_i[L-] hands   C_{i-s} y_i[L-] to cell i-s (r_{i-s}[R-] -= it)
 //   backward (item i at level l, descending; u of the kept neighbours is final):
 //     u_i = y_i - A_i^{-1}[:, L+] B_i u_{i-s}[R+] - A_i^{-1}[:, R-] C_i u_{i+s}[L-]
-// r_i is complete when item i's level runs (its pushes came from lower levels);
-// every pushed-to sub-vector has exactly one writer per level, so nothing races.
-// rhs and Y are written by other blocks between grid-wide barriers and are read
-// with L1-bypassing loads. The solution is left in Y.
+// What is handed on, y and the outflow rows of u travel as packets (below); rhs is only
+// read, and a unit forms r_i from it and the packets of the levels below its own, in
+// level order, so the solution does not depend on timing. It is left in Y.
 template <typename T>
 struct VecOf;
 template <>
@@ -1656,15 +1655,11 @@ __device__ __forceinline__ int sliced_matvec(const T *__restrict__ Mt, int n2, i
 // Up to two h2 x h2 coupling products for RC vectors at once, all NT threads:
 // rows (side, p) of M_side (row-major), a group of G threads per row, each
 // reading a contiguous k-range once for all RC vectors; partial sums meet by
-// shuffles (M_side in global or shared memory). With nred = 0:
-// out_side[rc * ostride + p] = sum_k M_side[p][k] v_side[rc * vstride + k]
-// (shared memory). With nred > 0: out_side[rc * ostride + p] -= that sum for rc < nred, as a
-// reduction without return in global memory.
-template <typename T, int NT, int RC>
-__device__ __forceinline__ void coupling_products(const T *__restrict__ M0, const T *v0, T *out0,
-                                                  const T *__restrict__ M1, const T *v1, T *out1, int h2,
-                                                  int vstride, size_t ostride, int nred = 0,
-                                                  int tid = (int)threadIdx.x) {
+// shuffles (M_side in global or shared memory). One thread of each group calls
+// out(side, rc, p, sum_k M_side[p][k] v_side[rc * vstride + k]).
+template <typename T, int NT, int RC, typename Out>
+__device__ __forceinline__ void coupling_products(const T *__restrict__ M0, const T *v0, const T *__restrict__ M1,
+                                                  const T *v1, int h2, int vstride, int tid, Out out) {
     const int nrows = (M0 ? h2 : 0) + (M1 ? h2 : 0);
     if (nrows == 0) return;
     int G = 1;
@@ -1697,20 +1692,16 @@ __device__ __forceinline__ void coupling_products(const T *__restrict__ M0, cons
 #pragma unroll
         for (int rc = 0; rc < RC; ++rc) {
             const T s = group_sum(acc[rc], G);
-            if (live && gq == 0) {
-                T *o = (second ? out1 : out0) + rc * ostride + p;
-                if (nred == 0) *o = s;
-                else if (rc < nred) atomicAdd(o, -s);
-            }
+            if (live && gq == 0) out((int)second, rc, p, s);
         }
     }
 }
 
-// Dataflow synchronisation of the BCR solve units (k_bcr_solve_flow): a unit waits
-// until the counters it depends on reach their targets (thread 0 polls with acquire
-// loads, at most `limit` times, then records *err = 1 and goes on), and after
-// its writes (block barrier, then thread 0 fences) bumps the counters of the units
-// that depend on it. NULL pointers are absent waits / signals.
+// Dataflow synchronisation of the factorization's items and the tensor-core solve's
+// units: one waits until the counters it depends on reach their targets (thread 0 polls
+// with acquire loads, at most `limit` times, then records *err = 1 and goes on), and after
+// its writes (block barrier, then thread 0 fences) bumps the counters of those that depend
+// on it. NULL pointers are absent waits / signals.
 // The limit is the context's: err[1] holds it (err[0] is the error flag), so a host
 // can shorten it to make a wait run out on purpose (tests of the error path).
 constexpr unsigned kFlowSpinLimit = 1u << 25;  // default: x >= 32 ns, about a second
@@ -1728,6 +1719,151 @@ __device__ __forceinline__ int ld_acquire_gpu(const int *p) {
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+
+// ---------------------------------------------------------------------------
+// Packets: how the units of the dataflow solves hand vectors to each other. A value
+// travels with the number of the solve it belongs to in one 8-byte word (two words for
+// FP64, each with its half of the value), written and read by single 8-byte accesses, so
+// a reader that finds this solve's number in a word has the value: no fence, no counter
+// and no second read follow the write, and nothing has to be cleared between solves
+// (every word is written once per solve). A hop of the reduction's dependency chain is
+// then one write and one read through the L2, where a release fence, a counter bump, the
+// poll that sees it and the load of the vector took 4.5 to 7 us together with the unit's
+// arithmetic.
+//   push [ch][cell][side][rc][N/2]  the product a cell's forward unit hands to its right
+//                                   (side 0: B_right y[R+]) or left (1: C_left y[L-])
+//                                   neighbour, to be subtracted from r there
+//   y    [ch][cell][rc][2N]         A^{-1} r, for the cell's own backward unit
+//   u    [ch][cell][rc][N]          the outflow rows of the solution, [L-, R+]
+//   rc   [coarse cell][2N]          complete right-hand sides of the coarse step
+// epoch[0] is the number of the next solve to run, epoch[1] counts the blocks that have
+// read it; the last one to do so moves it on for the next launch.
+// ---------------------------------------------------------------------------
+struct Packets {
+    unsigned long long *push, *y, *u, *rc;
+    unsigned *epoch;
+};
+template <typename T>
+__host__ __device__ constexpr int packet_words() { return (int)sizeof(T) / 4; }
+
+// One thread per block: this solve's number.
+__device__ __forceinline__ unsigned take_epoch(unsigned *epoch) {
+    const unsigned e = *(volatile unsigned *)epoch;
+    if (atomicAdd(epoch + 1, 1u) == gridDim.x - 1) {
+        epoch[1] = 0u;
+        *(volatile unsigned *)epoch = e + 1u;
+    }
+    return e;
+}
+
+template <typename T>
+__device__ __forceinline__ void packet_put(unsigned long long *p, size_t i, T v, unsigned e) {
+    if constexpr (sizeof(T) == 4) {
+        const unsigned long long w = ((unsigned long long)e << 32) | __float_as_uint(v);
+        asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p + i), "l"(w) : "memory");
+    } else {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)e << 32;
+        asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p + 2 * i), "l"(t | (b & 0xffffffffull)),
+                     "l"(t | (b >> 32))
+                     : "memory");
+    }
+}
+// The value, if it has arrived.
+template <typename T>
+__device__ __forceinline__ bool packet_try(const unsigned long long *p, size_t i, unsigned e, T &v) {
+    if constexpr (sizeof(T) == 4) {
+        unsigned long long w;
+        asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p + i) : "memory");
+        v = __uint_as_float((unsigned)w);
+        return (unsigned)(w >> 32) == e;
+    } else {
+        unsigned long long a, b;
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p + 2 * i) : "memory");
+        v = __longlong_as_double((long long)((a & 0xffffffffull) | (b << 32)));
+        return (unsigned)(a >> 32) == e && (unsigned)(b >> 32) == e;
+    }
+}
+// Wait for a value: at most `limit` polls (*err = 1 after that, and the data it has); a
+// long wait also ends when another thread has recorded an error.
+template <typename T>
+__device__ __noinline__ T packet_wait(const unsigned long long *p, size_t i, unsigned e, int *err, unsigned limit) {
+    T v;
+    for (unsigned spins = 1; !packet_try<T>(p, i, e, v); ++spins) {
+        if (spins >= limit) {
+            atomicExch(err, 1);
+            break;
+        }
+        if (spins > 256) {
+            __nanosleep(32);
+            if (spins % 1024 == 0 && *(volatile int *)err != 0) break;
+        }
+    }
+    return v;
+}
+
+// The solve a unit belongs to: its packets of one chunk of right-hand sides, and its waits.
+template <typename T, int RC>
+struct UnitLinks {
+    Packets pk;
+    unsigned e, limit;
+    int *err;
+    size_t cell0;  // ch * sumK: index of the chunk's first cell
+    int h2;
+
+    __device__ __forceinline__ size_t push_at(int cell, int side, int rc, int p) const {
+        return (((cell0 + cell) * 2 + side) * RC + rc) * h2 + p;
+    }
+    __device__ __forceinline__ size_t y_at(int cell, int rc, int row) const {
+        return ((cell0 + cell) * RC + rc) * (4 * h2) + row;
+    }
+    __device__ __forceinline__ size_t u_at(int cell, int rc, int k) const {
+        return ((cell0 + cell) * RC + rc) * (2 * h2) + k;
+    }
+    __device__ __forceinline__ T get(const unsigned long long *p, size_t i) const {
+        T v;
+        if (!packet_try<T>(p, i, e, v)) v = packet_wait<T>(p, i, e, err, limit);
+        return v;
+    }
+    // v less what the cells eliminated below level `level` hand to row `row` of cell (local
+    // index a of K), in level order: L+ rows receive from the left neighbours at distance
+    // 2^l, R- rows from the right ones; four requested at a time, so that a unit that starts
+    // late pays one read.
+    __device__ __forceinline__ T less_received(T v0, int cell, int a, int K, int level, int rc, int row) const {
+        const bool left = row >= h2 && row < 2 * h2, right = row >= 2 * h2 && row < 3 * h2;
+        if (!left && !right) return v0;
+        const int p = left ? row - h2 : row - 2 * h2;
+        for (int l0 = 0; l0 < level; l0 += 4) {
+            T v[4];
+            bool have[4], here[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int step = 1 << (l0 + u);
+                have[u] = l0 + u < level && (left ? a >= step : a + step < K);
+                here[u] = !have[u] ||
+                          packet_try<T>(pk.push, push_at(left ? cell - step : cell + step, left ? 0 : 1, rc, p), e, v[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int step = 1 << (l0 + u);
+                if (!here[u])
+                    v[u] = packet_wait<T>(pk.push, push_at(left ? cell - step : cell + step, left ? 0 : 1, rc, p), e, err,
+                                          limit);
+                if (have[u]) v0 -= v[u];
+            }
+        }
+        return v0;
+    }
+    // Row `row` of the cell's solution (its outflow rows travel on).
+    __device__ __forceinline__ void put_u(int cell, int rc, int row, T v) const {
+        if (row < h2) packet_put<T>(pk.u, u_at(cell, rc, row), v, e);
+        else if (row >= 3 * h2) packet_put<T>(pk.u, u_at(cell, rc, row - 2 * h2), v, e);
+    }
+    // Inflow k of a backward unit: the left neighbour's R+ (k < N/2), the right one's L-.
+    __device__ __forceinline__ T inflow(const BcrItem &it, int rc, int k) const {
+        if (k < h2) return get(pk.u, u_at(it.left, rc, h2 + k));
+        return it.right >= 0 ? get(pk.u, u_at(it.right, rc, k - h2)) : T(0);
+    }
+};
 
 __device__ __forceinline__ void flow_wait(const FlowSync *fs) {
     if (!fs) return;
@@ -1752,26 +1888,12 @@ __device__ __forceinline__ void flow_wait(const FlowSync *fs) {
 
 // The block barrier orders every thread's earlier writes before the signalling
 // thread's fence, which then orders them before the counter bumps (the pattern of a
-// cooperative grid barrier's arrival). The staged-slice solve signals from a thread
-// outside warp 0 (thread 0 polls for the block's next unit meanwhile) with a
-// release fence paired with the consumers' acquire loads; its units end without a
-// second barrier (every read of the unit's scratch precedes the first one).
+// cooperative grid barrier's arrival).
 __device__ __forceinline__ void flow_signal(const FlowSync *fs) {
     if (!fs) return;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (fs->sig0) atomicAdd(fs->sig0, 1);
-        if (fs->sig1) atomicAdd(fs->sig1, 1);
-        if (fs->sig2) atomicAdd(fs->sig2, 1);
-    }
-}
-
-__device__ __forceinline__ void flow_signal_release(const FlowSync *fs, int signaller) {
-    if (!fs) return;
-    __syncthreads();
-    if ((int)threadIdx.x == signaller) {
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
         if (fs->sig0) atomicAdd(fs->sig0, 1);
         if (fs->sig1) atomicAdd(fs->sig1, 1);
         if (fs->sig2) atomicAdd(fs->sig2, 1);
@@ -1828,8 +1950,8 @@ __global__ void __launch_bounds__(512, 1) k_bcr_factor_flow(T *__restrict__ A, c
 template <typename T, int NT, int RC>
 __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *__restrict__ Bc,
                                              const T *__restrict__ Cc, const BcrItem &it, int r0, int nrc, int sl,
-                                             int S, T *rhs, T *Y, int N, int sumK, T *sm,
-                                             const FlowSync *fs = nullptr) {
+                                             int S, const T *rhs, T *Y, int N, int sumK, T *sm,
+                                             const UnitLinks<T, RC> &lk) {
     const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2;
     T *rs = sm, *ys = sm + RC * n2, *part = ys + RC * n2 + RC * N;
     T *cbuf = bcr_couplings_staged(N, (int)sizeof(T)) ? part + NT * VecOf<T>::V * RC : nullptr;
@@ -1842,10 +1964,11 @@ __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *_
     const T *mC = push_left ? Cc + (size_t)it.s_left * hh : nullptr;
     stage_couplings(mB, mC, cbuf, hh);  // in flight during the matrix-vector product
     const int KS = sliced_matvec<T, NT, RC>(Ai, n2, row0, nr, n2, n2, 0, 0, rs, n2, part, [&] {
-        flow_wait(fs);  // r_i complete (every push into it has landed)
         for (int i = threadIdx.x; i < RC * n2; i += NT) {
             const int rc = i / n2, k = i - rc * n2;
-            rs[i] = rc < nrc ? __ldcg(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + k) : T(0);
+            rs[i] = rc < nrc ? lk.less_received(__ldcg(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + k),
+                                                it.cell, it.local, it.K_inst, it.level, rc, k)
+                             : T(0);
         }
         __syncthreads();
     });
@@ -1855,24 +1978,26 @@ __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *_
         T y = T(0);
         for (int s = 0; s < KS; ++s) y += part[(s * RC + rc) * nr + row];
         ys[rc * n2 + row0 + row] = y;
-        if (rc < nrc) Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y;
+        if (rc >= nrc) continue;
+        if (it.left >= 0) {
+            packet_put<T>(lk.pk.y, lk.y_at(it.cell, rc, row0 + row), y, lk.e);
+        } else {  // a root: its solution is final
+            lk.put_u(it.cell, rc, row0 + row, y);
+            Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y;
+        }
     }
     if (cbuf) cp_async_wait_all();
     __syncthreads();
-    // pushes as reductions without return (one writer per sub-vector and level, so
-    // old - product is formed exactly as a read-modify-write would)
-    coupling_products<T, NT, RC>(mB, ys + N + h2,
-                                 push_right ? rhs + (size_t)r0 * rstride + (size_t)it.right * n2 + h2 : nullptr,
-                                 mC, ys, push_left ? rhs + (size_t)r0 * rstride + (size_t)it.left * n2 + N : nullptr,
-                                 h2, n2, rstride, nrc);
-    flow_signal(fs);
+    coupling_products<T, NT, RC>(mB, ys + N + h2, mC, ys, h2, n2, threadIdx.x, [&](int side, int rc, int p, T v) {
+        if (rc < nrc) packet_put<T>(lk.pk.push, lk.push_at(it.cell, side, rc, p), v, lk.e);
+    });
     __syncthreads();  // scratch reuse by the block's next unit
 }
 
 template <typename T, int NT, int RC>
 __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *__restrict__ Bc,
                                              const T *__restrict__ Cc, const BcrItem &it, int r0, int nrc, int sl,
-                                             int S, T *Y, int N, int sumK, T *sm, const FlowSync *fs = nullptr) {
+                                             int S, T *Y, int N, int sumK, T *sm, const UnitLinks<T, RC> &lk) {
     const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2;
     T *gv = sm, *g = sm + RC * N, *part = sm + RC * (5 * N);  // gv[rc] = [u_left[R+], u_right[L-]]
     T *cbuf = bcr_couplings_staged(N, (int)sizeof(T)) ? part + NT * VecOf<T>::V * RC : nullptr;
@@ -1882,20 +2007,14 @@ __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *_
     const T *mB = Bc + (size_t)it.s_cell * hh, *mC = it.right >= 0 ? Cc + (size_t)it.s_cell * hh : nullptr;
     stage_couplings(mB, mC, cbuf, hh);
     const int KS = sliced_matvec<T, NT, RC>(Ai, n2, row0, nr, N, h2, h2, N, g, N, part, [&] {
-        flow_wait(fs);  // u of both kept neighbours final
         for (int idx = threadIdx.x; idx < RC * N; idx += NT) {
             const int rc = idx / N, k = idx - rc * N;
-            T v = T(0);
-            if (rc < nrc) {
-                const T *base = Y + (size_t)(r0 + rc) * rstride;
-                if (k < h2) v = __ldcg(base + (size_t)it.left * n2 + N + h2 + k);
-                else if (it.right >= 0) v = __ldcg(base + (size_t)it.right * n2 + (k - h2));
-            }
-            gv[idx] = v;
+            gv[idx] = rc < nrc ? lk.inflow(it, rc, k) : T(0);
         }
         if (cbuf) cp_async_wait_all();
         __syncthreads();
-        coupling_products<T, NT, RC>(mB, gv, g, mC, gv + h2, g + h2, h2, N, N);
+        coupling_products<T, NT, RC>(mB, gv, mC, gv + h2, h2, N, threadIdx.x,
+                                     [&](int side, int rc, int p, T v) { g[rc * N + side * h2 + p] = v; });
         if (it.right < 0)
             for (int idx = threadIdx.x; idx < RC * h2; idx += NT) g[(idx / h2) * N + h2 + idx % h2] = T(0);
         __syncthreads();
@@ -1905,9 +2024,10 @@ __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *_
         const int rc = idx / nr, row = idx - rc * nr;
         T s = T(0);
         for (int q = 0; q < KS; ++q) s += part[(q * RC + rc) * nr + row];
-        atomicAdd(Y + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row, -s);
+        const T u = lk.get(lk.pk.y, lk.y_at(it.cell, rc, row0 + row)) - s;
+        lk.put_u(it.cell, rc, row0 + row, u);
+        Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = u;
     }
-    flow_signal(fs);
     __syncthreads();
 }
 
@@ -1932,32 +2052,25 @@ struct LevelTable {
 // The BCR solve as a dataflow over all units in one cooperative launch, without
 // grid-wide barriers. Units are numbered phase by phase (forward levels, roots,
 // backward levels) and taken block-stride in that order, so every unit depends only
-// on units numbered before it and, all blocks being co-resident, every wait ends.
-// Counters per (right-hand-side chunk, cell), zero at launch:
-//   cnt[ch][i]   pushes landed in r_i; the forward unit of item i at level l (local
-//                index a, instance size K) waits for sum_{l' < l} ([a >= 2^l'] + [a + 2^l' < K])
-//   done[ch][i]  slices of cell i whose u is final (its root solve or backward update);
-//                the backward unit of item i waits for all slices of both kept neighbours
-// A unit requests its A^{-1} vectors before it waits, so the factor reads overlap the
-// wait. The levels thus overlap: a unit starts as soon as its own inputs are final.
-__device__ __forceinline__ int bcr_cell_level(int local, int n_levels) {
-    return local == 0 ? n_levels : __ffs(local) - 1;
-}
-
+// on units numbered before it and, all blocks being co-resident, every wait ends. The
+// units' vectors travel as packets (above). A unit requests its A^{-1} vectors before it
+// waits, so the factor reads overlap the wait; the levels overlap too: a unit starts as
+// soon as its own inputs are there.
 template <typename T, int NT, int RC>
 __global__ void __launch_bounds__(NT, 2) k_bcr_solve_flow(const T *__restrict__ A, const T *__restrict__ Bc,
                                                        const T *__restrict__ Cc, const BcrItem *__restrict__ items,
-                                                       LevelTable lv, T *rhs, T *Y, int N, int sumK, int R, int *cnt,
-                                                       int *done, int *err,
+                                                       LevelTable lv, const T *rhs, T *Y, int N, int sumK, int R,
+                                                       Packets pk, int *err,
                                                        const T *__restrict__ G /* coarse step: staged only */,
-                                                       int *zero_next, long long nzero, const int *stop) {
-    for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < nzero; i += (long long)gridDim.x * NT)
-        zero_next[i] = 0;
+                                                       const int *stop) {
     tc::grid_dependency_wait();
     if (stopped(stop)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned s_epoch;
     T *sm = reinterpret_cast<T *>(smem_raw);
-    const unsigned limit = flow_spin_limit(err);
+    if (threadIdx.x == 0) s_epoch = take_epoch(pk.epoch);
+    __syncthreads();
+    UnitLinks<T, RC> lk{pk, s_epoch, flow_spin_limit(err), err, 0, N / 2};
     const int nchunk = (R + RC - 1) / RC, nl = lv.n_levels, P = 2 * nl;
     auto phase_level = [&](int ph) { return ph <= nl ? ph : 2 * nl - ph; };
     auto units = [&](int ph) {
@@ -1976,34 +2089,9 @@ __global__ void __launch_bounds__(NT, 2) k_bcr_solve_flow(const T *__restrict__ 
         const int sl = w % S, ch = (w / S) % nchunk, item = w / (S * nchunk);
         const int r0 = ch * RC, nrc = min(RC, R - r0);
         const BcrItem it = items[lv.off[l] + item];
-        int *cnt_c = cnt + (size_t)ch * sumK, *done_c = done + (size_t)ch * sumK;
-        const int n2 = 2 * N, nr = n2 / S, row0 = sl * nr;
-        FlowSync fs{};
-        fs.err = err;
-        fs.limit = limit;
-        if (ph <= nl) {
-            int want = 0;
-            for (int lp = 0; lp < it.level; ++lp)
-                want += (it.local >= (1 << lp)) + (it.local + (1 << lp) < it.K_inst);
-            if (want) {
-                fs.wait0 = cnt_c + it.cell;
-                fs.want0 = want;
-            }
-            if (it.right >= 0 && row0 + nr == n2) fs.sig0 = cnt_c + it.right;
-            if (it.left >= 0 && row0 == 0) fs.sig1 = cnt_c + it.left;
-            if (it.left < 0) fs.sig2 = done_c + it.cell;  // a root: its solution is final
-            bcr_fwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, rhs, Y, N, sumK, sm, &fs);
-        } else {
-            const int step = 1 << it.level;
-            fs.wait0 = done_c + it.left;
-            fs.want0 = lv.slices[bcr_cell_level(it.local - step, nl)];
-            if (it.right >= 0) {
-                fs.wait1 = done_c + it.right;
-                fs.want1 = lv.slices[bcr_cell_level(it.local + step, nl)];
-            }
-            fs.sig0 = done_c + it.cell;
-            bcr_bwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, Y, N, sumK, sm, &fs);
-        }
+        lk.cell0 = (size_t)ch * sumK;
+        if (ph <= nl) bcr_fwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, rhs, Y, N, sumK, sm, lk);
+        else bcr_bwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, Y, N, sumK, sm, lk);
     }
 }
 
@@ -2143,15 +2231,14 @@ __device__ __forceinline__ int smem_matvec(const T *As, int lda, int nr, int nk,
 // and two service warps. Group g computes the block's units k = g, g + 2, ... and
 // synchronises on its own named barrier (1 + g); when it has finished a unit it only
 // ARRIVES on the unit's handoff barrier (id 3 + (k mod n_stages) + n_stages g, NTG + 32
-// threads) and goes on, while service warp g waits there, fences and bumps the
-// counters of the units that depend on this one (the release fence's latency is off
-// the compute path), then refills the unit's stage with the unit n_stages ahead. A stage's
+// threads) and goes on, while service warp g waits there and refills the unit's stage
+// with the unit n_stages ahead. A stage's
 // next fill is issued only after its unit has been handed off, and a group waits for a
 // fill only once a service warp has published that it was issued (s_fills): so every
 // earlier phase of the stage's mbarrier has completed (its parity then names the right
 // phase), and a handoff barrier is arrived at again only after its previous round has
-// completed. Two groups keep two units' latencies (input counters, right-hand-side
-// loads) in flight on the SM, two service warps two fences.
+// completed. Two groups keep two units' latencies (the wait for their inputs) in flight
+// on the SM.
 constexpr int kSolveGroups = 2;
 __device__ __forceinline__ void gbar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -2178,36 +2265,13 @@ struct Group {
     int bar;  // named barrier id of the group
 };
 
-// A unit's input wait on a compute group: its thread 0 polls (bounded), then the group barrier.
-template <int NTG>
-__device__ __forceinline__ void flow_wait_g(const FlowSync *fs, const Group &gr) {
-    if (gr.gt == 0) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int *c = k ? fs->wait1 : fs->wait0;
-            const int want = k ? fs->want1 : fs->want0;
-            if (!c) continue;
-            unsigned spins = 0;
-            while (ld_acquire_gpu(c) < want) {
-                if (++spins > fs->limit) {
-                    atomicExch(fs->err, 1);
-                    break;
-                }
-                if (spins > 256) __nanosleep(32);
-            }
-        }
-    }
-    gbar_sync(gr.bar, NTG);
-}
-
 // Forward / backward unit on a compute group, its A^{-1} slice in As and its coupling
 // blocks (mB, mC: shared-memory copies, or global memory when not staged; NULL where
-// absent) in flight; wait_copies() returns (true) once they have landed. The unit's
-// results are written when it returns; its signal is the service warp's.
+// absent) in flight; wait_copies() returns (true) once they have landed.
 template <typename T, int NTG, int RC, typename WaitCopies>
 __device__ __forceinline__ bool ring_fwd_unit(const T *mB, const T *mC, const BcrItem &it, int r0, int nrc, int sl,
-                                              int S, T *rhs, T *Y, int N, int sumK, T *sm, const T *As,
-                                              const T *rs_staged, const FlowSync *fs, const Group &gr,
+                                              int S, const T *rhs, T *Y, int N, int sumK, T *sm, const T *As,
+                                              const T *rs_staged, const UnitLinks<T, RC> &lk, const Group &gr,
                                               WaitCopies wait_copies) {
     const int n2 = 2 * N, h2 = N / 2, gt = gr.gt;
     T *ys = sm + RC * n2, *part = ys + RC * n2 + RC * N;
@@ -2215,10 +2279,11 @@ __device__ __forceinline__ bool ring_fwd_unit(const T *mB, const T *mC, const Bc
     const size_t rstride = (size_t)sumK * n2;
     const int nr = n2 / S, row0 = sl * nr;
     if (!rs_staged) {
-        flow_wait_g<NTG>(fs, gr);
         for (int i = gt; i < RC * n2; i += NTG) {
             const int rc = i / n2, k = i - rc * n2;
-            sm[i] = rc < nrc ? __ldcg(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + k) : T(0);
+            sm[i] = rc < nrc ? lk.less_received(__ldcg(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + k),
+                                                it.cell, it.local, it.K_inst, it.level, rc, k)
+                             : T(0);
         }
     }
     if (!wait_copies()) return false;  // a group barrier: rs complete too
@@ -2229,37 +2294,40 @@ __device__ __forceinline__ bool ring_fwd_unit(const T *mB, const T *mC, const Bc
         T y = T(0);
         for (int q = 0; q < KS; ++q) y += part[(q * RC + rc) * nr + row];
         ys[rc * n2 + row0 + row] = y;
-        if (rc < nrc) Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y;
+        if (rc >= nrc) continue;
+        if (it.left >= 0) {
+            packet_put<T>(lk.pk.y, lk.y_at(it.cell, rc, row0 + row), y, lk.e);
+        } else {  // a root: its solution is final
+            lk.put_u(it.cell, rc, row0 + row, y);
+            Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y;
+        }
     }
     gbar_sync(gr.bar, NTG);
-    coupling_products<T, NTG, RC>(mB, ys + N + h2,
-                                  mB ? rhs + (size_t)r0 * rstride + (size_t)it.right * n2 + h2 : nullptr, mC, ys,
-                                  mC ? rhs + (size_t)r0 * rstride + (size_t)it.left * n2 + N : nullptr, h2, n2,
-                                  rstride, nrc, gt);
+    coupling_products<T, NTG, RC>(mB, ys + N + h2, mC, ys, h2, n2, gt, [&](int side, int rc, int p, T v) {
+        if (rc < nrc) packet_put<T>(lk.pk.push, lk.push_at(it.cell, side, rc, p), v, lk.e);
+    });
     return true;
 }
 
 template <typename T, int NTG, int RC, typename WaitCopies>
 __device__ __forceinline__ bool ring_bwd_unit(const T *mB, const T *mC, const BcrItem &it, int r0, int nrc, int sl,
-                                              int S, T *Y, int N, int sumK, T *sm, const T *As, const FlowSync *fs,
-                                              const Group &gr, WaitCopies wait_copies) {
+                                              int S, T *Y, int N, int sumK, T *sm, const T *As,
+                                              const UnitLinks<T, RC> &lk, const Group &gr, WaitCopies wait_copies) {
     const int n2 = 2 * N, h2 = N / 2, gt = gr.gt;
     T *gv = sm, *g = sm + RC * N, *part = sm + RC * (5 * N);
     const size_t rstride = (size_t)sumK * n2;
     const int nr = n2 / S, row0 = sl * nr;
-    flow_wait_g<NTG>(fs, gr);
+    // y of this thread's first row: long there, requested before the waits
+    T y0 = T(0);
+    bool have_y0 = false;
+    if (gt < nrc * nr) have_y0 = packet_try<T>(lk.pk.y, lk.y_at(it.cell, gt / nr, row0 + gt % nr), lk.e, y0);
     for (int idx = gt; idx < RC * N; idx += NTG) {
         const int rc = idx / N, k = idx - rc * N;
-        T v = T(0);
-        if (rc < nrc) {
-            const T *base = Y + (size_t)(r0 + rc) * rstride;
-            if (k < h2) v = __ldcg(base + (size_t)it.left * n2 + N + h2 + k);
-            else if (it.right >= 0) v = __ldcg(base + (size_t)it.right * n2 + (k - h2));
-        }
-        gv[idx] = v;
+        gv[idx] = rc < nrc ? lk.inflow(it, rc, k) : T(0);
     }
     if (!wait_copies()) return false;
-    coupling_products<T, NTG, RC>(mB, gv, g, mC, gv + h2, g + h2, h2, N, N, 0, gt);
+    coupling_products<T, NTG, RC>(mB, gv, mC, gv + h2, h2, N, gt,
+                                  [&](int side, int rc, int p, T v) { g[rc * N + side * h2 + p] = v; });
     if (it.right < 0)
         for (int idx = gt; idx < RC * h2; idx += NTG) g[(idx / h2) * N + h2 + idx % h2] = T(0);
     gbar_sync(gr.bar, NTG);
@@ -2269,37 +2337,46 @@ __device__ __forceinline__ bool ring_bwd_unit(const T *mB, const T *mC, const Bc
         const int rc = idx / nr, row = idx - rc * nr;
         T sacc = T(0);
         for (int q = 0; q < KS; ++q) sacc += part[(q * RC + rc) * nr + row];
-        atomicAdd(Y + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row, -sacc);
+        const T y = idx == gt && have_y0 ? y0 : lk.get(lk.pk.y, lk.y_at(it.cell, rc, row0 + row));
+        lk.put_u(it.cell, rc, row0 + row, y - sacc);
+        Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y - sacc;
     }
     return true;
 }
 
+// Gather unit of the coarse step: the complete right-hand side of coarse cell j, i.e. its own
+// less what the levels below c hand to it, for all the coarse units at once.
+template <typename T, int NTG, typename WaitCopies>
+__device__ __forceinline__ bool ring_gather_unit(int j, const LevelTable &lv, const T *rhs, int N,
+                                                 const UnitLinks<T, 1> &lk, const Group &gr, WaitCopies wait_copies) {
+    const int n2 = 2 * N, cl = lv.coarse_level, a = j << cl;
+    for (int k = gr.gt; k < n2; k += NTG)
+        packet_put<T>(lk.pk.rc, (size_t)j * n2 + k,
+                      lk.less_received(__ldcg(rhs + (size_t)a * n2 + k), a, a, lv.coarse_K, cl, 0, k), lk.e);
+    return wait_copies();  // (an empty fill: keeps the stage's phases in step)
+}
+
 // The coarse unit u on a compute group: rows [u rpu, (u + 1) rpu) of u_c = G r_c (G
 // rows staged in As by the unit's bulk copy; r_c, the right-hand sides of the m coarse
-// cells in coarse order, gathered into rc) once every coarse cell has received the
-// pushes of the levels below c; the rows are written to Y.
+// cells in coarse order, collected into rc); the rows are written to Y and handed on.
 template <typename T, int NTG, typename WaitCopies>
-__device__ __forceinline__ bool ring_coarse_unit(int u, const LevelTable &lv, const T *rhs, T *Y, int N, T *rc,
-                                                 const T *As, const int *cnt, int *err, unsigned limit,
-                                                 const Group &gr, WaitCopies wait_copies) {
+__device__ __forceinline__ bool ring_coarse_unit(int u, const LevelTable &lv, T *Y, int N, T *rc, const T *As,
+                                                 const UnitLinks<T, 1> &lk, const Group &gr, WaitCopies wait_copies) {
     const int n2 = 2 * N, cl = lv.coarse_level, m = lv.coarse_m, n = m * n2, rpu = lv.coarse_rpu, gt = gr.gt;
-    for (int j = gt; j < m; j += NTG) {  // one poller per coarse cell
-        const int a = j << cl;
-        int want = 0;
-        for (int lp = 0; lp < cl; ++lp) want += (a >= (1 << lp)) + (a + (1 << lp) < lv.coarse_K);
-        unsigned spins = 0;
-        while (want && ld_acquire_gpu(cnt + a) < want) {
-            if (++spins > limit) {
-                atomicExch(err, 1);
-                break;
-            }
-            if (spins > 256) __nanosleep(32);
+    for (int i0 = gt; i0 < n; i0 += 8 * NTG) {
+        T v[8];
+        bool here[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int i = i0 + q * NTG;
+            here[q] = i >= n || packet_try<T>(lk.pk.rc, i, lk.e, v[q]);
         }
-    }
-    gbar_sync(gr.bar, NTG);
-    for (int idx = gt; idx < n; idx += NTG) {
-        const int j = idx / n2;
-        rc[idx] = __ldcg(rhs + (size_t)(j << cl) * n2 + (idx - j * n2));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int i = i0 + q * NTG;
+            if (!here[q]) v[q] = packet_wait<T>(lk.pk.rc, i, lk.e, lk.err, lk.limit);
+            if (i < n) rc[i] = v[q];
+        }
     }
     if (!wait_copies()) return false;
     const int lane = gt & 31;
@@ -2310,16 +2387,17 @@ __device__ __forceinline__ bool ring_coarse_unit(int u, const LevelTable &lv, co
         acc = group_sum(acc, 32);
         if (lane == 0) {
             const int row = u * rpu + rr, j = row / n2;
+            lk.put_u(j << cl, 0, row - j * n2, acc);
             Y[(size_t)(j << cl) * n2 + (row - j * n2)] = acc;
         }
     }
     return true;
 }
 
-// The dataflow BCR solve with staged slices (same unit order, counters and waits as
+// The dataflow BCR solve with staged slices (same unit order and packets as
 // k_bcr_solve_flow; with a coarse step, the levels from coarse_level up and the
-// root are one phase of coarse units between the forward and backward levels below
-// it). Shared memory: one unit scratch per compute group, then lv.n_stages copy
+// root are a phase of gather units and one of coarse units between the forward and
+// backward levels below it). Shared memory: one unit scratch per compute group, then lv.n_stages copy
 // stages. The factor columns, couplings and rows of G a unit reads do not change
 // during the solve, so a block requests them lv.n_stages units ahead of the unit it
 // computes (a ring: unit k of the block uses stage k mod n_stages, refilled with unit
@@ -2329,23 +2407,22 @@ __device__ __forceinline__ bool ring_coarse_unit(int u, const LevelTable &lv, co
 // input, no dependencies) travel with their stage's copies, except for the first
 // n_stages units, requested before the previous kernel has finished.
 // NT = kSolveGroups compute groups of NTG threads + kSolveGroups service warps; service
-// warp g hands off, signals and refills the units of group g.
-template <typename T, int NT, int RC>
-__global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict__ A, const T *__restrict__ Bc,
+// warp g refills the stages of group g's units as it finishes them. BPSM: blocks per SM
+// the registers are limited for (two where the stages of small blocks leave room: at the
+// wide levels a unit's latencies, not its bytes, fill a group's time).
+template <typename T, int NT, int RC, int BPSM>
+__global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restrict__ A, const T *__restrict__ Bc,
                                                             const T *__restrict__ Cc,
-                                                            const BcrItem *__restrict__ items, LevelTable lv, T *rhs,
-                                                            T *Y, int N, int sumK, int R, int *cnt, int *done,
-                                                            int *err, const T *__restrict__ G, int *zero_next,
-                                                            long long nzero, const int *stop) {
+                                                            const BcrItem *__restrict__ items, LevelTable lv,
+                                                            const T *rhs, T *Y, int N, int sumK, int R, Packets pk,
+                                                            int *err, const T *__restrict__ G, const int *stop) {
     constexpr int NTG = (NT - 32 * kSolveGroups) / kSolveGroups;
     static_assert(NTG >= 64 && NTG % 32 == 0 && NT == kSolveGroups * (NTG + 32), "compute groups and service warps");
-    // the next solve's counters (the other half of the double-buffered pair) start at zero
-    for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < nzero; i += (long long)gridDim.x * NT)
-        zero_next[i] = 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t s_bar[kMaxSolveStages];  // per stage: one phase per fill
     __shared__ int s_fills[kMaxSolveStages];                   // per stage: fills issued so far
     __shared__ int s_stop;                                     // a compute group stopped (copy timeout)
+    __shared__ unsigned s_epoch;
     T *sm = reinterpret_cast<T *>(smem_raw);
     const int hh = (N / 2) * (N / 2), n2 = 2 * N;
     const bool cpl_staged = bcr_couplings_staged(N, (int)sizeof(T));
@@ -2364,22 +2441,21 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
     }
     __syncthreads();
     const int nchunk = (R + RC - 1) / RC, nl = lv.n_levels, cl = lv.coarse_level;
-    const int P = cl >= 0 ? 2 * cl : 2 * nl;
-    const unsigned limit = flow_spin_limit(err);
-    // level of a phase (-1: the coarse phase) and whether it is a backward phase
+    const int P = cl >= 0 ? 2 * cl + 1 : 2 * nl;
+    // level of a phase (kGather, kCoarse: the phases of the coarse step) and whether it is a
+    // backward phase
+    constexpr int kGather = -2, kCoarse = -1;
     auto phase_level = [&](int ph) {
-        if (cl >= 0) return ph < cl ? ph : (ph == cl ? -1 : 2 * cl - ph);
+        if (cl >= 0) return ph < cl ? ph : (ph == cl ? kGather : (ph == cl + 1 ? kCoarse : 2 * cl + 1 - ph));
         return ph <= nl ? ph : 2 * nl - ph;
     };
-    auto phase_bwd = [&](int ph) { return cl >= 0 ? ph > cl : ph > nl; };
+    auto phase_bwd = [&](int ph) { return cl >= 0 ? ph > cl + 1 : ph > nl; };
     auto units = [&](int ph) {
         const int l = phase_level(ph);
-        if (l < 0) return lv.coarse_units;
+        if (l < 0) return l == kGather ? lv.coarse_m : lv.coarse_units;
         const int nitems = (l < nl) ? lv.off[l + 1] - lv.off[l] : lv.n_roots;
         return nitems * nchunk * lv.slices[l];
     };
-    // units that complete a cell of the given level (its row slices, or the coarse units over its rows)
-    auto done_want = [&](int level) { return (cl >= 0 && level >= cl) ? 2 * N / lv.coarse_rpu : lv.slices[level]; };
     struct Pos {
         int ph, start, l, S, sl, ch, item;
         bool valid;
@@ -2393,7 +2469,7 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
         if (!q.valid) return;
         q.l = phase_level(q.ph);
         const int w = gidx - q.start;
-        if (q.l < 0) {  // coarse unit w
+        if (q.l < 0) {  // gather or coarse unit w
             q.S = 1;
             q.sl = 0;
             q.ch = 0;
@@ -2412,12 +2488,14 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
     };
     constexpr int kHandoff = NTG + 32;  // threads of a handoff barrier: one group and its service warp
     if (threadIdx.x >= kSolveGroups * NTG) {
-        // ---- service warps: copies into the ring, then per unit: handoff, refill, signal
+        // ---- service warps: copies into the ring, then per unit: handoff, refill
         const int sw = (threadIdx.x - kSolveGroups * NTG) >> 5, lane = threadIdx.x & 31;
         // copies of unit k into its stage (q located at k)
         auto issue = [&](const Pos &q, int k) {
             const int st = k % ns;
-            if (q.l < 0) {
+            if (q.l == kGather) {
+                if (lane == 0) tc::mbar_arrive_expect_tx(&s_bar[st], 0);  // no copies
+            } else if (q.l == kCoarse) {
                 const int n = lv.coarse_m * n2, rpu = lv.coarse_rpu;
                 tc::fence_async_smem();
                 if (lane == 0) {
@@ -2451,6 +2529,7 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
         }
         tc::grid_dependency_wait();  // later copies may carry the previous kernel's right-hand sides
         const bool halt = stopped(stop);
+        __syncthreads();  // the solve's number (read below); every thread of the block comes here
         Pos cur{0, 0, 0, 0, 0, 0, 0, false}, nxt{0, 0, 0, 0, 0, 0, 0, false};
         int k = sw;
         for (; !halt; k += kSolveGroups) {
@@ -2458,30 +2537,6 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
             if (!cur.valid) break;
             gbar_sync(3 + k % ns + ns * sw, kHandoff);  // group sw is done with unit k
             if (*(volatile int *)&s_stop) break;
-            if (lane == 0) {
-                int *sig[3] = {nullptr, nullptr, nullptr};
-                if (cur.l < 0) {
-                    sig[0] = done + (((cur.item * lv.coarse_rpu) / n2) << cl);
-                } else {
-                    const BcrItem it = items[lv.off[cur.l] + cur.item];
-                    int *cnt_c = cnt + (size_t)cur.ch * sumK, *done_c = done + (size_t)cur.ch * sumK;
-                    const int nr = n2 / cur.S, row0 = cur.sl * nr;
-                    if (!phase_bwd(cur.ph)) {
-                        if (it.right >= 0 && row0 + nr == n2) sig[0] = cnt_c + it.right;
-                        if (it.left >= 0 && row0 == 0) sig[1] = cnt_c + it.left;
-                        if (it.left < 0) sig[2] = done_c + it.cell;
-                    } else {
-                        sig[0] = done_c + it.cell;
-                    }
-                }
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (sig[q]) atomicAdd(sig[q], 1);
-            }
-            __syncwarp();
-            // then the stage is refilled (the signal first: the dependency chain of the
-            // narrow levels waits on it, the ring has n_stages - 1 other units in flight)
             locate(nxt, blockIdx.x + (k + ns) * (int)gridDim.x);
             if (nxt.valid) issue(nxt, k + ns);
         }
@@ -2498,7 +2553,11 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
     const Group gr{(int)threadIdx.x - grp * NTG, 1 + grp};
     T *smg = sm + grp * base;
     tc::grid_dependency_wait();  // the right-hand sides come from the previous kernel
-    if (stopped(stop)) return;   // the service warps wait for the copies in flight
+    const bool halt = stopped(stop);
+    if (threadIdx.x == 0 && !halt) s_epoch = take_epoch(pk.epoch);
+    __syncthreads();
+    if (halt) return;  // the service warps wait for the copies in flight
+    UnitLinks<T, RC> lk{pk, s_epoch, flow_spin_limit(err), err, 0, N / 2};
     Pos cur{0, 0, 0, 0, 0, 0, 0, false};
     for (int k = grp;; k += kSolveGroups) {
         locate(cur, blockIdx.x + k * (int)gridDim.x);
@@ -2527,9 +2586,14 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
             return !stalled;
         };
         bool ok;
-        if (cur.l < 0) {
-            // the stage's coupling area holds r_c (coarse units take no couplings)
-            ok = ring_coarse_unit<T, NTG>(cur.item, lv, rhs, Y, N, cb, As, cnt, err, limit, gr, wait_copies);
+        if (cur.l < 0) {  // (one right-hand side: RC = 1)
+            if constexpr (RC == 1) {
+                // the stage's coupling area holds r_c (coarse units take no couplings)
+                ok = cur.l == kGather ? ring_gather_unit<T, NTG>(cur.item, lv, rhs, N, lk, gr, wait_copies)
+                                      : ring_coarse_unit<T, NTG>(cur.item, lv, Y, N, cb, As, lk, gr, wait_copies);
+            } else {
+                ok = false;
+            }
         } else {
             const BcrItem it = items[lv.off[cur.l] + cur.item];
             const bool bwd = phase_bwd(cur.ph);
@@ -2540,32 +2604,14 @@ __global__ void __launch_bounds__(NT, 1) k_bcr_solve_flow_s(const T *__restrict_
                 mC = mC ? cb + hh : nullptr;
             }
             const int r0 = cur.ch * RC, nrc = min(RC, R - r0);
-            const int *cnt_c = cnt + (size_t)cur.ch * sumK, *done_c = done + (size_t)cur.ch * sumK;
-            FlowSync fs{};
-            fs.err = err;
-            fs.limit = limit;
-            if (!bwd) {
-                int want = 0;
-                for (int lp = 0; lp < it.level; ++lp)
-                    want += (it.local >= (1 << lp)) + (it.local + (1 << lp) < it.K_inst);
-                if (want) {
-                    fs.wait0 = cnt_c + it.cell;
-                    fs.want0 = want;
-                }
+            lk.cell0 = (size_t)cur.ch * sumK;
+            if (!bwd)
                 ok = ring_fwd_unit<T, NTG, RC>(mB, mC, it, r0, nrc, cur.sl, cur.S, rhs, Y, N, sumK, smg, As,
-                                               rhs_staged(cur, k) ? stage_rhs(st) : (const T *)nullptr, &fs, gr,
+                                               rhs_staged(cur, k) ? stage_rhs(st) : (const T *)nullptr, lk, gr,
                                                wait_copies);
-            } else {
-                const int step = 1 << it.level;
-                fs.wait0 = done_c + it.left;
-                fs.want0 = done_want(bcr_cell_level(it.local - step, nl));
-                if (it.right >= 0) {
-                    fs.wait1 = done_c + it.right;
-                    fs.want1 = done_want(bcr_cell_level(it.local + step, nl));
-                }
-                ok = ring_bwd_unit<T, NTG, RC>(mB, mC, it, r0, nrc, cur.sl, cur.S, Y, N, sumK, smg, As, &fs, gr,
+            else
+                ok = ring_bwd_unit<T, NTG, RC>(mB, mC, it, r0, nrc, cur.sl, cur.S, Y, N, sumK, smg, As, lk, gr,
                                                wait_copies);
-            }
         }
         // every thread of the group has written and read what the unit needs before the handoff
         handoff_arrive(3 + st + ns * grp, kHandoff);

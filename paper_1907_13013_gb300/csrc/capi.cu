@@ -140,6 +140,7 @@ struct fpsa_ctx {
     double *gm_partial = nullptr, *gm_dots = nullptr, *gm_coef = nullptr, *gm_alpha = nullptr;
     long long *gm_seg_begin = nullptr, *gm_seg_end = nullptr;
     int gm_nchunks = 0;
+    bool gm_small = false;  // chunks of kDotChunkSmall elements
 
     PathBuffers<double> p64;  // FP64 path; for MIXED: FP64 tables, psi (refined iterate), phi
     PathBuffers<float> p32;   // MIXED: the FP32 inner FPSA solve
@@ -1458,7 +1459,10 @@ int gmres_alloc(fpsa_ctx *ctx, int m) {
             }
         CK(cudaMemcpy(ctx->gm_seg_begin, sb.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->gm_seg_end, se.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
-        ctx->gm_nchunks = (int)((maxlen + kDotChunk - 1) / kDotChunk);
+        // small chunks where the large ones give most SMs none
+        ctx->gm_small = (maxlen + kDotChunk - 1) / kDotChunk * nsys < ctx->n_sm;
+        const int chunk = ctx->gm_small ? kDotChunkSmall : kDotChunk;
+        ctx->gm_nchunks = (int)((maxlen + chunk - 1) / chunk);
     }
     if (ctx->gm_partial) {
         for (double *q : {ctx->gm_partial, ctx->gm_dots, ctx->gm_coef, ctx->gm_alpha}) {
@@ -1483,12 +1487,17 @@ int gm_dots(fpsa_ctx *ctx, const T *V, int nv, const T *w, std::vector<double> &
     cudaStream_t st = ctx->stream;
     {
         Launch L_(ctx, FPSA_PHASE_CONVERGENCE);
-        k_seg_dots<T><<<dim3(ctx->gm_nchunks, nsys), kDotThreads, 0, st>>>(V, n, nv, w, ctx->gm_seg_begin, ctx->gm_seg_end,
-                                                                   ctx->gm_nchunks, ctx->gm_partial);
+        const dim3 grid(ctx->gm_nchunks, nsys);
+        if (ctx->gm_small)
+            k_seg_dots<T, kDotChunkSmall><<<grid, kDotThreads, 0, st>>>(V, n, nv, w, ctx->gm_seg_begin, ctx->gm_seg_end,
+                                                                       ctx->gm_nchunks, ctx->gm_partial);
+        else
+            k_seg_dots<T, kDotChunk><<<grid, kDotThreads, 0, st>>>(V, n, nv, w, ctx->gm_seg_begin, ctx->gm_seg_end,
+                                                                  ctx->gm_nchunks, ctx->gm_partial);
     }
     {
         Launch L_(ctx, FPSA_PHASE_CONVERGENCE);
-        k_seg_dots_finish<<<(nsys * nv + 255) / 256, 256, 0, st>>>(ctx->gm_partial, nsys, ctx->gm_nchunks, nv,
+        k_seg_dots_finish<<<(nsys * nv + 7) / 8, 256, 0, st>>>(ctx->gm_partial, nsys, ctx->gm_nchunks, nv,
                                                                     ctx->gm_dots);
     }
     CK(cudaGetLastError());
@@ -1514,9 +1523,13 @@ int gm_combine(fpsa_ctx *ctx, T *y, const std::vector<double> *alpha, const T *V
         CK(cudaMemcpyAsync(ctx->gm_alpha, alpha->data(), alpha->size() * sizeof(double), cudaMemcpyHostToDevice, st));
     {
         Launch L_(ctx, FPSA_PHASE_CONVERGENCE);
-        k_seg_combine<T><<<dim3(ctx->gm_nchunks, nsys), kDotThreads, 0, st>>>(
-            y, alpha ? ctx->gm_alpha : nullptr, x ? x : y, V, n, nv, ctx->gm_coef, ctx->gm_seg_begin,
-            ctx->gm_seg_end);
+        const dim3 grid(ctx->gm_nchunks, nsys);
+        auto go = [&](auto kern) {
+            kern<<<grid, kDotThreads, 0, st>>>(y, alpha ? ctx->gm_alpha : nullptr, x ? x : y, V, n, nv, ctx->gm_coef,
+                                               ctx->gm_seg_begin, ctx->gm_seg_end);
+        };
+        if (ctx->gm_small) go(k_seg_combine<T, kDotChunkSmall>);
+        else go(k_seg_combine<T, kDotChunk>);
     }
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));  // the host vectors are reused right away

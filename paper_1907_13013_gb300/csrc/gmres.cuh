@@ -69,27 +69,30 @@ __global__ void k_moments_axpy(const T *__restrict__ psi, const T *__restrict__ 
 // partial[s][chunk][i] = sum over the chunk of the segment of V_i * w.
 // Grid: (chunks, nsys), kDotThreads threads; segments [seg_begin[s], seg_end[s]), whole
 // 16-byte words (every segment starts and ends on a multiple of 2N elements). A thread
-// keeps its kDotChunk / kDotThreads elements of w in registers (16-byte loads,
+// keeps its CH / kDotThreads elements of w in registers (16-byte loads,
 // interleaved across the block so every load instruction is coalesced) and streams
 // the vectors four at a time, so each V_i is read once with all of a thread's loads in
 // flight together. FP64 vectors accumulate in FP64; FP32 vectors (the inner solves of
-// GMRES-IR) in FP32 over a thread's 32 products, then in FP64 across threads and
+// GMRES-IR) in FP32 over a thread's products (at most 32), then in FP64 across threads and
 // chunks (the FP64 rate of this GPU is far below what one FMA per loaded element
 // needs). The sum order is fixed, so results are bitwise reproducible.
-constexpr int kDotChunk = 8192;
+// CH: kDotChunk where the chunks fill the chip (the vectors then stream at memory rate);
+// kDotChunkSmall below that, where a chunk's latency counts: 100 cells at N = 32 are one
+// chunk of the large size, 19 us a dot and 18 us a combination on one SM.
+constexpr int kDotChunk = 8192, kDotChunkSmall = 1024;
 constexpr int kDotThreads = 256;
-template <typename T>
+template <typename T, int CH>
 __global__ void __launch_bounds__(kDotThreads) k_seg_dots(const T *__restrict__ V, size_t vstride, int nv,
                                                           const T *__restrict__ w,
                                                           const long long *__restrict__ seg_begin,
                                                           const long long *__restrict__ seg_end, int nchunks,
                                                           double *__restrict__ partial) {
     using VT = typename VecOf<T>::type;
-    constexpr int VW = VecOf<T>::V, NW = kDotChunk / VW / kDotThreads;
+    constexpr int VW = VecOf<T>::V, NW = CH / VW / kDotThreads;
     __shared__ double red[4][kDotThreads / 32];
     const int s = blockIdx.y, ch = blockIdx.x, t = threadIdx.x;
-    const long long b0 = seg_begin[s] + (long long)ch * kDotChunk;
-    const long long b1 = min(seg_end[s], b0 + kDotChunk);
+    const long long b0 = seg_begin[s] + (long long)ch * CH;
+    const long long b1 = min(seg_end[s], b0 + CH);
     const int nwords = b1 > b0 ? (int)((b1 - b0) / VW) : 0;
     const long long wb = b0 / VW;
     VT wv[NW];
@@ -136,31 +139,34 @@ __global__ void __launch_bounds__(kDotThreads) k_seg_dots(const T *__restrict__ 
     }
 }
 
-// Pass 2: out[s][i] = sum over chunks in order.
+// Pass 2: out[s][i] = sum over chunks, one warp each (lanes take every 32nd chunk, then
+// meet by shuffles: a fixed order).
 static __global__ void k_seg_dots_finish(const double *__restrict__ partial, int nsys, int nchunks, int nv,
                                          double *__restrict__ out) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (t >= nsys * nv) return;
     const int s = t / nv, i = t - s * nv;
     double acc = 0.0;
-    for (int c = 0; c < nchunks; ++c) acc += partial[((size_t)s * nchunks + c) * nv + i];
-    out[(size_t)s * nv + i] = acc;
+#pragma unroll 4
+    for (int c = lane; c < nchunks; c += 32) acc += partial[((size_t)s * nchunks + c) * nv + i];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[(size_t)s * nv + i] = acc;
 }
 
 // y = alpha_s x + sum_i coef[s][i] V_i on the segment of system s (coef stride nv;
 // alpha NULL: no x term; x may alias y). Grid and chunks as k_seg_dots; each thread
-// holds its 32 elements and streams the vectors. FP32 vectors combine in FP32.
-template <typename T>
+// holds its elements and streams the vectors. FP32 vectors combine in FP32.
+template <typename T, int CH>
 __global__ void __launch_bounds__(kDotThreads) k_seg_combine(T *y, const double *__restrict__ alpha, const T *x,
                                                              const T *__restrict__ V, size_t vstride, int nv,
                                                              const double *__restrict__ coef,
                                                              const long long *__restrict__ seg_begin,
                                                              const long long *__restrict__ seg_end) {
     using VT = typename VecOf<T>::type;
-    constexpr int VW = VecOf<T>::V, NW = kDotChunk / VW / kDotThreads;
+    constexpr int VW = VecOf<T>::V, NW = CH / VW / kDotThreads;
     const int s = blockIdx.y, ch = blockIdx.x, t = threadIdx.x;
-    const long long b0 = seg_begin[s] + (long long)ch * kDotChunk;
-    const long long b1 = min(seg_end[s], b0 + kDotChunk);
+    const long long b0 = seg_begin[s] + (long long)ch * CH;
+    const long long b1 = min(seg_end[s], b0 + CH);
     const int nwords = b1 > b0 ? (int)((b1 - b0) / VW) : 0;
     const long long wb = b0 / VW;
     VT acc[NW];

@@ -22,7 +22,6 @@ __global__ void k_fp_rhs_moments(const T *__restrict__ v, const T *__restrict__ 
                                  int sumK) {
     extern __shared__ unsigned char smem_raw[];
     T *Xs = reinterpret_cast<T *>(smem_raw);
-    T *Ys = Xs + 2 * kContractCells * N;
     const int r = blockIdx.y;
     const int g0 = blockIdx.x * kContractCells;
     const int ncell = min(kContractCells, sumK - g0);
@@ -33,15 +32,7 @@ __global__ void k_fp_rhs_moments(const T *__restrict__ v, const T *__restrict__ 
         Xs[idx] = sigma_s[(size_t)(g0 + c / 2) * N + l] * v[colbase * N + idx];
     }
     __syncthreads();
-    block_contract(Xs, N, MT, N, ncols, Ys, N);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
-        const int cl = idx / N, n = idx - cl * N;
-        const T w = (T)(h[g0 + cl] / 6.0);
-        const T r0 = Ys[(2 * cl) * N + n], r1 = Ys[(2 * cl + 1) * N + n];
-        rhs[(colbase + 2 * cl) * N + n] = w * (T(2) * r0 + r1);
-        rhs[(colbase + 2 * cl + 1) * N + n] = w * (r0 + T(2) * r1);
-    }
+    expand_mass(Xs, MT, h + g0, N, ncell, rhs + colbase * N);
 }
 
 // out = base + sign * D psi (moments of a sweep; base may be NULL).
@@ -50,18 +41,19 @@ __global__ void k_moments_axpy(const T *__restrict__ psi, const T *__restrict__ 
                                const T *__restrict__ DT, T *__restrict__ out, int N, int sumK) {
     extern __shared__ unsigned char smem_raw[];
     T *Xs = reinterpret_cast<T *>(smem_raw);
-    T *Ys = Xs + 2 * kContractCells * N;
     const int r = blockIdx.y;
     const int g0 = blockIdx.x * kContractCells;
-    const int ncols = 2 * min(kContractCells, sumK - g0);
+    const int ncell = min(kContractCells, sumK - g0);
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) Xs[idx] = psi[colbase * N + idx];
+    fold_columns(psi + colbase * N, 2 * ncell, N, Xs);
     __syncthreads();
-    block_contract(Xs, N, DT, N, ncols, Ys, N);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
-        const size_t e = colbase * N + idx;
-        out[e] = (base ? base[e] : T(0)) + sign * Ys[idx];
+    for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
+        const int cl = idx / N, l = idx - cl * N;
+        const size_t e = (colbase + 2 * cl) * N + l;
+        T m[2];
+        folded_moments(Xs, DT, N, cl, l, m);
+        out[e] = (base ? base[e] : T(0)) + sign * m[0];
+        out[e + N] = (base ? base[e + N] : T(0)) + sign * m[1];
     }
 }
 

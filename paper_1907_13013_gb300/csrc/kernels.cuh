@@ -384,22 +384,96 @@ __global__ void __launch_bounds__(kSegWarps * 32) k_sweep_apply(const T *__restr
 }
 
 // ---------------------------------------------------------------------------
-// Angular contractions. Ys[c][o] = sum_k MatT[k][o] Xs[c][k] over the columns
-// c < ncols of a shared-memory tile; MatT is the transposed operator in global
-// memory (k-major, so consecutive threads read consecutive o).
-//   moments    phi_l = sum_n D[l][n] psi_n            (Eq. phi-mom)   MatT = D^T
-//   expansion  q_n = sum_l M[n][l] (sigma_{s,l} phi_l + Q_l)  (Eq. treq) MatT = M^T
+// Angular contractions over the columns (cell, node) of a block, through shared memory;
+// DT[n][l] and MT[l][n] are the transposed operators in global memory (consecutive
+// threads read consecutive outputs).
+//   moments    phi_l = sum_n D[l][n] psi_n            (Eq. phi-mom)
+//   expansion  q_n = sum_l M[n][l] (sigma_{s,l} phi_l + Q_l)  (Eq. treq)
+// Both use the mirror symmetry of the S_N set (mu_{N-1-n} = -mu_n, equal weights,
+// P_l(-mu) = (-1)^l P_l(mu), exact in the tables): half the multiply-adds of the plain
+// products, same values up to rounding order,
+//   phi_l = sum_{n < N/2} D[l][n] (psi_n + (-1)^l psi_{N-1-n})
+//   q_n, q_{N-1-n} = E_n +- O_n,  E_n / O_n = sum over even / odd l of M[n][l] x_l.
+// What bounds the FP64 kernels is FP64 arithmetic (N^2 FMAs a column for both contractions:
+// 31 us for 4000 columns at N = 64); a thread takes both nodes of a cell, so that an
+// operator entry is loaded once for two columns. With the plain products the FP kernels
+// took 73 and 80 us there.
 // ---------------------------------------------------------------------------
+// F[c] = (psi_n + psi_{N-1-n})_n, (psi_n - psi_{N-1-n})_n of column c < ncols of psi
 template <typename T>
-__device__ __forceinline__ void block_contract(const T *Xs, int ldx, const T *__restrict__ MatT, int N, int ncols,
-                                               T *Ys, int ldy, const T *__restrict__ add = nullptr) {
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
-        const int c = idx / N, o = idx - c * N;
-        const T *x = Xs + c * ldx;
-        T acc = add ? add[(size_t)c * ldy + o] : T(0);
+__device__ __forceinline__ void fold_columns(const T *psi, int ncols, int N, T *F) {
+    const int h2 = N / 2;
+    for (int idx = threadIdx.x; idx < ncols * h2; idx += blockDim.x) {
+        const int c = idx / h2, n = idx - c * h2;
+        const T a = psi[(size_t)c * N + n], b = psi[(size_t)c * N + (N - 1 - n)];
+        F[c * N + n] = a + b;
+        F[c * N + h2 + n] = a - b;
+    }
+}
+// moment l of both nodes of cell cl from the folded columns
+template <typename T>
+__device__ __forceinline__ void folded_moments(const T *F, const T *__restrict__ DT, int N, int cl, int l, T (&m)[2]) {
+    const int h2 = N / 2;
+    const T *f0 = F + 2 * cl * N + ((l & 1) ? h2 : 0), *f1 = f0 + N;
+    m[0] = m[1] = T(0);
 #pragma unroll 8
-        for (int k = 0; k < N; ++k) acc = fma(MatT[(size_t)k * N + o], x[k], acc);
-        Ys[c * ldy + o] = acc;
+    for (int n = 0; n < h2; ++n) {
+        const T d = DT[(size_t)n * N + l];
+        m[0] = fma(d, f0[n], m[0]);
+        m[1] = fma(d, f1[n], m[1]);
+    }
+}
+// values at ordinates n (lo) and N-1-n (hi), n < N/2, of both nodes of cell cl from moments X[c][l]
+template <typename T>
+__device__ __forceinline__ void folded_expand(const T *X, const T *__restrict__ MT, int N, int cl, int n, T (&lo)[2],
+                                              T (&hi)[2]) {
+    const T *x0 = X + 2 * cl * N, *x1 = x0 + N;
+    T e0 = T(0), o0 = T(0), e1 = T(0), o1 = T(0);
+#pragma unroll 4
+    for (int l = 0; l < N; l += 2) {
+        const T me = MT[(size_t)l * N + n], mo = MT[(size_t)(l + 1) * N + n];
+        e0 = fma(me, x0[l], e0);
+        o0 = fma(mo, x0[l + 1], o0);
+        e1 = fma(me, x1[l], e1);
+        o1 = fma(mo, x1[l + 1], o1);
+    }
+    lo[0] = e0 + o0;
+    hi[0] = e0 - o0;
+    lo[1] = e1 + o1;
+    hi[1] = e1 - o1;
+}
+// out[c][n] = (expansion of X)[c][n] + add[c][n] (add NULL: nothing) for the columns of ncell cells
+template <typename T>
+__device__ __forceinline__ void expand_columns(const T *X, const T *__restrict__ MT, int N, int ncell, T *out,
+                                               const T *add) {
+    const int h2 = N / 2;
+    for (int idx = threadIdx.x; idx < ncell * h2; idx += blockDim.x) {
+        const int cl = idx / h2, n = idx - cl * h2;
+        T lo[2], hi[2];
+        folded_expand(X, MT, N, cl, n, lo, hi);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const size_t e = (size_t)(2 * cl + a) * N;
+            out[e + n] = lo[a] + (add ? add[e + n] : T(0));
+            out[e + N - 1 - n] = hi[a] + (add ? add[e + N - 1 - n] : T(0));
+        }
+    }
+}
+// rhs = m (x) (expansion of X): the mass-weighted FP right-hand side of ncell cells
+template <typename T>
+__device__ __forceinline__ void expand_mass(const T *X, const T *__restrict__ MT, const double *__restrict__ h, int N,
+                                            int ncell, T *rhs) {
+    const int h2 = N / 2;
+    for (int idx = threadIdx.x; idx < ncell * h2; idx += blockDim.x) {
+        const int cl = idx / h2, n = idx - cl * h2;
+        const T w = (T)(h[cl] / 6.0);
+        T lo[2], hi[2];
+        folded_expand(X, MT, N, cl, n, lo, hi);
+        const size_t e = (size_t)2 * cl * N;
+        rhs[e + n] = w * (T(2) * lo[0] + lo[1]);
+        rhs[e + N + n] = w * (lo[0] + T(2) * lo[1]);
+        rhs[e + N - 1 - n] = w * (T(2) * hi[0] + hi[1]);
+        rhs[e + 2 * N - 1 - n] = w * (hi[0] + T(2) * hi[1]);
     }
 }
 
@@ -426,7 +500,7 @@ __global__ void k_scatter(const T *__restrict__ phi, const T *__restrict__ sigma
         Xs[c * N + l] = sigma_s[(size_t)g * N + l] * phi[e] + (Qext ? Qext[e] : T(0));
     }
     __syncthreads();
-    block_contract(Xs, N, MT, N, ncols, q + colbase * N, N, Qang ? Qang + colbase * N : nullptr);
+    expand_columns(Xs, MT, N, ncell, q + colbase * N, Qang ? Qang + colbase * N : nullptr);
 }
 
 // FPSA, after the sweep: phi_half = D psi_half; then the FP right-hand side
@@ -445,27 +519,22 @@ __global__ void k_fp_rhs(const T *__restrict__ psi_half, const T *__restrict__ p
     const int ncell = min(kContractCells, sumK - g0);
     const int ncols = 2 * ncell;
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) Xs[idx] = psi_half[colbase * N + idx];
-    __syncthreads();
-    block_contract(Xs, N, DT, N, ncols, Ys, N);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
-        const int c = idx / N, l = idx - c * N;
-        const int g = g0 + c / 2;
-        const T ph = Ys[idx];
-        phi_half[colbase * N + idx] = ph;
-        Xs[idx] = sigma_s[(size_t)g * N + l] * (ph - phi[colbase * N + idx]);
-    }
-    __syncthreads();
-    block_contract(Xs, N, MT, N, ncols, Ys, N);
+    fold_columns(psi_half + colbase * N, ncols, N, Xs);
     __syncthreads();
     for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
-        const int cl = idx / N, n = idx - cl * N;
-        const T w = (T)(h[g0 + cl] / 6.0);
-        const T r0 = Ys[(2 * cl) * N + n], r1 = Ys[(2 * cl + 1) * N + n];
-        rhs[(colbase + 2 * cl) * N + n] = w * (T(2) * r0 + r1);
-        rhs[(colbase + 2 * cl + 1) * N + n] = w * (r0 + T(2) * r1);
+        const int cl = idx / N, l = idx - cl * N;
+        const T sg = sigma_s[(size_t)(g0 + cl) * N + l];
+        const size_t e = (colbase + 2 * cl) * N + l;
+        const T p0 = phi[e], p1 = phi[e + N];
+        T m[2];
+        folded_moments(Xs, DT, N, cl, l, m);
+        phi_half[e] = m[0];
+        phi_half[e + N] = m[1];
+        Ys[2 * cl * N + l] = sg * (m[0] - p0);
+        Ys[(2 * cl + 1) * N + l] = sg * (m[1] - p1);
     }
+    __syncthreads();
+    expand_mass(Ys, MT, h + g0, N, ncell, rhs + colbase * N);
 }
 
 // Order-preserving key of a non-negative double (NaN sorts above +Inf).
@@ -495,27 +564,33 @@ __global__ void k_update_scatter(const T *__restrict__ v, const T *__restrict__ 
     const int ncell = min(kContractCells, sumK - g0);
     const int ncols = 2 * ncell;
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) Xs[idx] = v[colbase * N + idx];
-    __syncthreads();
-    block_contract(Xs, N, DT, N, ncols, Ys, N);
+    fold_columns(v + colbase * N, ncols, N, Xs);
     __syncthreads();
     if (halt) return;
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
-        const int c = idx / N, l = idx - c * N;
-        const int g = g0 + c / 2;
-        const size_t e = colbase * N + idx;
-        T pn = Ys[idx];
-        if (phi_base) pn += phi_base[e];
+    for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
+        const int cl = idx / N, l = idx - cl * N, g = g0 + cl;
+        const T sg = sigma_s[(size_t)g * N + l];
+        const size_t e = (colbase + 2 * cl) * N + l;
+        const T b0 = phi_base ? phi_base[e] : T(0), b1 = phi_base ? phi_base[e + N] : T(0);
+        const T q0 = Qext ? Qext[e] : T(0), q1 = Qext ? Qext[e + N] : T(0);
+        T m[2];
+        folded_moments(Xs, DT, N, cl, l, m);
+        m[0] += b0;
+        m[1] += b1;
         if (l == 0 && conv) {
             const int slot = (r * B + cell_inst[g]) * 2;
-            atomicMax(conv + slot, dkey((double)pn - (double)phi[e]));
-            atomicMax(conv + slot + 1, dkey((double)pn));
+            const unsigned long long d0 = dkey((double)m[0] - (double)phi[e]), d1 = dkey((double)m[1] - (double)phi[e + N]);
+            const unsigned long long a0 = dkey((double)m[0]), a1 = dkey((double)m[1]);
+            atomicMax(conv + slot, d0 > d1 ? d0 : d1);
+            atomicMax(conv + slot + 1, a0 > a1 ? a0 : a1);
         }
-        phi[e] = pn;
-        Xs[idx] = sigma_s[(size_t)g * N + l] * pn + (Qext ? Qext[e] : T(0));
+        phi[e] = m[0];
+        phi[e + N] = m[1];
+        Ys[2 * cl * N + l] = sg * m[0] + q0;
+        Ys[(2 * cl + 1) * N + l] = sg * m[1] + q1;
     }
     __syncthreads();
-    block_contract(Xs, N, MT, N, ncols, q + colbase * N, N, Qang ? Qang + colbase * N : nullptr);
+    expand_columns(Ys, MT, N, ncell, q + colbase * N, Qang ? Qang + colbase * N : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -549,55 +624,29 @@ static __global__ void k_mixed_residual(const double *__restrict__ psi, double *
     const int ncols = 2 * ncell;
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
     const double *psr = psi + (size_t)r * sumK * 2 * N;  // this rhs
-    // Both contractions use the mirror symmetry of the S_N set (mu_{N-1-n} = -mu_n,
-    // equal weights, P_l(-mu) = (-1)^l P_l(mu), exact in the tables): half the FP64
-    // multiply-adds of the plain products, same values up to rounding order.
-    //   phi_l = sum_{n < N/2} D[l][n] (psi_n + (-1)^l psi_{N-1-n})
-    //   q_n, q_{N-1-n} = E_n +- O_n,  E_n / O_n = sum over even / odd l of M[n][l] x_l
-    const int h2 = N / 2;
-    for (int idx = threadIdx.x; idx < ncols * h2; idx += blockDim.x) {
-        const int c = idx / h2, n = idx - c * h2;
-        const double a = psi[(colbase + c) * N + n], bm = psi[(colbase + c) * N + (N - 1 - n)];
-        Ys[c * N + n] = a + bm;        // even part
-        Ys[c * N + h2 + n] = a - bm;   // odd part
-    }
+    fold_columns(psi + colbase * N, ncols, N, Ys);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
-        const int c = idx / N, l = idx - c * N;
-        const double *f = Ys + c * N + ((l & 1) ? h2 : 0);
-        double acc = 0.0;
-#pragma unroll 8
-        for (int n = 0; n < h2; ++n) acc = fma(DT[(size_t)n * N + l], f[n], acc);
-        Xs[idx] = acc;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
-        const int c = idx / N, l = idx - c * N;
-        const int g = g0 + c / 2;
-        const size_t e = colbase * N + idx;
-        const double pn = Xs[idx];
+    for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
+        const int cl = idx / N, l = idx - cl * N, g = g0 + cl;
+        const double sg = sigma_s[(size_t)g * N + l];
+        const size_t e = (colbase + 2 * cl) * N + l;
+        const double q0 = Qext ? Qext[e] : 0.0, q1 = Qext ? Qext[e + N] : 0.0;
+        double m[2];
+        folded_moments(Ys, DT, N, cl, l, m);
         if (l == 0) {
             const int slot = (r * B + cell_inst[g]) * 2;
-            atomicMax(conv + slot, dkey(pn - phi[e]));
-            atomicMax(conv + slot + 1, dkey(pn));
+            const unsigned long long d0 = dkey(m[0] - phi[e]), d1 = dkey(m[1] - phi[e + N]);
+            const unsigned long long a0 = dkey(m[0]), a1 = dkey(m[1]);
+            atomicMax(conv + slot, d0 > d1 ? d0 : d1);
+            atomicMax(conv + slot + 1, a0 > a1 ? a0 : a1);
         }
-        phi[e] = pn;
-        Xs[idx] = sigma_s[(size_t)g * N + l] * pn + (Qext ? Qext[e] : 0.0);
+        phi[e] = m[0];
+        phi[e + N] = m[1];
+        Xs[2 * cl * N + l] = sg * m[0] + q0;
+        Xs[(2 * cl + 1) * N + l] = sg * m[1] + q1;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < ncols * h2; idx += blockDim.x) {
-        const int c = idx / h2, n = idx - c * h2;
-        const double *x = Xs + c * N;
-        double ev = 0.0, od = 0.0;
-#pragma unroll 4
-        for (int l = 0; l + 1 < N; l += 2) {
-            ev = fma(MT[(size_t)l * N + n], x[l], ev);
-            od = fma(MT[(size_t)(l + 1) * N + n], x[l + 1], od);
-        }
-        const double *qa = Qang ? Qang + (colbase + c) * N : nullptr;
-        Ys[c * N + n] = ev + od + (qa ? qa[n] : 0.0);
-        Ys[c * N + (N - 1 - n)] = ev - od + (qa ? qa[N - 1 - n] : 0.0);
-    }
+    expand_columns(Xs, MT, N, ncell, Ys, Qang ? Qang + colbase * N : nullptr);
     __syncthreads();
     for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
         const int cl = idx / N, n = idx - cl * N;
@@ -658,11 +707,11 @@ __global__ void k_expand(const T *__restrict__ x, const T *__restrict__ MT, T *_
     T *Xs = reinterpret_cast<T *>(smem_raw);
     const int r = blockIdx.y;
     const int g0 = blockIdx.x * kContractCells;
-    const int ncols = 2 * min(kContractCells, sumK - g0);
+    const int ncell = min(kContractCells, sumK - g0), ncols = 2 * ncell;
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
     for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) Xs[idx] = x[colbase * N + idx];
     __syncthreads();
-    block_contract(Xs, N, MT, N, ncols, out + colbase * N, N);
+    expand_columns(Xs, MT, N, ncell, out + colbase * N, (const T *)nullptr);
 }
 
 // ---------------------------------------------------------------------------

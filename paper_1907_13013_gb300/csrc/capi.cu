@@ -945,6 +945,15 @@ int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs, const int *stop = nullpt
     return FPSA_OK;
 }
 
+// Moments (padded to N) to the caller's layout (L+1). Rows without padding are one contiguous
+// copy: as a 2D copy into pageable host memory they moved at 3 GB/s.
+cudaError_t copy_moments(const Geometry &g, double *out, const double *phi, int mem, cudaStream_t st) {
+    const size_t ncol = (size_t)g.R * g.sumK * 2;
+    const cudaMemcpyKind kind = mem == FPSA_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    if (g.L1 == g.N) return cudaMemcpyAsync(out, phi, ncol * g.N * sizeof(double), kind, st);
+    return cudaMemcpy2DAsync(out, g.L1 * sizeof(double), phi, g.N * sizeof(double), g.L1 * sizeof(double), ncol, kind, st);
+}
+
 // The next report's target: the change of phi_0 against tol (a negative tol: reported only).
 ConvReport next_report(fpsa_ctx *ctx, double tol) {
     const unsigned seq = ++ctx->conv_seq;
@@ -1066,8 +1075,7 @@ int solve_fp64(fpsa_ctx *ctx, PathBuffers<T> &p, const fpsa_opts &o, const doubl
     stats.sweeps = it;
     stats.rel_change = e;
     if (phi_out)
-        CK(cudaMemcpy2DAsync(phi_out, L1 * sizeof(double), p.phi, N * sizeof(T), L1 * sizeof(double), ncol,
-                             mem == FPSA_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
+        CK(copy_moments(g, phi_out, (const double *)p.phi, mem, st));
     CK(cudaStreamSynchronize(st));
     if (status == FPSA_ENOTCONV)
         fail(ctx, FPSA_ENOTCONV, "not converged after " + std::to_string(o.max_iterations) + " iterations");
@@ -1418,8 +1426,7 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
     stats.sweeps = sweeps;
     stats.rel_change = e;
     if (phi_out)
-        CK(cudaMemcpy2DAsync(phi_out, L1 * sizeof(double), p.phi, N * sizeof(double), L1 * sizeof(double), ncol,
-                             mem == FPSA_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
+        CK(copy_moments(g, phi_out, (const double *)p.phi, mem, st));
     CK(cudaStreamSynchronize(st));
     if (status == FPSA_ENOTCONV)
         fail(ctx, FPSA_ENOTCONV, "not converged after " + std::to_string(o.max_iterations) + " refinement steps");
@@ -1788,8 +1795,7 @@ int solve_gmres(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
     stats.sweeps = sweeps;
     stats.rel_change = worst;
     if (phi_out)
-        CK(cudaMemcpy2DAsync(phi_out, g.L1 * sizeof(double), p.phi, g.N * sizeof(double), g.L1 * sizeof(double), ncol,
-                             mem == FPSA_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, ctx->stream));
+        CK(copy_moments(g, phi_out, p.phi, mem, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (status == FPSA_ENOTCONV)
         fail(ctx, FPSA_ENOTCONV, "GMRES not converged after " + std::to_string(it) + " iterations");
@@ -2416,8 +2422,7 @@ int fpsa_solve_batch(fpsa_ctx *const *ctxs, int32_t n, const fpsa_opts *opts, do
         else if (!(e < o.tol))
             status = fail(c, FPSA_ENOTCONV, "not converged after " + std::to_string(o.max_iterations) + " refinement steps");
         const size_t ncol = (size_t)g.R * g.sumK * 2;
-        CKB(cudaMemcpy2DAsync(phi[i], g.L1 * sizeof(double), c->p64.phi, g.N * sizeof(double), g.L1 * sizeof(double),
-                             ncol, mem == FPSA_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, cs));
+        CKB(copy_moments(g, phi[i], c->p64.phi, mem, cs));
         if (status == FPSA_OK) {
             CKB(cudaMemcpyAsync(c->d_phi_fwd, c->p64.phi, ncol * g.N * sizeof(double), cudaMemcpyDeviceToDevice, cs));
             c->fwd_ready = true;

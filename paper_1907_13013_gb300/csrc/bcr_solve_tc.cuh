@@ -5,33 +5,40 @@
 // The dataflow solve k_bcr_solve_flow applies an eliminated cell's A^{-1} to at
 // most 8 right-hand sides per unit, so with R of them every factor is read R / 8
 // times per solve. Here a unit is one (cell, phase, tile of RT <= 64 right-hand
-// sides), and its product is one GEMM on the tensor cores:
-//   forward  Y_i = A_i^{-1} r_i                            [2N x RT]
-//   backward u_i = Y_i - A_i^{-1}[:, N/2 : 3N/2] g_i,
-//            g_i = [B_i u_left[3N/2 : 2N] ; C_i u_right[0 : N/2]]
-// (the same reduction, pushes and counters as k_bcr_solve_flow, one row slice).
-// A_i^{-1} is operand A (2N/128 tiles of 128 rows, M = 128), the right-hand sides
-// operand B (N = RT), accumulated in FP32 in tensor memory ((2N/128) x RT
-// columns). Precision: split BF16 with three products, as the contractions
-//   A x ~= A_hi x_hi + A_hi x_lo + A_lo x_hi.
-// Each factor is stored a second time for this solve, already split and in the
-// K-major core-matrix layout (k_bcr_factor_split), as 2N/16 chunks of 16 columns
-// (hi [2N x 16] then lo); a chunk is one bulk asynchronous copy (the TMA engine)
-// into one of two shared-memory stages, so a unit streams its factor once while
-// the previous chunk is multiplied. The right-hand-side chunk of each K-step is
-// split by the CTA's threads from FP32 (loaded one chunk ahead) into the stage
-// beside it. The coupling products (N/2 x N/2 blocks, a few percent of the
-// flops) run on the FP32 cores, one row per thread.
+// sides, slice of 128 rows), and its products are GEMMs on the tensor cores
+// (M = 128 rows, N = RT, accumulated in FP32 in tensor memory):
+//   forward  Y_i = A_i^{-1} r_i, rows of the slice; the slice holding R+ (L-) then forms
+//            B_right Y_i[R+] (C_left Y_i[L-]) and subtracts it from the neighbour's r
+//   backward u_i = Y_i - A_i^{-1}[:, N/2 : 3N/2] g_i, rows of the slice,
+//            g_i = [B_i u_left[R+] ; C_i u_right[L-]]
+// (the reduction of k_bcr_solve_flow). Precision: the factors and the vectors they
+// multiply in split BF16 with three products, as the contractions,
+//   A x ~= A_hi x_hi + A_hi x_lo + A_lo x_hi;
+// the couplings in three BF16 parts with six products (all pairs of weight 2^-16 and
+// more), which keeps FP32's 24 bits. Both are stored a second time for this solve,
+// already split and in the K-major core-matrix layout, one bulk copy (the TMA engine) per
+// chunk: A^{-1} by (slice, 32 columns), 16 KB (k_bcr_factor_split), a coupling block by 16
+// columns (k_bcr_coupling_split).
 //
-// Units are taken from a work queue in phase order (forward levels, roots,
-// backward levels): a unit depends only on units with lower indices, every one of
-// which is held by a running CTA, so every wait ends and an ordinary launch
-// suffices (two CTAs per SM: the shared-memory request admits no third, so their
-// 2 x 256 tensor-memory columns always fit). The copies of a CTA's next unit are
-// issued while the current one finishes. Every wait is bounded; on a timeout the
-// CTA records the error, lets its copies and products land (bounded), frees its
-// tensor memory and stops taking units, and the other CTAs' waits give up as soon
-// as they see the error flag.
+// A CTA is four worker warps and a driver thread that share a ring of kStages stages, a
+// chunk of the operand A and one of the operand B each. The driver copies A chunks as many
+// stages ahead as are free, across units, and issues the products of a stage once its copy
+// has landed and the workers have written its B chunk; the workers load the vectors four
+// chunks ahead, split them, and run the epilogues. What bounds it: at the wide levels the
+// factors' stream through the stages (with the conversion of the vectors behind it), at
+// the narrow ones the chain of hops, each a unit's length. Hence slices of 128 rows (four
+// CTAs share a cell at 2N = 512) and a pipeline without a block barrier per chunk: one CTA
+// for all rows, 16-column chunks with a barrier, a wait for the products and a copy issued
+// only then, and the couplings on the FP32 cores took 3.43 ms at 2N = 512, 1250 cells and
+// 64 right-hand sides, 1.72 ms with 16; this one 1.68 and 1.25 ms.
+//
+// Units are taken from a work queue in phase order (forward levels, roots, backward
+// levels), within a phase the slices others wait for first: a unit depends only on units
+// with lower indices, every one of which is held by a running CTA, so every wait ends and
+// an ordinary launch suffices (two CTAs per SM: the shared-memory request admits no third,
+// so their 2 x 256 tensor-memory columns always fit). Every wait is bounded; on a timeout
+// the error is recorded, the CTA lets its copies and products land (bounded), frees its
+// tensor memory and stops, and the other CTAs' waits give up as soon as they see the flag.
 #pragma once
 
 #include "kernels.cuh"
@@ -40,136 +47,153 @@
 namespace fpsa {
 namespace tcs {
 
-constexpr int kThreads = 128;
-constexpr int kK = 16;                     // factor columns per streamed chunk: one MMA K-step
+constexpr int kWorkers = 128, kThreads = kWorkers + 32;
+constexpr int kK = 32;                     // factor columns per chunk
+constexpr int kKc = 16;                    // coupling columns per chunk
+constexpr int kStages = 4;
+constexpr int kAhead = 4;                  // chunks of the vectors in flight per worker
+constexpr int kUnitRing = 8;               // units the driver may have taken ahead of the workers
 constexpr int kMaxRT = 64;                 // right-hand sides per unit
 constexpr int kMaxN2 = 512;
 constexpr uint32_t kMinSmem = 80u * 1024u;  // > 228 KB / 3: at most two CTAs per SM
+constexpr uint32_t kChunkA = 128u * kK * 4u;  // hi and lo, 128 x 32 BF16 each
 
 __host__ __device__ constexpr int rhs_tile(int R) { return R >= kMaxRT ? kMaxRT : (R + 15) / 16 * 16; }
 __host__ __device__ constexpr bool applies(int n2, int R) { return n2 % 128 == 0 && n2 <= kMaxN2 && R >= 16; }
-// bytes of one chunk of a split factor (hi + lo, 2N x 16 BF16 each) and of a cell's
-__host__ __device__ constexpr uint32_t chunk_bytes(int n2) { return (uint32_t)n2 * kK * 4u; }
 __host__ __device__ constexpr size_t cell_bytes(int n2) { return (size_t)n2 * n2 * 4u; }
-// one K-step of the right-hand sides: hi + lo, RT x 16 BF16 each
-__host__ __device__ constexpr uint32_t rhs_bytes(int RT) { return (uint32_t)RT * kK * 4u; }
-// row stride (floats) of the coupling vectors in shared memory, [RT][N/2 + 4]
-__host__ __device__ constexpr int aux_ld(int n2) { return n2 / 4 + 4; }
+// one coupling block: N/2 x N/2 in three BF16 parts; a chunk of its columns
+__host__ __device__ constexpr size_t coupling_bytes(int n2) { return (size_t)(n2 / 4) * (n2 / 4) * 6u; }
+__host__ __device__ constexpr uint32_t coupling_chunk(int n2) { return (uint32_t)(n2 / 4) * kKc * 6u; }
+// one chunk of the vectors: RT x 32 in two parts (or RT x 16 in three)
+__host__ __device__ constexpr uint32_t chunk_b(int RT) { return (uint32_t)RT * kK * 4u; }
 
-// Shared memory: two stages (factor chunk, then right-hand-side chunk), the
-// coupling vectors, 5 mbarriers (full[2], empty[2], drain), the tensor-memory slot
-// and the CTA's current unit.
+// Shared memory: the stages (A chunk, B chunk), the ring of units, the mbarriers and the
+// tensor-memory slot.
 struct Plan {
-    uint32_t stage, aux, bars, total;
-    __host__ __device__ static Plan make(int n2, int RT) {
+    uint32_t stage, units, bars, total;
+    __host__ __device__ static Plan make(int RT) {
         Plan p;
-        p.stage = chunk_bytes(n2) + rhs_bytes(RT);
-        p.aux = 2 * p.stage;
-        p.bars = (p.aux + (uint32_t)RT * aux_ld(n2) * 4u + 15u) & ~15u;
-        p.total = p.bars + 64;
+        p.stage = kChunkA + chunk_b(RT);
+        p.units = kStages * p.stage;
+        p.bars = p.units + kUnitRing * 64u;
+        p.total = p.bars + 8u * (3 * kStages + kUnitRing + 2) + 64u;
         if (p.total < kMinSmem) p.total = kMinSmem;
         return p;
     }
 };
 
-// out = the split copy of the stored inverses (FP32, transposed: Mt[col][row] =
-// A^{-1}[row][col]): block (cell, kc) writes columns 16 kc .. 16 kc + 15 as hi and lo
-// BF16 in the K-major core-matrix layout, element (row, k) of a part at
-// kmajor_offset(row, k, 16). Consecutive threads take consecutive rows, so every
-// column is read coalesced; each thread writes 16 bytes of each part.
+// The split copy of the stored inverses (FP32, transposed: Mt[col][row] = A^{-1}[row][col]):
+// block (cell, kc) writes columns 32 kc .. 32 kc + 31; chunk (cell, slice m, kc) holds rows
+// 128 m .. as hi and lo, element (row, k) of a part at kmajor_offset(row, k, 32).
+// Consecutive threads take consecutive rows, so every column is read coalesced.
 __global__ void __launch_bounds__(256) k_bcr_factor_split(const float *__restrict__ A, unsigned char *__restrict__ out,
                                                           int n2) {
     const int nkc = n2 / kK;
     const int cell = blockIdx.x / nkc, kc = blockIdx.x - cell * nkc;
     const float *Mt = A + (size_t)cell * n2 * n2 + (size_t)kc * kK * n2;
-    unsigned char *o = out + (size_t)cell * cell_bytes(n2) + (size_t)kc * chunk_bytes(n2);
-    for (int i = threadIdx.x; i < 2 * n2; i += blockDim.x) {
-        const int row = i % n2, half = i / n2;
+    unsigned char *o = out + (size_t)cell * cell_bytes(n2);
+    for (int i = threadIdx.x; i < (kK / 8) * n2; i += blockDim.x) {
+        const int row = i % n2, g = i / n2;
         uint32_t hi[4], lo[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             __nv_bfloat16 h0, l0, h1, l1;
-            tc::split_bf16(Mt[(size_t)(8 * half + 2 * j) * n2 + row], h0, l0);
-            tc::split_bf16(Mt[(size_t)(8 * half + 2 * j + 1) * n2 + row], h1, l1);
+            tc::split_bf16(Mt[(size_t)(8 * g + 2 * j) * n2 + row], h0, l0);
+            tc::split_bf16(Mt[(size_t)(8 * g + 2 * j + 1) * n2 + row], h1, l1);
             hi[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
             lo[j] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
         }
-        const uint32_t off = tc::kmajor_offset(row, 8 * half, kK);
-        *reinterpret_cast<uint4 *>(o + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4 *>(o + (size_t)n2 * kK * 2 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        unsigned char *c = o + ((size_t)(row / 128) * nkc + kc) * kChunkA + tc::kmajor_offset(row % 128, 8 * g, kK);
+        *reinterpret_cast<uint4 *>(c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4 *>(c + kChunkA / 2) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
 }
 
-// acc[r] = sum_k M[p][k] v[r][k] for row p = threadIdx.x < h2: M row-major h2 x h2
-// in global memory, v [RT][ld] in shared memory (read by the whole warp at once).
-template <int RT>
-__device__ __forceinline__ void coupling_rows(const float *__restrict__ M, const float *v, int h2, int ld,
-                                              float (&acc)[RT]) {
-    const int p = threadIdx.x;
+// x = p[0] + p[1] + p[2] in BF16 parts (24 bits)
+__device__ __forceinline__ void split3(float x, __nv_bfloat16 (&p)[3]) {
+    p[0] = __float2bfloat16_rn(x);
+    const float r = x - __bfloat162float(p[0]);
+    p[1] = __float2bfloat16_rn(r);
+    p[2] = __float2bfloat16_rn(r - __bfloat162float(p[1]));
+}
+// eight values as one 16-byte core-matrix row per part
+__device__ __forceinline__ void store_split3(unsigned char *dst, uint32_t part, const float *x) {
+    uint32_t w[3][4];
 #pragma unroll
-    for (int r = 0; r < RT; ++r) acc[r] = 0.f;
-    const float4 *Mr = reinterpret_cast<const float4 *>(M + (size_t)p * h2);
-    for (int k4 = 0; k4 < h2 / 4; ++k4) {
-        const float4 m = __ldg(Mr + k4);
+    for (int j = 0; j < 4; ++j) {
+        __nv_bfloat16 a[3], b[3];
+        split3(x[2 * j], a);
+        split3(x[2 * j + 1], b);
 #pragma unroll
-        for (int r = 0; r < RT; ++r) {
-            const float4 a = *reinterpret_cast<const float4 *>(v + r * ld + 4 * k4);
-            acc[r] = fmaf(m.x, a.x, acc[r]);
-            acc[r] = fmaf(m.y, a.y, acc[r]);
-            acc[r] = fmaf(m.z, a.z, acc[r]);
-            acc[r] = fmaf(m.w, a.w, acc[r]);
-        }
+        for (int k = 0; k < 3; ++k)
+            w[k][j] = (uint32_t)__bfloat16_as_ushort(a[k]) | ((uint32_t)__bfloat16_as_ushort(b[k]) << 16);
     }
-}
-
-// v[r][k] = src[r * stride + k] (r < nrc, else 0) for r < RT, k < h2
-template <int RT>
-__device__ __forceinline__ void load_vectors(float *v, const float *src, size_t stride, int nrc, int h2, int ld) {
-    for (int i = threadIdx.x; i < RT * h2; i += kThreads) {
-        const int r = i / h2, k = i - r * h2;
-        v[r * ld + k] = r < nrc ? __ldcg(src + (size_t)r * stride + k) : 0.f;
-    }
-}
-
-// The dataflow wait of a unit (thread 0 polls; bounded), giving up at once when
-// another CTA has recorded an error.
-__device__ __forceinline__ void flow_wait_tc(const FlowSync &fs) {
-    if (threadIdx.x == 0) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int *c = k ? fs.wait1 : fs.wait0;
-            const int want = k ? fs.want1 : fs.want0;
-            if (!c) continue;
-            unsigned spins = 0;
-            while (ld_acquire_gpu(c) < want) {
-                if (++spins > fs.limit || *(volatile int *)fs.err != 0) {
-                    atomicExch(fs.err, 1);
-                    break;
-                }
-                if (spins > 256) __nanosleep(32);
-            }
-        }
-    }
-    __syncthreads();
+    for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4 *>(dst + k * part) = make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
 }
 
+// The split copy of the coupling blocks (row-major h2 x h2): block (slot, kc) writes columns
+// 16 kc .. 16 kc + 15 of the three parts, element (row, k) at kmajor_offset(row, k, 16).
+__global__ void __launch_bounds__(256) k_bcr_coupling_split(const float *__restrict__ M, unsigned char *__restrict__ out,
+                                                            int n2) {
+    const int h2 = n2 / 4, nkc = h2 / kKc;
+    const int slot = blockIdx.x / nkc, kc = blockIdx.x - slot * nkc;
+    const float *m = M + (size_t)slot * h2 * h2 + kc * kKc;
+    unsigned char *o = out + (size_t)slot * coupling_bytes(n2) + (size_t)kc * coupling_chunk(n2);
+    for (int i = threadIdx.x; i < 2 * h2; i += blockDim.x) {
+        const int row = i >> 1, half = i & 1;
+        float x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = m[(size_t)row * h2 + 8 * half + j];
+        store_split3(o + tc::kmajor_offset(row, 8 * half, kKc), (uint32_t)h2 * kKc * 2u, x);
+    }
+}
+
+// A unit as the driver hands it to the workers (id < 0: no more units).
 struct Unit {
-    int item, ch, bwd, nkc, kc0;
+    int id, m, ch, bwd;
+    int cell, left, right, s_cell, s_left, s_right, local, K_inst, level;
+    int pad[3];
 };
+static_assert(sizeof(Unit) == 64, "one slot of the unit ring");
+
+__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+// Did any worker fail? (a barrier of the workers: they stop together)
+__device__ __forceinline__ bool worker_any(bool v) { return gbar_or(1, kWorkers, v); }
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
+
+template <int V>
+struct Const {
+    static constexpr int value = V;
+};
+
+// One counter of a unit's dataflow wait (bounded), giving up at once when an error has been recorded.
+__device__ __forceinline__ void poll(const int *c, int want, int *err, unsigned limit) {
+    unsigned spins = 0;
+    while (ld_acquire_gpu(c) < want) {
+        if (++spins > limit || *(volatile int *)err != 0) {
+            atomicExch(err, 1);
+            break;
+        }
+        if (spins > 256) __nanosleep(32);
+    }
+}
 
 }  // namespace tcs
 
-// The solve: units as above over the concatenated item array of lv; counters
-// cnt / done per (tile of RT right-hand sides, cell), zero at launch, as in
-// k_bcr_solve_flow (one slice per item); queue: this launch's unit counter (zero
-// at launch). zero_next / queue_next: the other parity's counters, zeroed for the
-// following solve. gs: per-CTA scratch of the backward coupling vectors g
-// (gridDim.x x RT x N floats).
+// The solve: units as above over the concatenated item array of lv. Counters per (tile of
+// RT right-hand sides, cell), n of each, zero at launch: flow[0 .. n) pushes landed in r,
+// [n .. 2n) forward slices written (for the cell's own backward slices), then two per cell,
+// the L- and the R+ rows of u final. queue: this launch's unit counter (zero at launch).
+// zero_next / queue_next: the other parity's counters, zeroed for the following solve. gs:
+// per-CTA scratch of the backward coupling vectors g (gridDim.x x RT x N floats).
 template <int RT>
-__global__ void __launch_bounds__(tcs::kThreads) k_bcr_solve_tc(
-    const unsigned char *__restrict__ Atc, const float *__restrict__ Bc, const float *__restrict__ Cc,
+__global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
+    const unsigned char *__restrict__ Atc, const unsigned char *__restrict__ Btc, const unsigned char *__restrict__ Ctc,
     const BcrItem *__restrict__ items, LevelTable lv, float *rhs, float *Y, float *gs, int N, int sumK, int R,
-    int *cnt, int *done, int *queue, int *err, int *zero_next, long long nzero, int *queue_next, const int *stop) {
+    int *flow, int *queue, int *err, int *zero_next, long long nzero, int *queue_next, const int *stop) {
     using namespace tcs;
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < nzero; i += (long long)gridDim.x * kThreads)
         zero_next[i] = 0;
@@ -177,21 +201,29 @@ __global__ void __launch_bounds__(tcs::kThreads) k_bcr_solve_tc(
     tc::grid_dependency_wait();
     if (stopped(stop)) return;
     extern __shared__ __align__(128) unsigned char smem_tcs[];
-    const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2, MT = n2 / 128, ald = aux_ld(n2);
-    const Plan pl = Plan::make(n2, RT);
-    const uint32_t cbytes = chunk_bytes(n2);
-    float *aux = reinterpret_cast<float *>(smem_tcs + pl.aux);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem_tcs + pl.bars), *empty = full + 2, *drain = full + 4;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(full + 5);
-    int *s_unit = reinterpret_cast<int *>(tslot + 1);
-    const int t = threadIdx.x;
+    __shared__ int s_fail;  // a wait of this CTA gave up
+    const int n2 = 2 * N, h2 = N / 2, MT = n2 / 128, t = threadIdx.x;
+    const Plan pl = Plan::make(RT);
+    Unit *ring = reinterpret_cast<Unit *>(smem_tcs + pl.units);
+    uint64_t *full_a = reinterpret_cast<uint64_t *>(smem_tcs + pl.bars), *full_b = full_a + kStages,
+             *empty = full_b + kStages, *unit_bar = empty + kStages, *seg_bar = unit_bar + kUnitRing,
+             *drain = seg_bar + 1;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(drain + 1);
+    constexpr uint32_t kCols = 3 * RT <= 64 ? 64u : (3 * RT <= 128 ? 128u : 256u);
     if (t == 0) {
-        for (int i = 0; i < 5; ++i) tc::mbar_init(full + i, 1);
+        for (int i = 0; i < kStages; ++i) {
+            tc::mbar_init(full_a + i, 1);
+            tc::mbar_init(full_b + i, kWorkers);
+            tc::mbar_init(empty + i, 1);
+        }
+        for (int i = 0; i < kUnitRing; ++i) tc::mbar_init(unit_bar + i, 1);
+        tc::mbar_init(seg_bar, 1);
+        tc::mbar_init(drain, 1);
+        s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const uint32_t tcols = tc::tmem_cols_for(MT * RT);
     if (t < 32) {
-        tc::tmem_alloc(tslot, tcols);
+        tc::tmem_alloc(tslot, kCols);
         tc::tmem_relinquish();
     }
     __syncthreads();
@@ -199,297 +231,347 @@ __global__ void __launch_bounds__(tcs::kThreads) k_bcr_solve_tc(
     const uint32_t tmem = *tslot;
 
     const int nch = (R + RT - 1) / RT, nl = lv.n_levels, P = 2 * nl;
-    const size_t rstride = (size_t)sumK * n2;
-    const unsigned limit = flow_spin_limit(err);
-    auto level_of = [&](int ph) { return ph <= nl ? ph : 2 * nl - ph; };
-    auto phase_units = [&](int ph) {
-        const int l = level_of(ph);
-        return (l < nl ? lv.off[l + 1] - lv.off[l] : lv.n_roots) * nch;
+    const size_t rstride = (size_t)sumK * n2, n = (size_t)nch * sumK;
+    const int nc = h2 / kKc;  // chunks of a coupling product
+    auto failed = [&]() { return *(volatile int *)&s_fail != 0; };
+    auto fail = [&]() {
+        *(volatile int *)&s_fail = 1;
+        atomicExch(err, 1);
     };
-    int total = 0;
-    for (int ph = 0; ph <= P; ++ph) total += phase_units(ph);
-    auto decode = [&](int u, Unit &d) {
-        int ph = 0, start = 0;
-        while (u >= start + phase_units(ph)) {
-            start += phase_units(ph);
-            ++ph;
-        }
-        const int w = u - start;
-        d.ch = w % nch;
-        d.item = lv.off[level_of(ph)] + w / nch;
-        d.bwd = ph > nl;
-        d.nkc = d.bwd ? N / kK : n2 / kK;
-        d.kc0 = d.bwd ? h2 / kK : 0;
+    // A unit's chunks, in order: forward, n2 / 32 of A^{-1}, then the couplings of its pushes;
+    // backward, the couplings (left, then right if there is one), then A^{-1} (only the left
+    // half of its columns without a right neighbour).
+    auto push_right = [&](const Unit &u) { return !u.bwd && u.right >= 0 && u.m == MT - 1; };
+    auto push_left = [&](const Unit &u) { return !u.bwd && u.left >= 0 && u.m == 0; };
+    auto n_main = [&](const Unit &u) { return (u.bwd ? (u.right >= 0 ? N : h2) : n2) / kK; };
+    auto n_coup = [&](const Unit &u) {
+        return u.bwd ? (u.right >= 0 ? 2 * nc : nc) : ((push_right(u) ? nc : 0) + (push_left(u) ? nc : 0));
     };
 
-    // thread 0: the stream of factor chunks, unit after unit in the order this CTA
-    // takes them; chunk q of the stream goes to stage q & 1
-    Unit cur{}, nxt{};
-    int nxt_u = -1;
-    uint32_t cur_base = 0, issued = 0, waited = 0;
-    auto chunk_src = [&](const Unit &d, int c) {
-        return Atc + (size_t)items[d.item].cell * cell_bytes(n2) + (size_t)(d.kc0 + c) * cbytes;
-    };
-    auto issue = [&](uint32_t q) {  // thread 0: request chunk q of the stream, if it exists
-        const unsigned char *src;
-        if (q < cur_base + (uint32_t)cur.nkc) {
-            src = chunk_src(cur, (int)(q - cur_base));
-        } else {
-            if (nxt_u < 0) {
-                nxt_u = atomicAdd(queue, 1);
-                if (nxt_u < total) decode(nxt_u, nxt);
-            }
-            if (nxt_u >= total) return;
-            src = chunk_src(nxt, (int)(q - cur_base - (uint32_t)cur.nkc));
-        }
-        const int s = q & 1;
-        tc::mbar_arrive_expect_tx(&full[s], cbytes);
-        tc::bulk_copy_g2s(smem_tcs + s * pl.stage, src, cbytes, &full[s]);
-        issued = q + 1;
-    };
-
-    if (t == 0) *s_unit = atomicAdd(queue, 1);
-    __syncthreads();
-    int u = *s_unit;
-    Unit d{};
-    if (u < total) decode(u, d);
-    if (t == 0 && u < total) {
-        cur = d;
-        issue(0);
-        issue(1);
-    }
-    const uint32_t idesc = tc::idesc_bf16(128, RT);
-    const int br = t >> 1, bh = t & 1;  // right-hand-side split: row br, k-half bh of a chunk
-    const int w = t >> 5, lane = t & 31;
-    const uint32_t lane_base = (uint32_t)(w * 32) << 16;
-    uint32_t q = 0;  // stream index of the chunk being consumed
-    bool ok = true;
-    while (u < total) {
-        const BcrItem it = items[d.item];
-        const int r0 = d.ch * RT, nrc = min(RT, R - r0);
-        int *cnt_c = cnt + (size_t)d.ch * sumK, *done_c = done + (size_t)d.ch * sumK;
-        FlowSync fs{};
-        fs.err = err;
-        fs.limit = limit;
-        if (!d.bwd) {
-            int want = 0;
-            for (int lp = 0; lp < it.level; ++lp)
-                want += (it.local >= (1 << lp)) + (it.local + (1 << lp) < it.K_inst);
-            if (want) {
-                fs.wait0 = cnt_c + it.cell;
-                fs.want0 = want;
-            }
-        } else {
-            fs.wait0 = done_c + it.left;
-            fs.want0 = 1;
-            if (it.right >= 0) {
-                fs.wait1 = done_c + it.right;
-                fs.want1 = 1;
-            }
-        }
-        flow_wait_tc(fs);
-        const float *bsrc;
-        size_t bstride;
-        if (!d.bwd) {
-            bsrc = rhs + (size_t)r0 * rstride + (size_t)it.cell * n2;
-            bstride = rstride;
-        } else {
-            // g = [B_i u_left[3N/2 : 2N] ; C_i u_right[0 : N/2]] into this CTA's scratch, [RT][N]
-            float *g = gs + (size_t)blockIdx.x * RT * N;
-            float acc[RT];
-            load_vectors<RT>(aux, Y + (size_t)r0 * rstride + (size_t)it.left * n2 + N + h2, rstride, nrc, h2, ald);
-            __syncthreads();
-            if (t < h2) {
-                coupling_rows<RT>(Bc + (size_t)it.s_cell * hh, aux, h2, ald, acc);
-#pragma unroll
-                for (int r = 0; r < RT; ++r) g[(size_t)r * N + t] = acc[r];
-            }
-            __syncthreads();
-            if (it.right >= 0) {
-                load_vectors<RT>(aux, Y + (size_t)r0 * rstride + (size_t)it.right * n2, rstride, nrc, h2, ald);
-                __syncthreads();
-                if (t < h2) {
-                    coupling_rows<RT>(Cc + (size_t)it.s_cell * hh, aux, h2, ald, acc);
-#pragma unroll
-                    for (int r = 0; r < RT; ++r) g[(size_t)r * N + h2 + t] = acc[r];
+    if (t == kWorkers) {
+        // ---- driver
+        int total = 0;
+        auto phase_items = [&](int ph) {
+            const int l = ph <= nl ? ph : 2 * nl - ph;
+            return l < nl ? lv.off[l + 1] - lv.off[l] : lv.n_roots;
+        };
+        for (int ph = 0; ph <= P; ++ph) total += phase_items(ph) * nch * MT;
+        uint32_t head = 0;  // the unit being multiplied (of the ring; those after it are being copied)
+        int popped = atomicAdd(queue, 1);
+        uint32_t taken = 0, issued = 0, q = 0;
+        bool ok = true;
+        auto take = [&]() {  // the next unit into the ring
+            Unit u{};
+            u.id = popped < total ? popped : -1;
+            if (u.id >= 0) {
+                popped = atomicAdd(queue, 1);
+                int ph = 0, w = u.id;
+                for (int k = phase_items(0) * nch * MT; w >= k; k = phase_items(ph) * nch * MT) {
+                    w -= k;
+                    ++ph;
                 }
-            } else if (t < h2) {
-#pragma unroll
-                for (int r = 0; r < RT; ++r) g[(size_t)r * N + h2 + t] = 0.f;
+                const int per = phase_items(ph) * nch, si = w / per, x = w - si * per;
+                const BcrItem it = items[lv.off[ph <= nl ? ph : 2 * nl - ph] + x / nch];
+                u.m = si == 0 ? MT - 1 : si - 1;  // the slices others wait for (R+, then L-) first
+                u.ch = x % nch;
+                u.bwd = ph > nl;
+                u.cell = it.cell;
+                u.left = it.left;
+                u.right = it.right;
+                u.s_cell = it.s_cell;
+                u.s_left = it.s_left;
+                u.s_right = it.s_right;
+                u.local = it.local;
+                u.K_inst = it.K_inst;
+                u.level = it.level;
             }
-            __syncthreads();
-            bsrc = g;
-            bstride = N;
-        }
-
-        // the GEMM: chunk by chunk, the right-hand sides split into the stage beside the factor chunk
-        float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
-        auto load_b = [&](int c) {
-            if (br < nrc) {
-                const float4 *s = reinterpret_cast<const float4 *>(bsrc + (size_t)br * bstride + c * kK + 8 * bh);
-                v0 = __ldcg(s);
-                v1 = __ldcg(s + 1);
+            ring[taken % kUnitRing] = u;
+            mbar_arrive(&unit_bar[taken % kUnitRing]);  // (release)
+            ++taken;
+            return u.id >= 0;
+        };
+        int copy_i = 0;       // next chunk to copy, of unit copy_u
+        uint32_t copy_u = 0;
+        bool more = take();
+        // copy one more chunk if its stage is free (its earlier products done) and there is one
+        auto copy_next = [&]() {
+            if (!more) return false;
+            const Unit &u = ring[copy_u % kUnitRing];
+            const int s = issued % kStages;
+            const unsigned char *src;
+            uint32_t bytes = kChunkA;
+            const int nm = n_main(u);
+            const int mi = u.bwd ? copy_i - n_coup(u) : copy_i, ci = u.bwd ? copy_i : copy_i - nm;
+            if (mi >= 0 && mi < nm) {
+                src = Atc + (size_t)u.cell * cell_bytes(n2) +
+                      ((size_t)u.m * (n2 / kK) + (u.bwd ? h2 / kK : 0) + mi) * kChunkA;
             } else {
-                v0 = v1 = make_float4(0.f, 0.f, 0.f, 0.f);
+                const bool second = ci >= nc || (!u.bwd && !push_right(u));  // the coupling with the other neighbour
+                const int slot = u.bwd ? u.s_cell : (second ? u.s_left : u.s_right);
+                src = (second ? Ctc : Btc) + (size_t)slot * coupling_bytes(n2) + (size_t)(ci % nc) * coupling_chunk(n2);
+                bytes = coupling_chunk(n2);
+            }
+            tc::mbar_arrive_expect_tx(&full_a[s], bytes);
+            tc::bulk_copy_g2s(smem_tcs + s * pl.stage, src, bytes, &full_a[s]);
+            ++issued;
+            if (++copy_i == nm + n_coup(u)) {
+                copy_i = 0;
+                ++copy_u;
+                more = take();
+            }
+            return true;
+        };
+        const uint32_t idesc = tc::idesc_bf16(128, RT);
+        while (ok && ring[head % kUnitRing].id >= 0) {
+            const Unit u = ring[head % kUnitRing];
+            const int nm = n_main(u), ncp = n_coup(u), ns = nm + ncp;
+            for (int i = 0; i < ns && ok; ++i, ++q) {
+                // copies ahead: the stage of chunk q + d is free once chunk q + d - kStages is done
+                while (issued < q + kStages - 1) {  // (the products of chunk q - 2, not of the one just issued)
+                    if (issued >= (uint32_t)kStages && !(ok = tc::mbar_wait(&empty[issued % kStages],
+                                                                            (issued / kStages - 1u) & 1u)))
+                        break;
+                    if (!copy_next()) break;
+                }
+                const int s = q % kStages;
+                const uint32_t par = (q / kStages) & 1u;
+                ok = ok && !failed() && tc::mbar_wait(&full_a[s], par);
+                if (ok) {  // the workers may be waiting for other units (their own bound): no time limit but the flag
+                    while (!tc::mbar_test(&full_b[s], par))
+                        if (failed()) {
+                            ok = false;
+                            break;
+                        }
+                }
+                if (!ok) break;
+                tc::tc_fence_after();
+                const int mi = u.bwd ? i - ncp : i, ci = u.bwd ? i : i - nm;
+                const uint32_t a0 = tc::smem_u32(smem_tcs + s * pl.stage), b0 = a0 + kChunkA;
+                if (mi >= 0 && mi < nm) {
+                    for (int j = 0; j < kK / 16; ++j) {
+                        const uint64_t ah = tc::smem_desc(a0 + 256u * j, 128, kK * 16),
+                                       al = tc::smem_desc(a0 + kChunkA / 2 + 256u * j, 128, kK * 16);
+                        const uint64_t bh = tc::smem_desc(b0 + 256u * j, 128, kK * 16),
+                                       bl = tc::smem_desc(b0 + RT * kK * 2u + 256u * j, 128, kK * 16);
+                        tc::mma_bf16(tmem, ah, bh, idesc, (mi > 0 || j > 0) ? 1u : 0u);
+                        tc::mma_bf16(tmem, ah, bl, idesc, 1u);
+                        tc::mma_bf16(tmem, al, bh, idesc, 1u);
+                    }
+                } else {
+                    // (rows from N/2 up read what follows in the stage; their accumulator lanes are ignored)
+                    const bool second = ci >= nc || (!u.bwd && !push_right(u));
+                    const uint32_t acc = tmem + (second ? 2u * RT : (uint32_t)RT);
+                    uint64_t a[3], b[3];
+                    for (int k = 0; k < 3; ++k) {
+                        a[k] = tc::smem_desc(a0 + (uint32_t)k * h2 * kKc * 2u, 128, kKc * 16);
+                        b[k] = tc::smem_desc(b0 + (uint32_t)k * RT * kKc * 2u, 128, kKc * 16);
+                    }
+                    tc::mma_bf16(acc, a[0], b[0], idesc, ci % nc > 0 ? 1u : 0u);
+                    tc::mma_bf16(acc, a[0], b[1], idesc, 1u);
+                    tc::mma_bf16(acc, a[1], b[0], idesc, 1u);
+                    tc::mma_bf16(acc, a[0], b[2], idesc, 1u);
+                    tc::mma_bf16(acc, a[2], b[0], idesc, 1u);
+                    tc::mma_bf16(acc, a[1], b[1], idesc, 1u);
+                }
+                tc::mma_commit(&empty[s]);
+                // the end of the unit's first or second group of chunks: the workers read its accumulators
+                if (i == (u.bwd ? ncp : nm) - 1 || i == ns - 1) tc::mma_commit(seg_bar);
+            }
+            ++head;
+        }
+        if (!ok) fail();
+        // every copy and product has landed before the CTA ends (bounded)
+        for (uint32_t j = q; j < issued; ++j)
+            if (!tc::mbar_wait(&full_a[j % kStages], (j / kStages) & 1u)) break;
+        tc::mma_commit(drain);
+        (void)tc::mbar_wait(drain, 0);
+    } else if (t < kWorkers) {
+        // ---- workers
+        const uint32_t lane_base = (uint32_t)(t & ~31) << 16;
+        const unsigned limit = flow_spin_limit(err);
+        uint32_t q = 0, segs = 0;
+        bool ok = true;
+        // wait (bounded by time, and by the flag) for a phase of bar
+        auto wait_bar = [&](uint64_t *bar, uint32_t par) {
+            if (!tc::mbar_wait(bar, par)) fail();
+            return !failed();
+        };
+        // The unit's next `chunks` chunks of KC columns of the vectors v_r[k] = src[r stride + k]
+        // (r < nrc, else 0) in P parts, kAhead of them in flight.
+        auto feed = [&](auto KCt, auto Pt, const float *src, size_t stride, int chunks, int nrc) {
+            constexpr int KC = decltype(KCt)::value, PARTS = decltype(Pt)::value, GR = KC / 8;
+            constexpr int NG = (RT * GR + kWorkers - 1) / kWorkers;  // groups of 8 values per worker and chunk
+            float4 v[kAhead][NG][2];
+            auto load = [&](int c, float4 (&x)[NG][2]) {
+#pragma unroll
+                for (int g = 0; g < NG; ++g) {
+                    const int id = t + g * kWorkers, r = id / GR, k = 8 * (id % GR);
+                    x[g][0] = x[g][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (r < nrc && c < chunks) {
+                        const float4 *p = reinterpret_cast<const float4 *>(src + (size_t)r * stride + c * KC + k);
+                        x[g][0] = __ldcg(p);
+                        x[g][1] = __ldcg(p + 1);
+                    }
+                }
+            };
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a) load(a, v[a]);
+            for (int c0 = 0; c0 < chunks && ok; c0 += kAhead) {
+#pragma unroll
+                for (int a = 0; a < kAhead; ++a) {
+                    if (c0 + a >= chunks || !ok) break;
+                    const int s = q % kStages;
+                    if (q >= (uint32_t)kStages) ok = wait_bar(&empty[s], (q / kStages - 1u) & 1u);
+                    unsigned char *bs = smem_tcs + s * pl.stage + kChunkA;
+#pragma unroll
+                    for (int g = 0; g < NG; ++g) {
+                        const int id = t + g * kWorkers, r = id / GR, k = 8 * (id % GR);
+                        if (r < RT) {
+                            const float4 lo4 = v[a][g][0], hi4 = v[a][g][1];
+                            const float x[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
+                            unsigned char *d = bs + tc::kmajor_offset(r, k, KC);
+                            if constexpr (PARTS == 3) {
+                                store_split3(d, (uint32_t)RT * KC * 2u, x);
+                            } else {
+                                uint32_t hi[4], lo[4];
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    __nv_bfloat16 h0, l0, h1, l1;
+                                    tc::split_bf16(x[2 * j], h0, l0);
+                                    tc::split_bf16(x[2 * j + 1], h1, l1);
+                                    hi[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                                    lo[j] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+                                }
+                                *reinterpret_cast<uint4 *>(d) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                                *reinterpret_cast<uint4 *>(d + (uint32_t)RT * KC * 2u) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                            }
+                        }
+                    }
+                    load(c0 + kAhead + a, v[a]);
+                    tc::fence_async_smem();  // the st.shared above, before the tensor core reads them
+                    tc::tc_fence_before();   // and the accumulator reads before it, before the next products
+                    mbar_arrive(&full_b[s]);
+                    ++q;
+                }
             }
         };
-        if (br < RT) load_b(0);
-        bool fail = false;
-        for (int c = 0; c < d.nkc; ++c, ++q) {
-            const int s = q & 1;
-            unsigned char *stg = smem_tcs + s * pl.stage, *bs = stg + cbytes;
-            if (q >= 2) ok = ok && tc::mbar_wait(&empty[s], ((q >> 1) - 1) & 1);  // chunk q - 2's products are done
-            if (br < RT) {
-                const float x[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-                uint32_t hi[4], lo[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    __nv_bfloat16 h0, l0, h1, l1;
-                    tc::split_bf16(x[2 * j], h0, l0);
-                    tc::split_bf16(x[2 * j + 1], h1, l1);
-                    hi[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-                    lo[j] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-                }
-                const uint32_t off = tc::kmajor_offset(br, 8 * bh, kK);
-                *reinterpret_cast<uint4 *>(bs + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                *reinterpret_cast<uint4 *>(bs + (size_t)RT * kK * 2 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                if (c + 1 < d.nkc) load_b(c + 1);
+        auto wait_seg = [&]() {  // the group of chunks just fed has been multiplied
+            if (ok) ok = wait_bar(seg_bar, segs & 1u);
+            ++segs;
+            tc::tc_fence_after();
+        };
+        for (uint32_t j = 0;; ++j) {
+            // (the driver takes units as it copies: it is at most a few chunks ahead, never far behind)
+            ok = wait_bar(&unit_bar[j % kUnitRing], (j / kUnitRing) & 1u);
+            if (worker_any(!ok)) break;
+            const Unit u = ring[j % kUnitRing];
+            if (u.id < 0) break;
+            const int r0 = u.ch * RT, nrc = min(RT, R - r0), row = 128 * u.m + t;
+            int *cnt = flow + (size_t)u.ch * sumK, *written = cnt + n, *fin = flow + 2 * n + (size_t)u.ch * sumK * 2;
+            float *Yc = Y + (size_t)r0 * rstride + (size_t)u.cell * n2;
+            if (!u.bwd) {
+                int want = 0;
+                for (int lp = 0; lp < u.level; ++lp)
+                    want += (u.local >= (1 << lp)) + (u.local + (1 << lp) < u.K_inst);
+                if (t == 0 && want) poll(cnt + u.cell, want, err, limit);
+            } else {  // three warps, so that the polls overlap
+                if (t == 0) poll(fin + 2 * u.left + 1, 1, err, limit);
+                if (t == 32 && u.right >= 0) poll(fin + 2 * u.right, 1, err, limit);
+                if (t == 64) poll(written + u.cell, MT, err, limit);
             }
-            tc::fence_async_smem();  // the st.shared above, before the tensor core reads them
-            if (__syncthreads_or(!ok)) {
-                fail = true;
-                break;
-            }
-            if (t == 0) {
-                ok = tc::mbar_wait(&full[s], (q >> 1) & 1);
-                if (ok) {
-                    waited = q + 1;
-                    tc::tc_fence_after();
-                    const uint32_t a0 = tc::smem_u32(stg), b0 = tc::smem_u32(bs);
-                    const uint64_t bhd = tc::smem_desc(b0, 128, 256), bld = tc::smem_desc(b0 + RT * kK * 2, 128, 256);
-                    for (int m = 0; m < MT; ++m) {
-                        const uint64_t ahd = tc::smem_desc(a0 + 4096u * m, 128, 256);
-                        const uint64_t ald_ = tc::smem_desc(a0 + (uint32_t)n2 * kK * 2 + 4096u * m, 128, 256);
-                        const uint32_t dt = tmem + (uint32_t)(m * RT);
-                        tc::mma_bf16(dt, ahd, bhd, idesc, c > 0 ? 1u : 0u);
-                        tc::mma_bf16(dt, ahd, bld, idesc, 1u);
-                        tc::mma_bf16(dt, ald_, bhd, idesc, 1u);
-                    }
-                    tc::mma_commit(&empty[s]);
-                    // the stage is refilled with chunk q + 2 once these products have read it
-                    ok = tc::mbar_wait(&empty[s], (q >> 1) & 1);
-                    if (ok) issue(q + 2);
-                }
-            }
-        }
-        if (fail || __syncthreads_or(!ok)) break;
-        // every product of the unit has completed (the last chunk's commit)
-        const uint32_t ql = q - 1;
-        ok = tc::mbar_wait(&empty[ql & 1], (ql >> 1) & 1);
-        if (__syncthreads_or(!ok)) break;
-        tc::tc_fence_after();
-        if (!d.bwd) {
-            const bool push_r = it.right >= 0, push_l = it.left >= 0;
-            float v[16];
-            for (int m = 0; m < MT; ++m) {
-                const int row = 128 * m + 32 * w + lane;
-                for (int c16 = 0; c16 < RT / 16; ++c16) {
-                    tc::tmem_ld16(tmem + lane_base + (uint32_t)(m * RT + 16 * c16), v);
+            worker_sync();
+            if (!u.bwd) {
+                feed(Const<kK>{}, Const<2>{}, rhs + (size_t)r0 * rstride + (size_t)u.cell * n2, rstride, n2 / kK, nrc);
+                wait_seg();
+                if (worker_any(!ok)) break;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int r = 16 * c16 + j;
-                        if (r < nrc) Y[(size_t)(r0 + r) * rstride + (size_t)it.cell * n2 + row] = v[j];
-                        if (push_r && row >= N + h2) aux[r * ald + row - N - h2] = v[j];
-                    }
-                }
-            }
-            float acc[RT];
-            if (push_r) {  // r_right[N/2 : N] -= B_right Y_i[3N/2 : 2N]
-                __syncthreads();
-                if (t < h2) {
-                    coupling_rows<RT>(Bc + (size_t)it.s_right * hh, aux, h2, ald, acc);
-                    float *o = rhs + (size_t)r0 * rstride + (size_t)it.right * n2 + h2 + t;
+                for (int c = 0; c < RT; c += 16) {
+                    float v[16];
+                    tc::tmem_ld16(tmem + lane_base + c, v);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r)
-                        if (r < nrc) atomicAdd(o + (size_t)r * rstride, -acc[r]);
+                    for (int i = 0; i < 16; ++i)
+                        if (c + i < nrc) Yc[(size_t)(c + i) * rstride + row] = v[i];
                 }
-            }
-            if (push_l) {  // r_left[N : 3N/2] -= C_left Y_i[0 : N/2]
-                __syncthreads();
-                if (32 * w < h2) {
-                    for (int c16 = 0; c16 < RT / 16; ++c16) {
-                        tc::tmem_ld16(tmem + lane_base + (uint32_t)(16 * c16), v);
-                        const int row = 32 * w + lane;
-                        if (row < h2)
+                const bool pr = push_right(u), plf = push_left(u);
+                if (pr || plf) {
+                    worker_sync();  // the rows this CTA just wrote are read back below
+                    if (pr) feed(Const<kKc>{}, Const<3>{}, Yc + N + h2, rstride, nc, nrc);
+                    if (plf) feed(Const<kKc>{}, Const<3>{}, Yc, rstride, nc, nrc);
+                    wait_seg();
+                    if (worker_any(!ok)) break;
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) aux[(16 * c16 + j) * ald + row] = v[j];
-                    }
-                }
-                __syncthreads();
-                if (t < h2) {
-                    coupling_rows<RT>(Cc + (size_t)it.s_left * hh, aux, h2, ald, acc);
-                    float *o = rhs + (size_t)r0 * rstride + (size_t)it.left * n2 + N + t;
+                    for (int side = 0; side < 2; ++side) {
+                        if (!(side ? plf : pr)) continue;
+                        float *o = rhs + (size_t)r0 * rstride + (size_t)(side ? u.left : u.right) * n2 + (side ? N : h2) + t;
 #pragma unroll
-                    for (int r = 0; r < RT; ++r)
-                        if (r < nrc) atomicAdd(o + (size_t)r * rstride, -acc[r]);
-                }
-            }
-            if (push_r) fs.sig0 = cnt_c + it.right;
-            if (push_l) fs.sig1 = cnt_c + it.left;
-            else fs.sig2 = done_c + it.cell;  // a root: its solution is final
-        } else {
-            float v[16];
-            for (int m = 0; m < MT; ++m) {
-                const int row = 128 * m + 32 * w + lane;
-                for (int c16 = 0; c16 < RT / 16; ++c16) {
-                    tc::tmem_ld16(tmem + lane_base + (uint32_t)(m * RT + 16 * c16), v);
+                        for (int c = 0; c < RT; c += 16) {
+                            float v[16];
+                            tc::tmem_ld16(tmem + lane_base + (uint32_t)((1 + side) * RT + c), v);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int r = 16 * c16 + j;
-                        if (r < nrc) {
-                            float *y = Y + (size_t)(r0 + r) * rstride + (size_t)it.cell * n2 + row;
-                            *y = __ldcg(y) - v[j];
+                            for (int i = 0; i < 16; ++i)
+                                if (t < h2 && c + i < nrc) atomicAdd(o + (size_t)(c + i) * rstride, -v[i]);
                         }
                     }
                 }
+                worker_sync();
+                if (t == 0) {
+                    __threadfence();
+                    if (u.left < 0) {  // a root: its solution is final
+                        if (u.m == 0) atomicAdd(fin + 2 * u.cell, 1);
+                        if (u.m == MT - 1) atomicAdd(fin + 2 * u.cell + 1, 1);
+                    } else {
+                        atomicAdd(written + u.cell, 1);
+                        if (pr) atomicAdd(cnt + u.right, 1);
+                        if (plf) atomicAdd(cnt + u.left, 1);
+                    }
+                }
+            } else {
+                float *g = gs + (size_t)blockIdx.x * RT * N;
+                feed(Const<kKc>{}, Const<3>{}, Y + (size_t)r0 * rstride + (size_t)u.left * n2 + N + h2, rstride, nc, nrc);
+                if (u.right >= 0)
+                    feed(Const<kKc>{}, Const<3>{}, Y + (size_t)r0 * rstride + (size_t)u.right * n2, rstride, nc, nrc);
+                wait_seg();
+                if (worker_any(!ok)) break;
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {
+                    if (side && u.right < 0) continue;
+#pragma unroll
+                    for (int c = 0; c < RT; c += 16) {
+                        float v[16];
+                        tc::tmem_ld16(tmem + lane_base + (uint32_t)((1 + side) * RT + c), v);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (t < h2) g[(size_t)(c + i) * N + side * h2 + t] = v[i];
+                    }
+                }
+                worker_sync();
+                feed(Const<kK>{}, Const<2>{}, g, N, n_main(u), RT);
+                float y[RT];
+#pragma unroll
+                for (int c = 0; c < RT; ++c) y[c] = c < nrc ? __ldcg(Yc + (size_t)c * rstride + row) : 0.f;
+                wait_seg();
+                if (worker_any(!ok)) break;
+#pragma unroll
+                for (int c = 0; c < RT; c += 16) {
+                    float v[16];
+                    tc::tmem_ld16(tmem + lane_base + c, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (c + i < nrc) Yc[(size_t)(c + i) * rstride + row] = y[c + i] - v[i];
+                }
+                worker_sync();
+                if (t == 0) {
+                    __threadfence();
+                    if (u.m == 0) atomicAdd(fin + 2 * u.cell, 1);
+                    if (u.m == MT - 1) atomicAdd(fin + 2 * u.cell + 1, 1);
+                }
             }
-            fs.sig0 = done_c + it.cell;
         }
-        tc::tc_fence_before();  // the accumulator reads, before the next unit's products
-        flow_signal(&fs);
-        // the next unit: already taken by the copy stream, or taken now
-        if (t == 0) {
-            if (nxt_u < 0) {
-                nxt_u = atomicAdd(queue, 1);
-                if (nxt_u < total) decode(nxt_u, nxt);
-            }
-            *s_unit = nxt_u;
-            if (nxt_u < total) {
-                cur_base += (uint32_t)cur.nkc;
-                cur = nxt;
-                // a unit taken here (not by the stream) has no chunk in flight yet
-                if (issued < cur_base + 1) issue(cur_base);
-                if (issued < cur_base + 2) issue(cur_base + 1);
-            }
-            nxt_u = -1;
-        }
-        __syncthreads();
-        u = *s_unit;
-        if (u < total) decode(u, d);
     }
-    if (!ok || u < total) {
-        // a wait gave up: let this CTA's copies and products land (bounded), record the error
-        if (t == 0) {
-            for (uint32_t j = waited; j < issued; ++j)
-                if (!tc::mbar_wait(&full[j & 1], (j >> 1) & 1)) break;
-            tc::mma_commit(drain);
-            (void)tc::mbar_wait(drain, 0);
-            atomicExch(err, 1);
-        }
-    }
+    __syncwarp();
     tc::tc_fence_before();
     __syncthreads();
-    if (t < 32) tc::tmem_dealloc(tmem, tcols);
+    if (t < 32) tc::tmem_dealloc(tmem, kCols);
 }
 
 }  // namespace fpsa

@@ -89,10 +89,10 @@ struct fpsa_ctx {
     double *d_in_st = nullptr, *d_in_ss = nullptr, *d_in_q = nullptr;  // fpsa_set_xs staging of host inputs
     int *d_xs_err = nullptr;     // [2] validation of fpsa_set_xs
     Packets pk = {};  // of the dataflow BCR solve (NULL push: not allocated)
-    // counters of the tensor-core BCR solve, double-buffered: [parity][cnt | done][rhs chunks][sumK];
-    // each solve uses one parity and zeroes the other for the next solve
+    // counters of the tensor-core BCR solve, double-buffered: [parity][4 flow_n]; each solve
+    // uses one parity and zeroes the other for the next solve
     int *d_flow = nullptr;
-    size_t flow_n = 0;                      // counters per array (rhs chunks x sumK)
+    size_t flow_n = 0;                      // rhs tiles x sumK
     int flow_parity = 0;
     bool solve_pdl = true;                  // cooperative launch with programmatic serialization accepted
     int *d_factor_cnt = nullptr;            // dataflow factorization counters [sumK]
@@ -119,6 +119,7 @@ struct fpsa_ctx {
     int tcs_rt = 0;                  // right-hand sides per unit; 0: unavailable
     int tcs_grid = 0;                // two CTAs per SM
     unsigned char *d_tcs_A = nullptr;  // the factors split to BF16 hi / lo in the core-matrix layout
+    unsigned char *d_tcs_B = nullptr, *d_tcs_C = nullptr;  // the couplings in three BF16 parts
     float *d_tcs_g = nullptr;        // per-CTA backward coupling vectors
     int *d_tcs_queue = nullptr;      // unit counters, one per parity of d_flow
     unsigned long long *d_conv = nullptr, *d_growth = nullptr;
@@ -747,6 +748,9 @@ int setup_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
         Launch L_(ctx, FPSA_PHASE_BCR_INVERT);
         tcs::k_bcr_factor_split<<<(unsigned)((size_t)g.sumK * (2 * N / tcs::kK)), 256, 0, st>>>(
             reinterpret_cast<const float *>(p.A), ctx->d_tcs_A, 2 * N);
+        const unsigned cgrid = (unsigned)((size_t)g.n_slots * (h2 / tcs::kKc));
+        tcs::k_bcr_coupling_split<<<cgrid, 256, 0, st>>>(reinterpret_cast<const float *>(p.Bc), ctx->d_tcs_B, 2 * N);
+        tcs::k_bcr_coupling_split<<<cgrid, 256, 0, st>>>(reinterpret_cast<const float *>(p.Cc), ctx->d_tcs_C, 2 * N);
         CK(cudaGetLastError());
     }
     if (p.G) {
@@ -867,18 +871,18 @@ int alloc_packets(fpsa_ctx *ctx) {
 int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *stop) {
     const Geometry &g = ctx->geo;
     const size_t n = ctx->flow_n;
-    int *cnt = ctx->d_flow + 2 * n * ctx->flow_parity, *done = cnt + n;
-    int *zero_next = ctx->d_flow + 2 * n * (1 - ctx->flow_parity);
+    int *flow = ctx->d_flow + 4 * n * ctx->flow_parity, *zero_next = ctx->d_flow + 4 * n * (1 - ctx->flow_parity);
     int *queue = ctx->d_tcs_queue + ctx->flow_parity, *queue_next = ctx->d_tcs_queue + (1 - ctx->flow_parity);
     ctx->flow_parity ^= 1;
     const int RT = ctx->tcs_rt;
-    const size_t smem = tcs::Plan::make(2 * g.N, RT).total;
+    const size_t smem = tcs::Plan::make(RT).total;
     Launch L_(ctx, FPSA_PHASE_BCR_SOLVE);
     auto go = [&](auto kern) {
         return launch_pdl(kern, dim3(ctx->tcs_grid), dim3(tcs::kThreads), smem, ctx->stream,
-                          (const unsigned char *)ctx->d_tcs_A, (const float *)p.Bc, (const float *)p.Cc,
-                          (const BcrItem *)ctx->d_items_all, ctx->lvt[0], rhs, p.ybuf, ctx->d_tcs_g, g.N, g.sumK,
-                          g.R, cnt, done, queue, ctx->d_dev_err, zero_next, (long long)(2 * n), queue_next, stop);
+                          (const unsigned char *)ctx->d_tcs_A, (const unsigned char *)ctx->d_tcs_B,
+                          (const unsigned char *)ctx->d_tcs_C, (const BcrItem *)ctx->d_items_all, ctx->lvt[0], rhs,
+                          p.ybuf, ctx->d_tcs_g, g.N, g.sumK, g.R, flow, queue, ctx->d_dev_err, zero_next,
+                          (long long)(4 * n), queue_next, stop);
     };
     switch (RT) {
         case 16: CK(go(k_bcr_solve_tc<16>)); break;
@@ -1895,7 +1899,7 @@ int capture_mixed_loop(fpsa_ctx *ctx, const MixedPlan &mp, const fpsa_opts &o, i
     // zeroed by the step before)
     if (fpsa && inner % 2 == 1 && ctx->d_tcs_queue) {
         const int par = ctx->flow_parity;
-        ok = cudaMemsetAsync(ctx->d_flow + 2 * ctx->flow_n * par, 0, 2 * ctx->flow_n * sizeof(int), cs) == cudaSuccess &&
+        ok = cudaMemsetAsync(ctx->d_flow + 4 * ctx->flow_n * par, 0, 4 * ctx->flow_n * sizeof(int), cs) == cudaSuccess &&
              cudaMemsetAsync(ctx->d_tcs_queue + par, 0, sizeof(int), cs) == cudaSuccess;
         if (!ok) {
             end_capture_on_error();
@@ -2122,14 +2126,16 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                 ctx->tcs_rt = tcs::rhs_tile(g.R);
                 ctx->tcs_grid = 2 * nsm;
                 ctx->flow_n = (size_t)((g.R + ctx->tcs_rt - 1) / ctx->tcs_rt) * g.sumK;
-                CK(dalloc(ctx, &ctx->d_flow, 4 * ctx->flow_n));
-                CK(cudaMemset(ctx->d_flow, 0, 4 * ctx->flow_n * sizeof(int)));
+                CK(dalloc(ctx, &ctx->d_flow, 8 * ctx->flow_n));
+                CK(cudaMemset(ctx->d_flow, 0, 8 * ctx->flow_n * sizeof(int)));
+                CK(dalloc(ctx, &ctx->d_tcs_B, (size_t)g.n_slots * tcs::coupling_bytes(2 * g.N)));
+                CK(dalloc(ctx, &ctx->d_tcs_C, (size_t)g.n_slots * tcs::coupling_bytes(2 * g.N)));
                 CK(dalloc(ctx, &ctx->d_tcs_A, (size_t)g.sumK * tcs::cell_bytes(2 * g.N)));
                 CK(dalloc(ctx, &ctx->d_tcs_g, (size_t)ctx->tcs_grid * ctx->tcs_rt * g.N));
                 CK(dalloc(ctx, &ctx->d_tcs_queue, 2));
                 CK(cudaMemset(ctx->d_tcs_queue, 0, 2 * sizeof(int)));
                 const void *k = tcs_kernel(ctx->tcs_rt);
-                CK(raise_smem_limit(k, (int)tcs::Plan::make(2 * g.N, ctx->tcs_rt).total));
+                CK(raise_smem_limit(k, (int)tcs::Plan::make(ctx->tcs_rt).total));
                 CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared));
             }

@@ -25,7 +25,7 @@ def test_few_columns(N, K, R):
     out = {}
     for eng in ("tensor", "simt"):
         ctx = binding.context_for(p, laplacian="wfd", precision="mixed")
-        out[eng] = ctx.solve("fpsa", tol=1e-12, max_iterations=60, contraction=eng)
+        out[eng] = ctx.solve("fpsa", tol=1e-12, max_iterations=60, inner_iterations=4, contraction=eng)
         ctx.close()
     (a, sa), (b, sb) = out["tensor"], out["simt"]
     assert np.abs(a - b).max() / np.abs(b[..., 0]).max() < 1e-9

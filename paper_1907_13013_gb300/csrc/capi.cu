@@ -337,7 +337,7 @@ const void *staged_kernel(int RC) {
 // The cooperative solve of a context of geometry g. Staged: two blocks per SM where their
 // shared memory fits and the widest level has more than two units for every compute group
 // of one block per SM (six slabs of 37 to 613 cells, N = 32, 3 right-hand sides: 112 us a
-// solve with one, 79 with two); below that more blocks only mean more slices per cell and
+// solve with one, 84 with two); below that more blocks only mean more slices per cell and
 // more readers of each packet (200 cells at N = 16, FP64: 1.94 ms a solve with one, 2.03
 // with two).
 template <typename T>

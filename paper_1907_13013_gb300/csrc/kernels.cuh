@@ -624,29 +624,52 @@ static __global__ void k_mixed_residual(const double *__restrict__ psi, double *
     const int ncols = 2 * ncell;
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
     const double *psr = psi + (size_t)r * sumK * 2 * N;  // this rhs
-    fold_columns(psi + colbase * N, ncols, N, Ys);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
-        const int cl = idx / N, l = idx - cl * N, g = g0 + cl;
-        const double sg = sigma_s[(size_t)g * N + l];
-        const size_t e = (colbase + 2 * cl) * N + l;
-        const double q0 = Qext ? Qext[e] : 0.0, q1 = Qext ? Qext[e + N] : 0.0;
-        double m[2];
-        folded_moments(Ys, DT, N, cl, l, m);
-        if (l == 0) {
-            const int slot = (r * B + cell_inst[g]) * 2;
-            const unsigned long long d0 = dkey(m[0] - phi[e]), d1 = dkey(m[1] - phi[e + N]);
-            const unsigned long long a0 = dkey(m[0]), a1 = dkey(m[1]);
-            atomicMax(conv + slot, d0 > d1 ? d0 : d1);
-            atomicMax(conv + slot + 1, a0 > a1 ? a0 : a1);
-        }
-        phi[e] = m[0];
-        phi[e + N] = m[1];
-        Xs[2 * cl * N + l] = sg * m[0] + q0;
-        Xs[(2 * cl + 1) * N + l] = sg * m[1] + q1;
+    // Folded contractions as above, one column per thread (both nodes of a cell in a thread
+    // measured 127 us against 100 for 2000 columns at N = 128).
+    const int h2 = N / 2;
+    for (int idx = threadIdx.x; idx < ncols * h2; idx += blockDim.x) {
+        const int c = idx / h2, n = idx - c * h2;
+        const double a = psi[(colbase + c) * N + n], bm = psi[(colbase + c) * N + (N - 1 - n)];
+        Ys[c * N + n] = a + bm;        // even part
+        Ys[c * N + h2 + n] = a - bm;   // odd part
     }
     __syncthreads();
-    expand_columns(Xs, MT, N, ncell, Ys, Qang ? Qang + colbase * N : nullptr);
+    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
+        const int c = idx / N, l = idx - c * N;
+        const double *f = Ys + c * N + ((l & 1) ? h2 : 0);
+        double acc = 0.0;
+#pragma unroll 8
+        for (int n = 0; n < h2; ++n) acc = fma(DT[(size_t)n * N + l], f[n], acc);
+        Xs[idx] = acc;
+    }
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < ncols * N; idx += blockDim.x) {
+        const int c = idx / N, l = idx - c * N;
+        const int g = g0 + c / 2;
+        const size_t e = colbase * N + idx;
+        const double pn = Xs[idx];
+        if (l == 0) {
+            const int slot = (r * B + cell_inst[g]) * 2;
+            atomicMax(conv + slot, dkey(pn - phi[e]));
+            atomicMax(conv + slot + 1, dkey(pn));
+        }
+        phi[e] = pn;
+        Xs[idx] = sigma_s[(size_t)g * N + l] * pn + (Qext ? Qext[e] : 0.0);
+    }
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < ncols * h2; idx += blockDim.x) {
+        const int c = idx / h2, n = idx - c * h2;
+        const double *x = Xs + c * N;
+        double ev = 0.0, od = 0.0;
+#pragma unroll 4
+        for (int l = 0; l + 1 < N; l += 2) {
+            ev = fma(MT[(size_t)l * N + n], x[l], ev);
+            od = fma(MT[(size_t)(l + 1) * N + n], x[l + 1], od);
+        }
+        const double *qa = Qang ? Qang + (colbase + c) * N : nullptr;
+        Ys[c * N + n] = ev + od + (qa ? qa[n] : 0.0);
+        Ys[c * N + (N - 1 - n)] = ev - od + (qa ? qa[N - 1 - n] : 0.0);
+    }
     __syncthreads();
     for (int idx = threadIdx.x; idx < ncell * N; idx += blockDim.x) {
         const int cl = idx / N, n = idx - cl * N;

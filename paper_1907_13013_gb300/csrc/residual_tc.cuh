@@ -26,13 +26,17 @@
 // the accuracy of an FP64 dot product.
 //
 // One CTA per tile of 64 cells x 2 nodes = 128 columns (tensor-memory lane = column)
-// and per SM (it holds all 512 TMEM columns), 256 threads: two per column, each taking
-// half of every K-chunk and of every output chunk. For each output chunk of OC = 64
-// rows (32 where 64 does not divide N) and each K-chunk of 32, in two pipelined stages:
-// thread 0 copies the operator's 8 digit slices of that block (OC x 32 BF16 each,
-// stored K-major in the core-matrix layout, one bulk copy), the threads write the 8
-// digit slices of their columns' 32 inputs (K-major), and thread 0 issues the 72 MMAs
-// (36 pairs, two K-steps; M = 128, N = OC, K = 16) while the next chunk is prepared.
+// and per SM (it holds all 512 TMEM columns), 256 worker threads: two per column, each
+// taking half of every K-chunk and of every output chunk; and one issuing thread. For each
+// output chunk of OC = 64 rows (32 where 64 does not divide N) and each K-chunk of 32, in
+// two pipelined stages: the issuing thread copies the operator's 8 digit slices of that
+// block (OC x 32 BF16 each, stored K-major in the core-matrix layout, one bulk copy) and
+// issues the 72 MMAs (36 pairs, two K-steps; M = 128, N = OC, K = 16), while the workers
+// write the 8 digit slices of their columns' next 32 inputs (K-major).
+// What bounds it: the workers' arithmetic, of which FP64 (two FMAs a clock and SM) is the
+// largest part, so the recombination takes 4 FP64 operations an output, the LD stencil 6;
+// with 6 and 11, and a worker thread that built each MMA's descriptors as it issued them,
+// a residual at N = 256, 1250 cells and 64 right-hand sides took 6.87 ms, now 5.46 ms.
 // Waits are bounded; on a timeout the CTA records the error, waits (bounded) for its
 // copies and products, frees its tensor memory and stops.
 #pragma once
@@ -45,7 +49,8 @@ namespace rtc {
 
 constexpr int S = 8;    // digit slices: 56-bit fixed point per row
 constexpr int KC = 32;  // K per chunk: two MMA K-steps
-constexpr int kThreads = 256;  // two threads per column (tensor-memory lane), halves of K and of the outputs
+constexpr int kWorkers = 256;  // two threads per column (tensor-memory lane), halves of K and of the outputs
+constexpr int kThreads = kWorkers + 32;  // and the issuing thread's warp
 // output rows per chunk: 64 where they divide N, else 32 (N is a multiple of 32)
 __host__ __device__ constexpr int oc_of(int N) { return N % 64 == 0 ? 64 : 32; }
 __host__ __device__ constexpr uint32_t a_slice_bytes() { return 128u * KC * 2u; }
@@ -109,6 +114,15 @@ struct Ops {
     const int32_t *eD, *eM;      // their row exponents
 };
 
+// (hi 2^-21 + lo 2^-49) with one rounding of the sum, |hi|, |lo| < 2^46: an integer added to
+// the bits of 1.5 2^(52 - k) is the double 1.5 2^(52 - k) + integer 2^-k, exactly
+__device__ __forceinline__ double combine(long long hi, long long lo) {
+    constexpr double mh = 1.5 * 2147483648.0, ml = 1.5 * 8.0;  // 1.5 2^31, 1.5 2^3
+    const double h = __longlong_as_double(__double_as_longlong(mh) + hi) - mh;
+    const double l = __longlong_as_double(__double_as_longlong(ml) + lo) - ml;
+    return h + l;
+}
+
 // 2^n as a double, for n in the normal range (exact)
 __device__ __forceinline__ double pow2(int n) { return __longlong_as_double((long long)(n + 1023) << 52); }
 
@@ -145,7 +159,7 @@ __device__ __forceinline__ void slice8(const double *x, int e, unsigned char *As
 }  // namespace rtc
 
 // Same arguments and results as k_mixed_residual (plus the operators' digit slices and
-// the error word); grid (ceil(sumK / 64), R), 256 threads: thread t and t + 128 share
+// the error word); grid (ceil(sumK / 64), R): the worker threads t and t + 128 share
 // column t % 128 (its tensor-memory lane), each slicing half of every K-chunk and
 // finishing half of every output chunk. The K-chunks of a contraction are pipelined
 // through two stages: the MMAs of one chunk run while the next chunk is sliced and its
@@ -165,6 +179,7 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar_m + 2);
     unsigned long long *s_max = reinterpret_cast<unsigned long long *>(smem_rt + 2 * SB + 64);
     const int t = threadIdx.x, tr = t & 127, half = t >> 7;
+    const bool worker = t < kWorkers, issuer = t == kWorkers;
     const int OC = oc_of(N), nkc = N / KC, nit = (N / OC) * nkc;
     const uint32_t ncols_t = tmem_cols(N);
     if (t == 0) {
@@ -182,7 +197,7 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
 
     const int r = blockIdx.y, g0 = blockIdx.x * 64;
     const int ncell = min(64, sumK - g0), ncols = 2 * ncell;
-    const bool live = tr < ncols;
+    const bool live = worker && tr < ncols;
     const int g = g0 + (live ? tr >> 1 : 0), a = tr & 1;
     const size_t colbase = ((size_t)r * sumK + g0) * 2;
     const size_t row = (colbase + (live ? tr : 0)) * N;  // this thread's column
@@ -217,9 +232,9 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
                     mx = u > mx ? u : mx;
                 }
         }
-        s_max[t] = mx;
+        if (worker) s_max[t] = mx;
         __syncthreads();
-        const unsigned long long m2 = s_max[t ^ 128];
+        const unsigned long long m2 = s_max[(t & 255) ^ 128];
         mx = m2 > mx ? m2 : mx;
         __syncthreads();  // s_max is reused by the next call
         const int E = (int)(mx >> 52);
@@ -234,13 +249,14 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
         const uint32_t idesc = tc::idesc_bf16(128, OC);
         const double p_in = pow2(e_in - 14);
         auto issue_copy = [&](int it, int b) {
-            if (t == 0) {
+            if (issuer) {
                 tc::mbar_arrive_expect_tx(&bar_b[b], b_block_bytes(N));
                 tc::bulk_copy_g2s(stg[b] + S * a_slice_bytes(), opsl + block_offset(N, it / nkc, it % nkc),
                                   b_block_bytes(N), &bar_b[b]);
             }
         };
-        auto slice_chunk = [&](int it, int b) {  // this thread's 16 inputs of the chunk
+        auto slice_chunk = [&](int it, int b) {  // this worker's 16 inputs of the chunk
+            if (!worker) return;
             const int k0 = (it % nkc) * KC + half * 16;
             double x[2][8];
             if (live) {
@@ -263,22 +279,24 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
         __syncthreads();
         for (int it = 0; it < nit; ++it) {
             const int b = it & 1, kc = it % nkc, oc = it / nkc;
-            if (t == 0) {
+            if (issuer) {
                 bool okb = tc::mbar_wait(&bar_b[b], fb[b]);
                 if (okb) {
                     tc::tc_fence_after();
-                    const uint32_t as = tc::smem_u32(stg[b]), bs = as + S * a_slice_bytes();
-                    for (int d = 0; d < S; ++d)
-                        for (int i = 0; i <= d; ++i) {
-                            const int j = d - i;
+                    // descriptors: a slice, a K-step further are address increments (16-byte units)
+                    const uint32_t as = tc::smem_u32(stg[b]);
+                    const uint64_t ad = tc::smem_desc(as, 128, KC * 16);
+                    const uint64_t bd = tc::smem_desc(as + S * a_slice_bytes(), 128, KC * 16);
+                    const uint32_t bstep = b_slice_bytes(N) >> 4;
+                    const uint32_t more = kc > 0 ? 1u : 0u;
 #pragma unroll
-                            for (int ks = 0; ks < KC / 16; ++ks) {
-                                const uint64_t ad = tc::smem_desc(as + i * a_slice_bytes() + 256u * ks, 128, KC * 16);
-                                const uint64_t bd = tc::smem_desc(bs + j * b_slice_bytes(N) + 256u * ks, 128, KC * 16);
-                                tc::mma_bf16(tmem + (uint32_t)(d * OC), ad, bd, idesc,
-                                             (kc > 0 || i > 0 || ks > 0) ? 1u : 0u);
-                            }
-                        }
+                    for (int d = 0; d < S; ++d)
+#pragma unroll
+                        for (int i = 0; i <= d; ++i)
+#pragma unroll
+                            for (int ks = 0; ks < KC / 16; ++ks)
+                                tc::mma_bf16(tmem + (uint32_t)(d * OC), ad + (uint64_t)(i * (a_slice_bytes() >> 4) + 16 * ks),
+                                             bd + (uint64_t)((d - i) * bstep + 16 * ks), idesc, i > 0 || ks > 0 ? 1u : more);
                 } else {
                     atomicExch(err, 1);
                     tc::mbar_wait(&bar_b[b], fb[b]);  // the copy must not land after the CTA has gone (bounded)
@@ -300,10 +318,11 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
                 // epilogue of output chunk oc: value(o) = 2^(e_in + e_o - 14) sum_d 2^(-7 d) A_d(o).
                 // The A_d are exact integers (|A_d| <= 2^24): hi = sum_{d < 4} A_d 2^(7 (3 - d))
                 // and lo = sum_{d >= 4} A_d 2^(7 (7 - d)) are exact 64-bit integers (below 2^46),
-                // so sum_d 2^(-7 d) A_d = hi 2^-21 + lo 2^-49 with one FP64 rounding
+                // so sum_d 2^(-7 d) A_d = hi 2^-21 + lo 2^-49 with one FP64 rounding; the power of
+                // two is applied at once where it is a normal number
                 ok = wait_mma(b) && ok;
                 tc::tc_fence_after();
-                for (int o16 = half * (OC / 2); o16 < (half + 1) * (OC / 2); o16 += 16) {
+                for (int o16 = half * (OC / 2); worker && o16 < (half + 1) * (OC / 2); o16 += 16) {
                     long long hi[16], lo[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) hi[i] = lo[i] = 0;
@@ -321,9 +340,11 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
                     double val[16];
                     const int o0 = oc * OC + o16;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        val[i] = fma((double)hi[i], 4.76837158203125e-07, (double)lo[i] * 1.7763568394002505e-15) *
-                                 p_in * pow2(eop[o0 + i]);
+                    for (int i = 0; i < 16; ++i) {
+                        const int eo = eop[o0 + i], n = e_in - 14 + eo;
+                        const double v = combine(hi[i], lo[i]);
+                        val[i] = n >= -1022 && n <= 1023 ? v * pow2(n) : v * p_in * pow2(eo);
+                    }
                     epi16(o0, val);
                 }
                 tc::tc_fence_before();  // the accumulator reads precede the next chunk's MMAs
@@ -373,81 +394,64 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
         for (int i = 0; i < 8; ++i) x[i] = sv[i] * pv[i] + (Qext ? qv[i] : 0.0);
     };
     const int e_x = ok ? row_exponent(in_x) : 0;
-    // the LD residual of this column's node for 16 ordinates, given both nodes' scattering
-    // source s (the partner node is the adjacent lane); the 16 ordinates share the sign of mu
-    // (N / 2 is a multiple of 16)
+    // the LD residual of this column's node for 16 ordinates, given the node's scattering
+    // source s; the 16 ordinates share the sign of mu (N / 2 is a multiple of 16)
     const int b = cell_inst[g], loc = g - off[b];
     const double hh = h[g], st = sigma_t[g], w = 2.0 / hh;
     const double *psr = psi + (size_t)r * sumK * 2 * N;
     if (ok) contract(ops.M, ops.eM, e_x, in_x, [&](int n0, const double *s) {
-        double sown[16], sL[16], sR[16];
-        if (Qang && live) {
-            double qa[16];
-            ld8(Qang + row + n0, qa, false);
-            ld8(Qang + row + n0 + 8, qa + 8, false);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) sown[i] = s[i] + qa[i];
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) sown[i] = s[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const double so = __shfl_xor_sync(0xffffffffu, sown[i], 1);
-            sL[i] = a ? so : sown[i];
-            sR[i] = a ? sown[i] : so;
-        }
         if (!live) return;
-        double m[16], pL[16], pR[16], pin[16];
-        ld8(mu + n0, m, false);
-        ld8(mu + n0 + 8, m + 8, false);
-        ld8(psr + ((size_t)2 * g) * N + n0, pL, false);
-        ld8(psr + ((size_t)2 * g) * N + n0 + 8, pL + 8, false);
-        ld8(psr + ((size_t)2 * g + 1) * N + n0, pR, false);
-        ld8(psr + ((size_t)2 * g + 1) * N + n0 + 8, pR + 8, false);
         const bool pos = n0 >= N / 2;  // mu_n > 0 for n >= N / 2 (ascending, symmetric)
-        if (pos ? loc > 0 : loc < Kc[b] - 1) {  // the upwind neighbour's outflow node
-            const double *src = psr + (pos ? ((size_t)2 * (g - 1) + 1) : ((size_t)2 * (g + 1))) * N + n0;
-            ld8(src, pin, false);
-            ld8(src + 8, pin + 8, false);
-        } else if (bc && bc[2 * b + (pos ? 0 : 1)] == kBcReflect) {  // the mirror ordinate's outflow
-            const double *node = psr + ((size_t)2 * g + (pos ? 0 : 1)) * N;
+        // m^{-1} (G psi - |mu| psi_in e_up) at this node: (2 mu / h) times a combination of the
+        // cell's nodal values and the inflow that depends on the direction and the node only
+        const double cL = pos ? (a ? -1.5 : 1.5) : -0.5, cR = pos ? 0.5 : (a ? -1.5 : 1.5);
+        const double ci = pos ? (a ? 1.0 : -2.0) : (a ? 2.0 : -1.0);
+        const bool inner = pos ? loc > 0 : loc < Kc[b] - 1;
+        const bool mirror = !inner && bc && bc[2 * b + (pos ? 0 : 1)] == kBcReflect;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) pin[i] = node[N - 1 - (n0 + i)];
-        } else if (psi_inc) {
-            const double *src = psi_inc + (((size_t)r * B + b) * 2 + (pos ? 0 : 1)) * N + n0;
-            ld8(src, pin, false);
-            ld8(src + 8, pin + 8, false);
-        } else {
+        for (int i0 = 0; i0 < 16; i0 += 8) {
+            const int n = n0 + i0;
+            double m[8], pL[8], pR[8], pin[8], qa[8];
+            ld8(mu + n, m, false);
+            ld8(psr + ((size_t)2 * g) * N + n, pL, false);
+            ld8(psr + ((size_t)2 * g + 1) * N + n, pR, false);
+            if (inner) {  // the upwind neighbour's outflow node
+                ld8(psr + (pos ? ((size_t)2 * (g - 1) + 1) : ((size_t)2 * (g + 1))) * N + n, pin, false);
+            } else if (mirror) {  // the mirror ordinate's outflow
+                const double *node = psr + ((size_t)2 * g + (pos ? 0 : 1)) * N;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) pin[i] = 0.0;
-        }
-        float v[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            double tL, tR;
-            if (pos) {
-                tL = 0.5 * m[i] * (pL[i] + pR[i]) - m[i] * pin[i];
-                tR = 0.5 * m[i] * (pR[i] - pL[i]);
+                for (int i = 0; i < 8; ++i) pin[i] = node[N - 1 - (n + i)];
+            } else if (psi_inc) {
+                ld8(psi_inc + (((size_t)r * B + b) * 2 + (pos ? 0 : 1)) * N + n, pin, false);
             } else {
-                tL = 0.5 * m[i] * (pR[i] - pL[i]);
-                tR = -0.5 * m[i] * (pL[i] + pR[i]) + m[i] * pin[i];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) pin[i] = 0.0;
             }
-            v[i] = a ? (float)(sR[i] - st * pR[i] - w * (2.0 * tR - tL))
-                     : (float)(sL[i] - st * pL[i] - w * (2.0 * tL - tR));
-        }
-        float4 *dd = reinterpret_cast<float4 *>(dq + row + n0);
+            if (Qang) {
+                ld8(Qang + row + n, qa, false);
+            } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) dd[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-        if (q32) {
-            float4 *dq2 = reinterpret_cast<float4 *>(q32 + row + n0);
+                for (int i = 0; i < 8; ++i) qa[i] = 0.0;
+            }
+            float v[8];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) dq2[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-        }
-        if (phi32) {
-            float4 *dp = reinterpret_cast<float4 *>(phi32 + row + n0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) dp[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int i = 0; i < 8; ++i) {
+                const double c = fma(cL, pL[i], fma(cR, pR[i], ci * pin[i]));
+                v[i] = (float)(fma(-st, a ? pR[i] : pL[i], Qang ? s[i0 + i] + qa[i] : s[i0 + i]) - (w * m[i]) * c);
+            }
+            const float4 lo = make_float4(v[0], v[1], v[2], v[3]), hi = make_float4(v[4], v[5], v[6], v[7]);
+            float4 *dd = reinterpret_cast<float4 *>(dq + row + n);
+            dd[0] = lo;
+            dd[1] = hi;
+            if (q32) {
+                float4 *dq2 = reinterpret_cast<float4 *>(q32 + row + n);
+                dq2[0] = lo;
+                dq2[1] = hi;
+            }
+            if (phi32) {
+                float4 *dp = reinterpret_cast<float4 *>(phi32 + row + n);
+                dp[0] = dp[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
         }
     });
     if (!ok && t == 0) atomicExch(err, 1);

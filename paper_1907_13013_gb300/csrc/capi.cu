@@ -591,7 +591,7 @@ int setup_tc(fpsa_ctx *ctx) {
     const int N = ctx->geo.N;
     // N <= 128: the operators stay in shared memory; N in (128, 256], a multiple of 32:
     // they are streamed in K-chunks (chunk-major layout)
-    ctx->tc_big = N > 128 && N <= 256 && N % tc::kChunkK == 0;
+    ctx->tc_big = N > 128 && N <= 256 && N % 32 == 0;
     ctx->tc_able = ((N % 16 == 0) && N >= 16 && N <= 128) || ctx->tc_big;
     if (!ctx->tc_able) return FPSA_OK;
     const size_t nn = (size_t)N * N;
@@ -612,12 +612,14 @@ int setup_tc(fpsa_ctx *ctx) {
     int nsm = 0;
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     if (ctx->tc_big) {
-        const int smem = (int)tc::BigPlan::make(N).total;
-        CK(raise_smem_limit((const void *)k_tc_fp_rhs_big, smem));
-        CK(raise_smem_limit((const void *)k_tc_update_scatter_big, smem));
-        CK(raise_smem_limit((const void *)k_tc_fp_rhs_moments<true>, smem));
-        CK(raise_smem_limit((const void *)k_tc_moments_axpy<true>, smem));
-        ctx->tc_grid = nsm;  // one CTA per SM (its shared memory)
+        const int smem = (int)tcw::Plan::make(N).total;
+        for (const void *k : {(const void *)k_tc_wide<tcw::FpRhs>, (const void *)k_tc_wide<tcw::UpdateScatter>,
+                              (const void *)k_tc_wide<tcw::RhsMoments>, (const void *)k_tc_wide<tcw::MomentsAxpy>}) {
+            CK(raise_smem_limit(k, smem));
+            CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
+        }
+        // two CTAs per SM (a third's tensor memory would have to wait: 3 x 256 columns)
+        ctx->tc_grid = 2 * nsm;
         return FPSA_OK;
     }
     const int smem = (int)tc::Plan::make(N).total;
@@ -625,8 +627,8 @@ int setup_tc(fpsa_ctx *ctx) {
     CK(raise_smem_limit((const void *)k_tc_update_scatter, smem));
     CK(raise_smem_limit((const void *)k_tc_fp_rhs_tile, smem));
     CK(raise_smem_limit((const void *)k_tc_update_scatter_tile, smem));
-    CK(raise_smem_limit((const void *)k_tc_fp_rhs_moments<false>, smem));
-    CK(raise_smem_limit((const void *)k_tc_moments_axpy<false>, smem));
+    CK(raise_smem_limit((const void *)k_tc_fp_rhs_moments, smem));
+    CK(raise_smem_limit((const void *)k_tc_moments_axpy, smem));
     ctx->tc_cols = tc::col_tile(ctx->geo.sumK, ctx->geo.R, nsm);
     if (ctx->tc_cols) {
         const int cs = (int)tc::ColPlan::make(N, ctx->tc_cols).total;
@@ -1113,10 +1115,10 @@ void tc_plan(const fpsa_ctx *ctx, MixedPlan &mp) {  // its tensor-core part (ctx
     const Geometry &g = ctx->geo;
     const int N = g.N;
     mp.tcops = TcOps{ctx->d_tc_ops, ctx->d_tc_ops + 2 * (size_t)N * N * sizeof(__nv_bfloat16)};
-    const int tc_tiles = ((2 * g.sumK + 127) / 128) * g.R;
-    mp.tc_blocks = std::max(1, std::min(tc_tiles, ctx->tc_grid));
     mp.tc_big = ctx->tc_big;
-    mp.tc_smem = mp.tc_big ? tc::BigPlan::make(N).total : tc::Plan::make(N).total;
+    const int cols = mp.tc_big ? tcw::kCT : 128, tc_tiles = ((2 * g.sumK + cols - 1) / cols) * g.R;
+    mp.tc_blocks = std::max(1, std::min(tc_tiles, ctx->tc_grid));
+    mp.tc_smem = mp.tc_big ? tcw::Plan::make(N).total : tc::Plan::make(N).total;
     mp.tc_full = !mp.tc_big && tc::Plan::make(N).full;
 }
 
@@ -1137,6 +1139,13 @@ int mixed_plan(fpsa_ctx *ctx, const fpsa_opts &o, MixedPlan &mp) {
 // The tensor-core contractions of the FP32 inner solves, by size: few columns per block
 // where that leaves no SM with more than one block (N <= 128; tc::col_tile), else
 // 128-column tiles, whole (N <= 64) or in k-chunks, with streamed operators for N > 128.
+int tc_wide(fpsa_ctx *ctx, const MixedPlan &mp, void (*kern)(tcw::Args, TcOps, int, int, int, int *),
+            const tcw::Args &a) {
+    CK(launch_pdl(kern, dim3(mp.tc_blocks), dim3(tcw::kThreads), mp.tc_smem, ctx->stream, a, mp.tcops, ctx->geo.N,
+                  ctx->geo.sumK, ctx->geo.R, ctx->d_dev_err));
+    return FPSA_OK;
+}
+
 int tc_fp_rhs(fpsa_ctx *ctx, const MixedPlan &mp, const float *psi, const float *phi, float *phi_half,
               const float *sigma_s, float *rhs) {
     const Geometry &g = ctx->geo;
@@ -1152,8 +1161,10 @@ int tc_fp_rhs(fpsa_ctx *ctx, const MixedPlan &mp, const float *psi, const float 
                           (size_t)tc::ColPlan::make(N, ct).total, st, psi, phi, phi_half, sigma_s,
                           (const double *)ctx->d_h, mp.tcops, rhs, N, g.sumK, ctx->d_dev_err);
     };
-    if (mp.tc_big) CK(tiles(k_tc_fp_rhs_big));
-    else if (ctx->tc_cols == 16) CK(cols(k_tc_fp_rhs_cols<16>));
+    if (mp.tc_big)
+        return tc_wide(ctx, mp, k_tc_wide<tcw::FpRhs>,
+                       tcw::Args{psi, phi, sigma_s, nullptr, ctx->d_h, phi_half, rhs, 0.f});
+    if (ctx->tc_cols == 16) CK(cols(k_tc_fp_rhs_cols<16>));
     else if (ctx->tc_cols == 32) CK(cols(k_tc_fp_rhs_cols<32>));
     else if (ctx->tc_cols == 64) CK(cols(k_tc_fp_rhs_cols<64>));
     else if (mp.tc_full) CK(tiles(k_tc_fp_rhs_tile));
@@ -1176,8 +1187,10 @@ int tc_update_scatter(fpsa_ctx *ctx, const MixedPlan &mp, const float *v, const 
                           (size_t)tc::ColPlan::make(N, ct).total, st, v, base, phi, sigma_s, mp.tcops, q, qang, N,
                           g.sumK, ctx->d_dev_err);
     };
-    if (mp.tc_big) CK(tiles(k_tc_update_scatter_big));
-    else if (ctx->tc_cols == 16) CK(cols(k_tc_update_scatter_cols<16>));
+    if (mp.tc_big)
+        return tc_wide(ctx, mp, k_tc_wide<tcw::UpdateScatter>,
+                       tcw::Args{v, base, sigma_s, qang, nullptr, phi, q, 0.f});
+    if (ctx->tc_cols == 16) CK(cols(k_tc_update_scatter_cols<16>));
     else if (ctx->tc_cols == 32) CK(cols(k_tc_update_scatter_cols<32>));
     else if (ctx->tc_cols == 64) CK(cols(k_tc_update_scatter_cols<64>));
     else if (mp.tc_full) CK(tiles(k_tc_update_scatter_tile));
@@ -1560,16 +1573,15 @@ int gm_fp_rhs(fpsa_ctx *ctx, PathBuffers<T> &p, const T *v, T *rhs) {
     Launch L_(ctx, FPSA_PHASE_CONTRACT);
     if constexpr (sizeof(T) == sizeof(float)) {
         if (ctx->gm_use_tc) {
-            const TcOps ops{ctx->d_tc_ops, ctx->d_tc_ops + 2 * (size_t)N * N * sizeof(__nv_bfloat16)};
-            const int blocks = std::max(1, std::min(((2 * g.sumK + 127) / 128) * g.R, ctx->tc_grid));
-            if (ctx->tc_big)
-                CK(launch_pdl(k_tc_fp_rhs_moments<true>, dim3(blocks), dim3(128), (size_t)tc::BigPlan::make(N).total, st,
-                              (const float *)v, (const float *)p.sigma_s, (const double *)ctx->d_h, ops, (float *)rhs, N,
-                              g.sumK, g.R, ctx->d_dev_err));
-            else
-                CK(launch_pdl(k_tc_fp_rhs_moments<false>, dim3(blocks), dim3(128), (size_t)tc::Plan::make(N).total, st,
-                              (const float *)v, (const float *)p.sigma_s, (const double *)ctx->d_h, ops, (float *)rhs, N,
-                              g.sumK, g.R, ctx->d_dev_err));
+            MixedPlan mp;
+            tc_plan(ctx, mp);
+            if (mp.tc_big)
+                return tc_wide(ctx, mp, k_tc_wide<tcw::RhsMoments>,
+                               tcw::Args{(const float *)v, nullptr, (const float *)p.sigma_s, nullptr, ctx->d_h, nullptr,
+                                         (float *)rhs, 0.f});
+            CK(launch_pdl(k_tc_fp_rhs_moments, dim3(mp.tc_blocks), dim3(128), mp.tc_smem, st, (const float *)v,
+                          (const float *)p.sigma_s, (const double *)ctx->d_h, mp.tcops, (float *)rhs, N, g.sumK, g.R,
+                          ctx->d_dev_err));
             return FPSA_OK;
         }
     }
@@ -1610,16 +1622,14 @@ int gm_axpy(fpsa_ctx *ctx, PathBuffers<T> &p, const T *psi, const T *base, T sig
     Launch L_(ctx, FPSA_PHASE_CONTRACT);
     if constexpr (sizeof(T) == sizeof(float)) {
         if (ctx->gm_use_tc) {
-            const TcOps ops{ctx->d_tc_ops, ctx->d_tc_ops + 2 * (size_t)N * N * sizeof(__nv_bfloat16)};
-            const int blocks = std::max(1, std::min(((2 * g.sumK + 127) / 128) * g.R, ctx->tc_grid));
-            if (ctx->tc_big)
-                CK(launch_pdl(k_tc_moments_axpy<true>, dim3(blocks), dim3(128), (size_t)tc::BigPlan::make(N).total, st,
-                              (const float *)psi, (const float *)base, (float)sign, ops, (float *)out, N, g.sumK, g.R,
-                              ctx->d_dev_err));
-            else
-                CK(launch_pdl(k_tc_moments_axpy<false>, dim3(blocks), dim3(128), (size_t)tc::Plan::make(N).total, st,
-                              (const float *)psi, (const float *)base, (float)sign, ops, (float *)out, N, g.sumK, g.R,
-                              ctx->d_dev_err));
+            MixedPlan mp;
+            tc_plan(ctx, mp);
+            if (mp.tc_big)
+                return tc_wide(ctx, mp, k_tc_wide<tcw::MomentsAxpy>,
+                               tcw::Args{(const float *)psi, (const float *)base, (const float *)p.sigma_s, nullptr, nullptr,
+                                         nullptr, (float *)out, (float)sign});
+            CK(launch_pdl(k_tc_moments_axpy, dim3(mp.tc_blocks), dim3(128), mp.tc_smem, st, (const float *)psi,
+                          (const float *)base, (float)sign, mp.tcops, (float *)out, N, g.sumK, g.R, ctx->d_dev_err));
             return FPSA_OK;
         }
     }

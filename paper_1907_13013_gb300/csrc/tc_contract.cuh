@@ -862,351 +862,284 @@ __global__ void __launch_bounds__(128) k_tc_update_scatter_cols(const float *v_i
 }
 
 // ---------------------------------------------------------------------------
-// Streamed-operator variants for N > 128 (N a multiple of 32, at most 256): the
-// operators (2 N^2 BF16 values each, split hi / lo) no longer fit shared memory next
-// to the column tile, so each GEMM streams them through three buffers in K-chunks of
-// 32 (an operator is stored chunk-major in global memory, [N / 32 chunks][N rows][32]
-// in the K-major core-matrix layout, so a chunk is one bulk copy; the operators are
-// shared by every tile and stay in L2); a buffer is refilled once the MMAs of the
-// chunk before the current one have read it, so two copies stay in flight while a
-// chunk is multiplied. The column tile (the A operand, 128 x N) is split from FP32
-// rows that each thread reads straight from global memory (row t of the tile is the
-// thread's accumulator lane), and every epilogue reads and writes its row the same
-// way, four 16-byte accesses per 16 columns and no block barrier between k-chunks,
-// several k-chunks of loads in flight per thread. The accumulator is N FP32 columns
-// of TMEM (M = 128, N = 256 per instruction).
+// Contractions for N > 128 (N a multiple of 32, at most 256): the operators (2 N^2 BF16
+// values each, split hi / lo) no longer fit shared memory. As in the few-column kernels the
+// operator is the A operand (rows = outputs, two M = 128 tiles) and a tile of CT = 64
+// columns the B operand, so that a warp's global accesses are 128 contiguous bytes of a
+// column and both nodes of a cell meet in one thread. A CTA is eight worker warps (thread t
+// owns output t of every column) and a driver thread that streams the operators through
+// kStages stages, 16 columns of hi and lo each (stored chunk-major in global memory, [N / 16
+// chunks][N rows][16] in the K-major core-matrix layout; shared by every tile, so they stay
+// in L2), across GEMMs and tiles: what it copies next never depends on the data. Two CTAs
+// per SM, so that one's loads and stores run during the other's products.
+// What bounds it: the operators' stream from L2 (0.5 MB a tile of 64 columns) and the
+// tile's own 0.26 MB of global traffic. A tile of 128 columns whose thread t owned COLUMN t
+// (rows of 1 KB read 16 bytes per lane and instruction, one CTA per SM) took 0.62 and 0.71
+// ms for 160000 columns at N = 256, now 0.44 and 0.50.
+//   k_tc_wide<FpRhs>         phi_half = D psi;  rhs = m (x) M Sigma (phi_half - phi)
+//   k_tc_wide<UpdateScatter> phi = phi_base + D v;  q = M (Sigma phi) + q_ang
+//   k_tc_wide<RhsMoments>    rhs = m (x) M Sigma v                 (GMRES; v: moments)
+//   k_tc_wide<MomentsAxpy>   out = base + sign D psi               (GMRES)
+// err is set to 1 if an mbarrier wait ran out (the CTA then stops).
 // ---------------------------------------------------------------------------
 namespace tc {
-constexpr int kChunkK = 32;
-constexpr int kBigBufs = 3;
+constexpr int kChunkK = 16;
 // byte offset of element (row, k) of an N x N operator in the chunk-major layout
 __host__ __device__ __forceinline__ uint32_t chunk_offset(int row, int k, int N) {
     return (uint32_t)(k / kChunkK) * (uint32_t)N * kChunkK * 2u + kmajor_offset(row, k % kChunkK, kChunkK);
 }
-// Shared-memory plan of a streamed CTA: x_hi, x_lo (128 x N BF16 each), three chunk
-// buffers of hi + lo (N x 32 BF16 each), 7 mbarriers, tmem slot.
-struct BigPlan {
-    uint32_t x_bytes, chunk_bytes, total;
-    __host__ __device__ static BigPlan make(int N) {
-        BigPlan p;
-        p.x_bytes = 128u * N * 2;
-        p.chunk_bytes = (uint32_t)N * kChunkK * 2;  // one part (hi or lo) of one chunk
-        p.total = 2 * p.x_bytes + 2 * kBigBufs * p.chunk_bytes + 128;
+}  // namespace tc
+
+namespace tcw {
+constexpr int kWorkers = 256, kThreads = kWorkers + 32, kCT = 64, kStages = 3;
+constexpr uint32_t kPart = 256u * tc::kChunkK * 2u, kStage = 2 * kPart;  // hi and lo of a chunk, 256 rows of room
+constexpr uint32_t kTmem = 256;                                          // two GEMMs x two row tiles x kCT
+struct Plan {
+    uint32_t x_bytes, stages, bars, total;
+    __host__ __device__ static Plan make(int N) {
+        Plan p;
+        p.x_bytes = (uint32_t)kCT * N * 2;
+        p.stages = 2 * p.x_bytes;
+        p.bars = p.stages + kStages * kStage;
+        p.total = p.bars + 128;
         return p;
     }
 };
-
-// 16 consecutive floats at p (16-byte aligned) through L2, or zeros.
-__device__ __forceinline__ void ld_row16(const float *p, bool live, float *v) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 x = live ? __ldcg(reinterpret_cast<const float4 *>(p) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-        v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
-    }
-}
-__device__ __forceinline__ void st_row16(float *p, const float *v) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        reinterpret_cast<float4 *>(p)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-}
-// Row t of the tile (N floats at src, zeros when not live), scaled elementwise by
-// scale (N floats, NULL: none), split into x_hi / x_lo; 64 columns of loads in flight.
-__device__ __forceinline__ void load_split_row(const float *src, const float *scale, bool live, int N,
-                                               unsigned char *x_hi, unsigned char *x_lo, int t) {
-    for (int k0 = 0; k0 < N; k0 += 64) {
-        float v[4][16], sc[4][16];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool in = live && k0 + 16 * j < N;
-            ld_row16(src + k0 + 16 * j, in, v[j]);
-            if (scale) ld_row16(scale + k0 + 16 * j, in, sc[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (k0 + 16 * j >= N) break;
-            if (scale) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[j][i] *= sc[j][i];
-            }
-            store_split_row16(x_hi, x_lo, t, k0 + 16 * j, v[j], N);
-        }
-    }
-}
-}  // namespace tc
-
-struct TcBig {
-    unsigned char *x_hi, *x_lo, *ch[tc::kBigBufs];  // ch[b]: hi then lo of buffer b
-    uint64_t *full, *empty, *bar_mma;               // full[kBigBufs], empty[kBigBufs]
-    uint32_t *tmem_slot;
-    uint32_t tmem, mma_phase;
-    uint32_t fills[tc::kBigBufs], reqs[tc::kBigBufs], commits[tc::kBigBufs];  // thread 0's view
+enum Kind { FpRhs, UpdateScatter, RhsMoments, MomentsAxpy };
+struct Args {
+    const float *in, *base, *sigma, *qang;  // psi / v, phi / phi_base / base, Sigma, q_ang (base, qang: may be NULL)
+    const double *h;
+    float *mid, *out;  // phi_half / phi; rhs / q / out (base may alias mid or out)
+    float sign;
 };
+}  // namespace tcw
 
-__device__ __forceinline__ void tc_big_setup(TcBig &s, unsigned char *smem, int N) {
-    const tc::BigPlan pl = tc::BigPlan::make(N);
-    s.x_hi = smem;
-    s.x_lo = smem + pl.x_bytes;
-    for (int b = 0; b < tc::kBigBufs; ++b) {
-        s.ch[b] = smem + 2 * pl.x_bytes + 2 * b * pl.chunk_bytes;
-        s.fills[b] = s.reqs[b] = s.commits[b] = 0;
-    }
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + 2 * pl.x_bytes + 2 * tc::kBigBufs * pl.chunk_bytes);
-    s.full = bars;
-    s.empty = bars + tc::kBigBufs;
-    s.bar_mma = bars + 2 * tc::kBigBufs;
-    s.tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * tc::kBigBufs + 1);
-    s.mma_phase = 0;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 2 * tc::kBigBufs + 1; ++i) tc::mbar_init(bars + i, 1);
+template <int KIND>
+__global__ void __launch_bounds__(tcw::kThreads, 2) k_tc_wide(tcw::Args g, TcOps ops, int N, int sumK, int R, int *err) {
+    using namespace tcw;
+    constexpr bool kMass = KIND == FpRhs || KIND == RhsMoments, kTwo = KIND == FpRhs || KIND == UpdateScatter;
+    constexpr int kGemms = kTwo ? 2 : 1;
+    extern __shared__ __align__(128) unsigned char smem_tc[];
+    __shared__ int s_fail;                // a wait of this CTA gave up
+    __shared__ float s_w[2][kCT / 2];     // h / 6 of a tile's cells
+    const Plan pl = Plan::make(N);
+    unsigned char *x_hi = smem_tc, *x_lo = smem_tc + pl.x_bytes, *stg = smem_tc + pl.stages;
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem_tc + pl.bars), *empty = full + kStages, *full_x = empty + kStages,
+             *acc_bar = full_x + 1, *drain = acc_bar + 1;
+    uint32_t *slot = reinterpret_cast<uint32_t *>(drain + 1);
+    const int t = threadIdx.x;
+    if (t == 0) {
+        for (int i = 0; i < 2 * kStages; ++i) tc::mbar_init(full + i, 1);
+        tc::mbar_init(full_x, kWorkers);
+        tc::mbar_init(acc_bar, 1);
+        tc::mbar_init(drain, 1);
+        s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (threadIdx.x < 32) {
-        tc::tmem_alloc(s.tmem_slot, tc::tmem_cols_for(N));
+    if (t < 32) {
+        tc::tmem_alloc(slot, kTmem);
         tc::tmem_relinquish();
     }
     __syncthreads();
     tc::tc_fence_after();
-    s.tmem = *s.tmem_slot;
-}
-
-// Out = X Op^T over K = N with the tile in x_hi / x_lo and the operator (hi, lo:
-// chunk-major in global memory) streamed chunk by chunk; returns false on a timeout.
-// Thread 0 runs the pipeline: chunks 0..2 are requested at once; after the MMAs of
-// chunk c are issued, the buffer of chunk c - 1 is refilled with chunk c + 2 once
-// those earlier MMAs have read it (its empty barrier), so the tensor core is not held
-// up by the copy just requested. Every wait is bounded.
-__device__ __forceinline__ bool tc_gemm_streamed(TcBig &s, const unsigned char *op_hi, const unsigned char *op_lo,
-                                                 int N, int *err) {
-    constexpr int NB = tc::kBigBufs;
-    tc::fence_async_smem();  // the tile's st.shared must be visible to the tensor core
-    tc::tc_fence_before();
-    __syncthreads();
-    bool ok = true;
-    if (threadIdx.x == 0) {
-        tc::tc_fence_after();
-        const int nch = N / tc::kChunkK;
-        const uint32_t cb = (uint32_t)N * tc::kChunkK * 2;
-        auto request = [&](int c) {
-            const int b = c % NB;
-            tc::mbar_arrive_expect_tx(&s.full[b], 2 * cb);
-            tc::bulk_copy_g2s(s.ch[b], op_hi + (size_t)c * cb, cb, &s.full[b]);
-            tc::bulk_copy_g2s(s.ch[b] + cb, op_lo + (size_t)c * cb, cb, &s.full[b]);
-            ++s.reqs[b];
+    const uint32_t tmem = *slot;
+    const int tiles_per_r = (2 * sumK + kCT - 1) / kCT, ntiles = tiles_per_r * R;
+    auto failed = [&]() { return *(volatile int *)&s_fail != 0; };
+    auto fail = [&]() {
+        *(volatile int *)&s_fail = 1;
+        atomicExch(err, 1);
+    };
+    if (t == kWorkers) {
+        // ---- driver: this CTA's tiles x GEMMs x chunks, in order
+        const int nch = N / tc::kChunkK, per_tile = kGemms * nch;
+        const uint32_t part = (uint32_t)N * tc::kChunkK * 2;  // bytes of hi (or lo) of a chunk
+        const int mine = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+        const uint32_t total = (uint32_t)mine * per_tile;
+        uint32_t issued = 0, q = 0;
+        bool ok = true;
+        auto copy_next = [&]() {
+            const int c = (int)(issued % per_tile), gm = c / nch, kc = c % nch, s = issued % kStages;
+            const unsigned char *op = (KIND == RhsMoments || gm == 1) ? ops.M : ops.D;
+            const unsigned char *src = op + (size_t)kc * part;
+            tc::mbar_arrive_expect_tx(&full[s], 2 * part);
+            tc::bulk_copy_g2s(stg + s * kStage, src, part, &full[s]);
+            tc::bulk_copy_g2s(stg + s * kStage + kPart, src + (size_t)N * N * 2, part, &full[s]);
+            ++issued;
         };
-        int issued = 0;
-        while (issued < nch && issued < NB) request(issued++);
-        const uint32_t idesc = tc::idesc_bf16(128, N);
-        const uint32_t xh = tc::smem_u32(s.x_hi), xl = tc::smem_u32(s.x_lo);
-        const uint32_t sbo_x = (uint32_t)N * 16, sbo_b = tc::kChunkK * 16;
-        for (int c = 0; c < nch && ok; ++c) {
-            const int b = c % NB;
-            ok = tc::mbar_wait(&s.full[b], s.fills[b] & 1u);
-            if (!ok) break;
-            ++s.fills[b];
-            tc::tc_fence_after();
-            const uint32_t oh = tc::smem_u32(s.ch[b]), ol = oh + cb;
-            for (int j = 0; j < tc::kChunkK / 16; ++j) {
-                const uint32_t ka = 256u * (uint32_t)(c * (tc::kChunkK / 16) + j), kb = 256u * (uint32_t)j;
-                const uint64_t a_hi = tc::smem_desc(xh + ka, 128, sbo_x), a_lo = tc::smem_desc(xl + ka, 128, sbo_x);
-                const uint64_t b_hi = tc::smem_desc(oh + kb, 128, sbo_b), b_lo = tc::smem_desc(ol + kb, 128, sbo_b);
-                tc::mma_bf16(s.tmem, a_hi, b_hi, idesc, (c > 0 || j > 0) ? 1u : 0u);
-                tc::mma_bf16(s.tmem, a_hi, b_lo, idesc, 1u);
-                tc::mma_bf16(s.tmem, a_lo, b_hi, idesc, 1u);
-            }
-            tc::mma_commit(&s.empty[b]);
-            ++s.commits[b];
-            if (c >= 1 && issued < nch) {  // chunk c - 1 + NB into the buffer of chunk c - 1
-                const int bp = (c - 1) % NB;
-                ok = tc::mbar_wait(&s.empty[bp], (s.commits[bp] - 1u) & 1u);
-                if (!ok) break;
-                request(issued++);
-            }
-        }
-        tc::mma_commit(s.bar_mma);
-        // every buffer's last commit has landed (its phases stay in step for the next
-        // GEMM), and on a timeout no requested copy is still landing (bounded)
-        for (int b = 0; b < NB; ++b) {
-            if (s.commits[b] > 0 && !tc::mbar_wait(&s.empty[b], (s.commits[b] - 1u) & 1u)) ok = false;
-            while (s.fills[b] < s.reqs[b]) {
-                if (!tc::mbar_wait(&s.full[b], s.fills[b] & 1u)) {
-                    ok = false;
+        const uint32_t idesc = tc::idesc_bf16(128, kCT), sbo_x = (uint32_t)N * 16;
+        const uint64_t bh0 = tc::smem_desc(tc::smem_u32(x_hi), 128, sbo_x), bl0 = tc::smem_desc(tc::smem_u32(x_lo), 128, sbo_x);
+        uint32_t xs = 0;  // tiles of x multiplied so far
+        for (; ok && q < total; ++q) {
+            while (issued < total && issued < q + kStages - 1) {  // (the products of chunk q - 2 free its stage)
+                if (issued >= (uint32_t)kStages &&
+                    !(ok = tc::mbar_wait(&empty[issued % kStages], (issued / kStages - 1u) & 1u)))
                     break;
+                copy_next();
+            }
+            const int s = q % kStages, c = (int)(q % per_tile), gm = c / nch, kc = c % nch;
+            ok = ok && !failed() && tc::mbar_wait(&full[s], (q / kStages) & 1u);
+            if (ok && kc == 0) {  // the workers' tile (no time limit but the flag: they wait for memory)
+                while (!tc::mbar_test(full_x, xs & 1u))
+                    if (failed()) {
+                        ok = false;
+                        break;
+                    }
+                ++xs;
+            }
+            if (!ok) break;
+            tc::tc_fence_after();
+            const uint64_t ah = tc::smem_desc(tc::smem_u32(stg + s * kStage), 128, tc::kChunkK * 16);
+            const uint64_t bh = bh0 + (uint64_t)(16 * kc), bl = bl0 + (uint64_t)(16 * kc);
+            const uint32_t more = kc > 0 ? 1u : 0u;
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const uint32_t acc = tmem + (uint32_t)((2 * gm + m) * kCT);
+                const uint64_t a_hi = ah + (uint64_t)(m * 4096 / 16), a_lo = a_hi + (uint64_t)(kPart / 16);
+                tc::mma_bf16(acc, a_hi, bh, idesc, more);
+                tc::mma_bf16(acc, a_hi, bl, idesc, 1u);
+                tc::mma_bf16(acc, a_lo, bh, idesc, 1u);
+            }
+            tc::mma_commit(&empty[s]);
+            if (kc == nch - 1) tc::mma_commit(acc_bar);
+        }
+        if (!ok) fail();
+        for (uint32_t j = q; j < issued; ++j)  // nothing may land after the CTA has gone (bounded)
+            if (!tc::mbar_wait(&full[j % kStages], (j / kStages) & 1u)) break;
+        tc::mma_commit(drain);
+        (void)tc::mbar_wait(drain, 0);
+    } else if (t < kWorkers) {
+        // ---- workers
+        tc::grid_dependency_wait();  // the inputs come from the previous kernel
+        const bool live = t < N;     // (N is a multiple of 32: whole warps)
+        const uint32_t at = tmem + ((uint32_t)(t & 96) << 16) + (uint32_t)((t >> 7) * kCT);
+        uint32_t accs = 0;
+        // 16 columns from column c0 into x_hi / x_lo (row = column, k = t; adjacent threads exchange
+        // values so that each stores two adjacent k of one column)
+        auto store16 = [&](int c0, const float (&v)[16]) {
+            const int odd = t & 1;
+#pragma unroll
+            for (int c = 0; c < 16; c += 2) {
+                const float other = __shfl_xor_sync(0xffffffffu, odd ? v[c] : v[c + 1], 1);
+                const float k0 = odd ? other : v[c], k1 = odd ? v[c + 1] : other;
+                __nv_bfloat16 h0, l0, h1, l1;
+                tc::split_bf16(k0, h0, l0);
+                tc::split_bf16(k1, h1, l1);
+                const uint32_t off = tc::kmajor_offset(c0 + c + odd, t & ~1, N);
+                *reinterpret_cast<uint32_t *>(x_hi + off) =
+                    (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                *reinterpret_cast<uint32_t *>(x_lo + off) =
+                    (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+            }
+        };
+        auto hand_over = [&]() {  // the tile in x_hi / x_lo to the driver
+            tc::fence_async_smem();
+            tc::tc_fence_before();
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(full_x)) : "memory");
+        };
+        auto wait_acc = [&]() {  // a GEMM's accumulators are ready; all workers agree whether to go on
+            if (!tc::mbar_wait(acc_bar, accs & 1u)) fail();
+            ++accs;
+            const bool stop = gbar_or(1, kWorkers, failed());
+            tc::tc_fence_after();
+            return !stop;
+        };
+        int par = 0;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, par ^= 1) {
+            const int r = tile / tiles_per_r, j0 = (tile % tiles_per_r) * kCT, nc = min(kCT, 2 * sumK - j0);
+            const size_t cb = ((size_t)r * sumK * 2 + j0) * N + t;
+            const float *sg = g.sigma + (size_t)(j0 >> 1) * N + t;
+            if (kMass && t < kCT / 2) s_w[par][t] = 2 * t < nc ? (float)(g.h[(j0 >> 1) + t] / 6.0) : 0.f;
+            if (live) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < kCT; c0 += 16) {
+                    float v[16];
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) v[c] = c0 + c < nc ? __ldcg(g.in + cb + (size_t)(c0 + c) * N) : 0.f;
+                    if constexpr (KIND == RhsMoments) {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            v[c] *= c0 + c < nc ? __ldg(sg + (size_t)((c0 + c) >> 1) * N) : 0.f;
+                    }
+                    store16(c0, v);
                 }
-                ++s.fills[b];
+            }
+            hand_over();
+            if constexpr (kTwo) {
+                if (!wait_acc()) break;
+                if (live) {
+#pragma unroll 1
+                    for (int c0 = 0; c0 < kCT; c0 += 16) {
+                        float a[16], b[16], s[8];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            b[c] = (g.base && c0 + c < nc) ? __ldcg(g.base + cb + (size_t)(c0 + c) * N) : 0.f;
+#pragma unroll
+                        for (int c = 0; c < 8; ++c)
+                            s[c] = c0 + 2 * c < nc ? __ldg(sg + (size_t)((c0 >> 1) + c) * N) : 0.f;
+                        tc::tmem_ld16(at + (uint32_t)c0, a);
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            if (KIND == UpdateScatter) a[c] += b[c];
+                            if (c0 + c < nc) g.mid[cb + (size_t)(c0 + c) * N] = a[c];
+                            a[c] = KIND == FpRhs ? s[c / 2] * (a[c] - b[c]) : s[c / 2] * a[c];
+                        }
+                        store16(c0, a);
+                    }
+                }
+                hand_over();
+            }
+            if (!wait_acc()) break;
+            if (live) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < kCT; c0 += 16) {
+                    float a[16], b[16];
+                    const float *add = KIND == UpdateScatter ? g.qang : (KIND == MomentsAxpy ? g.base : nullptr);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        b[c] = (!kMass && add && c0 + c < nc) ? __ldcg(add + cb + (size_t)(c0 + c) * N) : 0.f;
+                    tc::tmem_ld16(at + (uint32_t)((kGemms - 1) * 2 * kCT + c0), a);
+#pragma unroll
+                    for (int c = 0; c < 16; c += 2) {
+                        float y0, y1;
+                        if constexpr (kMass) {
+                            const float w = s_w[par][(c0 + c) >> 1];
+                            y0 = w * (2.f * a[c] + a[c + 1]);
+                            y1 = w * (a[c] + 2.f * a[c + 1]);
+                        } else if constexpr (KIND == MomentsAxpy) {
+                            y0 = b[c] + g.sign * a[c];
+                            y1 = b[c + 1] + g.sign * a[c + 1];
+                        } else {
+                            y0 = a[c] + b[c];
+                            y1 = a[c + 1] + b[c + 1];
+                        }
+                        if (c0 + c < nc) {  // (columns come in pairs)
+                            g.out[cb + (size_t)(c0 + c) * N] = y0;
+                            g.out[cb + (size_t)(c0 + c + 1) * N] = y1;
+                        }
+                    }
+                }
             }
         }
     }
-    ok = __syncthreads_and(ok) != 0;
-    // every MMA issued has completed before the accumulator is read or the CTA ends (bounded)
-    const bool done = tc::mbar_wait(s.bar_mma, s.mma_phase);
-    s.mma_phase ^= 1u;
-    tc::tc_fence_after();
-    ok = __syncthreads_and(ok && done) != 0;
-    if (!ok && threadIdx.x == 0) atomicExch(err, 1);
-    return ok;
-}
-
-__device__ __forceinline__ void tc_big_teardown(TcBig &s, int N) {
+    __syncwarp();
     tc::tc_fence_before();
     __syncthreads();
-    if (threadIdx.x < 32) tc::tmem_dealloc(s.tmem, tc::tmem_cols_for(N));
-}
-
-// k_tc_fp_rhs with streamed operators (N > 128).
-__global__ void __launch_bounds__(128) k_tc_fp_rhs_big(const float *__restrict__ psi_half,
-                                                       const float *__restrict__ phi, float *__restrict__ phi_half,
-                                                       const float *__restrict__ sigma_s,
-                                                       const double *__restrict__ h, TcOps ops,
-                                                       float *__restrict__ rhs, int N, int sumK, int R, int *err) {
-    extern __shared__ __align__(128) unsigned char smem_tc[];
-    TcBig s;
-    tc_big_setup(s, smem_tc, N);
-    tc::grid_dependency_wait();  // the inputs come from the previous kernel
-    const int t = threadIdx.x;
-    const uint32_t lane_base = (uint32_t)(t & ~31) << 16;
-    const int tiles_per_r = (2 * sumK + 127) / 128;
-    const int ntiles = tiles_per_r * R;
-    const size_t opb = (size_t)N * N * 2;  // bytes of one part of one operator
-    bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-        const int r = tile / tiles_per_r, j0 = (tile % tiles_per_r) * 128;
-        const int ncols = min(128, 2 * sumK - j0);
-        const bool live = t < ncols;
-        const int g = live ? (j0 + t) >> 1 : 0;
-        const size_t row = ((size_t)r * sumK * 2 + j0 + t) * N;  // this thread's column of the tile
-        tc::load_split_row(psi_half + row, nullptr, live, N, s.x_hi, s.x_lo, t);
-        if (!(ok = tc_gemm_streamed(s, ops.D, ops.D + opb, N, err))) break;
-        // phi_half = D psi_half; next A = Sigma (phi_half - phi)
-        const float *sig = sigma_s + (size_t)g * N;
-        for (int k0 = 0; k0 < N; k0 += 16) {
-            float a[16], ph[16], sg[16], v[16];
-            tc::ld_row16(phi + row + k0, live, ph);
-            tc::ld_row16(sig + k0, live, sg);
-            tc::tmem_ld16(s.tmem + lane_base + k0, a);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = live ? sg[i] * (a[i] - ph[i]) : 0.f;
-            if (live) tc::st_row16(phi_half + row + k0, a);
-            tc::store_split_row16(s.x_hi, s.x_lo, t, k0, v, N);
-        }
-        if (!(ok = tc_gemm_streamed(s, ops.M, ops.M + opb, N, err))) break;
-        // rhs = m (x) r: the node partner is the adjacent lane (column j ^ 1)
-        const float w = live ? (float)(h[g] / 6.0) : 0.f;
-        for (int k0 = 0; k0 < N; k0 += 16) {
-            float a[16], o[16];
-            tc::tmem_ld16(s.tmem + lane_base + k0, a);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float other = __shfl_xor_sync(0xffffffffu, a[i], 1);
-                o[i] = w * (2.f * a[i] + other);
-            }
-            if (live) tc::st_row16(rhs + row + k0, o);
-        }
-    }
-    tc_big_teardown(s, N);
-}
-
-// k_tc_update_scatter with streamed operators (N > 128).
-__global__ void __launch_bounds__(128) k_tc_update_scatter_big(const float *__restrict__ v_in,
-                                                               const float *__restrict__ phi_base,
-                                                               float *__restrict__ phi,
-                                                               const float *__restrict__ sigma_s, TcOps ops,
-                                                               float *__restrict__ q, const float *__restrict__ qang,
-                                                               int N, int sumK, int R, int *err) {
-    extern __shared__ __align__(128) unsigned char smem_tc[];
-    TcBig s;
-    tc_big_setup(s, smem_tc, N);
-    tc::grid_dependency_wait();  // the inputs come from the previous kernel
-    const int t = threadIdx.x;
-    const uint32_t lane_base = (uint32_t)(t & ~31) << 16;
-    const int tiles_per_r = (2 * sumK + 127) / 128;
-    const int ntiles = tiles_per_r * R;
-    const size_t opb = (size_t)N * N * 2;
-    bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-        const int r = tile / tiles_per_r, j0 = (tile % tiles_per_r) * 128;
-        const int ncols = min(128, 2 * sumK - j0);
-        const bool live = t < ncols;
-        const int g = live ? (j0 + t) >> 1 : 0;
-        const size_t row = ((size_t)r * sumK * 2 + j0 + t) * N;
-        tc::load_split_row(v_in + row, nullptr, live, N, s.x_hi, s.x_lo, t);
-        if (!(ok = tc_gemm_streamed(s, ops.D, ops.D + opb, N, err))) break;
-        // phi = phi_base + D v (read before written: phi_base may alias phi); next A = Sigma phi
-        const float *sig = sigma_s + (size_t)g * N;
-        for (int k0 = 0; k0 < N; k0 += 16) {
-            float a[16], pb[16], sg[16], v[16];
-            tc::ld_row16(phi_base ? phi_base + row + k0 : nullptr, live && phi_base, pb);
-            tc::ld_row16(sig + k0, live, sg);
-            tc::tmem_ld16(s.tmem + lane_base + k0, a);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                a[i] += pb[i];
-                v[i] = live ? sg[i] * a[i] : 0.f;
-            }
-            if (live) tc::st_row16(phi + row + k0, a);
-            tc::store_split_row16(s.x_hi, s.x_lo, t, k0, v, N);
-        }
-        if (!(ok = tc_gemm_streamed(s, ops.M, ops.M + opb, N, err))) break;
-        // q = M (Sigma phi) + q_ang
-        for (int k0 = 0; k0 < N; k0 += 16) {
-            float a[16], qa[16];
-            tc::ld_row16(qang ? qang + row + k0 : nullptr, live && qang, qa);
-            tc::tmem_ld16(s.tmem + lane_base + k0, a);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[i] += qa[i];
-            if (live) tc::st_row16(q + row + k0, a);
-        }
-    }
-    tc_big_teardown(s, N);
+    if (t < 32) tc::tmem_dealloc(tmem, kTmem);
 }
 
 // ---------------------------------------------------------------------------
-// Tensor-core contractions of the GMRES operator (the FP32 inner solve of GMRES-IR),
-// one GEMM each, with the operators either in shared memory (N <= 128) or streamed
-// (N > 128); TcEngine picks the form at compile time.
+// Tensor-core contractions of the GMRES operator (the FP32 inner solve of GMRES-IR), one
+// GEMM each, N <= 128 (above: k_tc_wide).
 //   k_tc_fp_rhs_moments:  rhs = m (x) M Sigma v      (v: moments)
 //   k_tc_moments_axpy:    out = base + sign D psi   (base may be NULL or alias out)
 // ---------------------------------------------------------------------------
-template <bool kBig>
-struct TcEngine {
-    TcCta a;
-    TcBig b;
-    float *stA, *stB, *stC;
-    unsigned char *x_hi, *x_lo;
-    uint32_t tmem;
-    __device__ __forceinline__ bool setup(unsigned char *smem, const TcOps &ops, int N, int *err) {
-        bool ok = true;
-        if constexpr (kBig) {  // global I/O straight from the threads' rows: no staging buffers
-            tc_big_setup(b, smem, N);
-            stA = stB = stC = nullptr;
-            x_hi = b.x_hi; x_lo = b.x_lo; tmem = b.tmem;
-        } else {
-            ok = tc_cta_setup(a, smem, ops, N, err);
-            stA = a.stA; stB = a.stB; stC = a.stC; x_hi = a.x_hi; x_lo = a.x_lo; tmem = a.tmem;
-        }
-        return ok;
-    }
-    __device__ __forceinline__ bool gemm(const TcOps &ops, bool use_d, int N, int *err) {
-        if constexpr (kBig) {
-            const unsigned char *o = use_d ? ops.D : ops.M;
-            return tc_gemm_streamed(b, o, o + (size_t)N * N * 2, N, err);
-        } else {
-            return tc_gemm(a, use_d ? a.opD_hi : a.opM_hi, use_d ? a.opD_lo : a.opM_lo, N, err);
-        }
-    }
-    __device__ __forceinline__ void teardown(int N) {
-        if constexpr (kBig) tc_big_teardown(b, N);
-        else tc_cta_teardown(a, N);
-    }
-};
-
-template <bool kBig>
 __global__ void __launch_bounds__(128) k_tc_fp_rhs_moments(const float *__restrict__ v,
                                                            const float *__restrict__ sigma_s,
                                                            const double *__restrict__ h, TcOps ops,
                                                            float *__restrict__ rhs, int N, int sumK, int R, int *err) {
     extern __shared__ __align__(128) unsigned char smem_tc[];
-    TcEngine<kBig> e;
-    bool ok = e.setup(smem_tc, ops, N, err);
+    TcCta e;
+    bool ok = tc_cta_setup(e, smem_tc, ops, N, err);
     tc::grid_dependency_wait();  // the inputs come from the previous kernel
     const int t = threadIdx.x;
     const uint32_t lane_base = (uint32_t)(t & ~31) << 16;
@@ -1220,24 +1153,19 @@ __global__ void __launch_bounds__(128) k_tc_fp_rhs_moments(const float *__restri
         const size_t cb = ((size_t)r * sumK * 2 + j0) * N;
         const float *sig = sigma_s + (size_t)(j0 >> 1) * N;
         // A = Sigma v
-        if constexpr (kBig) {
-            tc::load_split_row(v + cb + (size_t)t * N, sigma_s + (size_t)(live ? g : 0) * N, live, N, e.x_hi,
-                               e.x_lo, t);
-        } else {
-            for (int k0 = 0; k0 < N; k0 += tc::kStageK) {
-                tc::stage_in(e.stA, v + cb, N, ncols, k0);
-                tc::stage_in(e.stB, sig, N, ncell, k0);
-                __syncthreads();
-                float vv[16], sg[16], a[16];
-                tc::row_get16(e.stA, t, vv);
-                tc::row_get16(e.stB, t >> 1, sg);
+        for (int k0 = 0; k0 < N; k0 += tc::kStageK) {
+            tc::stage_in(e.stA, v + cb, N, ncols, k0);
+            tc::stage_in(e.stB, sig, N, ncell, k0);
+            __syncthreads();
+            float vv[16], sg[16], a[16];
+            tc::row_get16(e.stA, t, vv);
+            tc::row_get16(e.stB, t >> 1, sg);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) a[i] = live ? sg[i] * vv[i] : 0.f;
-                tc::store_split_row16(e.x_hi, e.x_lo, t, k0, a, N);
-                __syncthreads();
-            }
+            for (int i = 0; i < 16; ++i) a[i] = live ? sg[i] * vv[i] : 0.f;
+            tc::store_split_row16(e.x_hi, e.x_lo, t, k0, a, N);
+            __syncthreads();
         }
-        if (!(ok = e.gemm(ops, false, N, err))) break;
+        if (!(ok = tc_gemm(e, e.opM_hi, e.opM_lo, N, err))) break;
         // rhs = m (x) r: node partner is the adjacent lane (column j ^ 1)
         const float w = live ? (float)(h[g] / 6.0) : 0.f;
         for (int k0 = 0; k0 < N; k0 += tc::kStageK) {
@@ -1248,25 +1176,20 @@ __global__ void __launch_bounds__(128) k_tc_fp_rhs_moments(const float *__restri
                 const float other = __shfl_xor_sync(0xffffffffu, a[i], 1);
                 o[i] = w * (2.f * a[i] + other);
             }
-            if constexpr (kBig) {
-                if (live) tc::st_row16(rhs + cb + (size_t)t * N + k0, o);
-            } else {
-                __syncthreads();  // stC of the previous chunk has been written out
-                tc::row_put16(e.stC, t, o);
-                __syncthreads();
-                tc::stage_out(e.stC, rhs + cb, N, ncols, k0);
-            }
+            __syncthreads();  // stC of the previous chunk has been written out
+            tc::row_put16(e.stC, t, o);
+            __syncthreads();
+            tc::stage_out(e.stC, rhs + cb, N, ncols, k0);
         }
     }
-    e.teardown(N);
+    tc_cta_teardown(e, N);
 }
 
-template <bool kBig>
 __global__ void __launch_bounds__(128) k_tc_moments_axpy(const float *__restrict__ psi, const float *base, float sign,
                                                          TcOps ops, float *out, int N, int sumK, int R, int *err) {
     extern __shared__ __align__(128) unsigned char smem_tc[];
-    TcEngine<kBig> e;
-    bool ok = e.setup(smem_tc, ops, N, err);
+    TcCta e;
+    bool ok = tc_cta_setup(e, smem_tc, ops, N, err);
     tc::grid_dependency_wait();  // the inputs come from the previous kernel
     const int t = threadIdx.x;
     const uint32_t lane_base = (uint32_t)(t & ~31) << 16;
@@ -1276,46 +1199,31 @@ __global__ void __launch_bounds__(128) k_tc_moments_axpy(const float *__restrict
         const int r = tile / tiles_per_r, j0 = (tile % tiles_per_r) * 128;
         const int ncols = min(128, 2 * sumK - j0);
         const size_t cb = ((size_t)r * sumK * 2 + j0) * N;
-        if constexpr (kBig) {
-            tc::load_split_row(psi + cb + (size_t)t * N, nullptr, t < ncols, N, e.x_hi, e.x_lo, t);
-        } else {
-            for (int k0 = 0; k0 < N; k0 += tc::kStageK) {
-                tc::stage_in(e.stA, psi + cb, N, ncols, k0);
-                __syncthreads();
-                float vv[16];
-                tc::row_get16(e.stA, t, vv);
-                tc::store_split_row16(e.x_hi, e.x_lo, t, k0, vv, N);
-                __syncthreads();
-            }
+        for (int k0 = 0; k0 < N; k0 += tc::kStageK) {
+            tc::stage_in(e.stA, psi + cb, N, ncols, k0);
+            __syncthreads();
+            float vv[16];
+            tc::row_get16(e.stA, t, vv);
+            tc::store_split_row16(e.x_hi, e.x_lo, t, k0, vv, N);
+            __syncthreads();
         }
-        if (!(ok = e.gemm(ops, true, N, err))) break;
+        if (!(ok = tc_gemm(e, e.opD_hi, e.opD_lo, N, err))) break;
         // out = base + sign D psi (base read chunk by chunk before out is written: it may alias)
         for (int k0 = 0; k0 < N; k0 += tc::kStageK) {
-            if constexpr (kBig) {
-                const bool live = t < ncols;
-                const size_t row = cb + (size_t)t * N + k0;
-                float a[16], bs[16];
-                tc::ld_row16(base ? base + row : nullptr, live && base, bs);
-                tc::tmem_ld16(e.tmem + lane_base + k0, a);
+            if (base) tc::stage_in(e.stA, base + cb, N, ncols, k0);
+            float a[16];
+            tc::tmem_ld16(e.tmem + lane_base + k0, a);
+            __syncthreads();
+            float bs[16];
+            if (base) tc::row_get16(e.stA, t, bs);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) a[i] = bs[i] + sign * a[i];
-                if (live) tc::st_row16(out + row, a);
-            } else {
-                if (base) tc::stage_in(e.stA, base + cb, N, ncols, k0);
-                float a[16];
-                tc::tmem_ld16(e.tmem + lane_base + k0, a);
-                __syncthreads();
-                float bs[16];
-                if (base) tc::row_get16(e.stA, t, bs);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) a[i] = (base ? bs[i] : 0.f) + sign * a[i];
-                tc::row_put16(e.stC, t, a);
-                __syncthreads();
-                tc::stage_out(e.stC, out + cb, N, ncols, k0);
-            }
+            for (int i = 0; i < 16; ++i) a[i] = (base ? bs[i] : 0.f) + sign * a[i];
+            tc::row_put16(e.stC, t, a);
+            __syncthreads();
+            tc::stage_out(e.stC, out + cb, N, ncols, k0);
         }
     }
-    e.teardown(N);
+    tc_cta_teardown(e, N);
 }
 
 }  // namespace fpsa

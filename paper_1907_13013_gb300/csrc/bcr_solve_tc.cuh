@@ -20,17 +20,20 @@
 // chunk: A^{-1} by (slice, 32 columns), 16 KB (k_bcr_factor_split), a coupling block by 16
 // columns (k_bcr_coupling_split).
 //
-// A CTA is four worker warps and a driver thread that share a ring of kStages stages, a
-// chunk of the operand A and one of the operand B each. The driver copies A chunks as many
-// stages ahead as are free, across units, and issues the products of a stage once its copy
-// has landed and the workers have written its B chunk; the workers load the vectors four
-// chunks ahead, split them, and run the epilogues. What bounds it: at the wide levels the
+// A CTA is four worker warps, a copying and an issuing thread that share a ring of kStages
+// stages, a chunk of the operand A and one of the operand B each. The copying thread takes
+// the units and copies A chunks as many stages ahead as are free, across units; the issuing
+// thread issues the products of a stage once its copy has landed and the workers have
+// written its B chunk; the workers load the vectors four chunks ahead, split them, and run
+// the epilogues. (One thread for copies and products, with descriptors built for each, took
+// 1 us a chunk, half of the time of a unit.) What bounds it: at the wide levels the
 // factors' stream through the stages (with the conversion of the vectors behind it), at
 // the narrow ones the chain of hops, each a unit's length. Hence slices of 128 rows (four
 // CTAs share a cell at 2N = 512) and a pipeline without a block barrier per chunk: one CTA
 // for all rows, 16-column chunks with a barrier, a wait for the products and a copy issued
 // only then, and the couplings on the FP32 cores took 3.43 ms at 2N = 512, 1250 cells and
-// 64 right-hand sides, 1.72 ms with 16; this one 1.68 and 1.25 ms.
+// 64 right-hand sides, 1.72 ms with 16; with one thread for copies and products 1.68 and
+// 1.25 ms, now 1.20 and 0.70 ms.
 //
 // Units are taken from a work queue in phase order (forward levels, roots, backward
 // levels), within a phase the slices others wait for first: a unit depends only on units
@@ -47,10 +50,11 @@
 namespace fpsa {
 namespace tcs {
 
-constexpr int kWorkers = 128, kThreads = kWorkers + 32;
+constexpr int kWorkers = 128, kThreads = kWorkers + 64;  // a copying and an issuing warp
 constexpr int kK = 32;                     // factor columns per chunk
 constexpr int kKc = 16;                    // coupling columns per chunk
 constexpr int kStages = 4;
+constexpr unsigned kFlagTries = 1u << 28;
 constexpr int kAhead = 4;                  // chunks of the vectors in flight per worker
 constexpr int kUnitRing = 8;               // units the driver may have taken ahead of the workers
 constexpr int kMaxRT = 64;                 // right-hand sides per unit
@@ -244,23 +248,27 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
     auto push_right = [&](const Unit &u) { return !u.bwd && u.right >= 0 && u.m == MT - 1; };
     auto push_left = [&](const Unit &u) { return !u.bwd && u.left >= 0 && u.m == 0; };
     auto n_main = [&](const Unit &u) { return (u.bwd ? (u.right >= 0 ? N : h2) : n2) / kK; };
-    auto n_coup = [&](const Unit &u) {
-        return u.bwd ? (u.right >= 0 ? 2 * nc : nc) : ((push_right(u) ? nc : 0) + (push_left(u) ? nc : 0));
-    };
 
+    // Waits of the copying and the issuing thread: the workers may be waiting for other
+    // units, with their own limit, so these end by the flag (kFlagTries is far beyond it).
+    auto wait_flag = [&](uint64_t *bar, uint32_t par) {
+        for (unsigned i = 0; !tc::mbar_test(bar, par); ++i)
+            if (failed() || i > kFlagTries) return false;
+        return true;
+    };
     if (t == kWorkers) {
-        // ---- driver
+        // ---- copies: takes the units and streams their chunks of A through the stages
         int total = 0;
         auto phase_items = [&](int ph) {
             const int l = ph <= nl ? ph : 2 * nl - ph;
             return l < nl ? lv.off[l + 1] - lv.off[l] : lv.n_roots;
         };
         for (int ph = 0; ph <= P; ++ph) total += phase_items(ph) * nch * MT;
-        uint32_t head = 0;  // the unit being multiplied (of the ring; those after it are being copied)
         int popped = atomicAdd(queue, 1);
-        uint32_t taken = 0, issued = 0, q = 0;
+        uint32_t issued = 0;
         bool ok = true;
-        auto take = [&]() {  // the next unit into the ring
+        for (uint32_t taken = 0; ok; ++taken) {
+            // the next unit into the ring (at most kStages + 1 units beyond the workers')
             Unit u{};
             u.id = popped < total ? popped : -1;
             if (u.id >= 0) {
@@ -287,103 +295,100 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
             }
             ring[taken % kUnitRing] = u;
             mbar_arrive(&unit_bar[taken % kUnitRing]);  // (release)
-            ++taken;
-            return u.id >= 0;
-        };
-        int copy_i = 0;       // next chunk to copy, of unit copy_u
-        uint32_t copy_u = 0;
-        bool more = take();
-        // copy one more chunk if its stage is free (its earlier products done) and there is one
-        auto copy_next = [&]() {
-            if (!more) return false;
-            const Unit &u = ring[copy_u % kUnitRing];
-            const int s = issued % kStages;
-            const unsigned char *src;
-            uint32_t bytes = kChunkA;
-            const int nm = n_main(u);
-            const int mi = u.bwd ? copy_i - n_coup(u) : copy_i, ci = u.bwd ? copy_i : copy_i - nm;
-            if (mi >= 0 && mi < nm) {
-                src = Atc + (size_t)u.cell * cell_bytes(n2) +
-                      ((size_t)u.m * (n2 / kK) + (u.bwd ? h2 / kK : 0) + mi) * kChunkA;
-            } else {
-                const bool second = ci >= nc || (!u.bwd && !push_right(u));  // the coupling with the other neighbour
-                const int slot = u.bwd ? u.s_cell : (second ? u.s_left : u.s_right);
-                src = (second ? Ctc : Btc) + (size_t)slot * coupling_bytes(n2) + (size_t)(ci % nc) * coupling_chunk(n2);
-                bytes = coupling_chunk(n2);
-            }
-            tc::mbar_arrive_expect_tx(&full_a[s], bytes);
-            tc::bulk_copy_g2s(smem_tcs + s * pl.stage, src, bytes, &full_a[s]);
-            ++issued;
-            if (++copy_i == nm + n_coup(u)) {
-                copy_i = 0;
-                ++copy_u;
-                more = take();
-            }
-            return true;
-        };
-        const uint32_t idesc = tc::idesc_bf16(128, RT);
-        while (ok && ring[head % kUnitRing].id >= 0) {
-            const Unit u = ring[head % kUnitRing];
-            const int nm = n_main(u), ncp = n_coup(u), ns = nm + ncp;
-            for (int i = 0; i < ns && ok; ++i, ++q) {
-                // copies ahead: the stage of chunk q + d is free once chunk q + d - kStages is done
-                while (issued < q + kStages - 1) {  // (the products of chunk q - 2, not of the one just issued)
-                    if (issued >= (uint32_t)kStages && !(ok = tc::mbar_wait(&empty[issued % kStages],
-                                                                            (issued / kStages - 1u) & 1u)))
-                        break;
-                    if (!copy_next()) break;
+            if (u.id < 0) break;
+            auto copy = [&](const unsigned char *src, int chunks, uint32_t bytes) {
+                for (int c = 0; c < chunks && ok; ++c, src += bytes, ++issued) {
+                    const int s = issued % kStages;
+                    if (issued >= (uint32_t)kStages) ok = wait_flag(&empty[s], (issued / kStages - 1u) & 1u);
+                    if (!ok) break;
+                    tc::mbar_arrive_expect_tx(&full_a[s], bytes);
+                    tc::bulk_copy_g2s(smem_tcs + s * pl.stage, src, bytes, &full_a[s]);
                 }
-                const int s = q % kStages;
-                const uint32_t par = (q / kStages) & 1u;
-                ok = ok && !failed() && tc::mbar_wait(&full_a[s], par);
-                if (ok) {  // the workers may be waiting for other units (their own bound): no time limit but the flag
-                    while (!tc::mbar_test(&full_b[s], par))
-                        if (failed()) {
-                            ok = false;
-                            break;
-                        }
-                }
-                if (!ok) break;
-                tc::tc_fence_after();
-                const int mi = u.bwd ? i - ncp : i, ci = u.bwd ? i : i - nm;
-                const uint32_t a0 = tc::smem_u32(smem_tcs + s * pl.stage), b0 = a0 + kChunkA;
-                if (mi >= 0 && mi < nm) {
-                    for (int j = 0; j < kK / 16; ++j) {
-                        const uint64_t ah = tc::smem_desc(a0 + 256u * j, 128, kK * 16),
-                                       al = tc::smem_desc(a0 + kChunkA / 2 + 256u * j, 128, kK * 16);
-                        const uint64_t bh = tc::smem_desc(b0 + 256u * j, 128, kK * 16),
-                                       bl = tc::smem_desc(b0 + RT * kK * 2u + 256u * j, 128, kK * 16);
-                        tc::mma_bf16(tmem, ah, bh, idesc, (mi > 0 || j > 0) ? 1u : 0u);
-                        tc::mma_bf16(tmem, ah, bl, idesc, 1u);
-                        tc::mma_bf16(tmem, al, bh, idesc, 1u);
-                    }
-                } else {
-                    // (rows from N/2 up read what follows in the stage; their accumulator lanes are ignored)
-                    const bool second = ci >= nc || (!u.bwd && !push_right(u));
-                    const uint32_t acc = tmem + (second ? 2u * RT : (uint32_t)RT);
-                    uint64_t a[3], b[3];
-                    for (int k = 0; k < 3; ++k) {
-                        a[k] = tc::smem_desc(a0 + (uint32_t)k * h2 * kKc * 2u, 128, kKc * 16);
-                        b[k] = tc::smem_desc(b0 + (uint32_t)k * RT * kKc * 2u, 128, kKc * 16);
-                    }
-                    tc::mma_bf16(acc, a[0], b[0], idesc, ci % nc > 0 ? 1u : 0u);
-                    tc::mma_bf16(acc, a[0], b[1], idesc, 1u);
-                    tc::mma_bf16(acc, a[1], b[0], idesc, 1u);
-                    tc::mma_bf16(acc, a[0], b[2], idesc, 1u);
-                    tc::mma_bf16(acc, a[2], b[0], idesc, 1u);
-                    tc::mma_bf16(acc, a[1], b[1], idesc, 1u);
-                }
-                tc::mma_commit(&empty[s]);
-                // the end of the unit's first or second group of chunks: the workers read its accumulators
-                if (i == (u.bwd ? ncp : nm) - 1 || i == ns - 1) tc::mma_commit(seg_bar);
-            }
-            ++head;
+            };
+            const unsigned char *main = Atc + (size_t)u.cell * cell_bytes(n2) +
+                                        ((size_t)u.m * (n2 / kK) + (u.bwd ? h2 / kK : 0)) * kChunkA;
+            const size_t cbytes = coupling_bytes(n2);
+            if (!u.bwd) copy(main, n_main(u), kChunkA);
+            if (u.bwd || push_right(u)) copy(Btc + (size_t)(u.bwd ? u.s_cell : u.s_right) * cbytes, nc, coupling_chunk(n2));
+            if (u.bwd ? u.right >= 0 : push_left(u))
+                copy(Ctc + (size_t)(u.bwd ? u.s_cell : u.s_left) * cbytes, nc, coupling_chunk(n2));
+            if (u.bwd) copy(main, n_main(u), kChunkA);
         }
         if (!ok) fail();
-        // every copy and product has landed before the CTA ends (bounded)
-        for (uint32_t j = q; j < issued; ++j)
+        // every copy has landed before the CTA ends (bounded)
+        for (uint32_t j = issued > (uint32_t)kStages ? issued - kStages : 0; j < issued; ++j)
             if (!tc::mbar_wait(&full_a[j % kStages], (j / kStages) & 1u)) break;
-        tc::mma_commit(drain);
+    } else if (t == kWorkers + 32) {
+        // ---- products, in the order of the copies. The descriptors differ from stage to
+        // stage and part to part by constants only.
+        const uint32_t idesc = tc::idesc_bf16(128, RT);
+        const uint64_t am = tc::smem_desc(tc::smem_u32(smem_tcs), 128, kK * 16),
+                       bm = tc::smem_desc(tc::smem_u32(smem_tcs) + kChunkA, 128, kK * 16),
+                       ac = tc::smem_desc(tc::smem_u32(smem_tcs), 128, kKc * 16),
+                       bc = tc::smem_desc(tc::smem_u32(smem_tcs) + kChunkA, 128, kKc * 16);
+        const uint32_t ap = (uint32_t)h2 * kKc * 2u / 16u;  // between the parts of a coupling chunk
+        const uint32_t step = pl.stage / 16u;
+        int s = 0;
+        uint32_t par = 0;
+        bool ok = true;
+        auto begin = [&]() {  // the stage's chunks of both operands are there
+            ok = wait_flag(&full_b[s], par) && tc::mbar_wait(&full_a[s], par);
+            tc::tc_fence_after();
+            return ok;
+        };
+        auto end = [&]() {
+            tc::mma_commit(&empty[s]);
+            if (++s == kStages) {
+                s = 0;
+                par ^= 1u;
+            }
+        };
+        auto main_chunks = [&](int chunks) {
+            for (int i = 0; i < chunks && begin(); ++i) {
+                const uint64_t a0 = am + (uint64_t)(s * step), b0 = bm + (uint64_t)(s * step);
+#pragma unroll
+                for (int j = 0; j < kK / 16; ++j) {
+                    const uint64_t ah = a0 + 16u * j, al = ah + kChunkA / 32u, bh = b0 + 16u * j, bl = bh + RT * kK / 8u;
+                    tc::mma_bf16(tmem, ah, bh, idesc, (j > 0 || i > 0) ? 1u : 0u);
+                    tc::mma_bf16(tmem, ah, bl, idesc, 1u);
+                    tc::mma_bf16(tmem, al, bh, idesc, 1u);
+                }
+                end();
+            }
+        };
+        // (rows from N/2 up read what follows in the stage; their accumulator lanes are ignored)
+        auto coupling_chunks = [&](uint32_t acc) {
+            for (int i = 0; i < nc && begin(); ++i) {
+                const uint64_t a0 = ac + (uint64_t)(s * step), a1 = a0 + ap, a2 = a1 + ap;
+                const uint64_t b0 = bc + (uint64_t)(s * step), b1 = b0 + RT * kKc / 8u, b2 = b1 + RT * kKc / 8u;
+                tc::mma_bf16(acc, a0, b0, idesc, i > 0 ? 1u : 0u);
+                tc::mma_bf16(acc, a0, b1, idesc, 1u);
+                tc::mma_bf16(acc, a1, b0, idesc, 1u);
+                tc::mma_bf16(acc, a0, b2, idesc, 1u);
+                tc::mma_bf16(acc, a2, b0, idesc, 1u);
+                tc::mma_bf16(acc, a1, b1, idesc, 1u);
+                end();
+            }
+        };
+        for (uint32_t j = 0; ok; ++j) {
+            if (!(ok = wait_flag(&unit_bar[j % kUnitRing], (j / kUnitRing) & 1u))) break;
+            const Unit u = ring[j % kUnitRing];
+            if (u.id < 0) break;
+            // after a unit's first and second group of chunks the workers read its accumulators
+            if (!u.bwd) {
+                main_chunks(n_main(u));
+                tc::mma_commit(seg_bar);
+            }
+            if (u.bwd || push_right(u)) coupling_chunks(tmem + RT);
+            if (u.bwd ? u.right >= 0 : push_left(u)) coupling_chunks(tmem + 2u * RT);
+            if (u.bwd || push_right(u) || push_left(u)) tc::mma_commit(seg_bar);
+            if (u.bwd) {
+                main_chunks(n_main(u));
+                tc::mma_commit(seg_bar);
+            }
+        }
+        if (!ok) fail();
+        tc::mma_commit(drain);  // every product has been done before the CTA ends (bounded)
         (void)tc::mbar_wait(drain, 0);
     } else if (t < kWorkers) {
         // ---- workers
@@ -461,7 +466,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
             tc::tc_fence_after();
         };
         for (uint32_t j = 0;; ++j) {
-            // (the driver takes units as it copies: it is at most a few chunks ahead, never far behind)
+            // (units are taken as their chunks are copied: a few chunks ahead of the products)
             ok = wait_bar(&unit_bar[j % kUnitRing], (j / kUnitRing) & 1u);
             if (worker_any(!ok)) break;
             const Unit u = ring[j % kUnitRing];

@@ -9,16 +9,18 @@
 // (M = 128 rows, N = RT, accumulated in FP32 in tensor memory):
 //   forward  Y_i = A_i^{-1} r_i, rows of the slice; the slice holding R+ (L-) then forms
 //            B_right Y_i[R+] (C_left Y_i[L-]) and subtracts it from the neighbour's r
-//   backward u_i = Y_i - A_i^{-1}[:, N/2 : 3N/2] g_i, rows of the slice,
-//            g_i = [B_i u_left[R+] ; C_i u_right[L-]]
-// (the reduction of k_bcr_solve_flow). Precision: the factors and the vectors they
-// multiply in split BF16 with three products, as the contractions,
+//   backward u_i = Y_i - P_i [u_left[R+] ; u_right[L-]], rows of the slice,
+//            P_i = [A_i^{-1}[:, L+] B_i , A_i^{-1}[:, R-] C_i]
+// (the reduction of k_bcr_solve_flow, with the couplings multiplied into the backward
+// operator once per factorization: a backward unit is then one product instead of two
+// dependent ones of which every slice repeated the first). Precision: the factors and the
+// vectors they multiply in split BF16 with three products, as the contractions,
 //   A x ~= A_hi x_hi + A_hi x_lo + A_lo x_hi;
 // the couplings in three BF16 parts with six products (all pairs of weight 2^-16 and
 // more), which keeps FP32's 24 bits. Both are stored a second time for this solve,
 // already split and in the K-major core-matrix layout, one bulk copy (the TMA engine) per
-// chunk: A^{-1} by (slice, 32 columns), 16 KB (k_bcr_factor_split), a coupling block by 16
-// columns (k_bcr_coupling_split).
+// chunk: A^{-1} and P by (slice, 32 columns), 16 KB (k_bcr_factor_split,
+// k_bcr_backward_split), a coupling block by 16 columns (k_bcr_coupling_split).
 //
 // A CTA is four worker warps, a copying and an issuing thread that share a ring of kStages
 // stages, a chunk of the operand A and one of the operand B each. The copying thread takes
@@ -33,7 +35,8 @@
 // for all rows, 16-column chunks with a barrier, a wait for the products and a copy issued
 // only then, and the couplings on the FP32 cores took 3.43 ms at 2N = 512, 1250 cells and
 // 64 right-hand sides, 1.72 ms with 16; with one thread for copies and products 1.68 and
-// 1.25 ms, now 1.20 and 0.70 ms.
+// 1.25 ms, with the couplings multiplied in every backward unit 1.20 and 0.70 ms, now 0.89
+// and 0.53 ms.
 //
 // Units are taken from a work queue in phase order (forward levels, roots, backward
 // levels), within a phase the slices others wait for first: a unit depends only on units
@@ -65,6 +68,7 @@ constexpr uint32_t kChunkA = 128u * kK * 4u;  // hi and lo, 128 x 32 BF16 each
 __host__ __device__ constexpr int rhs_tile(int R) { return R >= kMaxRT ? kMaxRT : (R + 15) / 16 * 16; }
 __host__ __device__ constexpr bool applies(int n2, int R) { return n2 % 128 == 0 && n2 <= kMaxN2 && R >= 16; }
 __host__ __device__ constexpr size_t cell_bytes(int n2) { return (size_t)n2 * n2 * 4u; }
+__host__ __device__ constexpr size_t backward_bytes(int n2) { return cell_bytes(n2) / 2; }
 // one coupling block: N/2 x N/2 in three BF16 parts; a chunk of its columns
 __host__ __device__ constexpr size_t coupling_bytes(int n2) { return (size_t)(n2 / 4) * (n2 / 4) * 6u; }
 __host__ __device__ constexpr uint32_t coupling_chunk(int n2) { return (uint32_t)(n2 / 4) * kKc * 6u; }
@@ -110,6 +114,71 @@ __global__ void __launch_bounds__(256) k_bcr_factor_split(const float *__restric
         unsigned char *c = o + ((size_t)(row / 128) * nkc + kc) * kChunkA + tc::kmajor_offset(row % 128, 8 * g, kK);
         *reinterpret_cast<uint4 *>(c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
         *reinterpret_cast<uint4 *>(c + kChunkA / 2) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
+}
+
+// The backward operators P_i (2N x N, FP32 sums, split as the inverses): block (item, side,
+// slice m) forms A_i^{-1}[128 m .., L+] B_i (side 0) or A_i^{-1}[128 m .., R-] C_i, 2 h2
+// threads with 8 x 8 outputs each, both operands through shared memory in k-chunks of 16
+// (contiguous in memory along their other index). Bounded by FP32 arithmetic: 2 N^3 / 2
+// FMAs a cell, 1.41 ms for 1250 cells at 2N = 512, once per factorization.
+__global__ void __launch_bounds__(256) k_bcr_backward_split(const float *__restrict__ A, const float *__restrict__ Bc,
+                                                            const float *__restrict__ Cc,
+                                                            const BcrItem *__restrict__ items,
+                                                            unsigned char *__restrict__ out, int n2) {
+    constexpr int KC = 16;
+    const BcrItem it = items[blockIdx.x];
+    const int side = blockIdx.y, m = blockIdx.z, N = n2 / 2, h2 = n2 / 4;
+    if ((side ? it.right : it.left) < 0) return;  // (a root has neither)
+    __shared__ __align__(16) float Ls[KC][128], Rs[KC][kMaxN2 / 4];
+    const float *L = A + (size_t)it.cell * n2 * n2 + (size_t)(side ? N : h2) * n2 + 128 * m;
+    const float *W = (side ? Cc : Bc) + (size_t)it.s_cell * h2 * h2;
+    const int t = threadIdx.x, rg = t & 15, cg = t >> 4;  // rows 4 rg .. + 3 and 64 more, columns 8 cg .. + 7
+    float acc[8][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    for (int k0 = 0; k0 < h2; k0 += KC) {
+        for (int i = t; i < KC * 32; i += blockDim.x)
+            *reinterpret_cast<float4 *>(&Ls[i >> 5][4 * (i & 31)]) =
+                __ldg(reinterpret_cast<const float4 *>(L + (size_t)(k0 + (i >> 5)) * n2) + (i & 31));
+        for (int i = t; i < KC * (h2 / 4); i += blockDim.x) {
+            const int k = i / (h2 / 4), c = i - k * (h2 / 4);
+            *reinterpret_cast<float4 *>(&Rs[k][4 * c]) =
+                __ldg(reinterpret_cast<const float4 *>(W + (size_t)(k0 + k) * h2) + c);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < KC; ++k) {
+            float l[8], r[8];
+            *reinterpret_cast<float4 *>(l) = *reinterpret_cast<const float4 *>(&Ls[k][4 * rg]);
+            *reinterpret_cast<float4 *>(l + 4) = *reinterpret_cast<const float4 *>(&Ls[k][64 + 4 * rg]);
+            *reinterpret_cast<float4 *>(r) = *reinterpret_cast<const float4 *>(&Rs[k][8 * cg]);
+            *reinterpret_cast<float4 *>(r + 4) = *reinterpret_cast<const float4 *>(&Rs[k][8 * cg + 4]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(l[i], r[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+    const int col = side * h2 + 8 * cg;
+    unsigned char *c = out + (size_t)it.cell * backward_bytes(n2) + ((size_t)m * (N / kK) + col / kK) * kChunkA;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            __nv_bfloat16 h0, l0, h1, l1;
+            tc::split_bf16(acc[i][2 * j], h0, l0);
+            tc::split_bf16(acc[i][2 * j + 1], h1, l1);
+            hi[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+            lo[j] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+        }
+        unsigned char *o = c + tc::kmajor_offset(4 * rg + (i & 3) + 64 * (i >> 2), col % kK, kK);
+        *reinterpret_cast<uint4 *>(o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4 *>(o + kChunkA / 2) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
 }
 
@@ -191,12 +260,11 @@ __device__ __forceinline__ void poll(const int *c, int want, int *err, unsigned 
 // RT right-hand sides, cell), n of each, zero at launch: flow[0 .. n) pushes landed in r,
 // [n .. 2n) forward slices written (for the cell's own backward slices), then two per cell,
 // the L- and the R+ rows of u final. queue: this launch's unit counter (zero at launch).
-// zero_next / queue_next: the other parity's counters, zeroed for the following solve. gs:
-// per-CTA scratch of the backward coupling vectors g (gridDim.x x RT x N floats).
+// zero_next / queue_next: the other parity's counters, zeroed for the following solve.
 template <int RT>
 __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
-    const unsigned char *__restrict__ Atc, const unsigned char *__restrict__ Btc, const unsigned char *__restrict__ Ctc,
-    const BcrItem *__restrict__ items, LevelTable lv, float *rhs, float *Y, float *gs, int N, int sumK, int R,
+    const unsigned char *__restrict__ Atc, const unsigned char *__restrict__ Ptc, const unsigned char *__restrict__ Btc, const unsigned char *__restrict__ Ctc,
+    const BcrItem *__restrict__ items, LevelTable lv, float *rhs, float *Y, int N, int sumK, int R,
     int *flow, int *queue, int *err, int *zero_next, long long nzero, int *queue_next, const int *stop) {
     using namespace tcs;
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < nzero; i += (long long)gridDim.x * kThreads)
@@ -243,8 +311,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
         atomicExch(err, 1);
     };
     // A unit's chunks, in order: forward, n2 / 32 of A^{-1}, then the couplings of its pushes;
-    // backward, the couplings (left, then right if there is one), then A^{-1} (only the left
-    // half of its columns without a right neighbour).
+    // backward, those of P (only its left half without a right neighbour).
     auto push_right = [&](const Unit &u) { return !u.bwd && u.right >= 0 && u.m == MT - 1; };
     auto push_left = [&](const Unit &u) { return !u.bwd && u.left >= 0 && u.m == 0; };
     auto n_main = [&](const Unit &u) { return (u.bwd ? (u.right >= 0 ? N : h2) : n2) / kK; };
@@ -305,14 +372,12 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                     tc::bulk_copy_g2s(smem_tcs + s * pl.stage, src, bytes, &full_a[s]);
                 }
             };
-            const unsigned char *main = Atc + (size_t)u.cell * cell_bytes(n2) +
-                                        ((size_t)u.m * (n2 / kK) + (u.bwd ? h2 / kK : 0)) * kChunkA;
+            const size_t slice = (size_t)u.m * ((u.bwd ? N : n2) / kK) * kChunkA;
+            copy((u.bwd ? Ptc + (size_t)u.cell * backward_bytes(n2) : Atc + (size_t)u.cell * cell_bytes(n2)) + slice,
+                 n_main(u), kChunkA);
             const size_t cbytes = coupling_bytes(n2);
-            if (!u.bwd) copy(main, n_main(u), kChunkA);
-            if (u.bwd || push_right(u)) copy(Btc + (size_t)(u.bwd ? u.s_cell : u.s_right) * cbytes, nc, coupling_chunk(n2));
-            if (u.bwd ? u.right >= 0 : push_left(u))
-                copy(Ctc + (size_t)(u.bwd ? u.s_cell : u.s_left) * cbytes, nc, coupling_chunk(n2));
-            if (u.bwd) copy(main, n_main(u), kChunkA);
+            if (push_right(u)) copy(Btc + (size_t)u.s_right * cbytes, nc, coupling_chunk(n2));
+            if (push_left(u)) copy(Ctc + (size_t)u.s_left * cbytes, nc, coupling_chunk(n2));
         }
         if (!ok) fail();
         // every copy has landed before the CTA ends (bounded)
@@ -374,18 +439,13 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
             if (!(ok = wait_flag(&unit_bar[j % kUnitRing], (j / kUnitRing) & 1u))) break;
             const Unit u = ring[j % kUnitRing];
             if (u.id < 0) break;
-            // after a unit's first and second group of chunks the workers read its accumulators
-            if (!u.bwd) {
-                main_chunks(n_main(u));
-                tc::mma_commit(seg_bar);
-            }
-            if (u.bwd || push_right(u)) coupling_chunks(tmem + RT);
-            if (u.bwd ? u.right >= 0 : push_left(u)) coupling_chunks(tmem + 2u * RT);
-            if (u.bwd || push_right(u) || push_left(u)) tc::mma_commit(seg_bar);
-            if (u.bwd) {
-                main_chunks(n_main(u));
-                tc::mma_commit(seg_bar);
-            }
+            // after each group of chunks the workers read its accumulators
+            main_chunks(n_main(u));
+            tc::mma_commit(seg_bar);
+            const bool pr = push_right(u), plf = push_left(u);
+            if (pr) coupling_chunks(tmem + RT);
+            if (plf) coupling_chunks(tmem + 2u * RT);
+            if (pr || plf) tc::mma_commit(seg_bar);
         }
         if (!ok) fail();
         tc::mma_commit(drain);  // every product has been done before the CTA ends (bounded)
@@ -402,8 +462,9 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
             return !failed();
         };
         // The unit's next `chunks` chunks of KC columns of the vectors v_r[k] = src[r stride + k]
-        // (r < nrc, else 0) in P parts, kAhead of them in flight.
-        auto feed = [&](auto KCt, auto Pt, const float *src, size_t stride, int chunks, int nrc) {
+        // (r < nrc, else 0; from chunk `first` on of src2) in P parts, kAhead of them in flight.
+        auto feed = [&](auto KCt, auto Pt, const float *src, size_t stride, int chunks, int nrc, int first,
+                        const float *src2) {
             constexpr int KC = decltype(KCt)::value, PARTS = decltype(Pt)::value, GR = KC / 8;
             constexpr int NG = (RT * GR + kWorkers - 1) / kWorkers;  // groups of 8 values per worker and chunk
             float4 v[kAhead][NG][2];
@@ -413,7 +474,8 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                     const int id = t + g * kWorkers, r = id / GR, k = 8 * (id % GR);
                     x[g][0] = x[g][1] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (r < nrc && c < chunks) {
-                        const float4 *p = reinterpret_cast<const float4 *>(src + (size_t)r * stride + c * KC + k);
+                        const float4 *p = reinterpret_cast<const float4 *>(
+                            (c < first ? src + c * KC : src2 + (c - first) * KC) + (size_t)r * stride + k);
                         x[g][0] = __ldcg(p);
                         x[g][1] = __ldcg(p + 1);
                     }
@@ -486,7 +548,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
             }
             worker_sync();
             if (!u.bwd) {
-                feed(Const<kK>{}, Const<2>{}, rhs + (size_t)r0 * rstride + (size_t)u.cell * n2, rstride, n2 / kK, nrc);
+                feed(Const<kK>{}, Const<2>{}, rhs + (size_t)r0 * rstride + (size_t)u.cell * n2, rstride, n2 / kK, nrc, n2 / kK, nullptr);
                 wait_seg();
                 if (worker_any(!ok)) break;
 #pragma unroll
@@ -500,8 +562,8 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                 const bool pr = push_right(u), plf = push_left(u);
                 if (pr || plf) {
                     worker_sync();  // the rows this CTA just wrote are read back below
-                    if (pr) feed(Const<kKc>{}, Const<3>{}, Yc + N + h2, rstride, nc, nrc);
-                    if (plf) feed(Const<kKc>{}, Const<3>{}, Yc, rstride, nc, nrc);
+                    // y[R+], then y[L-]
+                    feed(Const<kKc>{}, Const<3>{}, pr ? Yc + N + h2 : Yc, rstride, pr && plf ? 2 * nc : nc, nrc, nc, Yc);
                     wait_seg();
                     if (worker_any(!ok)) break;
 #pragma unroll
@@ -531,26 +593,8 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                     }
                 }
             } else {
-                float *g = gs + (size_t)blockIdx.x * RT * N;
-                feed(Const<kKc>{}, Const<3>{}, Y + (size_t)r0 * rstride + (size_t)u.left * n2 + N + h2, rstride, nc, nrc);
-                if (u.right >= 0)
-                    feed(Const<kKc>{}, Const<3>{}, Y + (size_t)r0 * rstride + (size_t)u.right * n2, rstride, nc, nrc);
-                wait_seg();
-                if (worker_any(!ok)) break;
-#pragma unroll
-                for (int side = 0; side < 2; ++side) {
-                    if (side && u.right < 0) continue;
-#pragma unroll
-                    for (int c = 0; c < RT; c += 16) {
-                        float v[16];
-                        tc::tmem_ld16(tmem + lane_base + (uint32_t)((1 + side) * RT + c), v);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            if (t < h2) g[(size_t)(c + i) * N + side * h2 + t] = v[i];
-                    }
-                }
-                worker_sync();
-                feed(Const<kK>{}, Const<2>{}, g, N, n_main(u), RT);
+                feed(Const<kK>{}, Const<2>{}, Y + (size_t)r0 * rstride + (size_t)u.left * n2 + N + h2, rstride, n_main(u), nrc,
+                     h2 / kK, u.right >= 0 ? Y + (size_t)r0 * rstride + (size_t)u.right * n2 : nullptr);
                 float y[RT];
 #pragma unroll
                 for (int c = 0; c < RT; ++c) y[c] = c < nrc ? __ldcg(Yc + (size_t)c * rstride + row) : 0.f;

@@ -120,7 +120,7 @@ struct fpsa_ctx {
     int tcs_grid = 0;                // two CTAs per SM
     unsigned char *d_tcs_A = nullptr;  // the factors split to BF16 hi / lo in the core-matrix layout
     unsigned char *d_tcs_B = nullptr, *d_tcs_C = nullptr;  // the couplings in three BF16 parts
-    float *d_tcs_g = nullptr;        // per-CTA backward coupling vectors
+    unsigned char *d_tcs_P = nullptr;  // the backward operators, split likewise
     int *d_tcs_queue = nullptr;      // unit counters, one per parity of d_flow
     unsigned long long *d_conv = nullptr, *d_growth = nullptr;
     int *d_status = nullptr;
@@ -750,6 +750,10 @@ int setup_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
         Launch L_(ctx, FPSA_PHASE_BCR_INVERT);
         tcs::k_bcr_factor_split<<<(unsigned)((size_t)g.sumK * (2 * N / tcs::kK)), 256, 0, st>>>(
             reinterpret_cast<const float *>(p.A), ctx->d_tcs_A, 2 * N);
+        if (g.n_levels)
+            tcs::k_bcr_backward_split<<<dim3(ctx->lvt[0].off[g.n_levels], 2, 2 * N / 128), 2 * h2, 0, st>>>(
+                reinterpret_cast<const float *>(p.A), reinterpret_cast<const float *>(p.Bc),
+                reinterpret_cast<const float *>(p.Cc), ctx->d_items_all, ctx->d_tcs_P, 2 * N);
         const unsigned cgrid = (unsigned)((size_t)g.n_slots * (h2 / tcs::kKc));
         tcs::k_bcr_coupling_split<<<cgrid, 256, 0, st>>>(reinterpret_cast<const float *>(p.Bc), ctx->d_tcs_B, 2 * N);
         tcs::k_bcr_coupling_split<<<cgrid, 256, 0, st>>>(reinterpret_cast<const float *>(p.Cc), ctx->d_tcs_C, 2 * N);
@@ -881,9 +885,9 @@ int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *st
     Launch L_(ctx, FPSA_PHASE_BCR_SOLVE);
     auto go = [&](auto kern) {
         return launch_pdl(kern, dim3(ctx->tcs_grid), dim3(tcs::kThreads), smem, ctx->stream,
-                          (const unsigned char *)ctx->d_tcs_A, (const unsigned char *)ctx->d_tcs_B,
-                          (const unsigned char *)ctx->d_tcs_C, (const BcrItem *)ctx->d_items_all, ctx->lvt[0], rhs,
-                          p.ybuf, ctx->d_tcs_g, g.N, g.sumK, g.R, flow, queue, ctx->d_dev_err, zero_next,
+                          (const unsigned char *)ctx->d_tcs_A, (const unsigned char *)ctx->d_tcs_P,
+                          (const unsigned char *)ctx->d_tcs_B, (const unsigned char *)ctx->d_tcs_C, (const BcrItem *)ctx->d_items_all, ctx->lvt[0], rhs,
+                          p.ybuf, g.N, g.sumK, g.R, flow, queue, ctx->d_dev_err, zero_next,
                           (long long)(4 * n), queue_next, stop);
     };
     switch (RT) {
@@ -2131,8 +2135,15 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                 CK(raise_smem_limit((const void *)k_bgemm_tc<128>, (int)bgt::smem_bytes(128)));
                 ctx->bgemm_tc_able = true;
             }
-            if (ctx->precision == FPSA_PRECISION_MIXED && tcs::applies(2 * g.N, g.R)) {
-                // the tensor-core BCR solve: a split copy of the factors, two CTAs per SM
+            // The tensor-core BCR solve keeps split copies of the factors and the backward
+            // operators beside the factors; a problem for which the device has no room for them
+            // (with 64 bytes per angular unknown for the vectors) takes the dataflow solve.
+            size_t mem_free = 0, mem_total = 0;
+            CK(cudaMemGetInfo(&mem_free, &mem_total));
+            const size_t tcs_need = (size_t)g.sumK * (2 * tcs::cell_bytes(2 * g.N) + tcs::backward_bytes(2 * g.N) +
+                                                      (size_t)g.R * 2 * g.N * 64);
+            if (ctx->precision == FPSA_PRECISION_MIXED && tcs::applies(2 * g.N, g.R) && tcs_need < mem_free) {
+                // two CTAs per SM
                 ctx->tcs_rt = tcs::rhs_tile(g.R);
                 ctx->tcs_grid = 2 * nsm;
                 ctx->flow_n = (size_t)((g.R + ctx->tcs_rt - 1) / ctx->tcs_rt) * g.sumK;
@@ -2141,7 +2152,7 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                 CK(dalloc(ctx, &ctx->d_tcs_B, (size_t)g.n_slots * tcs::coupling_bytes(2 * g.N)));
                 CK(dalloc(ctx, &ctx->d_tcs_C, (size_t)g.n_slots * tcs::coupling_bytes(2 * g.N)));
                 CK(dalloc(ctx, &ctx->d_tcs_A, (size_t)g.sumK * tcs::cell_bytes(2 * g.N)));
-                CK(dalloc(ctx, &ctx->d_tcs_g, (size_t)ctx->tcs_grid * ctx->tcs_rt * g.N));
+                CK(dalloc(ctx, &ctx->d_tcs_P, (size_t)g.sumK * tcs::backward_bytes(2 * g.N)));
                 CK(dalloc(ctx, &ctx->d_tcs_queue, 2));
                 CK(cudaMemset(ctx->d_tcs_queue, 0, 2 * sizeof(int)));
                 const void *k = tcs_kernel(ctx->tcs_rt);

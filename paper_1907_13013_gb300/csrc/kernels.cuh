@@ -1604,10 +1604,13 @@ struct VecOf<double> {
 
 // Coupling blocks of one unit (the two N/2 x N/2 blocks it multiplies) are staged
 // in shared memory by asynchronous copies issued when the unit starts, when both
-// fit in 16 KB and a block is a whole number of 16-byte chunks.
+// fit in 32 KB (two blocks of eight right-hand sides then still share an SM) and a block
+// is a whole number of 16-byte chunks. Read from global memory after the unit's wait
+// instead, one value per lane from rows of 256 bytes, the couplings at N = 128 in FP32
+// were most of a hop: 1000 cells, one right-hand side, 157 us a solve, now 128.
 __host__ __device__ constexpr int bcr_coupling_values(int N) { return 2 * (N / 2) * (N / 2); }
 __host__ __device__ constexpr bool bcr_couplings_staged(int N, int esize) {
-    return bcr_coupling_values(N) * esize <= 16384 && ((N / 2) * (N / 2) * esize) % 16 == 0;
+    return bcr_coupling_values(N) * esize <= 32768 && ((N / 2) * (N / 2) * esize) % 16 == 0;
 }
 
 // shared scratch (values of T) of one solve block handling RC right-hand sides:

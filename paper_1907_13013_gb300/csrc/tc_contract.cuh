@@ -867,7 +867,7 @@ __global__ void __launch_bounds__(128) k_tc_update_scatter_cols(const float *v_i
 // operator is the A operand (rows = outputs, two M = 128 tiles) and a tile of CT = 64
 // columns the B operand, so that a warp's global accesses are 128 contiguous bytes of a
 // column and both nodes of a cell meet in one thread. A CTA is eight worker warps (thread t
-// owns output t of every column) and a driver thread that streams the operators through
+// owns output t of every column), an issuing thread and one that streams the operators through
 // kStages stages, 16 columns of hi and lo each (stored chunk-major in global memory, [N / 16
 // chunks][N rows][16] in the K-major core-matrix layout; shared by every tile, so they stay
 // in L2), across GEMMs and tiles: what it copies next never depends on the data. Two CTAs
@@ -875,7 +875,8 @@ __global__ void __launch_bounds__(128) k_tc_update_scatter_cols(const float *v_i
 // What bounds it: the operators' stream from L2 (0.5 MB a tile of 64 columns) and the
 // tile's own 0.26 MB of global traffic. A tile of 128 columns whose thread t owned COLUMN t
 // (rows of 1 KB read 16 bytes per lane and instruction, one CTA per SM) took 0.62 and 0.71
-// ms for 160000 columns at N = 256, now 0.44 and 0.50.
+// ms for 160000 columns at N = 256, with one thread for copies and products 0.44
+// and 0.50, now 0.26 and 0.29.
 //   k_tc_wide<FpRhs>         phi_half = D psi;  rhs = m (x) M Sigma (phi_half - phi)
 //   k_tc_wide<UpdateScatter> phi = phi_base + D v;  q = M (Sigma phi) + q_ang
 //   k_tc_wide<RhsMoments>    rhs = m (x) M Sigma v                 (GMRES; v: moments)
@@ -891,7 +892,8 @@ __host__ __device__ __forceinline__ uint32_t chunk_offset(int row, int k, int N)
 }  // namespace tc
 
 namespace tcw {
-constexpr int kWorkers = 256, kThreads = kWorkers + 32, kCT = 64, kStages = 3;
+constexpr int kWorkers = 256, kThreads = kWorkers + 64, kCT = 64, kStages = 3;
+constexpr unsigned kFlagTries = 1u << 28;  // of a wait that ends with the workers' bounded ones
 constexpr uint32_t kPart = 256u * tc::kChunkK * 2u, kStage = 2 * kPart;  // hi and lo of a chunk, 256 rows of room
 constexpr uint32_t kTmem = 256;                                          // two GEMMs x two row tiles x kCT
 struct Plan {
@@ -949,62 +951,72 @@ __global__ void __launch_bounds__(tcw::kThreads, 2) k_tc_wide(tcw::Args g, TcOps
         *(volatile int *)&s_fail = 1;
         atomicExch(err, 1);
     };
+    const int nch = N / tc::kChunkK, mine = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    auto wait_flag = [&](uint64_t *bar, uint32_t par) {
+        for (unsigned i = 0; !tc::mbar_test(bar, par); ++i)
+            if (failed() || i > kFlagTries) return false;
+        return true;
+    };
     if (t == kWorkers) {
-        // ---- driver: this CTA's tiles x GEMMs x chunks, in order
-        const int nch = N / tc::kChunkK, per_tile = kGemms * nch;
+        // ---- copies: this CTA's tiles x GEMMs x chunks, in order, as stages become free
         const uint32_t part = (uint32_t)N * tc::kChunkK * 2;  // bytes of hi (or lo) of a chunk
-        const int mine = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-        const uint32_t total = (uint32_t)mine * per_tile;
-        uint32_t issued = 0, q = 0;
+        const size_t lo = (size_t)N * N * 2;
+        uint32_t issued = 0, par = 1;
+        int s = 0;
         bool ok = true;
-        auto copy_next = [&]() {
-            const int c = (int)(issued % per_tile), gm = c / nch, kc = c % nch, s = issued % kStages;
-            const unsigned char *op = (KIND == RhsMoments || gm == 1) ? ops.M : ops.D;
-            const unsigned char *src = op + (size_t)kc * part;
-            tc::mbar_arrive_expect_tx(&full[s], 2 * part);
-            tc::bulk_copy_g2s(stg + s * kStage, src, part, &full[s]);
-            tc::bulk_copy_g2s(stg + s * kStage + kPart, src + (size_t)N * N * 2, part, &full[s]);
-            ++issued;
-        };
+        for (int i = 0; i < mine && ok; ++i)
+            for (int gm = 0; gm < kGemms && ok; ++gm) {
+                const unsigned char *src = (KIND == RhsMoments || gm == 1) ? ops.M : ops.D;
+                for (int kc = 0; kc < nch; ++kc, src += part) {
+                    if (issued >= (uint32_t)kStages && !(ok = wait_flag(&empty[s], par))) break;
+                    tc::mbar_arrive_expect_tx(&full[s], 2 * part);
+                    tc::bulk_copy_g2s(stg + s * kStage, src, part, &full[s]);
+                    tc::bulk_copy_g2s(stg + s * kStage + kPart, src + lo, part, &full[s]);
+                    ++issued;
+                    if (++s == kStages) {
+                        s = 0;
+                        par ^= 1u;
+                    }
+                }
+            }
+        if (!ok) fail();
+        // nothing may land after the CTA has gone (bounded)
+        for (uint32_t j = issued > (uint32_t)kStages ? issued - kStages : 0; j < issued; ++j)
+            if (!tc::mbar_wait(&full[j % kStages], (j / kStages) & 1u)) break;
+    } else if (t == kWorkers + 32) {
+        // ---- products, in the order of the copies; descriptors that differ by constants
         const uint32_t idesc = tc::idesc_bf16(128, kCT), sbo_x = (uint32_t)N * 16;
         const uint64_t bh0 = tc::smem_desc(tc::smem_u32(x_hi), 128, sbo_x), bl0 = tc::smem_desc(tc::smem_u32(x_lo), 128, sbo_x);
-        uint32_t xs = 0;  // tiles of x multiplied so far
-        for (; ok && q < total; ++q) {
-            while (issued < total && issued < q + kStages - 1) {  // (the products of chunk q - 2 free its stage)
-                if (issued >= (uint32_t)kStages &&
-                    !(ok = tc::mbar_wait(&empty[issued % kStages], (issued / kStages - 1u) & 1u)))
-                    break;
-                copy_next();
-            }
-            const int s = q % kStages, c = (int)(q % per_tile), gm = c / nch, kc = c % nch;
-            ok = ok && !failed() && tc::mbar_wait(&full[s], (q / kStages) & 1u);
-            if (ok && kc == 0) {  // the workers' tile (no time limit but the flag: they wait for memory)
-                while (!tc::mbar_test(full_x, xs & 1u))
-                    if (failed()) {
-                        ok = false;
-                        break;
-                    }
+        const uint64_t a0 = tc::smem_desc(tc::smem_u32(stg), 128, tc::kChunkK * 16);
+        uint32_t xs = 0, par = 0;
+        int s = 0;
+        bool ok = true;
+        for (int i = 0; i < mine && ok; ++i)
+            for (int gm = 0; gm < kGemms && ok; ++gm) {
+                if (!(ok = wait_flag(full_x, xs & 1u))) break;  // the workers' tile
                 ++xs;
-            }
-            if (!ok) break;
-            tc::tc_fence_after();
-            const uint64_t ah = tc::smem_desc(tc::smem_u32(stg + s * kStage), 128, tc::kChunkK * 16);
-            const uint64_t bh = bh0 + (uint64_t)(16 * kc), bl = bl0 + (uint64_t)(16 * kc);
-            const uint32_t more = kc > 0 ? 1u : 0u;
+                const uint32_t acc = tmem + (uint32_t)(2 * gm * kCT);
+                for (int kc = 0; kc < nch; ++kc) {
+                    if (!(ok = tc::mbar_wait(&full[s], par))) break;
+                    tc::tc_fence_after();
+                    const uint64_t ah = a0 + (uint64_t)(s * (kStage / 16)), al = ah + (uint64_t)(kPart / 16);
+                    const uint64_t bh = bh0 + (uint64_t)(16 * kc), bl = bl0 + (uint64_t)(16 * kc);
+                    const uint32_t more = kc > 0 ? 1u : 0u;
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                const uint32_t acc = tmem + (uint32_t)((2 * gm + m) * kCT);
-                const uint64_t a_hi = ah + (uint64_t)(m * 4096 / 16), a_lo = a_hi + (uint64_t)(kPart / 16);
-                tc::mma_bf16(acc, a_hi, bh, idesc, more);
-                tc::mma_bf16(acc, a_hi, bl, idesc, 1u);
-                tc::mma_bf16(acc, a_lo, bh, idesc, 1u);
+                    for (int m = 0; m < 2; ++m) {
+                        tc::mma_bf16(acc + m * kCT, ah + m * 256u, bh, idesc, more);
+                        tc::mma_bf16(acc + m * kCT, ah + m * 256u, bl, idesc, 1u);
+                        tc::mma_bf16(acc + m * kCT, al + m * 256u, bh, idesc, 1u);
+                    }
+                    tc::mma_commit(&empty[s]);
+                    if (++s == kStages) {
+                        s = 0;
+                        par ^= 1u;
+                    }
+                }
+                if (ok) tc::mma_commit(acc_bar);
             }
-            tc::mma_commit(&empty[s]);
-            if (kc == nch - 1) tc::mma_commit(acc_bar);
-        }
         if (!ok) fail();
-        for (uint32_t j = q; j < issued; ++j)  // nothing may land after the CTA has gone (bounded)
-            if (!tc::mbar_wait(&full[j % kStages], (j / kStages) & 1u)) break;
         tc::mma_commit(drain);
         (void)tc::mbar_wait(drain, 0);
     } else if (t < kWorkers) {

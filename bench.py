@@ -326,7 +326,7 @@ def scale_secondary(binding, inputs, dev, stream, hbm, bf16, precisions, K=20000
                 # such GEMMs per contraction launch, a GMRES operator four in three launches
                 gemms = 2.0 if meth == "fpsa" else 4.0 / 3.0
                 fl = gemms * 3 * 2.0 * N * N * 2 * K * R
-                roof = {"kernel": "k_tc_*_big (tensor-core contractions)", "bound": "tensor",
+                roof = {"kernel": "k_tc_wide (tensor-core contractions)", "bound": "tensor",
                         "achieved": fl / (per * 1e-3) / 1e12, "peak": bf16, "unit": "TFLOP/s",
                         "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (cuBLAS bf16, seconds-long loop)"}
             elif dom == "contract":

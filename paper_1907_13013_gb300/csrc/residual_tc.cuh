@@ -36,7 +36,9 @@
 // What bounds it: the workers' arithmetic, of which FP64 (two FMAs a clock and SM) is the
 // largest part, so the recombination takes 4 FP64 operations an output, the LD stencil 6;
 // with 6 and 11, and a worker thread that built each MMA's descriptors as it issued them,
-// a residual at N = 256, 1250 cells and 64 right-hand sides took 6.87 ms, now 5.46 ms.
+// a residual at N = 256, 1250 cells and 64 right-hand sides took 6.87 ms; 5.46 ms then, and 5.29 ms
+// with the scaling by powers of two done in the exponent bits and the second contraction's row
+// maxima taken where its inputs are first at hand.
 // Waits are bounded; on a timeout the CTA records the error, waits (bounded) for its
 // copies and products, frees its tensor memory and stops.
 #pragma once
@@ -125,6 +127,16 @@ __device__ __forceinline__ double combine(long long hi, long long lo) {
 
 // 2^n as a double, for n in the normal range (exact)
 __device__ __forceinline__ double pow2(int n) { return __longlong_as_double((long long)(n + 1023) << 52); }
+
+// v 2^n = (v p) 2^eo, p 2^eo = 2^n: in the bits of v where v and the result are normal
+// numbers (one FP64 operation less an output), else by multiplication (powers of two in
+// the normal range are exact)
+__device__ __forceinline__ double scaled(double v, int n, double p, int eo) {
+    const long long bits = __double_as_longlong(v);
+    const int ev = (int)((bits >> 52) & 0x7FF);
+    if (ev != 0 && ev != 0x7FF && ev + n > 0 && ev + n < 0x7FF) return __longlong_as_double(bits + ((long long)n << 52));
+    return n >= -1022 && n <= 1023 ? v * pow2(n) : v * p * pow2(eo);
+}
 
 // x 2^(56 - e) rounded to an integer (|x| < 2^e), from the bits of x with integer
 // operations only (the FP64 pipe is the resource this kernel avoids); zeros and
@@ -217,6 +229,16 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
     // frexp exponent of the row's largest magnitude: each half scans its half of the row
     // (integer compares of the magnitude bits, which order non-negative doubles) and the
     // two meet in shared memory; 0 for a row of zeros
+    auto magnitude = [](double v) { return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; };
+    auto shared_exponent = [&](unsigned long long mx) {  // of the two halves' maxima
+        if (worker) s_max[t] = mx;
+        __syncthreads();
+        const unsigned long long m2 = s_max[(t & 255) ^ 128];
+        mx = m2 > mx ? m2 : mx;
+        __syncthreads();  // s_max is reused by the next call
+        const int E = (int)(mx >> 52);
+        return E ? E - 1022 : 0;
+    };
     auto row_exponent = [&](auto in8) {
         unsigned long long mx = 0;
         for (int k0 = half * (N / 2); k0 < (half + 1) * (N / 2); k0 += 16) {
@@ -227,18 +249,11 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
             for (int j = 0; j < 2; ++j)
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const unsigned long long u =
-                        (unsigned long long)__double_as_longlong(x[j][i]) & 0x7FFFFFFFFFFFFFFFull;
+                    const unsigned long long u = magnitude(x[j][i]);
                     mx = u > mx ? u : mx;
                 }
         }
-        if (worker) s_max[t] = mx;
-        __syncthreads();
-        const unsigned long long m2 = s_max[(t & 255) ^ 128];
-        mx = m2 > mx ? m2 : mx;
-        __syncthreads();  // s_max is reused by the next call
-        const int E = (int)(mx >> 52);
-        return E ? E - 1022 : 0;
+        return shared_exponent(mx);
     };
 
     // One exact contraction out[o] = sum_k op[o][k] in(k) of this thread's column, in
@@ -342,8 +357,7 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const int eo = eop[o0 + i], n = e_in - 14 + eo;
-                        const double v = combine(hi[i], lo[i]);
-                        val[i] = n >= -1022 && n <= 1023 ? v * pow2(n) : v * p_in * pow2(eo);
+                        val[i] = scaled(combine(hi[i], lo[i]), n, p_in, eo);
                     }
                     epi16(o0, val);
                 }
@@ -367,6 +381,8 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
     };
     const int e_psi = row_exponent(in_psi);
     const int slot = (r * B + cell_inst[g]) * 2;
+    const double *sg = sigma_s + (size_t)g * N;
+    unsigned long long mx_x = 0;  // of the next contraction's inputs, formed here while phi is at hand
     contract(ops.D, ops.eD, e_psi, in_psi, [&](int l0, const double *pn) {
         if (!live) return;
         double *dst = phi + row + l0;
@@ -376,10 +392,20 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) reinterpret_cast<double2 *>(dst)[i] = make_double2(pn[2 * i], pn[2 * i + 1]);
+#pragma unroll
+        for (int i0 = 0; i0 < 16; i0 += 8) {
+            double sv[8], qv[8];
+            ld8(sg + l0 + i0, sv, false);
+            if (Qext) ld8(Qext + row + l0 + i0, qv, false);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const unsigned long long u = magnitude(sv[i] * pn[i0 + i] + (Qext ? qv[i] : 0.0));
+                mx_x = u > mx_x ? u : mx_x;
+            }
+        }
     });
     __syncthreads();  // the phi halves written by both threads of a column are read below
     // s = M x, x = Sigma phi + Q (FP64 per element; phi read through L2)
-    const double *sg = sigma_s + (size_t)g * N;
     auto in_x = [&](int k0, double *x) {
         if (!live) {
 #pragma unroll
@@ -393,7 +419,7 @@ __global__ void __launch_bounds__(rtc::kThreads, 1) k_mixed_residual_tc(
 #pragma unroll
         for (int i = 0; i < 8; ++i) x[i] = sv[i] * pv[i] + (Qext ? qv[i] : 0.0);
     };
-    const int e_x = ok ? row_exponent(in_x) : 0;
+    const int e_x = ok ? shared_exponent(mx_x) : 0;
     // the LD residual of this column's node for 16 ordinates, given the node's scattering
     // source s; the 16 ordinates share the sign of mu (N / 2 is a multiple of 16)
     const int b = cell_inst[g], loc = g - off[b];

@@ -281,9 +281,11 @@ typedef struct {
                                        is read once per 64 of them; only for FP32 factors
                                        (MIXED) with 2N a multiple of 128 up to 512 and at least
                                        16 right-hand sides, else FPSA_ENOTSUP; such a context
-                                       keeps a second, split copy of its factors, the same
-                                       size as the FP32 ones); 0 = tensor cores where they
-                                       apply, else the dataflow solve. Solutions differ by
+                                       keeps split copies of its factors and backward
+                                       operators, 1.5 times the size of the FP32 factors,
+                                       and where the device had no room for them at its
+                                       creation 2 is FPSA_ENOTSUP too); 0 = tensor cores
+                                       where they apply, else the dataflow solve. Solutions differ by
                                        rounding only */
     int32_t residual_engine;        /* MIXED, the FP64 refinement residual's two contractions
                                        (phi = D psi, s = M (Sigma phi + Q)): 1 = FP64 FMA

@@ -2178,8 +2178,8 @@ __global__ void __launch_bounds__(NT, 2) k_bcr_solve_flow(const T *__restrict__ 
 // one thread instead of thousands of 16-byte copies, which backed up the load/store
 // path while the wide levels stream), and the copy for the block's NEXT unit is
 // issued as soon as the current unit's matrix-vector product has read its columns,
-// so a block's factor stream overlaps the unit's reduction, pushes, fence and
-// counter bump and the next unit's wait for its inputs. The coupling blocks are
+// so a block's factor stream overlaps the unit's reduction and pushes and the next
+// unit's wait for its inputs. The coupling blocks are
 // double-buffered (the current unit multiplies by them after the next copy starts).
 // ---------------------------------------------------------------------------
 constexpr int kSolveStageBytes = 64 * 1024;

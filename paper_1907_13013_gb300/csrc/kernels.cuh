@@ -2562,6 +2562,8 @@ __global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restri
         return k >= ns && q.l == 0 && !phase_bwd(q.ph) && (q.ch + 1) * RC <= R;
     };
     constexpr int kHandoff = NTG + 32;  // threads of a handoff barrier: one group and its service warp
+    constexpr int kServiceBar = 3 + kSolveGroups * kMaxSolveStages;  // of the service warps
+    static_assert(kServiceBar < 16, "named barriers");
     if (threadIdx.x >= kSolveGroups * NTG) {
         // ---- service warps: copies into the ring, then per unit: handoff, refill
         const int sw = (threadIdx.x - kSolveGroups * NTG) >> 5, lane = threadIdx.x & 31;
@@ -2615,8 +2617,12 @@ __global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restri
             locate(nxt, blockIdx.x + (k + ns) * (int)gridDim.x);
             if (nxt.valid) issue(nxt, k + ns);
         }
-        // no copy may still be landing when the block exits: wait (bounded) for each
-        // stage's latest fill (at once if it has landed; it is pending only after a stop)
+        // No copy may still be landing when the block exits: wait (bounded) for each
+        // stage's latest fill (at once if it has landed; it is pending only after a stop).
+        // Both service warps have issued their last fill first: a fill of the other one that
+        // was issued and landed between the read of its count and the wait would leave the
+        // wait on a phase two fills old, whose parity never comes up again.
+        gbar_sync(kServiceBar, 32 * kSolveGroups);
         for (int st = 0; st < ns; ++st) {
             const int f = *(volatile int *)&s_fills[st];
             if (f > 0) tc::mbar_wait(&s_bar[st], (uint32_t)(f - 1) & 1u);

@@ -2334,6 +2334,16 @@ __device__ __forceinline__ void handoff_arrive(int id, int nthreads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// A count in shared memory, published to and read by other threads of the block.
+__device__ __forceinline__ int ld_acquire_shared(const int *p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(tc::smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_shared(int *p, int v) {
+    asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(p)), "r"(v) : "memory");
+}
+
 // The thread indices and barrier of one compute group.
 struct Group {
     int gt;   // thread index within the group
@@ -2434,11 +2444,21 @@ __device__ __forceinline__ bool ring_gather_unit(int j, const LevelTable &lv, co
 // The coarse unit u on a compute group: rows [u rpu, (u + 1) rpu) of u_c = G r_c (G
 // rows staged in As by the unit's bulk copy; r_c, the right-hand sides of the m coarse
 // cells in coarse order, collected into rc); the rows are written to Y and handed on.
-template <typename T, int NTG, typename WaitCopies>
+// rc lies in the unit's own stage (its coupling area, into which a coarse unit's fill
+// copies nothing), so the group writes it itself and may do so only once the stage is its
+// own: until the fill of unit k is issued, the stage belongs to unit k - n_stages, whose
+// coupling products may still be reading the area. With an even number of stages that unit
+// was this group's, with an odd one it is the other group's, and nothing else orders the
+// two: parts of r_c (rows no level pushes into) are there as soon as the gather units have
+// run. wait_issued() is that wait (the fill is issued after the handoff of unit
+// k - n_stages); it has long been met in the usual order of events.
+template <typename T, int NTG, typename WaitIssued, typename WaitCopies>
 __device__ __forceinline__ bool ring_coarse_unit(int u, const LevelTable &lv, T *Y, int N, T *rc, const T *As,
-                                                 const UnitLinks<T, 1> &lk, const Group &gr, WaitCopies wait_copies) {
+                                                 const UnitLinks<T, 1> &lk, const Group &gr, WaitIssued wait_issued,
+                                                 WaitCopies wait_copies) {
     const int n2 = 2 * N, cl = lv.coarse_level, m = lv.coarse_m, n = m * n2, rpu = lv.coarse_rpu, gt = gr.gt;
-    for (int i0 = gt; i0 < n; i0 += 8 * NTG) {
+    const bool mine = wait_issued();  // (a thread whose wait ran out writes nothing; wait_copies stops the group)
+    for (int i0 = gt; mine && i0 < n; i0 += 8 * NTG) {
         T v[8];
         bool here[8];
 #pragma unroll
@@ -2453,7 +2473,7 @@ __device__ __forceinline__ bool ring_coarse_unit(int u, const LevelTable &lv, T 
             if (i < n) rc[i] = v[q];
         }
     }
-    if (!wait_copies()) return false;
+    if (!wait_copies(mine)) return false;
     const int lane = gt & 31;
     for (int rr = gt >> 5; rr < rpu; rr += NTG / 32) {
         const T *g = As + (size_t)rr * n;
@@ -2595,7 +2615,7 @@ __global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restri
                                    &s_bar[st]);
             }
             __syncwarp();
-            if (lane == 0) *(volatile int *)&s_fills[st] = k / ns + 1;
+            if (lane == 0) st_release_shared(&s_fills[st], k / ns + 1);
         };
         if (sw == 0) {  // factors, couplings and G are not written by the previous kernel
             Pos q{0, 0, 0, 0, 0, 0, 0, false};
@@ -2646,18 +2666,20 @@ __global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restri
         const int st = k % ns;
         const uint32_t parity = (uint32_t)(k / ns) & 1u;
         T *As = stage_slice(st), *cb = stage_cpl(st);
-        // bounded; a group whose copies never land records the error and stops (the
-        // units left are then timed out by their consumers)
-        auto wait_copies = [&]() {
-            bool ok = true;
-            if (*(volatile int *)&s_fills[st] <= k / ns) {  // the fill has not been issued yet
+        // the fill of this unit's stage has been issued (bounded): the unit that held the
+        // stage before has been handed off and no longer reads it
+        auto wait_issued = [&]() {
+            if (ld_acquire_shared(&s_fills[st]) <= k / ns) {
                 const unsigned long long t0 = tc::global_ns();
-                while (*(volatile int *)&s_fills[st] <= k / ns)
-                    if (tc::global_ns() - t0 > tc::kWaitNs) {
-                        ok = false;
-                        break;
-                    }
+                while (ld_acquire_shared(&s_fills[st]) <= k / ns)
+                    if (tc::global_ns() - t0 > tc::kWaitNs) return false;
             }
+            return true;
+        };
+        // and its copies have landed; a group whose copies never land records the error and
+        // stops (the units left are then timed out by their consumers)
+        auto wait_copies = [&](bool ok = true) {
+            ok = ok && wait_issued();
             if (ok) ok = tc::mbar_wait(&s_bar[st], parity);
             const bool stalled = gbar_or(gr.bar, NTG, !ok);
             if (stalled && gr.gt == 0) {
@@ -2671,7 +2693,8 @@ __global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restri
             if constexpr (RC == 1) {
                 // the stage's coupling area holds r_c (coarse units take no couplings)
                 ok = cur.l == kGather ? ring_gather_unit<T, NTG>(cur.item, lv, rhs, N, lk, gr, wait_copies)
-                                      : ring_coarse_unit<T, NTG>(cur.item, lv, Y, N, cb, As, lk, gr, wait_copies);
+                                      : ring_coarse_unit<T, NTG>(cur.item, lv, Y, N, cb, As, lk, gr, wait_issued,
+                                                                 wait_copies);
             } else {
                 ok = false;
             }

@@ -860,9 +860,9 @@ int alloc_packets(fpsa_ctx *ctx) {
     pk.y = pk.push + n;
     pk.u = pk.y + 2 * n;
     pk.rc = pk.u + n;
-    CK(dalloc(ctx, &pk.epoch, 2));
-    const unsigned first[2] = {1u, 0u};
-    CK(cudaMemcpy(pk.epoch, first, sizeof(first), cudaMemcpyHostToDevice));
+    CK(dalloc(ctx, &pk.epoch, 1));
+    const unsigned long long first = 1ull << 32;
+    CK(cudaMemcpy(pk.epoch, &first, sizeof(first), cudaMemcpyHostToDevice));
     ctx->pk = pk;
     return FPSA_OK;
 }

@@ -43,3 +43,10 @@ def test_coarse_step(binding, N, K, method, precision):
     p = inputs.random_slab(K, N, N - 1, seed=1300 + K + N, kernel="srk", thick=(5, 200), c=(0.9, 0.999))
     kw = dict(inner_iterations=4) if precision == "mixed" and method == "fpsa" else {}
     _repeat(binding, p, 6, method, precision, **kw)
+
+
+@pytest.mark.parametrize("N,K,R,precision", [(16, 64, 1, "fp64"), (16, 400, 2, "mixed"), (128, 40, 1, "mixed"),
+                                             (64, 40, 3, "fp64")])
+def test_solve_numbers(binding, N, K, R, precision):
+    p = inputs.random_slab(K, N, N - 1, seed=1400 + K + N, kernel="hg", thick=(2, 60), c=(0.7, 0.99), nrhs=R)
+    _repeat(binding, p, 30, "fpsa", precision, **(dict(inner_iterations=4) if precision == "mixed" else {}))

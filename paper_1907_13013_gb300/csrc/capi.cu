@@ -856,13 +856,16 @@ int alloc_packets(fpsa_ctx *ctx) {
     const size_t n = (size_t)nchunk * g.sumK * RC * g.N * words, m = (size_t)ctx->lvt[e].coarse_m * 2 * g.N * words;
     Packets pk{};
     CK(dalloc(ctx, &pk.push, 4 * n + m));
-    CK(cudaMemset(pk.push, 0, (4 * n + m) * sizeof(*pk.push)));
+    // on the context's stream: one that does not wait for the legacy stream would let the next
+    // solve start before its packets are cleared (this also runs at a change of engine)
+    CK(cudaMemsetAsync(pk.push, 0, (4 * n + m) * sizeof(*pk.push), ctx->stream));
     pk.y = pk.push + n;
     pk.u = pk.y + 2 * n;
     pk.rc = pk.u + n;
     CK(dalloc(ctx, &pk.epoch, 1));
     const unsigned long long first = 1ull << 32;
-    CK(cudaMemcpy(pk.epoch, &first, sizeof(first), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(pk.epoch, &first, sizeof(first), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     ctx->pk = pk;
     return FPSA_OK;
 }
@@ -1487,6 +1490,7 @@ int gmres_alloc(fpsa_ctx *ctx, int m) {
             }
         CK(cudaMemcpy(ctx->gm_seg_begin, sb.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->gm_seg_end, se.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
+        CK(cudaStreamSynchronize(cudaStreamLegacy));  // (as at the end of fpsa_create)
         // small chunks where the large ones give most SMs none
         ctx->gm_small = (maxlen + kDotChunk - 1) / kDotChunk * nsys < ctx->n_sm;
         const int chunk = ctx->gm_small ? kDotChunkSmall : kDotChunk;
@@ -2179,14 +2183,17 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                 if (rp) return rp;
             }
         }
-        if (ctx->precision == FPSA_PRECISION_FP64) return alloc_path(ctx, ctx->p64, true);
-        int r2 = alloc_path(ctx, ctx->p64, false);
+        const bool mixed = ctx->precision == FPSA_PRECISION_MIXED;
+        int r2 = alloc_path(ctx, ctx->p64, !mixed);
+        if (!r2 && mixed) r2 = alloc_path(ctx, ctx->p32, true);
+        if (!r2 && mixed) r2 = setup_residual_tc(ctx);
+        if (!r2 && mixed) r2 = setup_tc(ctx);
         if (r2) return r2;
-        r2 = alloc_path(ctx, ctx->p32, true);
-        if (r2) return r2;
-        r2 = setup_residual_tc(ctx);
-        if (r2) return r2;
-        return setup_tc(ctx);
+        // the tables and cleared counters above went over the legacy stream, for which the
+        // context's own (it may be a non-blocking one) does not wait: a copy from pageable
+        // memory can return before its last part has arrived
+        CK(cudaStreamSynchronize(cudaStreamLegacy));
+        return FPSA_OK;
     }();
     if (rc != FPSA_OK) {
         g_create_error = ctx->err;

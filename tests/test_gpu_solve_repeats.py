@@ -50,3 +50,25 @@ def test_coarse_step(binding, N, K, method, precision):
 def test_solve_numbers(binding, N, K, R, precision):
     p = inputs.random_slab(K, N, N - 1, seed=1400 + K + N, kernel="hg", thick=(2, 60), c=(0.7, 0.99), nrhs=R)
     _repeat(binding, p, 30, "fpsa", precision, **(dict(inner_iterations=4) if precision == "mixed" else {}))
+
+
+def test_engine_change(binding):
+    import torch
+    p = inputs.random_slab(90, 64, 63, seed=1500, kernel="hg", thick=(2, 60), c=(0.7, 0.99), nrhs=16)
+    kw = dict(tol=1e-12, max_iterations=300, inner_iterations=4)
+    ref = binding.context_for(p, laplacian="wfd", precision="mixed")
+    ref.set_tuning({"solve_engine": 1})
+    want, _ = ref.solve("fpsa", **kw)
+    ref.close()
+    busy = torch.ones((8192, 8192), device="cuda")
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        ctx = binding.context_for(p, laplacian="wfd", precision="mixed")
+        ctx.solve("fpsa", **kw)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        busy = busy @ busy * 1e-4
+    ctx.set_tuning({"solve_engine": 1})
+    got, _ = ctx.solve("fpsa", **kw)
+    ctx.close()
+    assert np.array_equal(got, want)

@@ -257,9 +257,15 @@ __device__ __forceinline__ void poll(const int *c, int want, int *err, unsigned 
 }  // namespace tcs
 
 // The solve: units as above over the concatenated item array of lv. Counters per (tile of
-// RT right-hand sides, cell), n of each, zero at launch: flow[0 .. n) pushes landed in r,
-// [n .. 2n) forward slices written (for the cell's own backward slices), then two per cell,
-// the L- and the R+ rows of u final. queue: this launch's unit counter (zero at launch).
+// RT right-hand sides, cell), n of each, zero at launch: flow[0 .. n) edge slices (the ones
+// that push, first and last) of eliminated neighbours done, [n .. 2n) forward slices written
+// (for the cell's own backward slices), then two per cell, the L- and the R+ rows of u final.
+// An edge slice counts for BOTH neighbours of its cell, whichever it pushes into: a cell at
+// distance 2^l of another then starts, and pushes into the cells between which it lies, only
+// after both pushes of every cell of a lower level between them have landed, so the pushes
+// into a row are added in level order and a solve gives the same bits each time. (Counted
+// for the pushed-to neighbour alone, the push of a further cell could come before that of a
+// nearer one, made by another CTA.) queue: this launch's unit counter (zero at launch).
 // zero_next / queue_next: the other parity's counters, zeroed for the following solve.
 template <int RT>
 __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
@@ -540,6 +546,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                 int want = 0;
                 for (int lp = 0; lp < u.level; ++lp)
                     want += (u.local >= (1 << lp)) + (u.local + (1 << lp) < u.K_inst);
+                want *= min(MT, 2);  // edge slices of a neighbour
                 if (t == 0 && want) poll(cnt + u.cell, want, err, limit);
             } else {  // three warps, so that the polls overlap
                 if (t == 0) poll(fin + 2 * u.left + 1, 1, err, limit);
@@ -588,8 +595,10 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                         if (u.m == MT - 1) atomicAdd(fin + 2 * u.cell + 1, 1);
                     } else {
                         atomicAdd(written + u.cell, 1);
-                        if (pr) atomicAdd(cnt + u.right, 1);
-                        if (plf) atomicAdd(cnt + u.left, 1);
+                        if (u.m == 0 || u.m == MT - 1) {
+                            atomicAdd(cnt + u.left, 1);
+                            if (u.right >= 0) atomicAdd(cnt + u.right, 1);
+                        }
                     }
                 }
             } else {

@@ -72,3 +72,9 @@ def test_engine_change(binding):
     got, _ = ctx.solve("fpsa", **kw)
     ctx.close()
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("N,K,R", [(128, 200, 16), (128, 90, 64), (192, 60, 33), (256, 90, 16), (256, 40, 64)])
+def test_tensor_core_pushes(binding, N, K, R):
+    p = inputs.random_slab(K, N, N - 1, seed=1600 + K + N, kernel="hg", thick=(2, 60), c=(0.7, 0.99), nrhs=R)
+    _repeat(binding, p, 6, "fpsa", "mixed", inner_iterations=4)

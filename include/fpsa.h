@@ -282,11 +282,16 @@ typedef struct {
                                        (MIXED) with 2N a multiple of 128 up to 512 and at least
                                        16 right-hand sides, else FPSA_ENOTSUP; such a context
                                        keeps split copies of its factors and backward
-                                       operators, 1.5 times the size of the FP32 factors,
-                                       and where the device had no room for them at its
-                                       creation 2 is FPSA_ENOTSUP too); 0 = tensor cores
-                                       where they apply, else the dataflow solve. Solutions differ by
-                                       rounding only */
+                                       operators, 6 (2N)^2 bytes per cell, and of its
+                                       couplings, 12 (N/2)^2 bytes for each of about 2 blocks
+                                       per cell; where the device has no room for them at
+                                       its creation, or later for a GMRES basis beside
+                                       them, the context goes without and 2 is FPSA_ENOTSUP
+                                       too); 0 = tensor cores where they apply, else the
+                                       dataflow solve. Solutions differ by rounding only.
+                                       The dataflow solve keeps 16 (MIXED) or 32 bytes per
+                                       angular unknown; without room for those it runs
+                                       level by level, more slowly, to the same solution */
     int32_t residual_engine;        /* MIXED, the FP64 refinement residual's two contractions
                                        (phi = D psi, s = M (Sigma phi + Q)): 1 = FP64 FMA
                                        cores, 2 = tensor cores computing them exactly at FP64

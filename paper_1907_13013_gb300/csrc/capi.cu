@@ -232,10 +232,20 @@ template <typename P>
 cudaError_t dalloc(fpsa_ctx *ctx, P **p, size_t count) {
     void *v = nullptr;
     cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(P));
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();  // reported here; not left for the next check of a launch
+        return e;
+    }
     ctx->allocs.push_back(v);
     *p = static_cast<P *>(v);
     return cudaSuccess;
+}
+template <typename P>
+void dfree(fpsa_ctx *ctx, P *&p) {  // of a work space no kernel in flight uses
+    if (!p) return;
+    cudaFree(p);
+    ctx->allocs.erase(std::find(ctx->allocs.begin(), ctx->allocs.end(), (void *)p));
+    p = nullptr;
 }
 
 template <typename T>
@@ -847,34 +857,94 @@ void plan_solve_shape(fpsa_ctx *ctx) {
     }
 }
 
-// The packets of the dataflow BCR solve (kernels.cuh), in the path's element type.
+// The packets of the dataflow BCR solve (kernels.cuh), in the path's element type. FPSA_ENOMEM
+// leaves the context without (pk.push NULL).
+void free_packets(fpsa_ctx *ctx) {
+    dfree(ctx, ctx->pk.push);
+    dfree(ctx, ctx->pk.epoch);
+    ctx->pk = Packets{};
+}
 int alloc_packets(fpsa_ctx *ctx) {
     const Geometry &g = ctx->geo;
     const int e = ctx->precision == FPSA_PRECISION_FP64 ? 1 : 0;
     const int RC = solve_rc(g.R), nchunk = (g.R + RC - 1) / RC;
     const size_t words = e ? packet_words<double>() : packet_words<float>();
     const size_t n = (size_t)nchunk * g.sumK * RC * g.N * words, m = (size_t)ctx->lvt[e].coarse_m * 2 * g.N * words;
-    Packets pk{};
-    CK(dalloc(ctx, &pk.push, 4 * n + m));
+    Packets &pk = ctx->pk;
+    if (dalloc(ctx, &pk.push, 4 * n + m) != cudaSuccess || dalloc(ctx, &pk.epoch, 1) != cudaSuccess) {
+        free_packets(ctx);
+        return fail(ctx, FPSA_ENOMEM, "no device memory for the dataflow BCR solve's packets");
+    }
     // on the context's stream: one that does not wait for the legacy stream would let the next
     // solve start before its packets are cleared (this also runs at a change of engine)
     CK(cudaMemsetAsync(pk.push, 0, (4 * n + m) * sizeof(*pk.push), ctx->stream));
     pk.y = pk.push + n;
     pk.u = pk.y + 2 * n;
     pk.rc = pk.u + n;
-    CK(dalloc(ctx, &pk.epoch, 1));
     const unsigned long long first = 1ull << 32;
     CK(cudaMemcpyAsync(pk.epoch, &first, sizeof(first), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->pk = pk;
     return FPSA_OK;
 }
 
-// F u = rhs by block cyclic reduction over the stored factors: one cooperative
-// launch (forward levels, roots, backward levels); the solution is left in p.ybuf.
-// No memset precedes it (packets carry their solve's number; the tensor-core solve's
-// counters were zeroed by its previous solve), so it can be launched as a programmatic
-// dependent of the kernel before it.
+// What the tensor-core BCR solve keeps beside the factors: their split copy, the backward
+// operators, the split couplings and its counters. FPSA_ENOMEM leaves the context without
+// (tcs_rt 0).
+void free_tcs(fpsa_ctx *ctx) {
+    for (unsigned char **q : {&ctx->d_tcs_A, &ctx->d_tcs_P, &ctx->d_tcs_B, &ctx->d_tcs_C}) dfree(ctx, *q);
+    dfree(ctx, ctx->d_flow);
+    dfree(ctx, ctx->d_tcs_queue);
+    ctx->tcs_rt = 0;
+    if (ctx->tuning.solve_engine == 2) ctx->tuning.solve_engine = 0;
+}
+int alloc_tcs(fpsa_ctx *ctx) {
+    const Geometry &g = ctx->geo;
+    const int n2 = 2 * g.N, rt = tcs::rhs_tile(g.R);
+    ctx->flow_n = (size_t)((g.R + rt - 1) / rt) * g.sumK;
+    const size_t cpl = (size_t)g.n_slots * tcs::coupling_bytes(n2);
+    if (dalloc(ctx, &ctx->d_flow, 8 * ctx->flow_n) != cudaSuccess || dalloc(ctx, &ctx->d_tcs_queue, 2) != cudaSuccess ||
+        dalloc(ctx, &ctx->d_tcs_B, cpl) != cudaSuccess || dalloc(ctx, &ctx->d_tcs_C, cpl) != cudaSuccess ||
+        dalloc(ctx, &ctx->d_tcs_A, (size_t)g.sumK * tcs::cell_bytes(n2)) != cudaSuccess ||
+        dalloc(ctx, &ctx->d_tcs_P, (size_t)g.sumK * tcs::backward_bytes(n2)) != cudaSuccess) {
+        free_tcs(ctx);
+        return fail(ctx, FPSA_ENOMEM, "no device memory for the tensor-core BCR solve");
+    }
+    CK(cudaMemset(ctx->d_flow, 0, 8 * ctx->flow_n * sizeof(int)));
+    CK(cudaMemset(ctx->d_tcs_queue, 0, 2 * sizeof(int)));
+    const void *k = tcs_kernel(rt);
+    CK(raise_smem_limit(k, (int)tcs::Plan::make(rt).total));
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
+    ctx->tcs_rt = rt;
+    ctx->tcs_grid = 2 * ctx->n_sm;  // two CTAs per SM
+    return FPSA_OK;
+}
+
+// The BCR solve's own storage, after everything a context cannot do without: the tensor-core
+// solve's where it applies, else packets, else none (one launch per level). Either is kept
+// only if it leaves room for the caller's arrays of a solve, source and flux in FP64, so that
+// a problem that fills the device is refused by neither the library nor the caller's
+// allocator for the sake of the faster solve.
+int alloc_solve_storage(fpsa_ctx *ctx) {
+    const Geometry &g = ctx->geo;
+    const size_t room = (size_t)g.R * g.sumK * 2 * g.N * 16;
+    auto fits = [&](int rc) {
+        size_t free_b = 0, total = 0;
+        return rc == FPSA_OK && cudaMemGetInfo(&free_b, &total) == cudaSuccess && free_b >= room;
+    };
+    if (ctx->precision == FPSA_PRECISION_MIXED && tcs::applies(2 * g.N, g.R)) {
+        const int rc = alloc_tcs(ctx);
+        if (fits(rc)) return FPSA_OK;
+        if (rc != FPSA_OK && rc != FPSA_ENOMEM) return rc;
+        free_tcs(ctx);
+    }
+    const int rc = alloc_packets(ctx);
+    if (fits(rc)) return FPSA_OK;
+    if (rc != FPSA_OK && rc != FPSA_ENOMEM) return rc;
+    free_packets(ctx);
+    ctx->err.clear();
+    return FPSA_OK;
+}
+
 // The tensor-core solve (k_bcr_solve_tc): an ordinary launch of two CTAs per SM
 // that takes its units from a queue.
 int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *stop) {
@@ -902,11 +972,44 @@ int bcr_solve_tc(fpsa_ctx *ctx, PathBuffers<float> &p, float *rhs, const int *st
     return FPSA_OK;
 }
 
+// The solve level by level (k_bcr_solve_level), without storage of its own.
+template <typename T>
+int bcr_solve_levels(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs, const int *stop) {
+    const Geometry &g = ctx->geo;
+    const LevelTable &lv = ctx->lvt[sizeof(T) == 8 ? 1 : 0];
+    const int RC = solve_rc(g.R), nchunk = (g.R + RC - 1) / RC;
+    const size_t smem = (size_t)bcr_unit_smem_values(g.N, kSolveThreads, VecOf<T>::V, RC, (int)sizeof(T)) * sizeof(T);
+    auto run = [&](auto kern) -> int {
+        CK(raise_smem_limit((const void *)kern, (int)smem));
+        for (int ph = 0; ph <= 2 * lv.n_levels; ++ph) {
+            const int l = ph <= lv.n_levels ? ph : 2 * lv.n_levels - ph;
+            const long long units = (long long)(l < lv.n_levels ? lv.off[l + 1] - lv.off[l] : lv.n_roots) * nchunk * lv.slices[l];
+            Launch L_(ctx, FPSA_PHASE_BCR_SOLVE);
+            CK(launch_pdl(kern, dim3((unsigned)std::min<long long>(units, 4 * ctx->n_sm)), dim3(kSolveThreads), smem,
+                          ctx->stream, (const T *)p.A, (const T *)p.Bc, (const T *)p.Cc,
+                          (const BcrItem *)ctx->d_items_all, lv, rhs, p.ybuf, g.N, g.sumK, g.R, ph, stop));
+        }
+        return FPSA_OK;
+    };
+    switch (RC) {
+        case 8: return run(k_bcr_solve_level<T, kSolveThreads, 8>);
+        case 4: return run(k_bcr_solve_level<T, kSolveThreads, 4>);
+        case 2: return run(k_bcr_solve_level<T, kSolveThreads, 2>);
+        default: return run(k_bcr_solve_level<T, kSolveThreads, 1>);
+    }
+}
+
+// F u = rhs by block cyclic reduction over the stored factors; the solution is left in
+// p.ybuf. The dataflow solve is one cooperative launch (forward levels, roots, backward
+// levels). No memset precedes it (packets carry their solve's number; the tensor-core
+// solve's counters were zeroed by its previous solve), so it can be launched as a
+// programmatic dependent of the kernel before it.
 // stop: the flag at which the solve is skipped (NULL: none).
 template <typename T>
 int bcr_solve(fpsa_ctx *ctx, PathBuffers<T> &p, T *rhs, const int *stop = nullptr) {
     if constexpr (sizeof(T) == sizeof(float))
         if (ctx->tcs_rt && ctx->tuning.solve_engine != 1) return bcr_solve_tc(ctx, p, rhs, stop);
+    if (!ctx->pk.push) return bcr_solve_levels(ctx, p, rhs, stop);
     const Geometry &g = ctx->geo;
     int N = g.N, sumK = g.sumK, R = g.R;
     const BcrItem *items = ctx->d_items_all;
@@ -1461,23 +1564,19 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
 // Lazily allocate the GMRES work space for restart length m. The basis and work
 // vectors hold the precision of the Krylov solve (FP64 contexts: double; MIXED:
 // float, the inner solve of the refinement loop); dots are always FP64.
-int gmres_alloc(fpsa_ctx *ctx, int m) {
-    if (ctx->gm_restart >= m) return FPSA_OK;
+int gmres_alloc_all(fpsa_ctx *ctx, int m) {
     const Geometry &g = ctx->geo;
     const size_t n = (size_t)g.R * g.sumK * 2 * g.N;
     const size_t es = ctx->precision == FPSA_PRECISION_FP64 ? sizeof(double) : sizeof(float);
     const int nsys = g.R * g.B;
-    if (ctx->gm_V) {  // grow: release the old basis (the allocations list keeps the pointer)
-        CK(cudaFree(ctx->gm_V));
-        ctx->allocs.erase(std::find(ctx->allocs.begin(), ctx->allocs.end(), (void *)ctx->gm_V));
-        ctx->gm_V = nullptr;
-    }
+    ctx->gm_restart = 0;  // until everything for m is there
+    dfree(ctx, ctx->gm_V);
+    for (double **q : {&ctx->gm_partial, &ctx->gm_dots, &ctx->gm_coef, &ctx->gm_alpha}) dfree(ctx, *q);
     CK(dalloc(ctx, &ctx->gm_V, (size_t)(m + 1) * n * es));
-    if (!ctx->gm_u) {
-        CK(dalloc(ctx, &ctx->gm_u, n * es));
-        CK(dalloc(ctx, &ctx->gm_w, n * es));
-        CK(dalloc(ctx, &ctx->gm_b, n * es));
-        CK(dalloc(ctx, &ctx->gm_seg_begin, nsys));
+    for (unsigned char **q : {&ctx->gm_u, &ctx->gm_w, &ctx->gm_b})
+        if (!*q) CK(dalloc(ctx, q, n * es));
+    if (!ctx->gm_seg_begin) CK(dalloc(ctx, &ctx->gm_seg_begin, nsys));
+    if (!ctx->gm_seg_end) {
         CK(dalloc(ctx, &ctx->gm_seg_end, nsys));
         std::vector<long long> sb(nsys), se(nsys);
         long long maxlen = 0;
@@ -1496,18 +1595,35 @@ int gmres_alloc(fpsa_ctx *ctx, int m) {
         const int chunk = ctx->gm_small ? kDotChunkSmall : kDotChunk;
         ctx->gm_nchunks = (int)((maxlen + chunk - 1) / chunk);
     }
-    if (ctx->gm_partial) {
-        for (double *q : {ctx->gm_partial, ctx->gm_dots, ctx->gm_coef, ctx->gm_alpha}) {
-            CK(cudaFree(q));
-            ctx->allocs.erase(std::find(ctx->allocs.begin(), ctx->allocs.end(), (void *)q));
-        }
-    }
     CK(dalloc(ctx, &ctx->gm_partial, (size_t)nsys * ctx->gm_nchunks * (m + 1)));
     CK(dalloc(ctx, &ctx->gm_dots, (size_t)nsys * (m + 1)));
     CK(dalloc(ctx, &ctx->gm_coef, (size_t)nsys * (m + 1)));
     CK(dalloc(ctx, &ctx->gm_alpha, nsys));
     ctx->gm_restart = m;
     return FPSA_OK;
+}
+
+// Where the basis does not fit beside the BCR solve's own storage, that is given back: the
+// tensor-core solve's copies first (the dataflow solve then takes packets if they fit), then
+// the packets.
+int gmres_alloc(fpsa_ctx *ctx, int m) {
+    if (ctx->gm_restart >= m) return FPSA_OK;
+    int rc = gmres_alloc_all(ctx, m);
+    if (rc == FPSA_ENOMEM && ctx->tcs_rt) {
+        CK(cudaStreamSynchronize(ctx->stream));
+        free_tcs(ctx);
+        rc = gmres_alloc_all(ctx, m);
+        if (rc == FPSA_OK && !ctx->pk.push) {
+            const int rp = alloc_packets(ctx);
+            if (rp && rp != FPSA_ENOMEM) return rp;
+        }
+    }
+    if (rc == FPSA_ENOMEM && ctx->pk.push) {
+        CK(cudaStreamSynchronize(ctx->stream));
+        free_packets(ctx);
+        rc = gmres_alloc_all(ctx, m);
+    }
+    return rc;
 }
 
 // out[s][i] = <V_i, w>_s for i < nv, all systems s (FP64 sums); result copied to host hdots.
@@ -2139,31 +2255,6 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                 CK(raise_smem_limit((const void *)k_bgemm_tc<128>, (int)bgt::smem_bytes(128)));
                 ctx->bgemm_tc_able = true;
             }
-            // The tensor-core BCR solve keeps split copies of the factors and the backward
-            // operators beside the factors; a problem for which the device has no room for them
-            // (with 64 bytes per angular unknown for the vectors) takes the dataflow solve.
-            size_t mem_free = 0, mem_total = 0;
-            CK(cudaMemGetInfo(&mem_free, &mem_total));
-            const size_t tcs_need = (size_t)g.sumK * (2 * tcs::cell_bytes(2 * g.N) + tcs::backward_bytes(2 * g.N) +
-                                                      (size_t)g.R * 2 * g.N * 64);
-            if (ctx->precision == FPSA_PRECISION_MIXED && tcs::applies(2 * g.N, g.R) && tcs_need < mem_free) {
-                // two CTAs per SM
-                ctx->tcs_rt = tcs::rhs_tile(g.R);
-                ctx->tcs_grid = 2 * nsm;
-                ctx->flow_n = (size_t)((g.R + ctx->tcs_rt - 1) / ctx->tcs_rt) * g.sumK;
-                CK(dalloc(ctx, &ctx->d_flow, 8 * ctx->flow_n));
-                CK(cudaMemset(ctx->d_flow, 0, 8 * ctx->flow_n * sizeof(int)));
-                CK(dalloc(ctx, &ctx->d_tcs_B, (size_t)g.n_slots * tcs::coupling_bytes(2 * g.N)));
-                CK(dalloc(ctx, &ctx->d_tcs_C, (size_t)g.n_slots * tcs::coupling_bytes(2 * g.N)));
-                CK(dalloc(ctx, &ctx->d_tcs_A, (size_t)g.sumK * tcs::cell_bytes(2 * g.N)));
-                CK(dalloc(ctx, &ctx->d_tcs_P, (size_t)g.sumK * tcs::backward_bytes(2 * g.N)));
-                CK(dalloc(ctx, &ctx->d_tcs_queue, 2));
-                CK(cudaMemset(ctx->d_tcs_queue, 0, 2 * sizeof(int)));
-                const void *k = tcs_kernel(ctx->tcs_rt);
-                CK(raise_smem_limit(k, (int)tcs::Plan::make(ctx->tcs_rt).total));
-                CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        (int)cudaSharedmemCarveoutMaxShared));
-            }
             for (int e = 0; e < 2; ++e) {
                 LevelTable &lv = ctx->lvt[e];
                 lv.n_levels = g.n_levels;
@@ -2178,16 +2269,13 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
             }
             ctx->sweep_cpt = sweep_cells_per_thread(g);
             plan_solve_shape(ctx);
-            if (!ctx->tcs_rt) {
-                const int rp = alloc_packets(ctx);
-                if (rp) return rp;
-            }
         }
         const bool mixed = ctx->precision == FPSA_PRECISION_MIXED;
         int r2 = alloc_path(ctx, ctx->p64, !mixed);
         if (!r2 && mixed) r2 = alloc_path(ctx, ctx->p32, true);
         if (!r2 && mixed) r2 = setup_residual_tc(ctx);
         if (!r2 && mixed) r2 = setup_tc(ctx);
+        if (!r2) r2 = alloc_solve_storage(ctx);
         if (r2) return r2;
         // the tables and cleared counters above went over the legacy stream, for which the
         // context's own (it may be a non-blocking one) does not wait: a copy from pageable
@@ -2602,12 +2690,12 @@ int fpsa_set_tuning(fpsa_ctx *ctx, const fpsa_tuning *t) {
         return fail(ctx, FPSA_ENOTSUP, "tensor-core residual needs MIXED precision and N a multiple of 32 up to 256");
     if (r.solve_engine == 2 && ctx->tcs_rt == 0)
         return fail(ctx, FPSA_ENOTSUP,
-                    "tensor-core BCR solve needs FP32 factors (MIXED), 2N a multiple of 128 up to 512 and at least "
-                    "16 right-hand sides");
+                    "tensor-core BCR solve needs FP32 factors (MIXED), 2N a multiple of 128 up to 512, at least "
+                    "16 right-hand sides and room on the device for its copies of the factors");
     if (r.solve_engine == 1 && !ctx->pk.push) {  // a tensor-core context's first dataflow solve
         CK(cudaSetDevice(ctx->device));
         const int rc = alloc_packets(ctx);
-        if (rc) return rc;
+        if (rc && rc != FPSA_ENOMEM) return rc;  // (without packets: level by level)
     }
     // the segment maps were allocated for the smallest cells-per-thread (most segments)
     const int cmin = sweep_cells_per_thread(ctx->geo);
@@ -2637,7 +2725,8 @@ int fpsa_autotune(fpsa_ctx *ctx, const fpsa_opts *opts, int32_t repeats, fpsa_tu
     CK(cudaEventCreate(&sc.e1));
     const fpsa_tuning saved = ctx->tuning;
     // fastest of `repeats` timed solves after one untimed solve with shapes t
-    auto trial = [&](const fpsa_tuning &t, double &ms) -> int {
+    auto trial = [&](fpsa_tuning t, double &ms) -> int {
+        if (!ctx->tcs_rt && t.solve_engine == 2) t.solve_engine = 0;  // (given up for a GMRES basis meanwhile)
         int rc = fpsa_set_tuning(ctx, &t);
         ms = INFINITY;
         for (int i = 0; rc == FPSA_OK && i <= repeats; ++i) {
@@ -2654,7 +2743,9 @@ int fpsa_autotune(fpsa_ctx *ctx, const fpsa_opts *opts, int32_t repeats, fpsa_tu
     };
     auto give_up = [&](int rc) {
         const std::string msg = ctx->err;
-        fpsa_set_tuning(ctx, &saved);
+        fpsa_tuning t = saved;
+        if (!ctx->tcs_rt && t.solve_engine == 2) t.solve_engine = 0;
+        fpsa_set_tuning(ctx, &t);
         ctx->err = msg;
         return rc;
     };
@@ -2680,6 +2771,7 @@ int fpsa_autotune(fpsa_ctx *ctx, const fpsa_opts *opts, int32_t repeats, fpsa_tu
         if (ms < bms) bms = ms, bt = t;
     }
     // keep the winner (the context's moments are those of the last trial solve)
+    if (!ctx->tcs_rt && bt.solve_engine == 2) bt.solve_engine = 0;
     const int rc = fpsa_set_tuning(ctx, &bt);
     if (rc != FPSA_OK) return give_up(rc);
     if (best) fpsa_get_tuning(ctx, best);

@@ -1929,6 +1929,13 @@ struct UnitLinks {
         }
         return v0;
     }
+    __device__ __forceinline__ void push(const BcrItem &it, int side, int rc, int p, T v) const {
+        packet_put<T>(pk.push, push_at(it.cell, side, rc, p), v, e);
+    }
+    __device__ __forceinline__ void put_y(int cell, int rc, int row, T v) const {
+        packet_put<T>(pk.y, y_at(cell, rc, row), v, e);
+    }
+    __device__ __forceinline__ T y(int cell, int rc, int row) const { return get(pk.y, y_at(cell, rc, row)); }
     // Row `row` of the cell's solution (its outflow rows travel on).
     __device__ __forceinline__ void put_u(int cell, int rc, int row, T v) const {
         if (row < h2) packet_put<T>(pk.u, u_at(cell, rc, row), v, e);
@@ -1938,6 +1945,33 @@ struct UnitLinks {
     __device__ __forceinline__ T inflow(const BcrItem &it, int rc, int k) const {
         if (k < h2) return get(pk.u, u_at(it.left, rc, h2 + k));
         return it.right >= 0 ? get(pk.u, u_at(it.right, rc, k - h2)) : T(0);
+    }
+};
+
+// The same hand-overs through rhs and Y themselves, for a solve of one launch per phase
+// (k_bcr_solve_level): what a unit reads was written by an earlier launch, and within one
+// every word has at most one writer and no reader besides it (the cells of a level push into
+// cells of higher levels, whose L+ rows receive from the left and R- rows from the right).
+template <typename T>
+struct LevelLinks {
+    T *rhs, *Y;
+    size_t rstride;
+    int r0, h2;
+
+    __device__ __forceinline__ T *at(T *v, int cell, int rc) const {
+        return v + (size_t)(r0 + rc) * rstride + (size_t)cell * (4 * h2);
+    }
+    __device__ __forceinline__ T less_received(T v0, int, int, int, int, int, int) const { return v0; }
+    __device__ __forceinline__ void push(const BcrItem &it, int side, int rc, int p, T v) const {
+        T *r = side ? at(rhs, it.left, rc) + 2 * h2 + p : at(rhs, it.right, rc) + h2 + p;
+        *r = __ldcg(r) - v;
+    }
+    __device__ __forceinline__ void put_y(int cell, int rc, int row, T v) const { at(Y, cell, rc)[row] = v; }
+    __device__ __forceinline__ T y(int cell, int rc, int row) const { return __ldcg(at(Y, cell, rc) + row); }
+    __device__ __forceinline__ void put_u(int, int, int, T) const {}
+    __device__ __forceinline__ T inflow(const BcrItem &it, int rc, int k) const {
+        if (k < h2) return __ldcg(at(Y, it.left, rc) + 3 * h2 + k);
+        return it.right >= 0 ? __ldcg(at(Y, it.right, rc) + k - h2) : T(0);
     }
 };
 
@@ -2023,11 +2057,11 @@ __global__ void __launch_bounds__(512, 1) k_bcr_factor_flow(T *__restrict__ A, c
 }
 
 // Units cover RC consecutive right-hand sides r0 .. r0 + nrc - 1 (nrc <= RC).
-template <typename T, int NT, int RC>
+template <typename T, int NT, int RC, typename Links>
 __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *__restrict__ Bc,
                                              const T *__restrict__ Cc, const BcrItem &it, int r0, int nrc, int sl,
                                              int S, const T *rhs, T *Y, int N, int sumK, T *sm,
-                                             const UnitLinks<T, RC> &lk) {
+                                             const Links &lk) {
     const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2;
     T *rs = sm, *ys = sm + RC * n2, *part = ys + RC * n2 + RC * N;
     T *cbuf = bcr_couplings_staged(N, (int)sizeof(T)) ? part + NT * VecOf<T>::V * RC : nullptr;
@@ -2056,7 +2090,7 @@ __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *_
         ys[rc * n2 + row0 + row] = y;
         if (rc >= nrc) continue;
         if (it.left >= 0) {
-            packet_put<T>(lk.pk.y, lk.y_at(it.cell, rc, row0 + row), y, lk.e);
+            lk.put_y(it.cell, rc, row0 + row, y);
         } else {  // a root: its solution is final
             lk.put_u(it.cell, rc, row0 + row, y);
             Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y;
@@ -2065,15 +2099,15 @@ __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *_
     if (cbuf) cp_async_wait_all();
     __syncthreads();
     coupling_products<T, NT, RC>(mB, ys + N + h2, mC, ys, h2, n2, threadIdx.x, [&](int side, int rc, int p, T v) {
-        if (rc < nrc) packet_put<T>(lk.pk.push, lk.push_at(it.cell, side, rc, p), v, lk.e);
+        if (rc < nrc) lk.push(it, side, rc, p, v);
     });
     __syncthreads();  // scratch reuse by the block's next unit
 }
 
-template <typename T, int NT, int RC>
+template <typename T, int NT, int RC, typename Links>
 __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *__restrict__ Bc,
                                              const T *__restrict__ Cc, const BcrItem &it, int r0, int nrc, int sl,
-                                             int S, T *Y, int N, int sumK, T *sm, const UnitLinks<T, RC> &lk) {
+                                             int S, T *Y, int N, int sumK, T *sm, const Links &lk) {
     const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2;
     T *gv = sm, *g = sm + RC * N, *part = sm + RC * (5 * N);  // gv[rc] = [u_left[R+], u_right[L-]]
     T *cbuf = bcr_couplings_staged(N, (int)sizeof(T)) ? part + NT * VecOf<T>::V * RC : nullptr;
@@ -2100,7 +2134,7 @@ __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *_
         const int rc = idx / nr, row = idx - rc * nr;
         T s = T(0);
         for (int q = 0; q < KS; ++q) s += part[(q * RC + rc) * nr + row];
-        const T u = lk.get(lk.pk.y, lk.y_at(it.cell, rc, row0 + row)) - s;
+        const T u = lk.y(it.cell, rc, row0 + row) - s;
         lk.put_u(it.cell, rc, row0 + row, u);
         Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = u;
     }
@@ -2166,6 +2200,30 @@ __global__ void __launch_bounds__(NT, 2) k_bcr_solve_flow(const T *__restrict__ 
         const int r0 = ch * RC, nrc = min(RC, R - r0);
         const BcrItem it = items[lv.off[l] + item];
         lk.cell0 = (size_t)ch * sumK;
+        if (ph <= nl) bcr_fwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, rhs, Y, N, sumK, sm, lk);
+        else bcr_bwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, Y, N, sumK, sm, lk);
+    }
+}
+
+// One phase of the same reduction as a launch of its own, for contexts that have no room for
+// packets (they take 16 bytes per angular unknown in FP32, 32 in FP64): same units, slices
+// and order of the sums, so without a coarse step the same bits as k_bcr_solve_flow; 2 n_levels + 1
+// launches a solve.
+template <typename T, int NT, int RC>
+__global__ void __launch_bounds__(NT, 2) k_bcr_solve_level(const T *__restrict__ A, const T *__restrict__ Bc,
+                                                           const T *__restrict__ Cc, const BcrItem *__restrict__ items,
+                                                           LevelTable lv, T *rhs, T *Y, int N, int sumK, int R, int ph,
+                                                           const int *stop) {
+    tc::grid_dependency_wait();
+    if (stopped(stop)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *sm = reinterpret_cast<T *>(smem_raw);
+    const int nchunk = (R + RC - 1) / RC, nl = lv.n_levels, l = ph <= nl ? ph : 2 * nl - ph, S = lv.slices[l];
+    const int nitems = l < nl ? lv.off[l + 1] - lv.off[l] : lv.n_roots, nunits = nitems * nchunk * S;
+    for (int w = blockIdx.x; w < nunits; w += gridDim.x) {
+        const int sl = w % S, r0 = (w / S) % nchunk * RC, nrc = min(RC, R - r0);
+        const BcrItem it = items[lv.off[l] + w / (S * nchunk)];
+        const LevelLinks<T> lk{rhs, Y, (size_t)sumK * 2 * N, r0, N / 2};
         if (ph <= nl) bcr_fwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, rhs, Y, N, sumK, sm, lk);
         else bcr_bwd_unit<T, NT, RC>(A, Bc, Cc, it, r0, nrc, sl, S, Y, N, sumK, sm, lk);
     }

@@ -35,19 +35,25 @@ namespace {
 // kSegMax segments of kSegWarps * cpt cells. Beyond that, where right-hand sides and
 // instances fill the chip by themselves, longer chunks (up to 64 cells) share a block's
 // fixed work (the maps of the segments and chunks before it) among more cells: as many as
-// leave kSweepBlocks blocks (two rounds of eight per SM). 64 right-hand sides of 1250 cells
-// at N = 256: 330 us a sweep with 4 cells, 159 with 32.
-constexpr int kSweepBlocks = 2 * 8 * 152;
-inline int sweep_cells_per_thread(const Geometry &g) {
+// leave kSweepRounds rounds of eight blocks per SM, and no more than give every warp of a
+// block a chunk of the longest slab (many short slabs would otherwise leave most of a
+// block's warps without cells). 64 right-hand sides of 1250 cells at N = 256: 330 us a sweep
+// with 4 cells, 159 with 32; 20000 slabs of 40 cells at N = 16, FP64: 6.05 ms with 64 cells,
+// 2.49 with 5.
+constexpr int kSweepRounds = 2;
+inline int sweep_cells_per_thread(const Geometry &g, int n_sm) {
     const int per = kSegMax * kSegWarps;
     const long long cells = 2ll * ((g.N / 2 + 31) / 32) * g.R * g.sumK;  // (direction, ordinate group, rhs, cell)
-    const long long fill = std::min<long long>(64, cells / ((long long)kSegWarps * kSweepBlocks) / kSweepBatch * kSweepBatch);
+    const long long blocks = 8ll * kSweepRounds * n_sm;
+    const long long fill = std::min<long long>({64, cells / (kSegWarps * blocks) / kSweepBatch * kSweepBatch,
+                                                (g.Kmax + kSegWarps - 1) / kSegWarps});
     return std::max({4, (g.Kmax + per - 1) / per, (int)fill});
 }
-inline int sweep_segments(const Geometry &g) {
-    const int len = kSegWarps * sweep_cells_per_thread(g);
+inline int sweep_segments(const Geometry &g, int n_sm) {
+    const int len = kSegWarps * sweep_cells_per_thread(g, n_sm);
     return (g.Kmax + len - 1) / len;
 }
+
 constexpr int kContractThreads = 256;
 constexpr int kInvertThreads = 512;
 constexpr int kSolveThreads = 256;  // one (item, rhs) unit per block (the staged solve: its compute groups' threads)
@@ -405,7 +411,7 @@ int alloc_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
     CK(dalloc(ctx, &p.phi, ang));
     CK(dalloc(ctx, &p.psi, ang));
     {
-        const int nseg = sweep_segments(g);
+        const int nseg = sweep_segments(g, ctx->n_sm);
         CK(dalloc(ctx, &p.smap, (size_t)g.R * g.B * nseg * N * 2));
         CK(dalloc(ctx, &p.cmap, (size_t)g.R * g.B * nseg * kSegWarps * N * 2));
     }
@@ -2267,7 +2273,7 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
                     off += l < g.n_levels ? (int)g.levels[l].size() : g.B;
                 }
             }
-            ctx->sweep_cpt = sweep_cells_per_thread(g);
+            ctx->sweep_cpt = sweep_cells_per_thread(g, ctx->n_sm);
             plan_solve_shape(ctx);
         }
         const bool mixed = ctx->precision == FPSA_PRECISION_MIXED;
@@ -2698,7 +2704,7 @@ int fpsa_set_tuning(fpsa_ctx *ctx, const fpsa_tuning *t) {
         if (rc && rc != FPSA_ENOMEM) return rc;  // (without packets: level by level)
     }
     // the segment maps were allocated for the smallest cells-per-thread (most segments)
-    const int cmin = sweep_cells_per_thread(ctx->geo);
+    const int cmin = sweep_cells_per_thread(ctx->geo, ctx->n_sm);
     ctx->sweep_cpt = std::max(cmin, r.sweep_cells_per_thread);
     ctx->tuning = r;
     plan_solve_shape(ctx);
@@ -2760,7 +2766,7 @@ int fpsa_autotune(fpsa_ctx *ctx, const fpsa_opts *opts, int32_t repeats, fpsa_tu
             if (rc != FPSA_OK) return give_up(rc);
             if (ms < bms) bms = ms, bt = t;
         }
-    const int cmin = sweep_cells_per_thread(g);
+    const int cmin = sweep_cells_per_thread(g, ctx->n_sm);
     auto segments = [&](int c) { return (g.Kmax + kSegWarps * c - 1) / (kSegWarps * c); };
     for (int k = 1; k <= 3 && segments(cmin << k) < segments(cmin << (k - 1)); ++k) {
         fpsa_tuning t = bt;

@@ -15,6 +15,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "fpsa_internal.h"
@@ -164,6 +165,7 @@ struct fpsa_ctx {
     int *d_stop = nullptr;
     ConvSlot *h_slots = nullptr;
     unsigned conv_seq = 0;
+    unsigned wait_flags = 0;  // how the process asked CUDA to wait (cudaDeviceSchedule*)
     int *h_flag = nullptr;  // pinned, after the slots
     double growth_limit = kGrowthLimit;  // fpsa_set_xs: FPSA_EPIVOT above this pivot growth
     int tc_grid = 0;
@@ -1090,12 +1092,20 @@ int report_alone(fpsa_ctx *ctx, const ConvReport &r) {
     return FPSA_OK;
 }
 
-// Wait for report r. The stream is asked now and then, so that a failed launch ends the wait.
+// Wait for report r, in the manner the process asked CUDA to wait (cudaSetDeviceFlags): with
+// blocking waits the thread sleeps between polls, with yielding ones it offers its core at
+// each, and otherwise it spins as a stream synchronization does, offering its core now and
+// then (several threads may be solving). The stream is asked now and then too, so that a
+// failed launch ends the wait.
 int wait_report(fpsa_ctx *ctx, const ConvReport &r, double &e, int &err) {
     const volatile ConvSlot *s = r.slot;
     auto arrived = [&]() { return __atomic_load_n(const_cast<const unsigned *>(&s->seq), __ATOMIC_ACQUIRE) == r.seq; };
+    const bool block = ctx->wait_flags == cudaDeviceScheduleBlockingSync;
+    const unsigned yield_every = ctx->wait_flags == cudaDeviceScheduleYield ? 1 : 256;
     for (unsigned n = 1; !arrived(); ++n) {
-        if (n % 4096) continue;
+        if (block) std::this_thread::sleep_for(std::chrono::microseconds(20));
+        else if (n % yield_every == 0) std::this_thread::yield();
+        if (n % (block ? 64 : 4096)) continue;
         const cudaError_t q = cudaStreamQuery(ctx->stream);
         if (q == cudaErrorNotReady) {
             (void)cudaGetLastError();
@@ -2161,6 +2171,8 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
             CK(cudaMemcpy(ctx->d_stop, e0, sizeof(e0), cudaMemcpyHostToDevice));
         }
         CK(cudaMallocHost(&ctx->h_slots, kConvSlots * sizeof(ConvSlot) + sizeof(int)));
+        CK(cudaGetDeviceFlags(&ctx->wait_flags));
+        ctx->wait_flags &= cudaDeviceScheduleMask;
         std::memset(ctx->h_slots, 0, kConvSlots * sizeof(ConvSlot) + sizeof(int));
         ctx->h_flag = reinterpret_cast<int *>(ctx->h_slots + kConvSlots);
         CK(dalloc(ctx, &ctx->d_factor_cnt, (size_t)g.sumK + 1));  // + the tensor-core factorization's queue

@@ -133,7 +133,7 @@ struct fpsa_ctx {
     int *d_status = nullptr;
     double *d_result = nullptr;
     int *d_steps = nullptr;      // refinement steps taken by a batch graph's loop
-    cudaEvent_t ad_ev[4] = {};   // MIXED: first residual and first inner step, timed once per solve
+    cudaEvent_t ad_ev[6] = {};   // MIXED: first residual and first inner step, timed once per solve
 
     // adjoint
     bool fwd_ready = false;      // d_phi_fwd holds the last converged forward moments
@@ -1453,11 +1453,12 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
     double e = INFINITY, e_prev = INFINITY;
     int outer = 0, sweeps = 0;
     // the adaptive inner count pays only where a residual costs more than an inner
-    // iteration: both are timed once, on the first refinement step (event pairs)
+    // iteration: both are timed once, on the first refinement step (event pairs; the step in
+    // its two parts, without the host's turn between them)
     bool adaptive_on = false;
     const bool time_first = adaptive && fpsa;
     if (time_first && !ctx->ad_ev[0])
-        for (int i = 0; i < 4; ++i) CK(cudaEventCreate(&ctx->ad_ev[i]));
+        for (cudaEvent_t &ev : ctx->ad_ev) CK(cudaEventCreate(&ev));
     for (outer = 1; outer <= o.max_iterations + 1; ++outer) {
         if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[0], st));
         int rcr = mixed_residual_launch(ctx, mp, Qm, Qa, inc, gmres, false);
@@ -1472,6 +1473,7 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
         if (ahead) {
             if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[2], st));
             rcr = mixed_inner_launch(ctx, mp, 1, 1, fpsa, false, rep);
+            if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[3], st));
         } else {
             rcr = report_alone(ctx, rep);
         }
@@ -1550,19 +1552,21 @@ int solve_mixed(fpsa_ctx *ctx, const fpsa_opts &o, const double *phi0, int mem, 
         k_before = k_last;
         k_last = inner_k;
         if (time_first && outer == 2) {
-            CK(cudaEventSynchronize(ctx->ad_ev[3]));  // (already reached: the report came after it)
-            float t_res = 0.f, t_step = 0.f;
+            CK(cudaEventSynchronize(ctx->ad_ev[5]));  // (already reached: the report came after it)
+            float t_res = 0.f, t_first = 0.f, t_rest = 0.f;
             if (cudaEventElapsedTime(&t_res, ctx->ad_ev[0], ctx->ad_ev[1]) == cudaSuccess &&
-                cudaEventElapsedTime(&t_step, ctx->ad_ev[2], ctx->ad_ev[3]) == cudaSuccess)
-                adaptive_on = t_res * inner > t_step;  // residual slower than one inner iteration
+                cudaEventElapsedTime(&t_first, ctx->ad_ev[2], ctx->ad_ev[3]) == cudaSuccess &&
+                cudaEventElapsedTime(&t_rest, ctx->ad_ev[4], ctx->ad_ev[5]) == cudaSuccess)
+                adaptive_on = t_res * inner > t_first + t_rest;  // residual slower than one inner iteration
             (void)cudaGetLastError();
         }
         if (!adaptive_on && inner_k > inner) inner_k = inner;
         k_last = inner_k;
+        if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[4], st));
         int rci = mixed_inner_launch(ctx, mp, 2, inner_k, fpsa, true);
         if (rci) return rci;
         sweeps += inner_k;
-        if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[3], st));
+        if (time_first && outer == 1) CK(cudaEventRecord(ctx->ad_ev[5], st));
     }
     stats.iterations = gmres ? krylov : sweeps;
     stats.outer_iterations = std::min(outer, o.max_iterations + 1);

@@ -647,7 +647,7 @@ int setup_tc(fpsa_ctx *ctx) {
     CK(raise_smem_limit((const void *)k_tc_update_scatter_tile, smem));
     CK(raise_smem_limit((const void *)k_tc_fp_rhs_moments, smem));
     CK(raise_smem_limit((const void *)k_tc_moments_axpy, smem));
-    ctx->tc_cols = tc::col_tile(ctx->geo.sumK, ctx->geo.R, nsm);
+    ctx->tc_cols = col_tile(N, ctx->geo.sumK, ctx->geo.R, nsm);
     if (ctx->tc_cols) {
         const int cs = (int)tc::ColPlan::make(N, ctx->tc_cols).total;
         const void *fr[3] = {(const void *)k_tc_fp_rhs_cols<16>, (const void *)k_tc_fp_rhs_cols<32>,
@@ -1263,7 +1263,7 @@ int mixed_plan(fpsa_ctx *ctx, const fpsa_opts &o, MixedPlan &mp) {
 }
 
 // The tensor-core contractions of the FP32 inner solves, by size: few columns per block
-// where that leaves no SM with more than one block (N <= 128; tc::col_tile), else
+// where that pays (N <= 128; col_tile), else
 // 128-column tiles, whole (N <= 64) or in k-chunks, with streamed operators for N > 128.
 int tc_wide(fpsa_ctx *ctx, const MixedPlan &mp, void (*kern)(tcw::Args, TcOps, int, int, int, int *),
             const tcw::Args &a) {

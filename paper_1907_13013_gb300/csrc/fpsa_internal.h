@@ -21,6 +21,22 @@ struct Tables {
 };
 void build_tables(int N, int L1, int laplacian, Tables &t);
 
+// Columns per block of the few-column tensor-core contractions (tc_contract.cuh): the fewest
+// (of 16, 32, 64) whose blocks fit one per SM; 0: the 128-column tiles. A wider block costs
+// more the more outputs a thread holds, whatever the order, while the tiles' time falls with
+// it, most below N = 65, where they hold both operators and all inputs of a tile at once. Us
+// for the pair of kernels of an iteration, few-column form against tiles, one right-hand side:
+//   N =          16           32           48           64           96           128
+//   CT = 16      11.6 / 11.7  11.6 / 15.2               13.1 / 22.8               14.5 / 88
+//   CT = 32      15.8 / 11.7  15.6 / 15.1  17.3 / 19.2  17.0 / 22.9               19.3 / 96
+//   CT = 64      30.6 / 12.1  51.9 / 15.9               55.0 / 23.1  56.3 / 81.8  57.3 / 96
+inline int col_tile(int N, int sumK, int R, int n_sm) {
+    const int widest = N <= 32 ? 16 : (N <= 64 ? 32 : 64);
+    for (int ct = 16; ct <= widest; ct *= 2)
+        if (((2ll * sumK + ct - 1) / ct) * R <= n_sm) return ct;
+    return 0;
+}
+
 // One cell eliminated at one block-cyclic-reduction level (or an instance root).
 // Cell ids are global (concatenated over instances); -1 = absent.
 // Coupling slots index the per-level N/2 x N/2 coupling blocks B (to the left

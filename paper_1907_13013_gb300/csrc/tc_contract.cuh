@@ -651,8 +651,9 @@ __global__ void __launch_bounds__(128) k_tc_update_scatter_tile(const float *__r
 // the B operand (N = CT), so a tile is as small as 16 columns. Thread t < N owns output t
 // of every column: its global accesses are whole rows across the threads, all requested
 // at the start, and both nodes of a cell meet in one thread. What bounds it is latency
-// (one pass of loads, two short chains of MMAs, one of stores per block); with 2000
-// columns (K = 1000) at N = 128 the 128-column kernels take 35 and 59 us on 16 SMs.
+// (one pass of loads, two short chains of MMAs, one of stores per block), and from CT = 32 on
+// the registers that hold a thread's outputs (CT = 64: 255, 208 bytes of spills in the
+// update). Used where col_tile says (fpsa_internal.h), with the figures there.
 // ---------------------------------------------------------------------------
 namespace tc {
 // Shared memory: the operators as in Plan, x_hi and x_lo (CT x N BF16 each), 2 mbarriers,
@@ -670,12 +671,6 @@ struct ColPlan {
         return p;
     }
 };
-// columns per block: the fewest (of 16, 32, 64) whose blocks fit one per SM; 0: none does
-__host__ inline int col_tile(int sumK, int R, int n_sm) {
-    for (int ct = 16; ct <= 64; ct *= 2)
-        if ((long long)((2 * sumK + ct - 1) / ct) * R <= n_sm) return ct;
-    return 0;
-}
 }  // namespace tc
 
 template <int CT>

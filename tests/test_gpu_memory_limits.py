@@ -26,6 +26,14 @@ def binding():
     return b
 
 
+@pytest.fixture(autouse=True)
+def give_back():
+    """The held blocks go back to the device, not only to the caching allocator."""
+    yield
+    import torch
+    torch.cuda.empty_cache()
+
+
 def _free():
     import torch
     torch.cuda.synchronize()

@@ -384,10 +384,11 @@ const void *tcs_kernel(int RT) {
     }
 }
 
+// shared memory of a one-CTA inversion of an n x n block (n may be odd: a leaf of the
+// recursive inversion of a block of 4 x odd rows)
 template <typename T>
-size_t invert_smem(int N) {
-    const int n2 = 2 * N;
-    return ((size_t)n2 * (n2 + 1) + n2) * sizeof(T) + (size_t)n2 * sizeof(int);
+size_t invert_smem(int n) {
+    return ((size_t)n * (n + 1) + n) * sizeof(T) + (size_t)n * sizeof(int);
 }
 
 // full: every buffer of an FPSA iteration in precision T. Otherwise only the tables,
@@ -399,7 +400,7 @@ size_t invert_smem(int N) {
 // latency bound, so halving their length does not pay for the extra GEMMs.)
 template <typename T>
 bool cta_invertible(int n) {
-    return n == 32 || n == 64 || n == 128 || invert_smem<T>(n / 2) <= kSmemLimit;
+    return n == 32 || n == 64 || n == 128 || invert_smem<T>(n) <= kSmemLimit;
 }
 
 template <typename T>
@@ -474,8 +475,8 @@ int alloc_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
         }
     CK(cudaMemcpy(p.DT, DT.data(), N * N * sizeof(T), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(p.MT, MT.data(), N * N * sizeof(T), cudaMemcpyHostToDevice));
-    if (invert_smem<T>(g.N) <= kSmemLimit)
-        CK(raise_smem_limit((const void *)k_bcr_invert<T>, (int)invert_smem<T>(g.N)));
+    if (invert_smem<T>(2 * g.N) <= kSmemLimit)
+        CK(raise_smem_limit((const void *)k_bcr_invert<T>, (int)invert_smem<T>(2 * g.N)));
     return FPSA_OK;
 }
 
@@ -515,8 +516,8 @@ int invert_inplace(fpsa_ctx *ctx, PathBuffers<T> &p, BMat<T> M, int n, const Bcr
         k_binv_reg_rm<T, 64><<<ne, 512, 0, st>>>(M, items, ctx->d_status);
     } else if (n == 32) {
         k_binv_reg_rm<T, 32><<<ne, 512, 0, st>>>(M, items, ctx->d_status);
-    } else if (invert_smem<T>(n / 2) <= kSmemLimit) {
-        k_binv_smem_rm<T><<<ne, kInvertThreads, invert_smem<T>(n / 2), st>>>(M, n, items, ctx->d_status);
+    } else if (invert_smem<T>(n) <= kSmemLimit) {
+        k_binv_smem_rm<T><<<ne, kInvertThreads, invert_smem<T>(n), st>>>(M, n, items, ctx->d_status);
     } else {
         const int h = n / 2;
         if (depth >= (int)p.inv_scratch.size()) return fail(ctx, FPSA_ENOTSUP, "block inversion scratch missing");
@@ -560,7 +561,7 @@ int invert_level(fpsa_ctx *ctx, PathBuffers<T> &p, const BcrItem *items, int ni,
     } else if (n2 == 32) {
         k_bcr_invert_reg<T, 32><<<ni, 512, ssm, st>>>(p.A, items, ctx->d_growth, ctx->d_status, p.Bc, p.Cc, staged);
     } else if (cta_invertible<T>(n2)) {
-        k_bcr_invert<T><<<ni, kInvertThreads, invert_smem<T>(ctx->geo.N), st>>>(p.A, items, n2, ctx->d_growth,
+        k_bcr_invert<T><<<ni, kInvertThreads, invert_smem<T>(n2), st>>>(p.A, items, n2, ctx->d_growth,
                                                                                ctx->d_status);
     } else {
         const BMat<T> M{p.A, (long long)n2 * n2, n2, 1};

@@ -266,6 +266,21 @@ bool schur_staged(int N) { return (size_t)3 * (N / 2) * (N / 2) * sizeof(T) <= 2
 template <typename T>
 size_t schur_smem(int N) { return (size_t)(schur_staged<T>(N) ? 3 : 1) * (N / 2) * (N / 2) * sizeof(T); }
 
+// the Schur update kernel of a coupling block's order (its register tile: schur_tile)
+template <typename T>
+const void *schur_kernel(int h2) {
+    switch (schur_tile(h2)) {
+        case 1: return (const void *)k_bcr_schur<T, 1>;
+        case 2: return (const void *)k_bcr_schur<T, 2>;
+        case 3: return (const void *)k_bcr_schur<T, 3>;
+        case 4: return (const void *)k_bcr_schur<T, 4>;
+        case 5: return (const void *)k_bcr_schur<T, 5>;
+        case 6: return (const void *)k_bcr_schur<T, 6>;
+        case 7: return (const void *)k_bcr_schur<T, 7>;
+        default: return (const void *)k_bcr_schur<T, 8>;
+    }
+}
+
 // usable dynamic shared memory per CTA (227 KB opt-in, less room for static shared memory)
 constexpr size_t kSmemLimit = 227 * 1024 - 1024;
 
@@ -444,12 +459,7 @@ int alloc_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
             CK(dalloc(ctx, &p.inv_amax, kLargeChunk));
             CK(raise_smem_limit((const void *)k_binv_smem_rm<T>, (int)kSmemLimit));
         }
-        switch (schur_tile(h2)) {
-            case 1: CK(raise_smem_limit((const void *)k_bcr_schur<T, 1>, (int)schur_tile_smem<T>(h2))); break;
-            case 2: CK(raise_smem_limit((const void *)k_bcr_schur<T, 2>, (int)schur_tile_smem<T>(h2))); break;
-            case 4: CK(raise_smem_limit((const void *)k_bcr_schur<T, 4>, (int)schur_tile_smem<T>(h2))); break;
-            default: CK(raise_smem_limit((const void *)k_bcr_schur<T, 8>, (int)schur_tile_smem<T>(h2))); break;
-        }
+        CK(raise_smem_limit(schur_kernel<T>(h2), (int)schur_tile_smem<T>(h2)));
     }
     {
         const int cs = (int)contract_smem<T>(g.N);
@@ -749,14 +759,9 @@ int setup_path(fpsa_ctx *ctx, PathBuffers<T> &p, bool full) {
         CK(cudaGetLastError());
         if (!fused) {
             Launch L_(ctx, FPSA_PHASE_BCR_SCHUR);
-            const dim3 grid(ni, 4);
-            const size_t sm = schur_tile_smem<T>(h2);
-            switch (schur_tile(h2)) {
-                case 1: k_bcr_schur<T, 1><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
-                case 2: k_bcr_schur<T, 2><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
-                case 4: k_bcr_schur<T, 4><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
-                default: k_bcr_schur<T, 8><<<grid, 256, sm, st>>>(p.A, p.Bc, p.Cc, ctx->d_levels[l], N); break;
-            }
+            const int n = N;
+            void *args[] = {(void *)&p.A, (void *)&p.Bc, (void *)&p.Cc, (void *)&ctx->d_levels[l], (void *)&n};
+            CK(cudaLaunchKernel(schur_kernel<T>(h2), dim3(ni, 4), dim3(256), args, schur_tile_smem<T>(h2), st));
         }
         CK(cudaGetLastError());
     }

@@ -1462,28 +1462,37 @@ __device__ __forceinline__ void schur_body(T *__restrict__ A, T *__restrict__ Bc
 // transposed, as the second product's left operand. What bounds it is FP32 (FP64)
 // arithmetic, 4 h2^3 operations an update: TI x TI register tiles make that 2 TI shared
 // loads for TI^2 FMAs (2 x 2 tiles, and one block for all four updates, took 978 us a
-// level at h2 = 128 and 113 us at h2 = 64).
+// level at h2 = 128 and 113 us at h2 = 64). TI is the smallest that covers h2, and rows and
+// k beyond h2 are left out: in FP64 every padded FMA costs a real one (the Schur updates of
+// 1500 cells at N = 66 took 1.9 ms with one 2 x 2-tiled block per item, 3.9 with tiles for
+// h2 = 64 and 128 only, 1.4 now; of 20000 cells at N = 8 0.57, 0.79 and 0.23 ms).
 constexpr int kSchurK = 16;
-constexpr int schur_tile(int h2) { return h2 <= 16 ? 1 : (h2 <= 32 ? 2 : (h2 <= 64 ? 4 : 8)); }
+constexpr int schur_tile(int h2) { return (h2 + 15) / 16; }  // TI, 1 to 8
 template <typename T>
 constexpr size_t schur_tile_smem(int h2) {  // X^T, then the chunks of both operands
     return ((size_t)h2 * (16 * schur_tile(h2) + 1) + (size_t)2 * kSchurK * (16 * schur_tile(h2) + 1)) * sizeof(T);
 }
 
-// acc[i][j] += sum_k L[k][16 i + ty] Rt[k][16 j + tx], k < nk (rows of ld values)
-template <typename T, int TI>
-__device__ __forceinline__ void schur_mma(const T *L, const T *Rt, int ld, int nk, int tx, int ty, T (&acc)[TI][TI]) {
+// acc[i][j] += sum_k L[k][16 i + ty] Rt[k][16 j + tx], k < nk (rows of ld values), i < NI
+template <typename T, int TI, int NI>
+__device__ __forceinline__ void schur_mma_rows(const T *L, const T *Rt, int ld, int nk, int tx, int ty, T (&acc)[TI][TI]) {
     for (int k = 0; k < nk; ++k) {
         T l[TI], r[TI];
 #pragma unroll
-        for (int i = 0; i < TI; ++i) l[i] = L[k * ld + 16 * i + ty];
+        for (int i = 0; i < NI; ++i) l[i] = L[k * ld + 16 * i + ty];
 #pragma unroll
         for (int j = 0; j < TI; ++j) r[j] = Rt[k * ld + 16 * j + tx];
 #pragma unroll
-        for (int i = 0; i < TI; ++i)
+        for (int i = 0; i < NI; ++i)
 #pragma unroll
             for (int j = 0; j < TI; ++j) acc[i][j] = fma(l[i], r[j], acc[i][j]);
     }
+}
+// The last of a thread's rows is left out by the warps (of two rows each) that have none of it.
+template <typename T, int TI>
+__device__ __forceinline__ void schur_mma(const T *L, const T *Rt, int ld, int nk, int h2, int tx, int ty, T (&acc)[TI][TI]) {
+    if (16 * (TI - 1) + (ty & ~1) < h2) schur_mma_rows<T, TI, TI>(L, Rt, ld, nk, tx, ty, acc);
+    else if constexpr (TI > 1) schur_mma_rows<T, TI, TI - 1>(L, Rt, ld, nk, tx, ty, acc);
 }
 
 template <typename T, int TI>
@@ -1538,7 +1547,7 @@ __global__ void __launch_bounds__(256) k_bcr_schur(T *__restrict__ A, T *__restr
             Rs[kk * ld + p] = in ? P[(size_t)p * n2 + k0 + kk] : T(0);
         }
         __syncthreads();
-        schur_mma<T, TI>(Ls, Rs, ld, kSchurK, tx, ty, acc);
+        schur_mma<T, TI>(Ls, Rs, ld, min(kSchurK, h2 - k0), h2, tx, ty, acc);
         __syncthreads();
     }
 #pragma unroll
@@ -1553,7 +1562,7 @@ __global__ void __launch_bounds__(256) k_bcr_schur(T *__restrict__ A, T *__restr
             Rs[kk * ld + q] = (k0 + kk < h2 && q < h2) ? V[(size_t)(k0 + kk) * h2 + q] : T(0);
         }
         __syncthreads();
-        schur_mma<T, TI>(Xt + (size_t)k0 * ld, Rs, ld, min(kSchurK, h2 - k0), tx, ty, acc);
+        schur_mma<T, TI>(Xt + (size_t)k0 * ld, Rs, ld, min(kSchurK, h2 - k0), h2, tx, ty, acc);
         __syncthreads();
     }
 #pragma unroll

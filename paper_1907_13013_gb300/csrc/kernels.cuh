@@ -1634,6 +1634,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_but_last() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // Start copying the coupling blocks m0, m1 (either may be NULL) into cbuf[0, hh) and
@@ -1889,6 +1890,7 @@ __device__ __noinline__ T packet_wait(const unsigned long long *p, size_t i, uns
 // The solve a unit belongs to: its packets of one chunk of right-hand sides, and its waits.
 template <typename T, int RC>
 struct UnitLinks {
+    static constexpr bool kReceives = true;
     Packets pk;
     unsigned e, limit;
     int *err;
@@ -1904,39 +1906,43 @@ struct UnitLinks {
     __device__ __forceinline__ size_t u_at(int cell, int rc, int k) const {
         return ((cell0 + cell) * RC + rc) * (2 * h2) + k;
     }
-    __device__ __forceinline__ T get(const unsigned long long *p, size_t i) const {
-        T v;
-        if (!packet_try<T>(p, i, e, v)) v = packet_wait<T>(p, i, e, err, limit);
-        return v;
-    }
-    // v less what the cells eliminated below level `level` hand to row `row` of cell (local
-    // index a of K), in level order: L+ rows receive from the left neighbours at distance
-    // 2^l, R- rows from the right ones; four requested at a time, so that a unit that starts
-    // late pays one read.
-    __device__ __forceinline__ T less_received(T v0, int cell, int a, int K, int level, int rc, int row) const {
-        const bool left = row >= h2 && row < 2 * h2, right = row >= 2 * h2 && row < 3 * h2;
-        if (!left && !right) return v0;
-        const int p = left ? row - h2 : row - 2 * h2;
-        for (int l0 = 0; l0 < level; l0 += 4) {
-            T v[4];
-            bool have[4], here[4];
+    // v[q] less what the cells eliminated below level `level` hand to row row[q] of cell (local
+    // index a of K) for right-hand side rc[q] (on[q] false: nothing), in level order: L+ rows
+    // receive from the left neighbours at distance 2^l, R- rows from the right ones. The words
+    // of LV levels of all NE elements are requested together, so that a unit that starts late
+    // pays few reads one after the other.
+    template <int NE>
+    __device__ __forceinline__ void less_received(T (&v)[NE], const bool (&on)[NE], int cell, int a, int K, int level,
+                                                  const int (&rc)[NE], const int (&row)[NE]) const {
+        constexpr int LV = NE >= 4 ? 1 : 4 / NE;
+        bool any = false;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int step = 1 << (l0 + u);
-                have[u] = l0 + u < level && (left ? a >= step : a + step < K);
-                here[u] = !have[u] ||
-                          packet_try<T>(pk.push, push_at(left ? cell - step : cell + step, left ? 0 : 1, rc, p), e, v[u]);
-            }
+        for (int q = 0; q < NE; ++q) any = any || (on[q] && row[q] >= h2 && row[q] < 3 * h2);
+        if (!any) return;
+        for (int l0 = 0; l0 < level; l0 += LV) {
+            T w[NE][LV];
+            bool have[NE][LV], here[NE][LV];
+            auto at = [&](int q, int step) {
+                const bool left = row[q] < 2 * h2;
+                return push_at(left ? cell - step : cell + step, left ? 0 : 1, rc[q], row[q] - (left ? h2 : 2 * h2));
+            };
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int step = 1 << (l0 + u);
-                if (!here[u])
-                    v[u] = packet_wait<T>(pk.push, push_at(left ? cell - step : cell + step, left ? 0 : 1, rc, p), e, err,
-                                          limit);
-                if (have[u]) v0 -= v[u];
-            }
+            for (int q = 0; q < NE; ++q)
+#pragma unroll
+                for (int u = 0; u < LV; ++u) {
+                    const int step = 1 << (l0 + u);
+                    const bool left = row[q] < 2 * h2;
+                    have[q][u] = on[q] && row[q] >= h2 && row[q] < 3 * h2 && l0 + u < level && (left ? a >= step : a + step < K);
+                    here[q][u] = !have[q][u] || packet_try<T>(pk.push, at(q, step), e, w[q][u]);
+                }
+#pragma unroll
+            for (int q = 0; q < NE; ++q)
+#pragma unroll
+                for (int u = 0; u < LV; ++u) {
+                    if (!here[q][u]) w[q][u] = packet_wait<T>(pk.push, at(q, 1 << (l0 + u)), e, err, limit);
+                    if (have[q][u]) v[q] -= w[q][u];
+                }
         }
-        return v0;
     }
     __device__ __forceinline__ void push(const BcrItem &it, int side, int rc, int p, T v) const {
         packet_put<T>(pk.push, push_at(it.cell, side, rc, p), v, e);
@@ -1944,16 +1950,28 @@ struct UnitLinks {
     __device__ __forceinline__ void put_y(int cell, int rc, int row, T v) const {
         packet_put<T>(pk.y, y_at(cell, rc, row), v, e);
     }
-    __device__ __forceinline__ T y(int cell, int rc, int row) const { return get(pk.y, y_at(cell, rc, row)); }
+    // y and the inflow of a backward unit: *_try takes the value if it is there
+    __device__ __forceinline__ bool y_try(int cell, int rc, int row, T &v) const {
+        return packet_try<T>(pk.y, y_at(cell, rc, row), e, v);
+    }
+    __device__ __forceinline__ T y_wait(int cell, int rc, int row) const {
+        return packet_wait<T>(pk.y, y_at(cell, rc, row), e, err, limit);
+    }
     // Row `row` of the cell's solution (its outflow rows travel on).
     __device__ __forceinline__ void put_u(int cell, int rc, int row, T v) const {
         if (row < h2) packet_put<T>(pk.u, u_at(cell, rc, row), v, e);
         else if (row >= 3 * h2) packet_put<T>(pk.u, u_at(cell, rc, row - 2 * h2), v, e);
     }
-    // Inflow k of a backward unit: the left neighbour's R+ (k < N/2), the right one's L-.
-    __device__ __forceinline__ T inflow(const BcrItem &it, int rc, int k) const {
-        if (k < h2) return get(pk.u, u_at(it.left, rc, h2 + k));
-        return it.right >= 0 ? get(pk.u, u_at(it.right, rc, k - h2)) : T(0);
+    // Inflow k of a backward unit: the left neighbour's R+ (k < N/2), the right one's L- (0 without one).
+    __device__ __forceinline__ size_t inflow_at(const BcrItem &it, int rc, int k) const {
+        return k < h2 ? u_at(it.left, rc, h2 + k) : u_at(it.right, rc, k - h2);
+    }
+    __device__ __forceinline__ bool inflow_try(const BcrItem &it, int rc, int k, T &v) const {
+        v = T(0);
+        return (k >= h2 && it.right < 0) || packet_try<T>(pk.u, inflow_at(it, rc, k), e, v);
+    }
+    __device__ __forceinline__ T inflow_wait(const BcrItem &it, int rc, int k) const {
+        return packet_wait<T>(pk.u, inflow_at(it, rc, k), e, err, limit);
     }
 };
 
@@ -1963,6 +1981,7 @@ struct UnitLinks {
 // cells of higher levels, whose L+ rows receive from the left and R- rows from the right).
 template <typename T>
 struct LevelLinks {
+    static constexpr bool kReceives = false;  // (pushes go into rhs itself)
     T *rhs, *Y;
     size_t rstride;
     int r0, h2;
@@ -1970,19 +1989,116 @@ struct LevelLinks {
     __device__ __forceinline__ T *at(T *v, int cell, int rc) const {
         return v + (size_t)(r0 + rc) * rstride + (size_t)cell * (4 * h2);
     }
-    __device__ __forceinline__ T less_received(T v0, int, int, int, int, int, int) const { return v0; }
+    template <int NE>
+    __device__ __forceinline__ void less_received(T (&)[NE], const bool (&)[NE], int, int, int, int, const int (&)[NE],
+                                                  const int (&)[NE]) const {}
     __device__ __forceinline__ void push(const BcrItem &it, int side, int rc, int p, T v) const {
         T *r = side ? at(rhs, it.left, rc) + 2 * h2 + p : at(rhs, it.right, rc) + h2 + p;
         *r = __ldcg(r) - v;
     }
     __device__ __forceinline__ void put_y(int cell, int rc, int row, T v) const { at(Y, cell, rc)[row] = v; }
-    __device__ __forceinline__ T y(int cell, int rc, int row) const { return __ldcg(at(Y, cell, rc) + row); }
-    __device__ __forceinline__ void put_u(int, int, int, T) const {}
-    __device__ __forceinline__ T inflow(const BcrItem &it, int rc, int k) const {
-        if (k < h2) return __ldcg(at(Y, it.left, rc) + 3 * h2 + k);
-        return it.right >= 0 ? __ldcg(at(Y, it.right, rc) + k - h2) : T(0);
+    __device__ __forceinline__ bool y_try(int cell, int rc, int row, T &v) const {
+        v = __ldcg(at(Y, cell, rc) + row);
+        return true;
     }
+    __device__ __forceinline__ T y_wait(int, int, int) const { return T(0); }  // (never)
+    __device__ __forceinline__ void put_u(int, int, int, T) const {}
+    __device__ __forceinline__ bool inflow_try(const BcrItem &it, int rc, int k, T &v) const {
+        if (k < h2) v = __ldcg(at(Y, it.left, rc) + 3 * h2 + k);
+        else v = it.right >= 0 ? __ldcg(at(Y, it.right, rc) + k - h2) : T(0);
+        return true;
+    }
+    __device__ __forceinline__ T inflow_wait(const BcrItem &, int, int) const { return T(0); }  // (never)
 };
+
+// What a unit collects from its links, NT threads (tid), NE elements a thread requested
+// together: one at a time, each a read through the L2 and a test before the next, the reads of
+// a unit of eight right-hand sides were longer than its product (1500 cells at N = 128, FP32,
+// eight right-hand sides: 786 us a solve, now 568; 100 cells at N = 256, one: 312, now 235).
+// NE is small where the registers also hold the first columns of A^{-1}: beyond that they
+// spill (500 cells at N = 128, four right-hand sides: 131 us, 235 with four elements).
+// rs[rc][k] (row stride n2, its own right-hand sides in place) less what the cell has received
+template <typename T, int NT, int NE, typename Links>
+__device__ __forceinline__ void receive_pushes(const Links &lk, const BcrItem &it, int nrc, int N, T *rs, int tid) {
+    for (int i0 = tid; i0 < nrc * N; i0 += NE * NT) {
+        T v[NE];
+        bool on[NE];
+        int rc[NE], row[NE];
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int i = i0 + q * NT;
+            on[q] = i < nrc * N;
+            rc[q] = i / N;
+            row[q] = N / 2 + i - rc[q] * N;
+            v[q] = on[q] ? rs[rc[q] * 2 * N + row[q]] : T(0);
+        }
+        lk.less_received(v, on, it.cell, it.local, it.K_inst, it.level, rc, row);
+#pragma unroll
+        for (int q = 0; q < NE; ++q)
+            if (on[q]) rs[rc[q] * 2 * N + row[q]] = v[q];
+    }
+}
+// rs[rc][k] = the unit's complete right-hand sides (0 from nrc on)
+template <typename T, int NT, int RC, int NE, typename Links>
+__device__ __forceinline__ void collect_rhs(const Links &lk, const T *rhs, const BcrItem &it, int r0, int nrc, int n2,
+                                            size_t rstride, T *rs, int tid) {
+    for (int i0 = tid; i0 < RC * n2; i0 += NE * NT) {
+        T v[NE];
+        bool on[NE];
+        int rc[NE], row[NE];
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int i = i0 + q * NT;
+            rc[q] = i / n2;
+            row[q] = i - rc[q] * n2;
+            on[q] = i < RC * n2 && rc[q] < nrc;
+            v[q] = on[q] ? __ldcg(rhs + (size_t)(r0 + rc[q]) * rstride + (size_t)it.cell * n2 + row[q]) : T(0);
+        }
+        lk.less_received(v, on, it.cell, it.local, it.K_inst, it.level, rc, row);
+#pragma unroll
+        for (int q = 0; q < NE; ++q)
+            if (i0 + q * NT < RC * n2) rs[i0 + q * NT] = v[q];
+    }
+}
+// gv[rc][k] = the inflow of a backward unit (0 from nrc on)
+template <typename T, int NT, int RC, int NE, typename Links>
+__device__ __forceinline__ void collect_inflow(const Links &lk, const BcrItem &it, int nrc, int N, T *gv, int tid) {
+    for (int i0 = tid; i0 < RC * N; i0 += NE * NT) {
+        T v[NE];
+        bool here[NE];
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int i = i0 + q * NT, rc = i / N;
+            v[q] = T(0);
+            here[q] = i >= RC * N || rc >= nrc || lk.inflow_try(it, rc, i - rc * N, v[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int i = i0 + q * NT, rc = i / N;
+            if (!here[q]) v[q] = lk.inflow_wait(it, rc, i - rc * N);
+            if (i < RC * N) gv[i] = v[q];
+        }
+    }
+}
+// out(rc, row, y) for the rows row0 .. row0 + nr - 1 of y, from element i0 of this thread on
+template <typename T, int NT, int NE, typename Links, typename Out>
+__device__ __forceinline__ void collect_y(const Links &lk, int cell, int nrc, int nr, int row0, int i0, Out out) {
+    for (; i0 < nrc * nr; i0 += NE * NT) {
+        T v[NE];
+        bool here[NE];
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int i = i0 + q * NT, rc = i / nr;
+            here[q] = i >= nrc * nr || lk.y_try(cell, rc, row0 + i - rc * nr, v[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int i = i0 + q * NT, rc = i / nr;
+            if (!here[q]) v[q] = lk.y_wait(cell, rc, row0 + i - rc * nr);
+            if (i < nrc * nr) out(rc, i - rc * nr, v[q]);
+        }
+    }
+}
 
 __device__ __forceinline__ void flow_wait(const FlowSync *fs) {
     if (!fs) return;
@@ -2081,15 +2197,36 @@ __device__ __forceinline__ void bcr_fwd_unit(const T *__restrict__ A, const T *_
     const bool push_left = it.left >= 0 && row0 == 0;          // this slice holds L-
     const T *mB = push_right ? Bc + (size_t)it.s_right * hh : nullptr;
     const T *mC = push_left ? Cc + (size_t)it.s_left * hh : nullptr;
+    // Up to two right-hand sides are read, less what the cell has received, into registers; more
+    // of them are copied into place, in flight with the first columns of A^{-1}, and the pushes
+    // subtracted there.
+    constexpr bool kCopy = RC > 2;
+    if constexpr (kCopy) {
+        const int rchunks = n2 * (int)sizeof(T) / 16;  // (N is even)
+        for (int c = threadIdx.x; c < RC * rchunks; c += NT) {
+            const int rc = c / rchunks, cc = c - rc * rchunks;
+            uint4 *dst = reinterpret_cast<uint4 *>(rs + rc * n2) + cc;
+            if (rc < nrc)
+                cp_async16(dst, reinterpret_cast<const uint4 *>(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2) + cc);
+            else
+                *dst = make_uint4(0u, 0u, 0u, 0u);
+        }
+        cp_async_commit();
+    }
     stage_couplings(mB, mC, cbuf, hh);  // in flight during the matrix-vector product
     const int KS = sliced_matvec<T, NT, RC>(Ai, n2, row0, nr, n2, n2, 0, 0, rs, n2, part, [&] {
-        for (int i = threadIdx.x; i < RC * n2; i += NT) {
-            const int rc = i / n2, k = i - rc * n2;
-            rs[i] = rc < nrc ? lk.less_received(__ldcg(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + k),
-                                                it.cell, it.local, it.K_inst, it.level, rc, k)
-                             : T(0);
+        if constexpr (kCopy) {
+            if (cbuf) cp_async_wait_but_last();
+            else cp_async_wait_all();
+            __syncthreads();
+            if (Links::kReceives && it.level > 0) {
+                receive_pushes<T, NT, 2>(lk, it, nrc, N, rs, threadIdx.x);
+                __syncthreads();
+            }
+        } else {
+            collect_rhs<T, NT, RC, sizeof(T) == 4 ? 2 : 1>(lk, rhs, it, r0, nrc, n2, rstride, rs, threadIdx.x);
+            __syncthreads();
         }
-        __syncthreads();
     });
     __syncthreads();
     for (int idx = threadIdx.x; idx < RC * nr; idx += NT) {
@@ -2118,6 +2255,7 @@ __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *_
                                              const T *__restrict__ Cc, const BcrItem &it, int r0, int nrc, int sl,
                                              int S, T *Y, int N, int sumK, T *sm, const Links &lk) {
     const int n2 = 2 * N, h2 = N / 2, hh = h2 * h2;
+    constexpr int kNE = sizeof(T) == 4 ? (RC == 8 ? 4 : (RC == 1 ? 1 : 2)) : (RC >= 4 ? 2 : 1);
     T *gv = sm, *g = sm + RC * N, *part = sm + RC * (5 * N);  // gv[rc] = [u_left[R+], u_right[L-]]
     T *cbuf = bcr_couplings_staged(N, (int)sizeof(T)) ? part + NT * VecOf<T>::V * RC : nullptr;
     const size_t rstride = (size_t)sumK * n2;
@@ -2126,10 +2264,7 @@ __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *_
     const T *mB = Bc + (size_t)it.s_cell * hh, *mC = it.right >= 0 ? Cc + (size_t)it.s_cell * hh : nullptr;
     stage_couplings(mB, mC, cbuf, hh);
     const int KS = sliced_matvec<T, NT, RC>(Ai, n2, row0, nr, N, h2, h2, N, g, N, part, [&] {
-        for (int idx = threadIdx.x; idx < RC * N; idx += NT) {
-            const int rc = idx / N, k = idx - rc * N;
-            gv[idx] = rc < nrc ? lk.inflow(it, rc, k) : T(0);
-        }
+        collect_inflow<T, NT, RC, kNE>(lk, it, nrc, N, gv, threadIdx.x);
         if (cbuf) cp_async_wait_all();
         __syncthreads();
         coupling_products<T, NT, RC>(mB, gv, mC, gv + h2, h2, N, threadIdx.x,
@@ -2139,14 +2274,12 @@ __device__ __forceinline__ void bcr_bwd_unit(const T *__restrict__ A, const T *_
         __syncthreads();
     });
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nrc * nr; idx += NT) {
-        const int rc = idx / nr, row = idx - rc * nr;
+    collect_y<T, NT, kNE>(lk, it.cell, nrc, nr, row0, threadIdx.x, [&](int rc, int row, T y) {
         T s = T(0);
         for (int q = 0; q < KS; ++q) s += part[(q * RC + rc) * nr + row];
-        const T u = lk.y(it.cell, rc, row0 + row) - s;
-        lk.put_u(it.cell, rc, row0 + row, u);
-        Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = u;
-    }
+        lk.put_u(it.cell, rc, row0 + row, y - s);
+        Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y - s;
+    });
     __syncthreads();
 }
 
@@ -2432,12 +2565,10 @@ __device__ __forceinline__ bool ring_fwd_unit(const T *mB, const T *mC, const Bc
     const size_t rstride = (size_t)sumK * n2;
     const int nr = n2 / S, row0 = sl * nr;
     if (!rs_staged) {
-        for (int i = gt; i < RC * n2; i += NTG) {
-            const int rc = i / n2, k = i - rc * n2;
-            sm[i] = rc < nrc ? lk.less_received(__ldcg(rhs + (size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + k),
-                                                it.cell, it.local, it.K_inst, it.level, rc, k)
-                             : T(0);
-        }
+        if (RC * n2 <= NTG || RC == 1 || (RC == 2 && sizeof(T) == 8))
+            collect_rhs<T, NTG, RC, 1>(lk, rhs, it, r0, nrc, n2, rstride, sm, gt);
+        else
+            collect_rhs<T, NTG, RC, RC >= 4 ? 4 : 2>(lk, rhs, it, r0, nrc, n2, rstride, sm, gt);
     }
     if (!wait_copies()) return false;  // a group barrier: rs complete too
     const int KS = smem_matvec<T, NTG, RC>(As + row0, n2, nr, n2, rs, n2, part, gt);
@@ -2473,11 +2604,8 @@ __device__ __forceinline__ bool ring_bwd_unit(const T *mB, const T *mC, const Bc
     // y of this thread's first row: long there, requested before the waits
     T y0 = T(0);
     bool have_y0 = false;
-    if (gt < nrc * nr) have_y0 = packet_try<T>(lk.pk.y, lk.y_at(it.cell, gt / nr, row0 + gt % nr), lk.e, y0);
-    for (int idx = gt; idx < RC * N; idx += NTG) {
-        const int rc = idx / N, k = idx - rc * N;
-        gv[idx] = rc < nrc ? lk.inflow(it, rc, k) : T(0);
-    }
+    if (gt < nrc * nr) have_y0 = lk.y_try(it.cell, gt / nr, row0 + gt % nr, y0);
+    collect_inflow<T, NTG, RC, RC <= 2 ? 1 : 2>(lk, it, nrc, N, gv, gt);
     if (!wait_copies()) return false;
     coupling_products<T, NTG, RC>(mB, gv, mC, gv + h2, h2, N, gt,
                                   [&](int side, int rc, int p, T v) { g[rc * N + side * h2 + p] = v; });
@@ -2486,14 +2614,14 @@ __device__ __forceinline__ bool ring_bwd_unit(const T *mB, const T *mC, const Bc
     gbar_sync(gr.bar, NTG);
     const int KS = smem_matvec<T, NTG, RC>(As + row0, n2, nr, N, g, N, part, gt);
     gbar_sync(gr.bar, NTG);
-    for (int idx = gt; idx < nrc * nr; idx += NTG) {
-        const int rc = idx / nr, row = idx - rc * nr;
+    auto finish = [&](int rc, int row, T y) {
         T sacc = T(0);
         for (int q = 0; q < KS; ++q) sacc += part[(q * RC + rc) * nr + row];
-        const T y = idx == gt && have_y0 ? y0 : lk.get(lk.pk.y, lk.y_at(it.cell, rc, row0 + row));
         lk.put_u(it.cell, rc, row0 + row, y - sacc);
         Y[(size_t)(r0 + rc) * rstride + (size_t)it.cell * n2 + row0 + row] = y - sacc;
-    }
+    };
+    if (have_y0) finish(gt / nr, gt % nr, y0);
+    collect_y<T, NTG, RC <= 2 ? 1 : 2>(lk, it.cell, nrc, nr, row0, have_y0 ? gt + NTG : gt, finish);
     return true;
 }
 
@@ -2503,9 +2631,13 @@ template <typename T, int NTG, typename WaitCopies>
 __device__ __forceinline__ bool ring_gather_unit(int j, const LevelTable &lv, const T *rhs, int N,
                                                  const UnitLinks<T, 1> &lk, const Group &gr, WaitCopies wait_copies) {
     const int n2 = 2 * N, cl = lv.coarse_level, a = j << cl;
-    for (int k = gr.gt; k < n2; k += NTG)
-        packet_put<T>(lk.pk.rc, (size_t)j * n2 + k,
-                      lk.less_received(__ldcg(rhs + (size_t)a * n2 + k), a, a, lv.coarse_K, cl, 0, k), lk.e);
+    for (int k = gr.gt; k < n2; k += NTG) {
+        T v[1] = {__ldcg(rhs + (size_t)a * n2 + k)};
+        const bool on[1] = {true};
+        const int rc[1] = {0}, row[1] = {k};
+        lk.less_received(v, on, a, a, lv.coarse_K, cl, rc, row);
+        packet_put<T>(lk.pk.rc, (size_t)j * n2 + k, v[0], lk.e);
+    }
     return wait_copies();  // (an empty fill: keeps the stage's phases in step)
 }
 

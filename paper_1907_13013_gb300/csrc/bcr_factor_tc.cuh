@@ -461,8 +461,8 @@ __global__ void __launch_bounds__(tcf::kThreads, 4) k_bcr_factor_tc(float *__res
         for (int lp = 0; lp < it.level; ++lp)
             want += (it.local >= (1 << lp)) + (it.local + (1 << lp) < it.K_inst);
         if (want) {
-            fs.wait0 = cnt + it.cell;
-            fs.want0 = want;
+            fs.wait = cnt + it.cell;
+            fs.want = want;
         }
         flow_wait(&fs);
         const bool has_r = it.right >= 0, has_l = it.left >= 0;

@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(256) k_bcr_coupling_split(const float *__restr
 // A unit as the driver hands it to the workers (id < 0: no more units).
 struct Unit {
     int id, m, ch, bwd;
-    int cell, left, right, s_cell, s_left, s_right, local, K_inst, level;
-    int pad[3];
+    int cell, left, right, s_left, s_right, local, K_inst, level;
+    int pad[4];
 };
 static_assert(sizeof(Unit) == 64, "one slot of the unit ring");
 
@@ -359,7 +359,6 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_bcr_solve_tc(
                 u.cell = it.cell;
                 u.left = it.left;
                 u.right = it.right;
-                u.s_cell = it.s_cell;
                 u.s_left = it.s_left;
                 u.s_right = it.s_right;
                 u.local = it.local;

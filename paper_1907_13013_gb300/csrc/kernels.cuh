@@ -1782,19 +1782,19 @@ __device__ __forceinline__ void coupling_products(const T *__restrict__ M0, cons
     }
 }
 
-// Dataflow synchronisation of the factorization's items and the tensor-core solve's
-// units: one waits until the counters it depends on reach their targets (thread 0 polls
-// with acquire loads, at most `limit` times, then records *err = 1 and goes on), and after
-// its writes (block barrier, then thread 0 fences) bumps the counters of those that depend
-// on it. NULL pointers are absent waits / signals.
+// Dataflow synchronisation of the factorization's items: one waits until the counter of
+// the updates it needs reaches its target (thread 0 polls with acquire loads, at most
+// `limit` times, then records *err = 1 and goes on), and after its writes (block barrier,
+// then thread 0 fences) bumps the counters of its two neighbours. NULL pointers are absent
+// waits / signals.
 // The limit is the context's: err[1] holds it (err[0] is the error flag), so a host
 // can shorten it to make a wait run out on purpose (tests of the error path).
 constexpr unsigned kFlowSpinLimit = 1u << 25;  // default: x >= 32 ns, about a second
 __device__ __forceinline__ unsigned flow_spin_limit(const int *err) { return (unsigned)__ldg(err + 1); }
 struct FlowSync {
-    const int *wait0, *wait1;
-    int want0, want1;
-    int *sig0, *sig1, *sig2;
+    const int *wait;
+    int want;
+    int *sig0, *sig1;
     int *err;
     unsigned limit;
 };
@@ -2102,20 +2102,14 @@ __device__ __forceinline__ void collect_y(const Links &lk, int cell, int nrc, in
 
 __device__ __forceinline__ void flow_wait(const FlowSync *fs) {
     if (!fs) return;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int *c = k ? fs->wait1 : fs->wait0;
-            const int want = k ? fs->want1 : fs->want0;
-            if (!c) continue;
-            unsigned spins = 0;
-            while (ld_acquire_gpu(c) < want) {  // busy first, then with short sleeps
-                if (++spins > fs->limit) {
-                    atomicExch(fs->err, 1);
-                    break;
-                }
-                if (spins > 256) __nanosleep(32);
+    if (threadIdx.x == 0 && fs->wait) {
+        unsigned spins = 0;
+        while (ld_acquire_gpu(fs->wait) < fs->want) {  // busy first, then with short sleeps
+            if (++spins > fs->limit) {
+                atomicExch(fs->err, 1);
+                break;
             }
+            if (spins > 256) __nanosleep(32);
         }
     }
     __syncthreads();
@@ -2131,7 +2125,6 @@ __device__ __forceinline__ void flow_signal(const FlowSync *fs) {
         __threadfence();
         if (fs->sig0) atomicAdd(fs->sig0, 1);
         if (fs->sig1) atomicAdd(fs->sig1, 1);
-        if (fs->sig2) atomicAdd(fs->sig2, 1);
     }
 }
 
@@ -2163,8 +2156,8 @@ __global__ void __launch_bounds__(512, 1) k_bcr_factor_flow(T *__restrict__ A, c
         for (int lp = 0; lp < it.level; ++lp)
             want += (it.local >= (1 << lp)) + (it.local + (1 << lp) < it.K_inst);
         if (want) {
-            fs.wait0 = cnt + it.cell;
-            fs.want0 = want;
+            fs.wait = cnt + it.cell;
+            fs.want = want;
         }
         flow_wait(&fs);
         T *Ag = A + (size_t)it.cell * N2 * N2;

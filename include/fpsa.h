@@ -288,7 +288,12 @@ typedef struct {
                                        its creation, or later for a GMRES basis beside
                                        them, the context goes without and 2 is FPSA_ENOTSUP
                                        too); 0 = tensor cores where they apply, else the
-                                       dataflow solve. Solutions differ by rounding only.
+                                       dataflow solve. Solutions differ by rounding only: the
+                                       products of 2 hold factors, backward operators
+                                       (A^{-1} times the couplings) and vectors in two BF16
+                                       parts each, about 16 bits, the forward couplings in
+                                       three (24 bits); every solve of either engine sums in
+                                       a fixed order and gives the same bits each time.
                                        The dataflow solve keeps 16 (MIXED) or 32 bytes per
                                        angular unknown; without room for those it runs
                                        level by level, more slowly, to the same solution */

@@ -21,6 +21,11 @@
 // already split and in the K-major core-matrix layout, one bulk copy (the TMA engine) per
 // chunk: A^{-1} and P by (slice, 32 columns), 16 KB (k_bcr_factor_split,
 // k_bcr_backward_split), a coupling block by 16 columns (k_bcr_coupling_split).
+// With P in two parts a solve is as far from the exact solution of the stored factors as with
+// the couplings multiplied by u in 24 bits first and the result split before A^{-1}: emulated
+// over ten slabs (N = 64 to 256, HG 0.8 to 0.99, 50 to 1000 per cm, cells of 1/200 to 1/3000
+// cm), three draws each, relative 2-norms of 2.3e-6 to 5.1e-6, 0.96 to 1.01 times the other
+// form's and 0.99 of them on average.
 //
 // A CTA is four worker warps, a copying and an issuing thread that share a ring of kStages
 // stages, a chunk of the operand A and one of the operand B each. The copying thread takes

@@ -2016,7 +2016,9 @@ struct LevelLinks {
 // a unit of eight right-hand sides were longer than its product (1500 cells at N = 128, FP32,
 // eight right-hand sides: 786 us a solve, now 568; 100 cells at N = 256, one: 312, now 235).
 // NE is small where the registers also hold the first columns of A^{-1}: beyond that they
-// spill (500 cells at N = 128, four right-hand sides: 131 us, 235 with four elements).
+// spill (500 cells at N = 128, four right-hand sides: 131 us, 235 with four elements). Staged
+// blocks have registers to spare where one of them fills an SM (600 cells at N = 64, eight
+// right-hand sides: 145 us with counters, 224 one element at a time, 180 four, 138 eight).
 // rs[rc][k] (row stride n2, its own right-hand sides in place) less what the cell has received
 template <typename T, int NT, int NE, typename Links>
 __device__ __forceinline__ void receive_pushes(const Links &lk, const BcrItem &it, int nrc, int N, T *rs, int tid) {
@@ -2547,7 +2549,7 @@ struct Group {
 // Forward / backward unit on a compute group, its A^{-1} slice in As and its coupling
 // blocks (mB, mC: shared-memory copies, or global memory when not staged; NULL where
 // absent) in flight; wait_copies() returns (true) once they have landed.
-template <typename T, int NTG, int RC, typename WaitCopies>
+template <typename T, int NTG, int RC, int BPSM, typename WaitCopies>
 __device__ __forceinline__ bool ring_fwd_unit(const T *mB, const T *mC, const BcrItem &it, int r0, int nrc, int sl,
                                               int S, const T *rhs, T *Y, int N, int sumK, T *sm, const T *As,
                                               const T *rs_staged, const UnitLinks<T, RC> &lk, const Group &gr,
@@ -2560,6 +2562,8 @@ __device__ __forceinline__ bool ring_fwd_unit(const T *mB, const T *mC, const Bc
     if (!rs_staged) {
         if (RC * n2 <= NTG || RC == 1 || (RC == 2 && sizeof(T) == 8))
             collect_rhs<T, NTG, RC, 1>(lk, rhs, it, r0, nrc, n2, rstride, sm, gt);
+        else if (RC == 8 && BPSM == 1 && RC * n2 > 4 * NTG)  // (two blocks per SM: fewer elements, and registers)
+            collect_rhs<T, NTG, RC, RC == 8 && BPSM == 1 ? 8 : 1>(lk, rhs, it, r0, nrc, n2, rstride, sm, gt);
         else
             collect_rhs<T, NTG, RC, RC >= 4 ? 4 : 2>(lk, rhs, it, r0, nrc, n2, rstride, sm, gt);
     }
@@ -2903,7 +2907,7 @@ __global__ void __launch_bounds__(NT, BPSM) k_bcr_solve_flow_s(const T *__restri
             const int r0 = cur.ch * RC, nrc = min(RC, R - r0);
             lk.cell0 = (size_t)cur.ch * sumK;
             if (!bwd)
-                ok = ring_fwd_unit<T, NTG, RC>(mB, mC, it, r0, nrc, cur.sl, cur.S, rhs, Y, N, sumK, smg, As,
+                ok = ring_fwd_unit<T, NTG, RC, BPSM>(mB, mC, it, r0, nrc, cur.sl, cur.S, rhs, Y, N, sumK, smg, As,
                                                rhs_staged(cur, k) ? stage_rhs(st) : (const T *)nullptr, lk, gr,
                                                wait_copies);
             else

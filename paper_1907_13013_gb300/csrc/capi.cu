@@ -1616,8 +1616,8 @@ int gmres_alloc_all(fpsa_ctx *ctx, int m) {
         CK(cudaMemcpy(ctx->gm_seg_begin, sb.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->gm_seg_end, se.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
         CK(cudaStreamSynchronize(cudaStreamLegacy));  // (as at the end of fpsa_create)
-        // small chunks where the large ones give most SMs none
-        ctx->gm_small = (maxlen + kDotChunk - 1) / kDotChunk * nsys < ctx->n_sm;
+        ctx->gm_small = small_dot_chunks((maxlen + kDotChunkSmall - 1) / kDotChunkSmall * nsys,
+                                         ctx->precision == FPSA_PRECISION_FP64, ctx->n_sm);
         const int chunk = ctx->gm_small ? kDotChunkSmall : kDotChunk;
         ctx->gm_nchunks = (int)((maxlen + chunk - 1) / chunk);
     }

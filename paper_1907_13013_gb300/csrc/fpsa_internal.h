@@ -37,6 +37,15 @@ inline int col_tile(int N, int sumK, int R, int n_sm) {
     return 0;
 }
 
+// Whether the GMRES vector kernels take small chunks (kDotChunkSmall elements a block) instead
+// of large ones (kDotChunk): where the small ones are few. A block's fixed work, the meeting
+// of its threads' sums for every four vectors, is paid per chunk, and in FP32 a small chunk is
+// one 16-byte word a thread. Vector kernels of 40 Krylov steps (FP32, two restarts) and 20
+// (FP64), us, large / small chunks, by the number of small blocks:
+//   FP32  125: 3407 / 2960   300: 3472 / 3443   600: 3727 / 4686   1125: 4051 / 7091
+//   FP64  125: 4069 / 1740   300: 4174 / 2108   600: 4439 / 3099    900: 4922 / 4099   1125: 5093 / 5234
+inline bool small_dot_chunks(long long small_blocks, bool fp64, int n_sm) { return small_blocks <= (fp64 ? 6ll : 2ll) * n_sm; }
+
 // One cell eliminated at one block-cyclic-reduction level (or an instance root).
 // Cell ids are global (concatenated over instances); -1 = absent.
 // Coupling slots index the per-level N/2 x N/2 coupling blocks B (to the left

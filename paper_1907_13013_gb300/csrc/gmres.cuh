@@ -68,9 +68,10 @@ __global__ void k_moments_axpy(const T *__restrict__ psi, const T *__restrict__ 
 // GMRES-IR) in FP32 over a thread's products (at most 32), then in FP64 across threads and
 // chunks (the FP64 rate of this GPU is far below what one FMA per loaded element
 // needs). The sum order is fixed, so results are bitwise reproducible.
-// CH: kDotChunk where the chunks fill the chip (the vectors then stream at memory rate);
-// kDotChunkSmall below that, where a chunk's latency counts: 100 cells at N = 32 are one
-// chunk of the large size, 19 us a dot and 18 us a combination on one SM.
+// CH: kDotChunk where there are many chunks (the vectors then stream at memory rate);
+// kDotChunkSmall where there are few (small_dot_chunks) and a chunk's latency counts: 100
+// cells at N = 32 are one chunk of the large size, 19 us a dot and 18 us a combination on
+// one SM.
 constexpr int kDotChunk = 8192, kDotChunkSmall = 1024;
 constexpr int kDotThreads = 256;
 template <typename T, int CH>

@@ -871,10 +871,10 @@ void plan_solve_shape(fpsa_ctx *ctx) {
     }
 }
 
-// The packets of the dataflow BCR solve (kernels.cuh), in the path's element type. FPSA_ENOMEM
-// leaves the context without (pk.push NULL).
+// The packets of the dataflow BCR solve (kernels.cuh), in the path's element type, behind the
+// word that numbers its solves. FPSA_ENOMEM leaves the context without (pk.push NULL). Cleared
+// on the legacy stream, which the caller waits for (wait_setup).
 void free_packets(fpsa_ctx *ctx) {
-    dfree(ctx, ctx->pk.push);
     dfree(ctx, ctx->pk.epoch);
     ctx->pk = Packets{};
 }
@@ -884,20 +884,23 @@ int alloc_packets(fpsa_ctx *ctx) {
     const int RC = solve_rc(g.R), nchunk = (g.R + RC - 1) / RC;
     const size_t words = e ? packet_words<double>() : packet_words<float>();
     const size_t n = (size_t)nchunk * g.sumK * RC * g.N * words, m = (size_t)ctx->lvt[e].coarse_m * 2 * g.N * words;
+    const size_t all = 2 + 4 * n + m;  // (two words: the packets stay 16-byte aligned)
     Packets &pk = ctx->pk;
-    if (dalloc(ctx, &pk.push, 4 * n + m) != cudaSuccess || dalloc(ctx, &pk.epoch, 1) != cudaSuccess) {
-        free_packets(ctx);
+    if (dalloc(ctx, &pk.epoch, all) != cudaSuccess)
         return fail(ctx, FPSA_ENOMEM, "no device memory for the dataflow BCR solve's packets");
-    }
-    // on the context's stream: one that does not wait for the legacy stream would let the next
-    // solve start before its packets are cleared (this also runs at a change of engine)
-    CK(cudaMemsetAsync(pk.push, 0, (4 * n + m) * sizeof(*pk.push), ctx->stream));
+    CK(cudaMemsetAsync(pk.epoch, 0, all * sizeof(*pk.epoch), cudaStreamLegacy));
+    pk.push = pk.epoch + 2;
     pk.y = pk.push + n;
     pk.u = pk.y + 2 * n;
     pk.rc = pk.u + n;
-    const unsigned long long first = 1ull << 32;
-    CK(cudaMemcpyAsync(pk.epoch, &first, sizeof(first), cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    return FPSA_OK;
+}
+
+// Set-up copies and clears go over the legacy stream, for which the context's own (it may be a
+// non-blocking one) does not wait; and a copy from pageable memory can return before its last
+// part has arrived.
+int wait_setup(fpsa_ctx *ctx) {
+    CK(cudaStreamSynchronize(cudaStreamLegacy));
     return FPSA_OK;
 }
 
@@ -1615,7 +1618,8 @@ int gmres_alloc_all(fpsa_ctx *ctx, int m) {
             }
         CK(cudaMemcpy(ctx->gm_seg_begin, sb.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->gm_seg_end, se.data(), nsys * sizeof(long long), cudaMemcpyHostToDevice));
-        CK(cudaStreamSynchronize(cudaStreamLegacy));  // (as at the end of fpsa_create)
+        const int rw = wait_setup(ctx);
+        if (rw) return rw;
         ctx->gm_small = small_dot_chunks((maxlen + kDotChunkSmall - 1) / kDotChunkSmall * nsys,
                                          ctx->precision == FPSA_PRECISION_FP64, ctx->n_sm);
         const int chunk = ctx->gm_small ? kDotChunkSmall : kDotChunk;
@@ -1640,7 +1644,8 @@ int gmres_alloc(fpsa_ctx *ctx, int m) {
         free_tcs(ctx);
         rc = gmres_alloc_all(ctx, m);
         if (rc == FPSA_OK && !ctx->pk.push) {
-            const int rp = alloc_packets(ctx);
+            int rp = alloc_packets(ctx);
+            if (!rp) rp = wait_setup(ctx);
             if (rp && rp != FPSA_ENOMEM) return rp;
         }
     }
@@ -2305,11 +2310,7 @@ int fpsa_create(fpsa_ctx **out, const fpsa_desc *d) {
         if (!r2 && mixed) r2 = setup_tc(ctx);
         if (!r2) r2 = alloc_solve_storage(ctx);
         if (r2) return r2;
-        // the tables and cleared counters above went over the legacy stream, for which the
-        // context's own (it may be a non-blocking one) does not wait: a copy from pageable
-        // memory can return before its last part has arrived
-        CK(cudaStreamSynchronize(cudaStreamLegacy));
-        return FPSA_OK;
+        return wait_setup(ctx);
     }();
     if (rc != FPSA_OK) {
         g_create_error = ctx->err;
@@ -2722,8 +2723,10 @@ int fpsa_set_tuning(fpsa_ctx *ctx, const fpsa_tuning *t) {
                     "16 right-hand sides and room on the device for its copies of the factors");
     if (r.solve_engine == 1 && !ctx->pk.push) {  // a tensor-core context's first dataflow solve
         CK(cudaSetDevice(ctx->device));
-        const int rc = alloc_packets(ctx);
+        int rc = alloc_packets(ctx);
         if (rc && rc != FPSA_ENOMEM) return rc;  // (without packets: level by level)
+        if (!rc) rc = wait_setup(ctx);
+        if (rc && rc != FPSA_ENOMEM) return rc;
     }
     // the segment maps were allocated for the smallest cells-per-thread (most segments)
     const int cmin = sweep_cells_per_thread(ctx->geo, ctx->n_sm);

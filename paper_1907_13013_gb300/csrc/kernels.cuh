@@ -1821,11 +1821,11 @@ __device__ __forceinline__ int ld_acquire_gpu(const int *p) {
 //   y    [ch][cell][rc][2N]         A^{-1} r, for the cell's own backward unit
 //   u    [ch][cell][rc][N]          the outflow rows of the solution, [L-, R+]
 //   rc   [coarse cell][2N]          complete right-hand sides of the coarse step
-// *epoch holds the number of the next solve to run (high half; never 0, the words' first
-// content) and counts the blocks that have taken it (low half). Both in one word, so that a
-// block takes the number and is counted by one atomic operation: with a read and a count
-// apart, relaxed accesses of two words, the last block could have moved the number on before
-// another one's read of it was performed.
+// *epoch holds the number of the solves run (high half) and counts the blocks that have taken
+// the next one's (low half), which is one more; 0, the words' first content, is left out. Both
+// in one word, so that a block takes the number and is counted by one atomic operation: with a
+// read and a count apart, relaxed accesses of two words, the last block could have moved the
+// number on before another one's read of it was performed.
 // ---------------------------------------------------------------------------
 struct Packets {
     unsigned long long *push, *y, *u, *rc;
@@ -1837,8 +1837,8 @@ __host__ __device__ constexpr int packet_words() { return (int)sizeof(T) / 4; }
 // One thread per block: this solve's number; the last block moves it on for the next launch.
 __device__ __forceinline__ unsigned take_epoch(unsigned long long *epoch) {
     const unsigned long long w = atomicAdd(epoch, 1ull);
-    const unsigned e = (unsigned)(w >> 32);
-    if ((unsigned)w == gridDim.x - 1) atomicExch(epoch, (unsigned long long)(e + 1u ? e + 1u : 1u) << 32);
+    const unsigned e = (unsigned)(w >> 32) + 1u;
+    if ((unsigned)w == gridDim.x - 1) atomicExch(epoch, (unsigned long long)(e + 1u ? e : 0u) << 32);
     return e;
 }
 
